@@ -911,6 +911,52 @@ __global__ void find_rep_two_kernel(const TwoParams P, const DevIndex I, const u
   }
 }
 
+// The configuration of every slot of the coset-arithmetic product (pair.cu), its basis index
+// and its weight: the two-level search once per slot, when a basis is built.
+template <int NSUB, bool kE2>
+__global__ void __launch_bounds__(256) pair_slots_kernel(const TwoParams P, const DevIndex I,
+                                                         const PairSlots Q, int n_up) {
+  extern __shared__ __align__(16) unsigned char sm[];
+  const Sm2 S = stage_two(P, sm, false, kE2);
+  const int n = P.n;
+  const uint32_t bmask = (1u << n) - 1u;
+  const int u0 = Q.hb[2 * Q.up_half], u1 = Q.hb[2 * Q.up_half + 1];
+  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < Q.n_slots;
+       p += (int64_t)gridDim.x * blockDim.x) {
+    uint32_t lo = 0, hi = Q.n_low - 1;
+    while (lo < hi) {   // the last class that starts at or before p (empty ones share a start)
+      const uint32_t mid = (lo + hi + 1) >> 1;
+      if (__ldg(Q.start + mid) <= (uint32_t)p) lo = mid; else hi = mid - 1;
+    }
+    const uint32_t r = (uint32_t)p - __ldg(Q.start + lo);
+    const uint32_t a = __ldg(Q.low + lo), b = __ldg(Q.up + __ldg(Q.first_up + lo) + r / Q.K);
+    const int g = __ldg(Q.kel + r % Q.K);
+    const uint32_t i0 = act(P, u0, u1 < 0 ? b : b >> n, g);
+    const uint32_t i1 = u1 < 0 ? 0u : act(P, u1, b & bmask, g);
+    const int d0 = S.dest[g * NSUB + u0], d1 = u1 < 0 ? -1 : S.dest[g * NSUB + u1];
+    uint32_t sub[NSUB];
+    int pc = 0;
+#pragma unroll
+    for (int X = 0; X < NSUB; X++) {
+      sub[X] = X == d0 ? i0 : X == d1 ? i1 : X == Q.hb[0] ? (u1 < 0 ? a : a >> n) : (a & bmask);
+      pc += __popc(sub[X]);
+    }
+    uint32_t idx = 0xFFFFFFFFu;
+    uint16_t meta = 0;
+    if (pc == n_up) {
+      const Rep2 R = find_rep_blocks<NSUB, kE2>(S, P, sub);
+      const int64_t j = R.mixed ? -1 : lookup_index(I, ((uint64_t)R.minrep << P.L) | R.low);
+      if (j >= 0) {
+        idx = (uint32_t)j;
+        meta = (uint16_t)(R.ph + P.denom * (int)__ldg(Q.tcode + R.t));
+        if (R.t > 1) *Q.any_weight = 1u;   // every writer stores the same value
+      }
+    }
+    Q.idx[p] = idx;
+    Q.meta[p] = meta;
+  }
+}
+
 size_t a16(size_t x) { return (x + 15) & ~(size_t)15; }
 
 // Parameters and shared-memory layout; e2 = stage the level-2 tables in shared memory.
@@ -1137,6 +1183,32 @@ int ed_launch_find_rep_two(const ed_basis *B, const uint64_t *states, int64_t n,
     L2CASE(3, 1)
     L2CASE(4, 1)
 #undef L2CASE
+  }
+  ED_CK(cudaGetLastError());
+  return ED_OK;
+}
+
+int ed_launch_pair_slots(const ed_basis *B, const PairSlots &Q, cudaStream_t st) {
+  TwoParams P;
+  bool e2 = true;
+  int rc = make_params(B, nullptr, nullptr, e2, P);
+  if (rc == ED_ERR_UNSUPPORTED) { e2 = false; rc = make_params(B, nullptr, nullptr, false, P); }
+  if (rc) return rc;
+  const int grid = (int)std::min<int64_t>(((int64_t)Q.n_slots + 255) / 256, (int64_t)B->sm_count * 4);
+  switch (B->nsub * 2 + (e2 ? 1 : 0)) {
+#define PSCASE(K, C)                                                                           \
+  case K * 2 + C: {                                                                            \
+    auto k = pair_slots_kernel<K, C>;                                                          \
+    ED_CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, P.smem_bytes)); \
+    k<<<grid, 256, P.smem_bytes, st>>>(P, B->I, Q, B->n_up);                                   \
+    break;                                                                                     \
+  }
+    PSCASE(2, 0)
+    PSCASE(4, 0)
+    PSCASE(2, 1)
+    PSCASE(4, 1)
+#undef PSCASE
+    default: return ED_ERR_UNSUPPORTED;
   }
   ED_CK(cudaGetLastError());
   return ED_OK;

@@ -424,6 +424,7 @@ int build_tables(ed_basis *B, cudaStream_t st, const ed_basis *share) {
 }
 
 void free_all(ed_basis *B) {
+  ed_free_pair(B);
   void *ptrs[] = {B->d_rep, B->d_sym_off, B->d_sym_list, B->d_action, B->d_dest, B->d_phase,
                   B->d_src, B->d_e1, B->d_rid, B->d_e2, B->d_off2, B->d_list2, B->d_bond_pad,
                   B->d_bond_blk, B->d_nib, B->d_pbit, B->d_flip,
@@ -561,6 +562,7 @@ extern "C" int ed_build_basis(const ed_lattice *L, const ed_group *G, const ed_i
   if ((rc = build_tables(B, st, opts ? opts->share_tables : nullptr))) { free_all(B); delete B; return rc; }
   const int bucket = (opts && opts->bucket_target > 0) ? opts->bucket_target : 1;
   if ((rc = ed_build_device(B, st, bucket))) { free_all(B); delete B; return rc; }
+  if ((rc = ed_build_pair(B, st))) { free_all(B); delete B; return rc; }
   B->n_partial = ED_MAXCLS * B->sm_count * 8;   // per-class partials of the widest grid
   if (cudaMalloc(&B->d_partial, (size_t)B->n_partial * 8) != cudaSuccess ||
       cudaMallocHost(&B->h_partial, (size_t)B->n_partial * 8) != cudaSuccess) {

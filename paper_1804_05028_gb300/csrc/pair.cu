@@ -1,0 +1,903 @@
+// pair.cu -- the product y = H x by coset arithmetic on the two halves of a configuration.
+//
+// Sublattice coding (Sec. III of arXiv:1804.05028) with two sublattices: when the blocks of
+// the split fall into two halves A and B that every group element carries onto themselves or
+// onto each other (the checkerboard halves of the four-block square clusters, the even and
+// odd blocks of a chain, or simply the two blocks of a two-block split), a configuration is
+// the pair (a, b) of its half patterns, and the orbit of a half pattern a is given by
+//     g_a a = R(class(a))          (class representative, placed on half A)
+// with g_a in H, the elements that keep the halves, and for b with g_b in the elements that
+// carry half B onto half A.  Both come from one table per half, 2^m entries of 32 bits
+// (m = N/2), small enough to stay in L2.
+//
+// Let the classes be ordered.  If class(a) <= class(b), h = g_a brings (a, b) to
+//     (R(class a), k R(class b)),   k = g_a g_b^-1,
+// and otherwise h = g_b to (R(class b), k R(class a)), k = g_b g_a^-1.  So the orbit is named
+// by (lower class, upper class, k): no candidate scan, no comparison of images, and no search
+// of the basis.  k is one lookup in the group's multiplication table (at most 2 |H|^2 bytes,
+// shared memory), and the triple has the position
+//     slot = off[lower] + K * upper + k
+// in a vector xs that holds x in slot order, K the number of elements between the halves.
+// The product first expands x into xs (one streaming pass over the slots: xs = chi(h2)
+// sqrt(|Stab_j|) x_j, j the basis index and h2 the element that carry the slot's
+// configuration to its representative, tabulated once per basis), then every row sums
+// chi(h) xs[slot] over its antiparallel bonds.
+//
+// Several slots may hold the same orbit: a lower class with a nontrivial stabiliser lists
+// every image of the upper pattern, an upper class with one lists the same pattern under
+// several k, and equal classes list both orders.  All of them receive the orbit's value, so
+// any of the equivalent choices of h gives the right term and no case is treated apart.
+// Slots whose configuration has another S^z or a vanishing projection hold 0.
+//
+// What a term costs: two half-table loads (L1/L2), one byte and one word from shared memory,
+// one gather of xs, and about 40 instructions; the two-level search it replaces executed
+// about 600 and 10 dependent loads (62.7 ms per product on the 3.2e7-state 6x6 sector, issue
+// bound).  One lane owns one row: without data-dependent searches the lanes of a warp differ
+// only in their number of antiparallel bonds.  Every y_i is written once, no atomics, fixed
+// summation order.
+#include "sced_internal.cuh"
+#include "dfloat.cuh"
+#include <algorithm>
+#include <cmath>
+#include <new>
+#include <type_traits>
+#include <vector>
+
+namespace {
+
+template <typename V> struct Pv;
+template <> struct Pv<double> { using A = double; static constexpr bool cplx = false; };
+template <> struct Pv<float> { using A = float; static constexpr bool cplx = false; };
+template <> struct Pv<double2> { using A = double; static constexpr bool cplx = true; };
+template <> struct Pv<float2> { using A = float; static constexpr bool cplx = true; };
+
+// half-table entry: class << 11 | special << 10 | sign << 9 | flip << 8 | element
+//   special: the class has a nontrivial stabiliser; sign: chi = -1 (real sectors);
+//   flip: the element also reverses every spin; element: its number in H (times the fixed
+//   swap for half B)
+constexpr uint32_t kClassShift = 11;
+constexpr uint32_t kSpecial = 1u << 10;
+constexpr uint32_t kSignBit = 9;
+constexpr uint32_t kFlip = 1u << 8;
+constexpr uint32_t kElem = 255u;
+
+struct PairParams {
+  int n_classes;
+  int cls_word[ED_MAXCLS + 1];
+  int nb_cls[ED_MAXCLS];
+  double jh[ED_MAXCLS], jzq[ED_MAXCLS];
+  // halves of a state: (((s >> sh[0]) & bmask_hi) << n) | ((s >> sh[1]) & bmask)
+  int n;
+  int shA0, shA1, shB0, shB1;
+  uint32_t bmask_hi, bmask;
+  const uint32_t *ta, *tb;       // half tables
+  const uint32_t *off;           // [n_cls] slot offset of the lower class
+  uint32_t n_cls, K, h0, sel_off;
+  const uint8_t *mult;           // k of (lower element, upper element)
+  uint32_t mult_bytes;
+  const uint2 *bond;             // per padded bond: bits flipped in A and in B
+  const uint32_t *nib;
+  uint32_t n_nib;
+  const double *rsqrt_tab;
+  uint32_t n_sq;
+  const double *chi;             // complex sectors: (cos, sin) of chi per half and element
+  uint32_t n_chi;
+  const uint64_t *basis;
+  const uint16_t *stab;
+  const void *x, *xs;
+  const float *xslo;             // fp32 real vectors: remainders of xs (null: all zero)
+  void *y;
+  void *ylo;
+  int64_t r0, r1;
+  double *partial;
+  uint32_t off_off, off_mult, off_bond, off_nib, off_rs, off_chi, off_mask, smem_bytes;
+};
+
+constexpr int kThreads = 512;
+constexpr int kMinBlocks = 2;
+
+template <typename T>
+__device__ __forceinline__ void cpy(unsigned char *sm, uint32_t off, const T *g, uint32_t n) {
+  T *d = reinterpret_cast<T *>(sm + off);
+  for (uint32_t k = threadIdx.x; k < n; k += blockDim.x) d[k] = g[k];
+}
+
+template <typename V>
+__device__ __forceinline__ V ld_slot(const V *p) {
+  if constexpr (std::is_same<V, float>::value) {
+    float f;
+    asm volatile("ld.global.nc.L1::no_allocate.f32 %0, [%1];" : "=f"(f) : "l"(p));
+    return f;
+  } else if constexpr (std::is_same<V, double>::value) {
+    double f;
+    asm volatile("ld.global.nc.L1::no_allocate.f64 %0, [%1];" : "=d"(f) : "l"(p));
+    return f;
+  } else if constexpr (std::is_same<V, float2>::value) {
+    float2 f;
+    asm volatile("ld.global.nc.L1::no_allocate.v2.f32 {%0,%1}, [%2];" : "=f"(f.x), "=f"(f.y) : "l"(p));
+    return f;
+  } else {
+    double2 f;
+    asm volatile("ld.global.nc.L1::no_allocate.v2.f64 {%0,%1}, [%2];" : "=d"(f.x), "=d"(f.y) : "l"(p));
+    return f;
+  }
+}
+
+// one row's running sum over a coupling class: fp64, or a double-float pair for fp32
+// vectors (the fp64 pipe of this GPU issues at a small fraction of the fp32 rate)
+template <typename V> struct Acc;
+template <> struct Acc<double> {
+  double s = 0;
+  __device__ __forceinline__ void add(double v, uint32_t neg) { s += neg ? -v : v; }
+  __device__ __forceinline__ double re() const { return s; }
+  __device__ __forceinline__ double im() const { return 0; }
+};
+template <> struct Acc<float> {
+  float h = 0, l = 0;
+  __device__ __forceinline__ void add(float v, uint32_t neg) {
+    df_add(h, l, __uint_as_float(__float_as_uint(v) ^ (neg << 31)));
+  }
+  __device__ __forceinline__ void add_lo(float v, uint32_t neg) {
+    l = __fadd_rn(l, __uint_as_float(__float_as_uint(v) ^ (neg << 31)));
+  }
+  __device__ __forceinline__ double re() const { return df_value(h, l); }
+  __device__ __forceinline__ double im() const { return 0; }
+};
+template <> struct Acc<double2> {
+  double r = 0, i = 0;
+  __device__ __forceinline__ void add(double2 v, uint32_t neg) {
+    r += neg ? -v.x : v.x;
+    i += neg ? -v.y : v.y;
+  }
+  __device__ __forceinline__ void add(double2 v, double2 c) {
+    r = fma(c.x, v.x, fma(-c.y, v.y, r));
+    i = fma(c.x, v.y, fma(c.y, v.x, i));
+  }
+  __device__ __forceinline__ double re() const { return r; }
+  __device__ __forceinline__ double im() const { return i; }
+};
+template <> struct Acc<float2> {
+  float rh = 0, rl = 0, ih = 0, il = 0;
+  __device__ __forceinline__ void add(float2 v, uint32_t neg) {
+    df_add(rh, rl, __uint_as_float(__float_as_uint(v.x) ^ (neg << 31)));
+    df_add(ih, il, __uint_as_float(__float_as_uint(v.y) ^ (neg << 31)));
+  }
+  // chi v with chi given as (cos, remainder, sin, remainder): exact products
+  __device__ __forceinline__ void add(float2 v, float4 c) {
+    df_add_prod(rh, rl, c.x, v.x);
+    df_add_prod(rh, rl, -c.z, v.y);
+    rl = __fmaf_rn(c.y, v.x, __fmaf_rn(-c.w, v.y, rl));
+    df_add_prod(ih, il, c.x, v.y);
+    df_add_prod(ih, il, c.z, v.x);
+    il = __fmaf_rn(c.y, v.y, __fmaf_rn(c.w, v.x, il));
+  }
+  __device__ __forceinline__ double re() const { return df_value(rh, rl); }
+  __device__ __forceinline__ double im() const { return df_value(ih, il); }
+};
+
+struct PairSm {
+  const uint32_t *off;
+  const uint8_t *mult;
+  const uint2 *bond;
+};
+
+// U terms of the row (A, B) given by their bonds; chi and the sum per term
+template <typename V, bool kChi, bool kFlips, int U>
+__device__ __forceinline__ void pair_terms(const PairParams &P, const PairSm &S, uint32_t A,
+                                           uint32_t B, const int (&kb)[U], int nu, const V *xs,
+                                           const unsigned char *chi_sm, Acc<V> &acc) {
+  uint32_t ea[U], eb[U];
+#pragma unroll
+  for (int u = 0; u < U; u++) {
+    const uint2 f = S.bond[kb[u]];
+    ea[u] = __ldg(P.ta + (A ^ f.x));
+    eb[u] = __ldg(P.tb + (B ^ f.y));
+  }
+  V v[U];
+  uint32_t lo[U], hi[U], slot[U];
+#pragma unroll
+  for (int u = 0; u < U; u++) {
+    lo[u] = min(ea[u], eb[u]);
+    hi[u] = max(ea[u], eb[u]);
+    const uint32_t mi = (lo[u] & kElem) * P.h0 + (hi[u] & kElem) + (ea[u] <= eb[u] ? 0u : P.sel_off);
+    slot[u] = S.off[lo[u] >> kClassShift] + P.K * (hi[u] >> kClassShift) + S.mult[mi];
+    if (kFlips) slot[u] += ((lo[u] ^ hi[u]) & kFlip) ? P.h0 : 0u;
+    v[u] = ld_slot(xs + slot[u]);
+  }
+#pragma unroll
+  for (int u = 0; u < U; u++) {
+    if (u < nu) {
+      if constexpr (kChi) {
+        const uint32_t ci = (lo[u] & (kElem | kFlip)) + (ea[u] <= eb[u] ? 0u : 512u);
+        if constexpr (sizeof(typename Pv<V>::A) == 4)
+          acc.add(v[u], reinterpret_cast<const float4 *>(chi_sm)[ci]);
+        else
+          acc.add(v[u], reinterpret_cast<const double2 *>(chi_sm)[ci]);
+      } else {
+        const uint32_t neg = (lo[u] >> kSignBit) & 1u;
+        acc.add(v[u], neg);
+        if constexpr (std::is_same<V, float>::value) {
+          // |Stab| > 1 needs a stabiliser on both halves, or halves that can be exchanged
+          if (P.xslo && ((lo[u] & hi[u] & kSpecial) || ((lo[u] ^ hi[u]) >> kClassShift) == 0))
+            acc.add_lo(__ldg(P.xslo + slot[u]), neg);
+        }
+      }
+    }
+  }
+}
+
+template <typename V, bool kChi, bool kFlips>
+__global__ void __launch_bounds__(kThreads, kMinBlocks) pair_kernel(const __grid_constant__ PairParams P) {
+  using A_ = typename Pv<V>::A;
+  constexpr bool kC = Pv<V>::cplx;
+  constexpr bool kF = sizeof(A_) == 4;
+  extern __shared__ __align__(16) unsigned char sm[];
+  cpy(sm, P.off_off, P.off, P.n_cls);
+  cpy(sm, P.off_mult, reinterpret_cast<const uint32_t *>(P.mult), P.mult_bytes / 4);
+  const int n_words = P.cls_word[P.n_classes];
+  cpy(sm, P.off_bond, P.bond, (uint32_t)n_words * 32);
+  cpy(sm, P.off_nib, P.nib, (uint32_t)n_words * P.n_nib * 16);
+  cpy(sm, P.off_rs, P.rsqrt_tab, P.n_sq);
+  if constexpr (kChi) {
+    for (uint32_t k = threadIdx.x; k < P.n_chi; k += blockDim.x) {
+      const double c = P.chi[2 * k], s = P.chi[2 * k + 1];
+      if constexpr (kF) {
+        const float ch = (float)c, sh = (float)s;
+        reinterpret_cast<float4 *>(sm + P.off_chi)[k] = make_float4(ch, (float)(c - (double)ch), sh, (float)(s - (double)sh));
+      } else {
+        reinterpret_cast<double2 *>(sm + P.off_chi)[k] = make_double2(c, s);
+      }
+    }
+  }
+  __syncthreads();
+  PairSm S;
+  S.off = reinterpret_cast<const uint32_t *>(sm + P.off_off);
+  S.mult = sm + P.off_mult;
+  S.bond = reinterpret_cast<const uint2 *>(sm + P.off_bond);
+  const uint32_t *nibs = reinterpret_cast<const uint32_t *>(sm + P.off_nib);
+  const double *rsd = reinterpret_cast<const double *>(sm + P.off_rs);
+  uint32_t *mask_s = reinterpret_cast<uint32_t *>(sm + P.off_mask) + threadIdx.x;
+  const V *xs = reinterpret_cast<const V *>(P.xs);
+  const V *x = reinterpret_cast<const V *>(P.x);
+  V *y = reinterpret_cast<V *>(P.y);
+  double dot_re = 0.0, dot_im = 0.0;
+  const int64_t stride = (int64_t)gridDim.x * kThreads;
+  for (int64_t i = P.r0 + (int64_t)blockIdx.x * kThreads + threadIdx.x; i < P.r1; i += stride) {
+    const uint64_t s = __ldcs(reinterpret_cast<const unsigned long long *>(P.basis) + i);
+    const uint32_t A = (((uint32_t)(s >> P.shA0) & P.bmask_hi) << P.n) | ((uint32_t)(s >> P.shA1) & P.bmask);
+    const uint32_t B = (((uint32_t)(s >> P.shB0) & P.bmask_hi) << P.n) | ((uint32_t)(s >> P.shB1) & P.bmask);
+    double diag = 0.0, row_re = 0.0, row_im = 0.0;
+    for (int c = 0; c < P.n_classes; c++) {
+      const int w0 = P.cls_word[c], w1 = P.cls_word[c + 1];
+      int nanti = 0;
+      for (int wd = w0; wd < w1; wd++) {
+        uint32_t m = 0;
+        const uint32_t *nw = nibs + (uint32_t)wd * P.n_nib * 16;
+        for (uint32_t q = 0; q < P.n_nib; q++) m ^= nw[q * 16 + (uint32_t)((s >> (4 * q)) & 15u)];
+        nanti += __popc(m);
+        mask_s[(wd - w0) * kThreads] = m;
+      }
+      Acc<V> acc;
+      int wd = w0;
+      uint32_t m = w0 < w1 ? mask_s[0] : 0u;
+      for (int left = nanti; left > 0;) {
+        while (m == 0) m = mask_s[(++wd - w0) * kThreads];
+        constexpr int U = 2;
+        int kb[U];
+        kb[0] = wd * 32 + __ffs(m) - 1;
+        m &= m - 1;
+        const int nu = left >= 2 ? 2 : 1;
+        kb[1] = kb[0];
+        if (nu == 2) {
+          while (m == 0) m = mask_s[(++wd - w0) * kThreads];
+          kb[1] = wd * 32 + __ffs(m) - 1;
+          m &= m - 1;
+        }
+        left -= nu;
+        pair_terms<V, kChi, kFlips, U>(P, S, A, B, kb, nu, xs, sm + P.off_chi, acc);
+      }
+      row_re += P.jh[c] * acc.re();
+      if constexpr (kC) row_im += P.jh[c] * acc.im();
+      diag += P.jzq[c] * (double)(P.nb_cls[c] - 2 * nanti);
+    }
+    const double rs = rsd[__ldcs(P.stab + i)];
+    // y_i in fp64, rounded once to the vector type; for fp32 vectors the rounding's
+    // remainder goes to ylo when asked, and <x, y> then uses the unrounded value
+    if constexpr (!kC) {
+      const double xi = (double)x[i];
+      const double yd = diag * xi + row_re * rs;
+      const A_ yi = (A_)yd;
+      __stcs(y + (i - P.r0), yi);
+      if (kF && P.ylo) reinterpret_cast<float *>(P.ylo)[i - P.r0] = (float)(yd - (double)yi);
+      if (P.partial) dot_re += xi * (kF && P.ylo ? yd : (double)yi);
+    } else {
+      const V xv = x[i];
+      const double yr = diag * (double)xv.x + row_re * rs;
+      const double yim = diag * (double)xv.y + row_im * rs;
+      V yv;
+      yv.x = (A_)yr;
+      yv.y = (A_)yim;
+      y[i - P.r0] = yv;
+      double ur = (double)yv.x, ui = (double)yv.y;
+      if (kF && P.ylo) {
+        float2 l;
+        l.x = (float)(yr - ur);
+        l.y = (float)(yim - ui);
+        reinterpret_cast<float2 *>(P.ylo)[i - P.r0] = l;
+        ur = yr;
+        ui = yim;
+      }
+      if (P.partial) {
+        dot_re += (double)xv.x * ur + (double)xv.y * ui;
+        dot_im += (double)xv.x * ui - (double)xv.y * ur;
+      }
+    }
+  }
+  if (P.partial) {
+    __shared__ double red[kThreads / 32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int part = 0; part < (kC ? 2 : 1); part++) {
+      double d = part ? dot_im : dot_re;
+      for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xFFFFFFFFu, d, o);
+      __syncthreads();
+      if (lane == 0) red[wid] = d;
+      __syncthreads();
+      if (wid == 0) {
+        d = lane < kThreads / 32 ? red[lane] : 0.0;
+        for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xFFFFFFFFu, d, o);
+        if (lane == 0) P.partial[part * gridDim.x + blockIdx.x] = d;
+      }
+    }
+  }
+}
+
+// xs[p] = w(meta[p]) x[idx[p]], w = chi sqrt(t); meta 0 is w = 1.  fp32 real vectors keep
+// the rounding's remainder in xslo, so that a weight sqrt(t) costs no precision.
+template <typename V>
+__global__ void __launch_bounds__(256) expand_kernel(const V *x, const uint32_t *idx, const uint16_t *meta,
+                                                     const double2 *w, uint32_t n, V *xs, float *xslo) {
+  using A_ = typename Pv<V>::A;
+  for (uint32_t p = blockIdx.x * 256 + threadIdx.x; p < n; p += gridDim.x * 256) {
+    const uint32_t j = __ldcs(idx + p);
+    const uint32_t mt = __ldcs(meta + p);
+    V v;
+    if constexpr (Pv<V>::cplx) { v.x = 0; v.y = 0; } else { v = 0; }
+    float lo = 0.f;
+    if (j != 0xFFFFFFFFu) {
+      v = __ldg(x + j);
+      if (mt) {
+        const double2 c = __ldg(w + mt);
+        if constexpr (Pv<V>::cplx) {
+          const double a = c.x * (double)v.x - c.y * (double)v.y, b = c.x * (double)v.y + c.y * (double)v.x;
+          v.x = (A_)a;
+          v.y = (A_)b;
+        } else {
+          const double a = c.x * (double)v;
+          v = (A_)a;
+          lo = (float)(a - (double)v);
+        }
+      }
+    }
+    xs[p] = v;
+    if (sizeof(V) == 4 && xslo) xslo[p] = lo;
+  }
+}
+
+// ------------------------------- tables (once per basis) -----------------------------
+// The half tables from the block tables: for every half pattern u the smallest image under
+// the listed elements, the number of the first of them in the list, and whether several
+// reach it.
+struct HalfParams {
+  const uint16_t *act;
+  const uint8_t *dest;
+  int n, nsub, nsym;
+  int b0, b1;          // blocks of the half (b0 most significant; b1 = -1: one block)
+  int t0;              // most significant block of the half it is carried onto
+  const uint16_t *list;
+  int n_list;
+};
+
+__device__ __forceinline__ uint32_t half_image(const HalfParams &Q, uint32_t u, int g) {
+  const uint32_t mask = (1u << Q.n) - 1u;
+  if (Q.b1 < 0) return Q.act[(((uint32_t)Q.b0 << Q.n) | u) * (uint32_t)Q.nsym + (uint32_t)g];
+  const uint32_t i0 = Q.act[(((uint32_t)Q.b0 << Q.n) | (u >> Q.n)) * (uint32_t)Q.nsym + (uint32_t)g];
+  const uint32_t i1 = Q.act[(((uint32_t)Q.b1 << Q.n) | (u & mask)) * (uint32_t)Q.nsym + (uint32_t)g];
+  return Q.dest[g * Q.nsub + Q.b0] == Q.t0 ? (i0 << Q.n) | i1 : (i1 << Q.n) | i0;
+}
+
+__global__ void half_reps(const HalfParams Q, uint32_t total, uint32_t *rep, uint32_t *first) {
+  for (uint32_t u = blockIdx.x * blockDim.x + threadIdx.x; u < total; u += gridDim.x * blockDim.x) {
+    uint32_t best = 0xFFFFFFFFu, at = 0, cnt = 0;
+    for (int j = 0; j < Q.n_list; j++) {
+      const uint32_t v = half_image(Q, u, Q.list[j]);
+      if (v < best) { best = v; at = (uint32_t)j; cnt = 1; }
+      else if (v == best) cnt++;
+    }
+    rep[u] = best;
+    first[u] = at | (cnt > 1 ? 0x80000000u : 0u);
+  }
+}
+
+__global__ void class_ids(const uint32_t *reps, uint32_t n, uint32_t base, uint32_t *id) {
+  for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x)
+    id[reps[c]] = base + c;
+}
+
+// code[j]: sign, flip and element number of list entry j
+__global__ void half_entries(const uint32_t *rep, const uint32_t *first, const uint32_t *id,
+                             const uint16_t *code, uint32_t total, uint32_t *t) {
+  for (uint32_t u = blockIdx.x * blockDim.x + threadIdx.x; u < total; u += gridDim.x * blockDim.x)
+    t[u] = (id[rep[u]] << kClassShift) | ((first[u] >> 31) ? kSpecial : 0u) |
+           code[first[u] & 0x7FFFFFFFu];
+}
+
+}  // namespace
+
+struct PairPlan {
+  int n = 0, m = 0;
+  int shA0 = 0, shA1 = 0, shB0 = 0, shB1 = 0;
+  uint32_t bmask_hi = 0, bmask = 0;
+  uint32_t n_cls = 0, K = 0, h0 = 0, sel_off = 0, mult_bytes = 0, n_slots = 0, n_w = 0;
+  bool flips = false, weights = false;
+  uint32_t *d_ta = nullptr, *d_tb = nullptr, *d_off = nullptr, *d_idx = nullptr;
+  uint8_t *d_mult = nullptr;
+  uint2 *d_bond = nullptr;
+  double *d_chi = nullptr, *d_w = nullptr;
+  uint16_t *d_meta = nullptr;
+  cudaMemPool_t pool = nullptr;   // xs of the calls in flight, stream-ordered
+  size_t bytes = 0;
+};
+
+void ed_free_pair(ed_basis *B) {
+  PairPlan *p = B->pair;
+  B->pair = nullptr;
+  if (!p) return;
+  for (void *q : {(void *)p->d_ta, (void *)p->d_tb, (void *)p->d_off, (void *)p->d_idx, (void *)p->d_mult,
+                  (void *)p->d_bond, (void *)p->d_chi, (void *)p->d_w, (void *)p->d_meta})
+    if (q) cudaFree(q);
+  if (p->pool) cudaMemPoolDestroy(p->pool);
+  delete p;
+}
+
+// Builds B->pair when the sector admits it; leaves it null (the search kernels serve the
+// sector) when the split has no two stable halves, the tables would be too large, or device
+// memory is short.  Only CUDA failures other than out-of-memory are errors.
+int ed_build_pair(ed_basis *B, cudaStream_t st) {
+  const int nsub = B->nsub, n = B->n, ns = B->nsym, N = B->N;
+  if (!B->two_level || (nsub != 2 && nsub != 4) || B->D == 0 || ns > 1024 || N > 44) return ED_OK;
+  const int m = N / 2;
+  std::vector<uint8_t> dest((size_t)ns * nsub);
+  for (int g = 0; g < ns; g++)
+    for (int X = 0; X < nsub; X++) dest[(size_t)g * nsub + X] = (uint8_t)(B->perm[(size_t)g * N + X * n] / n);
+  // halves: block sets {hb[0], hb[1]} and {hb[2], hb[3]} (one block each when nsub == 2)
+  static const int kSplit[3][4] = {{0, 1, 2, 3}, {0, 2, 1, 3}, {0, 3, 1, 2}};
+  int hb[4] = {0, -1, 1, -1};
+  std::vector<uint8_t> swaps(ns, 0);
+  bool found = false;
+  for (int t = 0; t < (nsub == 4 ? 3 : 1) && !found; t++) {
+    if (nsub == 4) for (int q = 0; q < 4; q++) hb[q] = kSplit[t][q];
+    auto half_of = [&](int X) { return X == hb[0] || X == hb[1] ? 0 : 1; };
+    found = true;
+    for (int g = 0; g < ns && found; g++) {
+      const int to = half_of(dest[(size_t)g * nsub + hb[0]]);
+      if (nsub == 4 && half_of(dest[(size_t)g * nsub + hb[1]]) != to) found = false;
+      swaps[g] = (uint8_t)to;
+    }
+  }
+  if (!found) return ED_OK;
+  // the group as G0 x {1, F} when it holds the pure spin flip F (its elements then carry a
+  // flip bit next to their number in G0), else all of it as it is
+  // Elements are told apart by their flip and the images of at most three sites (enough for
+  // affine lattice symmetries); products are then looked up without comparing permutations.
+  const int32_t *pm = B->perm.data();
+  int base[3] = {0, 0, 0}, nb = 0;
+  std::vector<int16_t> at;
+  auto key = [&](int i0, int i1, int i2, int f) { return ((size_t)(i0 * N + i1) * N + i2) * 2 + f; };
+  for (nb = 1; nb <= 3; nb++) {
+    // the next base site: the one that tells the most elements apart
+    int best = 0, most = -1;
+    for (int q = 0; q < N; q++) {
+      base[nb - 1] = q;
+      for (int r = nb; r < 3; r++) base[r] = base[0];
+      std::vector<size_t> ks(ns);
+      for (int g = 0; g < ns; g++) ks[g] = key(pm[g * N + base[0]], pm[g * N + base[1]], pm[g * N + base[2]], B->flip[g] ? 1 : 0);
+      std::sort(ks.begin(), ks.end());
+      const int d = (int)(std::unique(ks.begin(), ks.end()) - ks.begin());
+      if (d > most) { most = d; best = q; }
+      if (d == ns) break;
+    }
+    base[nb - 1] = best;
+    for (int r = nb; r < 3; r++) base[r] = base[0];
+    if (most == ns) break;
+  }
+  if (nb > 3) return ED_OK;
+  at.assign((size_t)N * N * N * 2, -1);
+  bool any_flip = false, pure = false;
+  for (int g = 0; g < ns; g++) {
+    const int f = B->flip[g] ? 1 : 0;
+    at[key(pm[g * N + base[0]], pm[g * N + base[1]], pm[g * N + base[2]], f)] = (int16_t)g;
+    any_flip = any_flip || f;
+    bool id = f == 1;
+    for (int q = 0; q < N && id; q++) id = pm[g * N + q] == q;
+    pure = pure || id;
+  }
+  auto mul = [&](int a, int b) -> int {   // (a b)[p] = a[b[p]]
+    const int32_t *pa = pm + (size_t)a * N, *pb = pm + (size_t)b * N;
+    return at[key(pa[pb[base[0]]], pa[pb[base[1]]], pa[pb[base[2]]], (B->flip[a] ? 1 : 0) ^ (B->flip[b] ? 1 : 0))];
+  };
+  std::vector<int> inverse(ns, -1);
+  {
+    std::vector<int32_t> q(N);
+    for (int g = 0; g < ns; g++) {
+      for (int p = 0; p < N; p++) q[pm[(size_t)g * N + p]] = p;
+      inverse[g] = at[key(q[base[0]], q[base[1]], q[base[2]], B->flip[g] ? 1 : 0)];
+      if (inverse[g] < 0) return ED_OK;
+    }
+  }
+  auto inv = [&](int a) { return inverse[a]; };
+  std::vector<int> H0, S0;   // elements keeping / exchanging the halves (without F)
+  for (int g = 0; g < ns; g++)
+    if (!(pure && B->flip[g])) (swaps[g] ? S0 : H0).push_back(g);
+  const uint32_t h0 = (uint32_t)H0.size();
+  if (h0 > 256) return ED_OK;
+  const bool has_swap = !S0.empty();
+  int tau = -1;
+  bool involution = false;
+  for (int s : S0) {
+    if (tau < 0) tau = s;
+    if (mul(s, s) == B->id_g) { tau = s; involution = true; break; }
+  }
+  const int nf = pure ? 2 : 1;
+  std::vector<int> num(ns, -1);                 // number of an element of H0
+  for (uint32_t q = 0; q < h0; q++) num[H0[q]] = (int)q;
+  // lists: half A by H; half B by H tau (or H when nothing exchanges the halves); K elements
+  // between the halves, numbered like the list of half B
+  auto with_flip = [&](int g, int f) -> int {
+    if (!f) return g;
+    const int32_t *q = pm + (size_t)g * N;
+    return at[key(q[base[0]], q[base[1]], q[base[2]], 1)];
+  };
+  std::vector<uint16_t> listA, listB, codeA, codeB;
+  std::vector<int> numK(ns, -1);
+  for (int f = 0; f < nf; f++)
+    for (uint32_t q = 0; q < h0; q++) {
+      const int ga = with_flip(H0[q], f), gb0 = has_swap ? mul(H0[q], tau) : H0[q], gb = with_flip(gb0, f);
+      if (ga < 0 || gb0 < 0 || gb < 0) return ED_OK;
+      if (!f) numK[gb0] = (int)q;
+      listA.push_back((uint16_t)ga);
+      listB.push_back((uint16_t)gb);
+      const uint32_t base = q | (f ? kFlip : 0u);
+      codeA.push_back((uint16_t)(base | (B->is_real && B->phase[ga] ? 1u << kSignBit : 0u)));
+      codeB.push_back((uint16_t)(base | (B->is_real && B->phase[gb] ? 1u << kSignBit : 0u)));
+    }
+  const uint32_t K = h0 * nf;
+  // k of (lower, upper): x tau^-1 y^-1 when half A is the lower one, x tau y^-1 when half B
+  // is (the same table when tau is an involution); x y^-1 when nothing exchanges the halves
+  const int itau = has_swap ? inv(tau) : -1;
+  const uint32_t n_tab = has_swap && !involution ? 2 : 1;
+  std::vector<uint8_t> mult(((size_t)n_tab * h0 * h0 + 3) / 4 * 4, 0);
+  for (uint32_t y = 0; y < h0; y++) {
+    const int iy = inv(H0[y]);
+    for (uint32_t t = 0; t < n_tab; t++) {
+      const int r = has_swap ? mul(t ? tau : itau, iy) : iy;
+      for (uint32_t x = 0; x < h0; x++) {
+        const int e = mul(H0[x], r);
+        const int k = e < 0 ? -1 : numK[e];
+        if (k < 0) return ED_OK;
+        mult[((size_t)t * h0 + x) * h0 + y] = (uint8_t)k;
+      }
+    }
+  }
+  PairPlan *p = new (std::nothrow) PairPlan();
+  if (!p) return ED_OK;
+  B->pair = p;
+  p->n = n; p->m = m;
+  p->h0 = h0; p->K = K;
+  p->flips = pure;
+  p->sel_off = n_tab == 2 ? h0 * h0 : 0u;
+  p->mult_bytes = (uint32_t)mult.size();
+  const int sh = N - n;   // block X sits at bit N - (X + 1) n
+  if (nsub == 4) {
+    p->shA0 = sh - hb[0] * n; p->shA1 = sh - hb[1] * n;
+    p->shB0 = sh - hb[2] * n; p->shB1 = sh - hb[3] * n;
+    p->bmask = p->bmask_hi = (1u << n) - 1u;
+  } else {
+    p->shA0 = p->shB0 = 0;
+    p->shA1 = n; p->shB1 = 0;
+    p->bmask = (1u << n) - 1u;
+    p->bmask_hi = 0;
+  }
+  struct Scratch {   // device scratch of the build, freed on every path
+    std::vector<void *> v;
+    ~Scratch() { for (void *q : v) cudaFree(q); }
+  } scratch;
+  bool oom = false;
+  auto dev = [&](size_t bytes, bool keep) -> void * {
+    void *q = nullptr;
+    if (oom || cudaMalloc(&q, std::max<size_t>(bytes, 16)) != cudaSuccess) {
+      cudaGetLastError();
+      oom = true;
+      return nullptr;
+    }
+    if (keep) p->bytes += bytes; else scratch.v.push_back(q);
+    return q;
+  };
+  const uint32_t total = 1u << m;
+  uint32_t *d_rep = (uint32_t *)dev((size_t)total * 4, false), *d_first = (uint32_t *)dev((size_t)total * 4, false);
+  uint32_t *d_id = (uint32_t *)dev((size_t)total * 4, false), *d_reps = (uint32_t *)dev((size_t)total * 4, false);
+  uint16_t *d_list = (uint16_t *)dev(listA.size() * 8, false);
+  p->d_ta = (uint32_t *)dev((size_t)total * 4, true);
+  p->d_tb = (uint32_t *)dev((size_t)total * 4, true);
+  if (oom) { ed_free_pair(B); return ED_OK; }
+  const size_t nl = listA.size();
+  ED_CK(cudaMemcpyAsync(d_list, listA.data(), nl * 2, cudaMemcpyHostToDevice, st));
+  ED_CK(cudaMemcpyAsync(d_list + nl, listB.data(), nl * 2, cudaMemcpyHostToDevice, st));
+  ED_CK(cudaMemcpyAsync(d_list + 2 * nl, codeA.data(), nl * 2, cudaMemcpyHostToDevice, st));
+  ED_CK(cudaMemcpyAsync(d_list + 3 * nl, codeB.data(), nl * 2, cudaMemcpyHostToDevice, st));
+  const int gt = (int)std::min<uint32_t>((total + 255) / 256, (uint32_t)B->sm_count * 8);
+  std::vector<uint32_t> rep(total);
+  std::vector<std::vector<uint32_t>> cls(2);      // representatives of half A's (and B's) classes
+  std::vector<uint32_t> bucket0[2];               // first class of each popcount
+  for (int half = 0; half < 2; half++) {
+    HalfParams Q{(const uint16_t *)B->d_action, B->d_dest, n, nsub, ns, hb[2 * half], hb[2 * half + 1],
+                 half && !has_swap ? hb[2] : hb[0], d_list + half * nl, (int)nl};
+    half_reps<<<gt, 256, 0, st>>>(Q, total, d_rep, d_first);
+    ED_CK(cudaGetLastError());
+    if (half == 0 || !has_swap) {
+      ED_CK(cudaMemcpyAsync(rep.data(), d_rep, (size_t)total * 4, cudaMemcpyDeviceToHost, st));
+      ED_CK(cudaStreamSynchronize(st));
+      // classes in order of (popcount of the representative, value); with spin flips the
+      // smaller of the popcounts of a pattern and its reverse
+      std::vector<std::vector<uint32_t>> by(m + 1);
+      for (uint32_t u = 0; u < total; u++)
+        if (rep[u] == u) {
+          const int pc = __builtin_popcount(u);
+          by[any_flip ? std::min(pc, m - pc) : pc].push_back(u);
+        }
+      bucket0[half].assign(m + 2, 0);
+      for (int q = 0; q <= m; q++) {
+        bucket0[half][q] = (uint32_t)cls[half].size();
+        cls[half].insert(cls[half].end(), by[q].begin(), by[q].end());
+      }
+      bucket0[half][m + 1] = (uint32_t)cls[half].size();
+      const uint32_t nc = (uint32_t)cls[half].size();
+      ED_CK(cudaMemcpyAsync(d_reps, cls[half].data(), (size_t)nc * 4, cudaMemcpyHostToDevice, st));
+      class_ids<<<gt, 256, 0, st>>>(d_reps, nc, half ? (uint32_t)cls[0].size() : 0u, d_id);
+      ED_CK(cudaGetLastError());
+    }
+    half_entries<<<gt, 256, 0, st>>>(d_rep, d_first, d_id, d_list + (2 + half) * nl, total, half ? p->d_tb : p->d_ta);
+    ED_CK(cudaGetLastError());
+  }
+  const uint32_t nA = (uint32_t)cls[0].size();
+  const std::vector<uint32_t> &up = has_swap ? cls[0] : cls[1];
+  const std::vector<uint32_t> &ub = has_swap ? bucket0[0] : bucket0[1];
+  const uint32_t ubase = has_swap ? 0u : nA;      // class number of the first upper class
+  p->n_cls = nA;
+  if (nA > 16384 || ubase + up.size() >= (1u << 21)) { ed_free_pair(B); return ED_OK; }
+  // slots of every lower class: the upper classes [lo, hi) that can share a configuration
+  // of the sector with it
+  std::vector<uint32_t> off(nA), start(nA + 1), first_up(nA);
+  uint64_t acc = 0;
+  for (uint32_t c = 0; c < nA; c++) {
+    int pc = __builtin_popcount(cls[0][c]);
+    if (any_flip) pc = std::min(pc, m - pc);
+    const int want = any_flip ? pc : B->n_up - pc;
+    uint32_t lo = 0, hi = 0;
+    if (want >= 0 && want <= m) { lo = ub[want]; hi = ub[want + 1]; }
+    if (has_swap) lo = std::max(lo, c);
+    if (lo >= hi) lo = hi = 0;
+    start[c] = (uint32_t)acc;
+    first_up[c] = lo;
+    off[c] = (uint32_t)acc - K * (ubase + lo);    // modulo 2^32: slot = off + K upper + k
+    acc += (uint64_t)K * (hi - lo);
+    if (acc >= 0xFFFFFF00ull) { ed_free_pair(B); return ED_OK; }
+  }
+  start[nA] = (uint32_t)acc;
+  const uint64_t cap = std::max<uint64_t>(4 * (uint64_t)B->D, 1u << 22);
+  if (acc == 0 || acc > cap) { ed_free_pair(B); return ED_OK; }
+  p->n_slots = (uint32_t)acc;
+  // weights chi sqrt(t): index phase + denom * (number of t among the divisors of |G|)
+  std::vector<uint8_t> tcode(ns + 1, 0);
+  std::vector<int> divs;
+  for (int t = 1; t <= ns; t++) if (ns % t == 0) { tcode[t] = (uint8_t)divs.size(); divs.push_back(t); }
+  p->n_w = (uint32_t)(B->denom * divs.size());
+  if (p->n_w > 65535 || divs.size() > 255) { ed_free_pair(B); return ED_OK; }
+  std::vector<double> wt(2 * (size_t)p->n_w);
+  for (size_t t = 0; t < divs.size(); t++)
+    for (int q = 0; q < B->denom; q++) {
+      const double a = 2.0 * M_PI * (double)q / (double)B->denom, r = std::sqrt((double)divs[t]);
+      double c = std::cos(a), s = std::sin(a);
+      if (B->is_real) { c = q ? -1.0 : 1.0; s = 0.0; }
+      wt[2 * (t * B->denom + q)] = r * c;
+      wt[2 * (t * B->denom + q) + 1] = r * s;
+    }
+  // chi of the lower half's element: [half][512] (flip bit above the element number)
+  std::vector<double> chi(2 * 1024, 0.0);
+  for (int half = 0; half < 2; half++)
+    for (size_t j = 0; j < nl; j++) {
+      const int g = half ? listB[j] : listA[j];
+      const uint32_t e = (half ? codeB[j] : codeA[j]) & (kElem | kFlip);
+      const double a = 2.0 * M_PI * (double)B->phase[g] / (double)B->denom;
+      chi[2 * (512 * half + e)] = std::cos(a);
+      chi[2 * (512 * half + e) + 1] = std::sin(a);
+    }
+  // bonds as flipped bits of the two halves
+  std::vector<uint2> bond(B->bond_pad.size() / 2, make_uint2(0, 0));
+  for (size_t b = 0; b < bond.size(); b++) {
+    const int pe[2] = {B->bond_pad[2 * b], B->bond_pad[2 * b + 1]};
+    if (pe[0] == pe[1]) continue;
+    for (int q = 0; q < 2; q++) {
+      const int lab = N - 1 - pe[q], X = lab / n, bit = n - 1 - lab % n;
+      const int pos = bit + ((nsub == 4 && (X == hb[0] || X == hb[2])) ? n : 0);
+      if (X == hb[0] || X == hb[1]) bond[b].x |= 1u << pos; else bond[b].y |= 1u << pos;
+    }
+  }
+  p->d_off = (uint32_t *)dev(4 * (size_t)nA, true);
+  p->d_mult = (uint8_t *)dev(mult.size(), true);
+  p->d_bond = (uint2 *)dev(bond.size() * 8, true);
+  p->d_chi = (double *)dev(chi.size() * 8, true);
+  p->d_w = (double *)dev(wt.size() * 8, true);
+  p->d_idx = (uint32_t *)dev((size_t)acc * 4, true);
+  p->d_meta = (uint16_t *)dev((size_t)acc * 2, true);
+  uint32_t *d_start = (uint32_t *)dev(4 * ((size_t)nA + 1), false);
+  uint32_t *d_fup = (uint32_t *)dev(4 * (size_t)nA, false);
+  uint32_t *d_up = (uint32_t *)dev(4 * up.size(), false);
+  uint32_t *d_low = (uint32_t *)dev(4 * (size_t)nA, false);
+  uint8_t *d_tcode = (uint8_t *)dev(tcode.size(), false);
+  uint32_t *d_any = (uint32_t *)dev(4, false);
+  if (oom) { ed_free_pair(B); return ED_OK; }
+  auto put = [&](void *d, const void *s, size_t bytes) { return cudaMemcpyAsync(d, s, bytes, cudaMemcpyHostToDevice, st); };
+  ED_CK(put(p->d_off, off.data(), 4 * (size_t)nA));
+  ED_CK(put(p->d_mult, mult.data(), mult.size()));
+  ED_CK(put(p->d_bond, bond.data(), bond.size() * 8));
+  ED_CK(put(p->d_chi, chi.data(), chi.size() * 8));
+  ED_CK(put(p->d_w, wt.data(), wt.size() * 8));
+  ED_CK(put(d_start, start.data(), 4 * ((size_t)nA + 1)));
+  ED_CK(put(d_fup, first_up.data(), 4 * (size_t)nA));
+  ED_CK(put(d_up, up.data(), 4 * up.size()));
+  ED_CK(put(d_low, cls[0].data(), 4 * (size_t)nA));
+  ED_CK(put(d_tcode, tcode.data(), tcode.size()));
+  ED_CK(cudaMemsetAsync(d_any, 0, 4, st));
+  PairSlots Q{};
+  Q.start = d_start; Q.first_up = d_fup; Q.low = d_low; Q.up = d_up; Q.n_low = nA; Q.n_slots = p->n_slots;
+  Q.K = K; Q.kel = d_list + nl; Q.tcode = d_tcode;
+  for (int q = 0; q < 4; q++) Q.hb[q] = hb[q];
+  Q.up_half = has_swap ? 0 : 1;
+  Q.idx = p->d_idx; Q.meta = p->d_meta; Q.any_weight = d_any;
+  int rc = ed_launch_pair_slots(B, Q, st);
+  if (rc == ED_ERR_UNSUPPORTED) { ed_free_pair(B); return ED_OK; }
+  if (rc) return rc;
+  uint32_t any = 0;
+  ED_CK(cudaMemcpyAsync(&any, d_any, 4, cudaMemcpyDeviceToHost, st));
+  ED_CK(cudaStreamSynchronize(st));
+  p->weights = any != 0;
+  cudaMemPoolProps props{};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = B->device;
+  if (cudaMemPoolCreate(&p->pool, &props) != cudaSuccess) {
+    cudaGetLastError();
+    p->pool = nullptr;
+    ed_free_pair(B);
+    return ED_OK;
+  }
+  uint64_t keep = ~0ull;
+  ED_CK(cudaMemPoolSetAttribute(p->pool, cudaMemPoolAttrReleaseThreshold, &keep));
+  // small sectors: the pool takes its first memory here rather than in the first product,
+  // where mapping it would cost several times the product itself
+  const size_t first = 8 * (size_t)p->n_slots;
+  if (first <= ((size_t)64 << 20)) {
+    void *q = nullptr;
+    if (cudaMallocFromPoolAsync(&q, first, p->pool, st) == cudaSuccess) ED_CK(cudaFreeAsync(q, st));
+    else cudaGetLastError();
+  }
+  B->table_bytes += p->bytes;
+  return ED_OK;
+}
+
+namespace {
+
+size_t al16(size_t x) { return (x + 15) & ~(size_t)15; }
+
+template <typename V, bool kChi, bool kFlips>
+int launch_pair_t(const ed_basis *B, PairParams &P, cudaStream_t st) {
+  auto k = pair_kernel<V, kChi, kFlips>;
+  ED_CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, P.smem_bytes));
+  const int need = kMinBlocks * ((int)P.smem_bytes + 1536);
+  const int pct = std::min(100, (need * 100 + 228 * 1024 - 1) / (228 * 1024));
+  ED_CK(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, pct));
+  const int64_t blocks = (P.r1 - P.r0 + kThreads - 1) / kThreads;
+  const int grid = (int)std::min<int64_t>(blocks, (int64_t)B->sm_count * kMinBlocks);
+  B->last_apply_grid = grid;
+  k<<<grid, kThreads, P.smem_bytes, st>>>(P);
+  ED_CK(cudaGetLastError());
+  return ED_OK;
+}
+
+template <typename V>
+int launch_pair_v(const ed_basis *B, PairParams &P, bool chi, bool flips, cudaStream_t st) {
+  if constexpr (Pv<V>::cplx) {
+    if (chi) return flips ? launch_pair_t<V, true, true>(B, P, st) : launch_pair_t<V, true, false>(B, P, st);
+  }
+  return flips ? launch_pair_t<V, false, true>(B, P, st) : launch_pair_t<V, false, false>(B, P, st);
+}
+
+}  // namespace
+
+int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, const void *x, void *y,
+                         int dtype, int64_t r0, int64_t r1, double *partial, cudaStream_t st, void *ylo,
+                         bool *ylo_done) {
+  const PairPlan *p = B->pair;
+  if (!p) return ED_ERR_UNSUPPORTED;
+  const size_t es = dtype == ED_F64 ? 8 : dtype == ED_F32 ? 4 : dtype == ED_C128 ? 16 : 8;
+  PairParams P{};
+  P.n_classes = B->n_classes;
+  int words = 0;
+  for (int c = 0; c <= B->n_classes; c++) P.cls_word[c] = B->cls_word[c];
+  for (int c = 0; c < B->n_classes; c++) {
+    words = std::max(words, B->cls_word[c + 1] - B->cls_word[c]);
+    P.nb_cls[c] = B->cls_off[c + 1] - B->cls_off[c];
+    P.jh[c] = 0.5 * J[c];
+    P.jzq[c] = 0.25 * J[c] * Jz[c];
+  }
+  P.n = p->n;
+  P.shA0 = p->shA0; P.shA1 = p->shA1; P.shB0 = p->shB0; P.shB1 = p->shB1;
+  P.bmask_hi = p->bmask_hi; P.bmask = p->bmask;
+  P.ta = p->d_ta; P.tb = p->d_tb; P.off = p->d_off;
+  P.n_cls = p->n_cls; P.K = p->K; P.h0 = p->h0; P.sel_off = p->sel_off;
+  P.mult = p->d_mult; P.mult_bytes = p->mult_bytes;
+  P.bond = p->d_bond;
+  P.nib = B->d_nib; P.n_nib = (uint32_t)B->n_nib;
+  P.rsqrt_tab = B->d_rsqrt; P.n_sq = (uint32_t)B->nsym + 1;
+  const bool cplx = dtype == ED_C128 || dtype == ED_C64;
+  const bool chi = cplx && !B->is_real;
+  P.chi = p->d_chi; P.n_chi = 1024;
+  P.basis = B->d_basis; P.stab = B->d_stab;
+  P.x = x; P.y = y; P.r0 = r0; P.r1 = r1; P.partial = partial;
+  P.ylo = (dtype == ED_F32 || dtype == ED_C64) ? ylo : nullptr;
+  size_t off = 0;
+  auto put = [&](uint32_t &o, size_t bytes) { o = (uint32_t)off; off += al16(bytes); };
+  const size_t n_words = (size_t)B->cls_word[B->n_classes];
+  put(P.off_off, 4 * (size_t)P.n_cls);
+  put(P.off_mult, P.mult_bytes);
+  put(P.off_bond, 8 * 32 * n_words);
+  put(P.off_nib, 4 * B->nib.size());
+  put(P.off_rs, 8 * (size_t)P.n_sq);
+  put(P.off_chi, chi ? 16 * 1024 : 0);
+  put(P.off_mask, 4 * (size_t)words * kThreads);
+  P.smem_bytes = (uint32_t)off;
+  if (off > 110 * 1024) return ED_ERR_UNSUPPORTED;
+  // xs (and its remainders) for this call, from the basis's own pool in stream order, so
+  // calls on several streams or threads never share it; without memory for it the search
+  // kernel takes the call
+  const bool lo = dtype == ED_F32 && p->weights;
+  const size_t xs_bytes = al16(es * (size_t)p->n_slots);
+  char *ws = nullptr;
+  if (cudaMallocFromPoolAsync((void **)&ws, xs_bytes + (lo ? 4 * (size_t)p->n_slots : 0), p->pool, st) != cudaSuccess) {
+    cudaGetLastError();
+    return ED_ERR_UNSUPPORTED;
+  }
+  float *xslo = lo ? reinterpret_cast<float *>(ws + xs_bytes) : nullptr;
+  const int eg = (int)std::min<uint32_t>((p->n_slots + 255) / 256, (uint32_t)B->sm_count * 16);
+  P.xs = ws;
+  P.xslo = xslo;
+  int rc = ED_OK;
+  switch (dtype) {
+#define PCASE(D, V)                                                                              \
+  case D:                                                                                        \
+    expand_kernel<V><<<eg, 256, 0, st>>>((const V *)x, p->d_idx, p->d_meta, (const double2 *)p->d_w, p->n_slots, (V *)ws, xslo); \
+    rc = cudaGetLastError() == cudaSuccess ? launch_pair_v<V>(B, P, chi, p->flips, st)            \
+                                           : ed_fail(ED_ERR_CUDA, "expand_kernel");              \
+    break;
+    PCASE(ED_F64, double)
+    PCASE(ED_F32, float)
+    PCASE(ED_C128, double2)
+    PCASE(ED_C64, float2)
+#undef PCASE
+    default: rc = ed_fail(ED_ERR_INVALID, "unknown dtype");
+  }
+  const cudaError_t fe = cudaFreeAsync(ws, st);
+  if (!rc && fe != cudaSuccess) rc = ed_cuda_fail(fe, "cudaFreeAsync");
+  if (!rc && ylo_done) *ylo_done = P.ylo != nullptr;
+  return rc;
+}

@@ -268,6 +268,8 @@ __device__ __forceinline__ uint64_t splitmix64_mix(uint64_t z) {
 #include <string>
 #include <vector>
 
+struct PairPlan;                       // pair.cu: the product by coset arithmetic
+
 struct ed_basis {
   int device = 0;
   int sm_count = 0;
@@ -333,6 +335,7 @@ struct ed_basis {
   cudaStream_t copy_stream = nullptr;   // device-to-host copies of ed_apply_H_host
   std::vector<cudaEvent_t> chunk_done;  // one per row chunk of ed_apply_H_host
   double build_ms = 0;
+  PairPlan *pair = nullptr;            // null: the split has no two stable halves
 };
 
 // error reporting (capi.cu)
@@ -376,6 +379,31 @@ int ed_launch_start(const ed_basis *B, void *v, uint64_t seed, int dtype, cudaSt
 int ed_launch_apply_fast(const ed_basis *B, const double *J, const double *Jz, const void *x,
                          void *y, int dtype, int64_t r0, int64_t r1, double *partial,
                          cudaStream_t st, int mode, void *ylo = nullptr, bool *ylo_done = nullptr);
+// pair.cu: the coset-arithmetic product, its tables (built once per basis) and their release;
+// ed_launch_apply_pair returns ED_ERR_UNSUPPORTED when the sector has no plan
+int ed_build_pair(ed_basis *B, cudaStream_t st);
+void ed_free_pair(ed_basis *B);
+int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, const void *x, void *y,
+                         int dtype, int64_t r0, int64_t r1, double *partial, cudaStream_t st, void *ylo,
+                         bool *ylo_done);
+// apply_fast.cu: representative, index and weight of every slot's configuration.  Slot p
+// belongs to the lower class c with start[c] <= p < start[c+1]; with r = p - start[c], the
+// upper class is first_up[c] + r / K and the element kel[r % K] carries its representative
+// (a pattern of half up_half) onto half 1; low[c] lies on half 0.  Half q consists of blocks
+// hb[2q], hb[2q+1] (-1: one block).  idx[p] = basis index or 0xFFFFFFFF, meta[p] = phase +
+// denom * tcode[|Stab|]; *any_weight is set when some |Stab| > 1.
+struct PairSlots {
+  const uint32_t *start, *first_up, *low, *up;
+  uint32_t n_low, n_slots, K;
+  const uint16_t *kel;
+  const uint8_t *tcode;
+  int hb[4];
+  int up_half;
+  uint32_t *idx;
+  uint16_t *meta;
+  uint32_t *any_weight;
+};
+int ed_launch_pair_slots(const ed_basis *B, const PairSlots &Q, cudaStream_t st);
 int ed_build_full_table(const uint8_t *d_pbit, const uint8_t *d_flip, int N, int nsym,
                         uint64_t *out, cudaStream_t st);
 struct ed_batch;

@@ -1,0 +1,99 @@
+"""The coset-arithmetic product (csrc/pair.cu) at the edges of what it accepts: splits of two
+and four blocks, halves that are exchanged by an involution, by none, or by no element at
+all, spin flips (as a factor of the group and tied to other elements), trivial, sign and
+complex characters, fillings whose halves hold no or all spins, every vector type, row ranges
+on both sides of the size rule, several streams at once and a captured call.  Reference: the
+oracle's explicit matrix.  Bounds: as in test_gpu_parity, a row sums at most a few hundred
+terms of size max|J| |x|, so fp64 stays near 1e-15 relative (1e-12 asked) and fp32 within a
+few roundings (2e-6 asked)."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+import oracle
+import workloads as w
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+T = w.square_torus
+
+
+def _sub(p, sel, name, **kw):
+    sel = np.asarray(sel)
+    return dataclasses.replace(p, perm=p.perm[sel], phase_num=p.phase_num[sel], name=name, **kw)
+
+
+SECTORS = [
+    w.chain(12, 2, k=5, n_up=6), w.chain(12, 4, k=6, n_up=5), w.chain(16, 4, k=3, n_up=8),
+    w.chain(20, 2, k=10, n_up=9),
+    w.chain(10, 2, k=0, n_up=0), w.chain(10, 2, k=0, n_up=1), w.chain(10, 2, k=5, n_up=9),
+    _sub(w.chain(12, 2, k=2, n_up=6), range(0, 12, 2), "chain12_even_translations"),
+    _sub(w.chain(12, 2, k=0, n_up=6), [0], "chain12_identity"),
+    dataclasses.replace(w.chain(12, 2, k=2, n_up=6), flip=(np.arange(12) % 2).astype(np.uint8), name="chain12_flip_tied"),
+    w.with_spin_flip(w.chain(12, 4, k=3, n_up=6), 1), w.with_spin_flip(w.chain(12, 2, k=0, n_up=6), 0),
+    T(4, momentum=(0, 0), point_irrep=3, J2=0.5, n_sublat=2, n_up=7),
+    T(4, momentum=(1, 0), point_irrep=1, J2=0.5, n_sublat=4, n_up=5),
+    T(4, momentum=(1, 2), point_irrep=0, J2=0.5, n_sublat=4, n_up=8),
+    w.with_spin_flip(T(4, momentum=(2, 2), point_irrep=1, J2=0.5, n_sublat=4, n_up=8), 1),
+    T(6, momentum=(0, 0), point_irrep=1, J2=0.5, n_sublat=4, n_up=4),
+]
+
+
+def _basis(p):
+    import paper_1804_05028_gb300 as ed
+    return ed.build_basis_from(p)
+
+
+def _vec(D, dtype, seed):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    return torch.randn(D, dtype=dtype, device="cuda", generator=g)
+
+
+@pytest.mark.parametrize("p", SECTORS, ids=lambda p: f"{p.name}_up{p.n_up}")
+def test_product_of_every_type(p):
+    B = _basis(p)
+    H, _, _ = oracle.hamiltonian(p)
+    real = [torch.float64, torch.float32] if B.is_real else []
+    for dt in real + [torch.complex128, torch.complex64]:
+        x = _vec(B.dim, dt, 3)
+        xd = x.cpu().to(torch.complex128).numpy()
+        ref = H @ xd
+        tol = (2e-6 if dt in (torch.float32, torch.complex64) else 1e-12) * max(np.abs(ref).max(), 1e-30)
+        assert np.abs(B.apply_H(x).cpu().numpy() - ref).max() <= tol
+        # the rows of a range, wide enough for this product and narrower than its rule
+        for r0, r1 in [(B.dim // 5, B.dim - B.dim // 7), (B.dim // 2, B.dim // 2 + max(1, B.dim // 40))]:
+            r1 = min(r1, B.dim)
+            if r0 < r1:
+                assert np.abs(B.apply_H_rows(x, r0, r1).cpu().numpy() - ref[r0:r1]).max() <= tol
+
+
+def test_streams_and_capture():
+    p = T(6, momentum=(0, 0), point_irrep=1, J2=0.5, n_sublat=4, n_up=6)
+    B = _basis(p)
+    xs = [_vec(B.dim, torch.float32, s) for s in range(4)]
+    ref = [B.apply_H(x).clone() for x in xs]
+    ys = [torch.empty_like(x) for x in xs]
+    streams = [torch.cuda.Stream() for _ in xs]
+    torch.cuda.synchronize()
+    for _ in range(20):
+        for x, y, s in zip(xs, ys, streams):
+            B.apply_H(x, y, stream=s)
+    torch.cuda.synchronize()
+    for y, r in zip(ys, ref):
+        assert torch.equal(y, r)
+    # captured once, replayed on other contents of the same buffers
+    x, y = torch.empty_like(xs[0]), torch.empty_like(xs[0])
+    g = torch.cuda.CUDAGraph()
+    x.copy_(xs[0])
+    torch.cuda.synchronize()
+    with torch.cuda.graph(g):
+        B.apply_H(x, y)
+    for v, r in zip(xs, ref):
+        x.copy_(v)
+        y.zero_()
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(y, r)
+    del g
