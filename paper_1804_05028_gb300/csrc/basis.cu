@@ -345,6 +345,10 @@ uint64_t binom_host(int n, int k) {
 
 }  // namespace
 
+int ed_exclusive_scan(const uint32_t *in, uint64_t n, uint64_t *out, uint64_t *total, cudaStream_t st) {
+  return exclusive_scan<uint32_t>(in, n, out, total, st);
+}
+
 int ed_build_full_table(const uint8_t *d_pbit, const uint8_t *d_flip, int N, int nsym,
                         uint64_t *out, cudaStream_t st) {
   const size_t sm = (size_t)nsym * N + nsym;

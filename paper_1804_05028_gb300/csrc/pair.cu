@@ -39,6 +39,7 @@
 #include "dfloat.cuh"
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <new>
 #include <type_traits>
 #include <vector>
@@ -91,10 +92,28 @@ struct PairParams {
   int64_t r0, r1;
   double *partial;
   uint32_t off_off, off_mult, off_bond, off_nib, off_rs, off_chi, off_mask, smem_bytes;
+  // rows in the order of (lower class, upper pattern): pair_rows_kernel
+  const uint32_t *low;           // [n_cls] representative of the class
+  const uint32_t *row0;          // [n_cls + 1] first row of the class
+  const uint32_t *slice0;        // [n_cls + 1] first 32-row slice of the class
+  uint32_t n_slices;
+  const uint32_t *row_b;         // upper pattern
+  const uint32_t *row_i;         // basis index
+  const uint16_t *row_m;         // weight of the row's configuration (meta of its slot)
+  const double2 *rw;             // conj(chi) / sqrt(t) per weight
+  const uint32_t *half_nib;      // antiparallel masks by the halves' nibbles, [half][word][n_hnib][16]
+  uint32_t n_hnib;
+  uint32_t off_et, et_words;
+  uint32_t *next;                // work counter, zeroed by expand_kernel
 };
 
 constexpr int kThreads = 512;
 constexpr int kMinBlocks = 2;
+constexpr int kRowThreads = 1024;      // pair_rows_kernel
+constexpr int kRowBlocks = 1;
+constexpr int kRowU = 4;
+constexpr int64_t kRowOrderMinDim = 1 << 21;
+constexpr size_t kRowOrderMinBytes = (size_t)24 << 20;
 
 template <typename T>
 __device__ __forceinline__ void cpy(unsigned char *sm, uint32_t off, const T *g, uint32_t n) {
@@ -178,31 +197,31 @@ template <> struct Acc<float2> {
 struct PairSm {
   const uint32_t *off;
   const uint8_t *mult;
-  const uint2 *bond;
+  const uint32_t *fa, *fb;   // bits flipped in A and in B, per padded bond
 };
 
-// U terms of the row (A, B) given by their bonds; chi and the sum per term
+// U terms of a row, given by the half-table entries of the exchanged configurations: the
+// first nu of them are added to acc
 template <typename V, bool kChi, bool kFlips, int U>
-__device__ __forceinline__ void pair_terms(const PairParams &P, const PairSm &S, uint32_t A,
-                                           uint32_t B, const int (&kb)[U], int nu, const V *xs,
+__device__ __forceinline__ void pair_terms(const PairParams &P, const PairSm &S, const uint32_t (&ea)[U],
+                                           const uint32_t (&eb)[U], int nu, const V *xs,
                                            const unsigned char *chi_sm, Acc<V> &acc) {
-  uint32_t ea[U], eb[U];
-#pragma unroll
-  for (int u = 0; u < U; u++) {
-    const uint2 f = S.bond[kb[u]];
-    ea[u] = __ldg(P.ta + (A ^ f.x));
-    eb[u] = __ldg(P.tb + (B ^ f.y));
-  }
   V v[U];
-  uint32_t lo[U], hi[U], slot[U];
+  float vl[U];
+  uint32_t lo[U];
 #pragma unroll
   for (int u = 0; u < U; u++) {
     lo[u] = min(ea[u], eb[u]);
-    hi[u] = max(ea[u], eb[u]);
-    const uint32_t mi = (lo[u] & kElem) * P.h0 + (hi[u] & kElem) + (ea[u] <= eb[u] ? 0u : P.sel_off);
-    slot[u] = S.off[lo[u] >> kClassShift] + P.K * (hi[u] >> kClassShift) + S.mult[mi];
-    if (kFlips) slot[u] += ((lo[u] ^ hi[u]) & kFlip) ? P.h0 : 0u;
-    v[u] = ld_slot(xs + slot[u]);
+    const uint32_t hi = max(ea[u], eb[u]);
+    const uint32_t mi = (lo[u] & kElem) * P.h0 + (hi & kElem) + (ea[u] <= eb[u] ? 0u : P.sel_off);
+    uint32_t slot = S.off[lo[u] >> kClassShift] + P.K * (hi >> kClassShift) + S.mult[mi];
+    if (kFlips) slot += ((lo[u] ^ hi) & kFlip) ? P.h0 : 0u;
+    v[u] = ld_slot(xs + slot);
+    vl[u] = 0.f;
+    if constexpr (std::is_same<V, float>::value) {
+      // |Stab| > 1 needs a stabiliser on both halves, or halves that can be exchanged
+      if (P.xslo && ((lo[u] & hi & kSpecial) || ((lo[u] ^ hi) >> kClassShift) == 0)) vl[u] = __ldg(P.xslo + slot);
+    }
   }
 #pragma unroll
   for (int u = 0; u < U; u++) {
@@ -216,32 +235,30 @@ __device__ __forceinline__ void pair_terms(const PairParams &P, const PairSm &S,
       } else {
         const uint32_t neg = (lo[u] >> kSignBit) & 1u;
         acc.add(v[u], neg);
-        if constexpr (std::is_same<V, float>::value) {
-          // |Stab| > 1 needs a stabiliser on both halves, or halves that can be exchanged
-          if (P.xslo && ((lo[u] & hi[u] & kSpecial) || ((lo[u] ^ hi[u]) >> kClassShift) == 0))
-            acc.add_lo(__ldg(P.xslo + slot[u]), neg);
-        }
+        if constexpr (std::is_same<V, float>::value) acc.add_lo(vl[u], neg);
       }
     }
   }
 }
 
-template <typename V, bool kChi, bool kFlips>
-__global__ void __launch_bounds__(kThreads, kMinBlocks) pair_kernel(const __grid_constant__ PairParams P) {
-  using A_ = typename Pv<V>::A;
-  constexpr bool kC = Pv<V>::cplx;
-  constexpr bool kF = sizeof(A_) == 4;
-  extern __shared__ __align__(16) unsigned char sm[];
+// The tables of the product in shared memory (not the masks and, in pair_rows_kernel, the
+// per-warp tables).
+template <typename V, bool kChi>
+__device__ __forceinline__ PairSm pair_stage(const PairParams &P, unsigned char *sm) {
   cpy(sm, P.off_off, P.off, P.n_cls);
   cpy(sm, P.off_mult, reinterpret_cast<const uint32_t *>(P.mult), P.mult_bytes / 4);
   const int n_words = P.cls_word[P.n_classes];
-  cpy(sm, P.off_bond, P.bond, (uint32_t)n_words * 32);
-  cpy(sm, P.off_nib, P.nib, (uint32_t)n_words * P.n_nib * 16);
+  uint32_t *fa = reinterpret_cast<uint32_t *>(sm + P.off_bond), *fb = fa + n_words * 32;
+  for (int k = threadIdx.x; k < n_words * 32; k += blockDim.x) {
+    const uint2 f = P.bond[k];
+    fa[k] = f.x;
+    fb[k] = f.y;
+  }
   cpy(sm, P.off_rs, P.rsqrt_tab, P.n_sq);
   if constexpr (kChi) {
     for (uint32_t k = threadIdx.x; k < P.n_chi; k += blockDim.x) {
       const double c = P.chi[2 * k], s = P.chi[2 * k + 1];
-      if constexpr (kF) {
+      if constexpr (sizeof(typename Pv<V>::A) == 4) {
         const float ch = (float)c, sh = (float)s;
         reinterpret_cast<float4 *>(sm + P.off_chi)[k] = make_float4(ch, (float)(c - (double)ch), sh, (float)(s - (double)sh));
       } else {
@@ -249,17 +266,95 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) pair_kernel(const __grid
       }
     }
   }
-  __syncthreads();
   PairSm S;
   S.off = reinterpret_cast<const uint32_t *>(sm + P.off_off);
   S.mult = sm + P.off_mult;
-  S.bond = reinterpret_cast<const uint2 *>(sm + P.off_bond);
+  S.fa = fa;
+  S.fb = fb;
+  return S;
+}
+
+// y_i in fp64, rounded once to the vector type; for fp32 vectors the rounding's remainder
+// goes to ylo when asked, and <x, y> then uses the unrounded value
+template <typename V>
+__device__ __forceinline__ void pair_store(const PairParams &P, const V *x, V *y, int64_t i, double diag,
+                                           double rs, double row_re, double row_im, double &dot_re,
+                                           double &dot_im) {
+  using A_ = typename Pv<V>::A;
+  constexpr bool kF = sizeof(A_) == 4;
+  if constexpr (!Pv<V>::cplx) {
+    const double xi = (double)x[i];
+    const double yd = diag * xi + row_re * rs;
+    const A_ yi = (A_)yd;
+    __stcs(y + (i - P.r0), yi);
+    if (kF && P.ylo) reinterpret_cast<float *>(P.ylo)[i - P.r0] = (float)(yd - (double)yi);
+    if (P.partial) dot_re += xi * (kF && P.ylo ? yd : (double)yi);
+  } else {
+    const V xv = x[i];
+    const double yr = diag * (double)xv.x + row_re * rs;
+    const double yim = diag * (double)xv.y + row_im * rs;
+    V yv;
+    yv.x = (A_)yr;
+    yv.y = (A_)yim;
+    y[i - P.r0] = yv;
+    double ur = (double)yv.x, ui = (double)yv.y;
+    if (kF && P.ylo) {
+      float2 l;
+      l.x = (float)(yr - ur);
+      l.y = (float)(yim - ui);
+      reinterpret_cast<float2 *>(P.ylo)[i - P.r0] = l;
+      ur = yr;
+      ui = yim;
+    }
+    if (P.partial) {
+      dot_re += (double)xv.x * ur + (double)xv.y * ui;
+      dot_im += (double)xv.x * ui - (double)xv.y * ur;
+    }
+  }
+}
+
+// per-block <x, y> in a fixed order
+template <bool kC, int kT>
+__device__ __forceinline__ void pair_dot(const PairParams &P, double dot_re, double dot_im) {
+  if (!P.partial) return;
+  __shared__ double red[kT / 32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (int part = 0; part < (kC ? 2 : 1); part++) {
+    double d = part ? dot_im : dot_re;
+    for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xFFFFFFFFu, d, o);
+    __syncthreads();
+    if (lane == 0) red[wid] = d;
+    __syncthreads();
+    if (wid == 0) {
+      d = lane < kT / 32 ? red[lane] : 0.0;
+      for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xFFFFFFFFu, d, o);
+      if (lane == 0) P.partial[part * gridDim.x + blockIdx.x] = d;
+    }
+  }
+}
+
+// the next antiparallel bond of a row whose masks of the words of one class lie at mask_s
+template <int kT>
+__device__ __forceinline__ int next_bond(uint32_t &m, int &wd, int w0, const uint32_t *mask_s) {
+  while (m == 0) m = mask_s[(++wd - w0) * kT];
+  const int k = wd * 32 + __ffs(m) - 1;
+  m &= m - 1;
+  return k;
+}
+
+// Rows in basis order: any range of rows, and sectors whose xs stays in L2.
+template <typename V, bool kChi, bool kFlips>
+__global__ void __launch_bounds__(kThreads, kMinBlocks) pair_kernel(const __grid_constant__ PairParams P) {
+  constexpr bool kC = Pv<V>::cplx;
+  constexpr int U = 2;
+  extern __shared__ __align__(16) unsigned char sm[];
+  const PairSm S = pair_stage<V, kChi>(P, sm);
+  cpy(sm, P.off_nib, P.nib, (uint32_t)P.cls_word[P.n_classes] * P.n_nib * 16);
+  __syncthreads();
   const uint32_t *nibs = reinterpret_cast<const uint32_t *>(sm + P.off_nib);
   const double *rsd = reinterpret_cast<const double *>(sm + P.off_rs);
   uint32_t *mask_s = reinterpret_cast<uint32_t *>(sm + P.off_mask) + threadIdx.x;
   const V *xs = reinterpret_cast<const V *>(P.xs);
-  const V *x = reinterpret_cast<const V *>(P.x);
-  V *y = reinterpret_cast<V *>(P.y);
   double dot_re = 0.0, dot_im = 0.0;
   const int64_t stride = (int64_t)gridDim.x * kThreads;
   for (int64_t i = P.r0 + (int64_t)blockIdx.x * kThreads + threadIdx.x; i < P.r1; i += stride) {
@@ -280,83 +375,130 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) pair_kernel(const __grid
       Acc<V> acc;
       int wd = w0;
       uint32_t m = w0 < w1 ? mask_s[0] : 0u;
-      for (int left = nanti; left > 0;) {
-        while (m == 0) m = mask_s[(++wd - w0) * kThreads];
-        constexpr int U = 2;
-        int kb[U];
-        kb[0] = wd * 32 + __ffs(m) - 1;
-        m &= m - 1;
-        const int nu = left >= 2 ? 2 : 1;
-        kb[1] = kb[0];
-        if (nu == 2) {
-          while (m == 0) m = mask_s[(++wd - w0) * kThreads];
-          kb[1] = wd * 32 + __ffs(m) - 1;
-          m &= m - 1;
+      for (int left = nanti; left > 0; left -= U) {
+        uint32_t ea[U], eb[U];
+        int kb = 0;
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+          if (u < left) kb = next_bond<kThreads>(m, wd, w0, mask_s);
+          ea[u] = __ldg(P.ta + (A ^ S.fa[kb]));
+          eb[u] = __ldg(P.tb + (B ^ S.fb[kb]));
         }
-        left -= nu;
-        pair_terms<V, kChi, kFlips, U>(P, S, A, B, kb, nu, xs, sm + P.off_chi, acc);
+        pair_terms<V, kChi, kFlips, U>(P, S, ea, eb, left, xs, sm + P.off_chi, acc);
       }
       row_re += P.jh[c] * acc.re();
       if constexpr (kC) row_im += P.jh[c] * acc.im();
       diag += P.jzq[c] * (double)(P.nb_cls[c] - 2 * nanti);
     }
-    const double rs = rsd[__ldcs(P.stab + i)];
-    // y_i in fp64, rounded once to the vector type; for fp32 vectors the rounding's
-    // remainder goes to ylo when asked, and <x, y> then uses the unrounded value
-    if constexpr (!kC) {
-      const double xi = (double)x[i];
-      const double yd = diag * xi + row_re * rs;
-      const A_ yi = (A_)yd;
-      __stcs(y + (i - P.r0), yi);
-      if (kF && P.ylo) reinterpret_cast<float *>(P.ylo)[i - P.r0] = (float)(yd - (double)yi);
-      if (P.partial) dot_re += xi * (kF && P.ylo ? yd : (double)yi);
-    } else {
-      const V xv = x[i];
-      const double yr = diag * (double)xv.x + row_re * rs;
-      const double yim = diag * (double)xv.y + row_im * rs;
-      V yv;
-      yv.x = (A_)yr;
-      yv.y = (A_)yim;
-      y[i - P.r0] = yv;
-      double ur = (double)yv.x, ui = (double)yv.y;
-      if (kF && P.ylo) {
-        float2 l;
-        l.x = (float)(yr - ur);
-        l.y = (float)(yim - ui);
-        reinterpret_cast<float2 *>(P.ylo)[i - P.r0] = l;
-        ur = yr;
-        ui = yim;
-      }
-      if (P.partial) {
-        dot_re += (double)xv.x * ur + (double)xv.y * ui;
-        dot_im += (double)xv.x * ui - (double)xv.y * ur;
-      }
-    }
+    pair_store<V>(P, reinterpret_cast<const V *>(P.x), reinterpret_cast<V *>(P.y), i, diag,
+                  rsd[__ldcs(P.stab + i)], row_re, row_im, dot_re, dot_im);
   }
-  if (P.partial) {
-    __shared__ double red[kThreads / 32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int part = 0; part < (kC ? 2 : 1); part++) {
-      double d = part ? dot_im : dot_re;
-      for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xFFFFFFFFu, d, o);
-      __syncthreads();
-      if (lane == 0) red[wid] = d;
-      __syncthreads();
-      if (wid == 0) {
-        d = lane < kThreads / 32 ? red[lane] : 0.0;
-        for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xFFFFFFFFu, d, o);
-        if (lane == 0) P.partial[part * gridDim.x + blockIdx.x] = d;
-      }
+  pair_dot<kC, kThreads>(P, dot_re, dot_im);
+}
+
+// Rows in the order of (lower class, upper pattern), for products whose xs is larger than the
+// L2 keeps.  In basis order the gathers of xs are random over the whole vector: on the 6x6
+// sector 59 bytes of DRAM traffic per gathered fp32 value and 77% of the DRAM's peak.  Rows
+// that share the lower half A reach few places: the exchanged half A' takes at most one value
+// per bond, and while class(A') stays the lower one the gather falls into that class's block
+// of slots; the whole GPU works on a few lower classes at a time, whose blocks stay in L2.
+// The half-table entries of A' are a table of the warp (one entry per bond), rows with
+// neighbouring upper patterns share the cache lines of the other half table.
+template <typename V, bool kChi, bool kFlips>
+__global__ void __launch_bounds__(kRowThreads, kRowBlocks) pair_rows_kernel(const __grid_constant__ PairParams P) {
+  constexpr bool kC = Pv<V>::cplx;
+  constexpr int U = kRowU;
+  extern __shared__ __align__(16) unsigned char sm[];
+  const PairSm S = pair_stage<V, kChi>(P, sm);
+  const int n_words = P.cls_word[P.n_classes];
+  cpy(sm, P.off_nib, P.half_nib, (uint32_t)n_words * P.n_hnib * 32);
+  __syncthreads();
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const uint32_t *nibA = reinterpret_cast<const uint32_t *>(sm + P.off_nib), *nibB = nibA + n_words * P.n_hnib * 16;
+  uint32_t *mask_s = reinterpret_cast<uint32_t *>(sm + P.off_mask) + threadIdx.x;
+  uint32_t *et = reinterpret_cast<uint32_t *>(sm + P.off_et) + wid * P.et_words;   // entries of A' by bond
+  uint32_t *ma = et + n_words * 32;                                                // masks of A by word
+  const V *xs = reinterpret_cast<const V *>(P.xs);
+  double dot_re = 0.0, dot_im = 0.0;
+  uint32_t cur = 0xFFFFFFFFu;
+  __shared__ uint32_t chunk_s;
+  for (;;) {
+    __syncthreads();
+    if (threadIdx.x == 0) chunk_s = atomicAdd(P.next, 1u);
+    __syncthreads();
+    if (chunk_s * (kRowThreads / 32) >= P.n_slices) break;
+    const uint32_t sl = chunk_s * (kRowThreads / 32) + wid;
+    if (sl >= P.n_slices) continue;
+    uint32_t lo = 0, hi = P.n_cls - 1;
+    while (lo < hi) {   // the last class that starts at or before the slice
+      const uint32_t mid = (lo + hi + 1) >> 1;
+      if (__ldg(P.slice0 + mid) <= sl) lo = mid; else hi = mid - 1;
     }
+    if (lo != cur) {
+      cur = lo;
+      const uint32_t A = __ldg(P.low + lo);
+      __syncwarp();
+      for (int k = lane; k < n_words * 32; k += 32) et[k] = __ldg(P.ta + (A ^ S.fa[k]));
+      for (int wd = lane; wd < n_words; wd += 32) {
+        uint32_t m = 0;
+        for (uint32_t q = 0; q < P.n_hnib; q++) m ^= nibA[(wd * P.n_hnib + q) * 16 + ((A >> (4 * q)) & 15u)];
+        ma[wd] = m;
+      }
+      __syncwarp();
+    }
+    const uint32_t r = __ldg(P.row0 + lo) + (sl - __ldg(P.slice0 + lo)) * 32 + lane;
+    if (r >= __ldg(P.row0 + lo + 1)) continue;
+    const uint32_t B = __ldcs(P.row_b + r);
+    double diag = 0.0, row_re = 0.0, row_im = 0.0;
+    for (int c = 0; c < P.n_classes; c++) {
+      const int w0 = P.cls_word[c], w1 = P.cls_word[c + 1];
+      int nanti = 0;
+      for (int wd = w0; wd < w1; wd++) {
+        uint32_t m = ma[wd];
+        const uint32_t *nw = nibB + (uint32_t)wd * P.n_hnib * 16;
+        for (uint32_t q = 0; q < P.n_hnib; q++) m ^= nw[q * 16 + ((B >> (4 * q)) & 15u)];
+        nanti += __popc(m);
+        mask_s[(wd - w0) * kRowThreads] = m;
+      }
+      Acc<V> acc;
+      int wd = w0;
+      uint32_t m = w0 < w1 ? mask_s[0] : 0u;
+      for (int left = nanti; left > 0; left -= U) {
+        uint32_t ea[U], eb[U];
+        int kb = 0;
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+          if (u < left) kb = next_bond<kRowThreads>(m, wd, w0, mask_s);
+          ea[u] = et[kb];
+          eb[u] = __ldg(P.tb + (B ^ S.fb[kb]));
+        }
+        pair_terms<V, kChi, kFlips, U>(P, S, ea, eb, left, xs, sm + P.off_chi, acc);
+      }
+      row_re += P.jh[c] * acc.re();
+      if constexpr (kC) row_im += P.jh[c] * acc.im();
+      diag += P.jzq[c] * (double)(P.nb_cls[c] - 2 * nanti);
+    }
+    // the sums belong to the configuration (R(lower), upper): conj(chi(h2)) takes them to the
+    // representative h2 carries it to
+    const double2 rw = __ldg(P.rw + __ldcs(P.row_m + r));
+    if constexpr (kChi) {
+      const double t = row_re * rw.x - row_im * rw.y;
+      row_im = row_re * rw.y + row_im * rw.x;
+      row_re = t;
+    }
+    pair_store<V>(P, reinterpret_cast<const V *>(P.x), reinterpret_cast<V *>(P.y), (int64_t)__ldcs(P.row_i + r), diag,
+                  kChi ? 1.0 : rw.x, row_re, row_im, dot_re, dot_im);
   }
+  pair_dot<kC, kRowThreads>(P, dot_re, dot_im);
 }
 
 // xs[p] = w(meta[p]) x[idx[p]], w = chi sqrt(t); meta 0 is w = 1.  fp32 real vectors keep
 // the rounding's remainder in xslo, so that a weight sqrt(t) costs no precision.
 template <typename V>
 __global__ void __launch_bounds__(256) expand_kernel(const V *x, const uint32_t *idx, const uint16_t *meta,
-                                                     const double2 *w, uint32_t n, V *xs, float *xslo) {
+                                                     const double2 *w, uint32_t n, V *xs, float *xslo, uint32_t *next) {
   using A_ = typename Pv<V>::A;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *next = 0;
   for (uint32_t p = blockIdx.x * 256 + threadIdx.x; p < n; p += gridDim.x * 256) {
     const uint32_t j = __ldcs(idx + p);
     const uint32_t mt = __ldcs(meta + p);
@@ -431,19 +573,112 @@ __global__ void half_entries(const uint32_t *rep, const uint32_t *first, const u
            code[first[u] & 0x7FFFFFFFu];
 }
 
+// The rows in slot-friendly order.  Candidates are (lower class c, pattern b of the other half
+// with the right number of up spins, in increasing order), in chunks of 1024 of one class; a
+// warp owns a chunk.  A candidate stands for the basis state of its slot.  Only a class with
+// a stabiliser, or two halves of one class, give the same state several candidates: those
+// claim it with their position, the lowest wins.
+struct RowEnum {
+  const uint32_t *ta, *tb, *low, *off, *chunk0, *list0, *list_n, *plist, *idx;
+  const uint8_t *mult;
+  uint32_t n_cls, n_chunks, K, h0;
+  uint32_t *first;       // [D] lowest claiming candidate
+  uint32_t *bits;        // [n_chunks][32] which candidates are rows
+  uint32_t *count;       // [n_chunks]
+  const uint64_t *at;    // [n_chunks] first row of the chunk
+  const uint16_t *meta;
+  uint32_t *row_b, *row_i;
+  uint16_t *row_m;
+};
+
+enum RowPass { kClaim, kCount, kFill };
+
+template <RowPass kPass>
+__global__ void __launch_bounds__(256) enum_rows(const RowEnum Q) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t nw = gridDim.x * (blockDim.x / 32);
+  for (uint32_t ch = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32; ch < Q.n_chunks; ch += nw) {
+    uint32_t lo = 0, hi = Q.n_cls - 1;
+    while (lo < hi) {
+      const uint32_t mid = (lo + hi + 1) >> 1;
+      if (__ldg(Q.chunk0 + mid) <= ch) lo = mid; else hi = mid - 1;
+    }
+    const uint32_t ea = __ldg(Q.ta + __ldg(Q.low + lo)), off = __ldg(Q.off + lo);
+    const uint32_t j0 = (ch - __ldg(Q.chunk0 + lo)) * 1024, n = __ldg(Q.list_n + lo), l0 = __ldg(Q.list0 + lo);
+    uint32_t total = 0;
+    uint64_t w = kPass == kFill ? Q.at[ch] : 0;
+    for (int step = 0; step < 32; step++) {
+      const uint32_t j = j0 + step * 32 + lane;
+      if (j0 + step * 32 >= n) {
+        if (kPass == kCount && lane == 0) Q.bits[ch * 32 + step] = 0;
+        continue;
+      }
+      uint32_t bits = 0;
+      if (kPass == kFill) {
+        bits = Q.bits[ch * 32 + step];
+        if (bits == 0) continue;
+      }
+      bool row = j < n && (kPass != kFill || ((bits >> lane) & 1u));
+      uint32_t i = 0, b = 0, slot = 0;
+      if (row) {
+        b = __ldg(Q.plist + l0 + j);
+        const uint32_t eb = __ldg(Q.tb + b);
+        row = (eb >> kClassShift) >= (ea >> kClassShift);
+        if (row) {
+          slot = off + Q.K * (eb >> kClassShift) + Q.mult[(ea & kElem) * Q.h0 + (eb & kElem)] +
+                                (((ea ^ eb) & kFlip) ? Q.h0 : 0u);
+          i = __ldg(Q.idx + slot);
+          row = i != 0xFFFFFFFFu;
+          if (row && kPass != kFill && ((ea & kSpecial) || ((ea ^ eb) >> kClassShift) == 0)) {
+            const uint32_t e = ch * 1024 + step * 32 + lane;
+            if (kPass == kClaim) atomicMin(Q.first + i, e);
+            else row = Q.first[i] == e;
+          }
+        }
+      }
+      if (kPass == kCount) {
+        const uint32_t m = __ballot_sync(0xFFFFFFFFu, row);
+        if (lane == 0) Q.bits[ch * 32 + step] = m;
+        total += __popc(m);
+      }
+      if (kPass == kFill) {
+        if (row) {
+          const uint64_t at = w + __popc(bits & ((1u << lane) - 1u));
+          Q.row_b[at] = b;
+          Q.row_i[at] = i;
+          Q.row_m[at] = __ldg(Q.meta + slot);
+        }
+        w += __popc(bits);
+      }
+    }
+    if (kPass == kCount && lane == 0) Q.count[ch] = total;
+  }
+}
+
+__global__ void class_rows(const uint64_t *at, const uint32_t *chunk0, uint32_t n_cls, uint32_t n_chunks,
+                           uint32_t total, uint32_t *row0) {
+  for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c <= n_cls; c += gridDim.x * blockDim.x)
+    row0[c] = c == n_cls || chunk0[c] >= n_chunks ? total : (uint32_t)at[chunk0[c]];
+}
+
 }  // namespace
 
 struct PairPlan {
   int n = 0, m = 0;
   int shA0 = 0, shA1 = 0, shB0 = 0, shB1 = 0;
   uint32_t bmask_hi = 0, bmask = 0;
-  uint32_t n_cls = 0, K = 0, h0 = 0, sel_off = 0, mult_bytes = 0, n_slots = 0, n_w = 0;
+  uint32_t n_cls = 0, K = 0, h0 = 0, sel_off = 0, mult_bytes = 0, n_slots = 0;
+  uint32_t n_hnib = 0, hnib_len = 0, n_slices = 0;
   bool flips = false, weights = false;
-  uint32_t *d_ta = nullptr, *d_tb = nullptr, *d_off = nullptr, *d_idx = nullptr;
-  uint8_t *d_mult = nullptr;
-  uint2 *d_bond = nullptr;
-  double *d_chi = nullptr, *d_w = nullptr;
-  uint16_t *d_meta = nullptr;
+  // device: the half tables, the small tables, the slots' indices and weights, the rows
+  void *d_half = nullptr, *d_small = nullptr, *d_slots = nullptr, *d_rows = nullptr;
+  uint32_t *ta = nullptr, *tb = nullptr, *off = nullptr, *idx = nullptr, *low = nullptr, *half_nib = nullptr;
+  uint32_t *row0 = nullptr, *slice0 = nullptr, *row_b = nullptr, *row_i = nullptr;
+  uint16_t *row_m = nullptr;
+  uint8_t *mult = nullptr;
+  uint2 *bond = nullptr;
+  double *chi = nullptr, *w = nullptr, *rw = nullptr;
+  uint16_t *meta = nullptr;
   cudaMemPool_t pool = nullptr;   // xs of the calls in flight, stream-ordered
   size_t bytes = 0;
 };
@@ -452,19 +687,120 @@ void ed_free_pair(ed_basis *B) {
   PairPlan *p = B->pair;
   B->pair = nullptr;
   if (!p) return;
-  for (void *q : {(void *)p->d_ta, (void *)p->d_tb, (void *)p->d_off, (void *)p->d_idx, (void *)p->d_mult,
-                  (void *)p->d_bond, (void *)p->d_chi, (void *)p->d_w, (void *)p->d_meta})
+  for (void *q : {p->d_half, p->d_small, p->d_slots, p->d_rows})
     if (q) cudaFree(q);
   if (p->pool) cudaMemPoolDestroy(p->pool);
   delete p;
 }
+
+namespace {
+
+// host tables gathered into one upload; at(k) is table k's place in it
+struct Blob {
+  std::vector<unsigned char> bytes;
+  template <typename T> size_t add(const T *v, size_t n) {
+    const size_t o = (bytes.size() + 15) / 16 * 16;
+    bytes.resize(o + sizeof(T) * n);
+    if (n) memcpy(bytes.data() + o, v, sizeof(T) * n);
+    return o;
+  }
+  template <typename T> size_t add(const std::vector<T> &v) { return add(v.data(), v.size()); }
+};
+
+// stream-ordered scratch of the build, returned on every path
+struct Scratch {
+  cudaStream_t st;
+  std::vector<void *> v;
+  explicit Scratch(cudaStream_t s) : st(s) {}
+  ~Scratch() { for (void *q : v) cudaFreeAsync(q, st); }
+  void *get(size_t bytes) {
+    void *q = nullptr;
+    if (cudaMallocAsync(&q, std::max<size_t>(bytes, 16), st) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    v.push_back(q);
+    return q;
+  }
+};
+
+// Row order for large sectors (see pair_rows_kernel); p->n_slices stays 0 when it is not made.
+int build_rows(ed_basis *B, PairPlan *p, const std::vector<uint32_t> &low, const std::vector<uint32_t> &off,
+               cudaStream_t st) {
+  const uint32_t nA = p->n_cls, total = 1u << p->m;
+  std::vector<uint32_t> plist(total), at(p->m + 2, 0);
+  for (uint32_t u = 0; u < total; u++) at[__builtin_popcount(u) + 1]++;
+  for (int q = 0; q <= p->m; q++) at[q + 1] += at[q];
+  std::vector<uint32_t> pos(at.begin(), at.end() - 1);
+  for (uint32_t u = 0; u < total; u++) plist[pos[__builtin_popcount(u)]++] = u;
+  std::vector<uint32_t> list0(nA), list_n(nA), chunk0(nA);
+  uint64_t chunks = 0;
+  for (uint32_t c = 0; c < nA; c++) {
+    const int want = B->n_up - __builtin_popcount(low[c]);
+    list0[c] = list_n[c] = 0;
+    if (want >= 0 && want <= p->m) { list0[c] = at[want]; list_n[c] = at[want + 1] - at[want]; }
+    chunk0[c] = (uint32_t)chunks;
+    chunks += (list_n[c] + 1023) / 1024;
+  }
+  if (chunks >= (1u << 22) || chunks == 0) return ED_OK;
+  Blob blob;
+  const size_t o_pl = blob.add(plist), o_l0 = blob.add(list0), o_ln = blob.add(list_n), o_c0 = blob.add(chunk0);
+  Scratch sc(st);
+  unsigned char *d = (unsigned char *)sc.get(blob.bytes.size());
+  uint32_t *d_first = (uint32_t *)sc.get(4 * (size_t)B->D), *d_bits = (uint32_t *)sc.get(128 * chunks);
+  uint32_t *d_count = (uint32_t *)sc.get(4 * chunks);
+  uint64_t *d_at = (uint64_t *)sc.get(8 * chunks);
+  if (!d || !d_first || !d_bits || !d_count || !d_at) return ED_OK;
+  const size_t rows_bytes = 10 * (size_t)B->D + 8 * ((size_t)nA + 1);
+  if (cudaMalloc(&p->d_rows, rows_bytes) != cudaSuccess) { cudaGetLastError(); p->d_rows = nullptr; return ED_OK; }
+  p->row_b = (uint32_t *)p->d_rows;
+  p->row_i = p->row_b + B->D;
+  p->row0 = p->row_i + B->D;
+  p->slice0 = p->row0 + nA + 1;
+  p->row_m = (uint16_t *)(p->slice0 + nA + 1);
+  ED_CK(cudaMemcpyAsync(d, blob.bytes.data(), blob.bytes.size(), cudaMemcpyHostToDevice, st));
+  ED_CK(cudaMemsetAsync(d_first, 0xFF, 4 * (size_t)B->D, st));
+  RowEnum Q{};
+  Q.ta = p->ta; Q.tb = p->tb; Q.low = p->low; Q.off = p->off; Q.idx = p->idx; Q.mult = p->mult;
+  Q.plist = (const uint32_t *)(d + o_pl); Q.list0 = (const uint32_t *)(d + o_l0);
+  Q.list_n = (const uint32_t *)(d + o_ln); Q.chunk0 = (const uint32_t *)(d + o_c0);
+  Q.n_cls = nA; Q.n_chunks = (uint32_t)chunks; Q.K = p->K; Q.h0 = p->h0;
+  Q.first = d_first; Q.bits = d_bits; Q.count = d_count; Q.at = d_at; Q.meta = p->meta;
+  Q.row_b = p->row_b; Q.row_i = p->row_i; Q.row_m = p->row_m;
+  const int grid = (int)std::min<uint64_t>((chunks + 7) / 8, (uint64_t)B->sm_count * 8);
+  enum_rows<kClaim><<<grid, 256, 0, st>>>(Q);
+  ED_CK(cudaGetLastError());
+  enum_rows<kCount><<<grid, 256, 0, st>>>(Q);
+  ED_CK(cudaGetLastError());
+  uint64_t found = 0;
+  int rc = ed_exclusive_scan(d_count, chunks, d_at, &found, st);
+  if (rc) return rc;
+  if (found != (uint64_t)B->D) return ed_fail(ED_ERR_CUDA, "row order does not cover the basis");
+  enum_rows<kFill><<<grid, 256, 0, st>>>(Q);
+  ED_CK(cudaGetLastError());
+  class_rows<<<16, 256, 0, st>>>(d_at, Q.chunk0, nA, Q.n_chunks, (uint32_t)B->D, p->row0);
+  ED_CK(cudaGetLastError());
+  std::vector<uint32_t> row0(nA + 1), slice0(nA + 1);
+  ED_CK(cudaMemcpyAsync(row0.data(), p->row0, 4 * ((size_t)nA + 1), cudaMemcpyDeviceToHost, st));
+  ED_CK(cudaStreamSynchronize(st));
+  uint64_t sl = 0;
+  for (uint32_t c = 0; c < nA; c++) {
+    slice0[c] = (uint32_t)sl;
+    sl += (row0[c + 1] - row0[c] + 31) / 32;
+  }
+  slice0[nA] = (uint32_t)sl;
+  ED_CK(cudaMemcpyAsync(p->slice0, slice0.data(), 4 * ((size_t)nA + 1), cudaMemcpyHostToDevice, st));
+  ED_CK(cudaStreamSynchronize(st));
+  p->n_slices = (uint32_t)sl;
+  p->bytes += rows_bytes;
+  return ED_OK;
+}
+
+}  // namespace
 
 // Builds B->pair when the sector admits it; leaves it null (the search kernels serve the
 // sector) when the split has no two stable halves, the tables would be too large, or device
 // memory is short.  Only CUDA failures other than out-of-memory are errors.
 int ed_build_pair(ed_basis *B, cudaStream_t st) {
   const int nsub = B->nsub, n = B->n, ns = B->nsym, N = B->N;
-  if (!B->two_level || (nsub != 2 && nsub != 4) || B->D == 0 || ns > 1024 || N > 44) return ED_OK;
+  if (!B->two_level || (nsub != 2 && nsub != 4) || B->D == 0 || ns > 1000 || N > 44) return ED_OK;
   const int m = N / 2;
   std::vector<uint8_t> dest((size_t)ns * nsub);
   for (int g = 0; g < ns; g++)
@@ -607,40 +943,33 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
     p->bmask = (1u << n) - 1u;
     p->bmask_hi = 0;
   }
-  struct Scratch {   // device scratch of the build, freed on every path
-    std::vector<void *> v;
-    ~Scratch() { for (void *q : v) cudaFree(q); }
-  } scratch;
-  bool oom = false;
-  auto dev = [&](size_t bytes, bool keep) -> void * {
+  Scratch sc(st);
+  auto keep = [&](size_t bytes) -> void * {
     void *q = nullptr;
-    if (oom || cudaMalloc(&q, std::max<size_t>(bytes, 16)) != cudaSuccess) {
-      cudaGetLastError();
-      oom = true;
-      return nullptr;
-    }
-    if (keep) p->bytes += bytes; else scratch.v.push_back(q);
+    if (cudaMalloc(&q, bytes) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    p->bytes += bytes;
     return q;
   };
   const uint32_t total = 1u << m;
-  uint32_t *d_rep = (uint32_t *)dev((size_t)total * 4, false), *d_first = (uint32_t *)dev((size_t)total * 4, false);
-  uint32_t *d_id = (uint32_t *)dev((size_t)total * 4, false), *d_reps = (uint32_t *)dev((size_t)total * 4, false);
-  uint16_t *d_list = (uint16_t *)dev(listA.size() * 8, false);
-  p->d_ta = (uint32_t *)dev((size_t)total * 4, true);
-  p->d_tb = (uint32_t *)dev((size_t)total * 4, true);
-  if (oom) { ed_free_pair(B); return ED_OK; }
   const size_t nl = listA.size();
-  ED_CK(cudaMemcpyAsync(d_list, listA.data(), nl * 2, cudaMemcpyHostToDevice, st));
-  ED_CK(cudaMemcpyAsync(d_list + nl, listB.data(), nl * 2, cudaMemcpyHostToDevice, st));
-  ED_CK(cudaMemcpyAsync(d_list + 2 * nl, codeA.data(), nl * 2, cudaMemcpyHostToDevice, st));
-  ED_CK(cudaMemcpyAsync(d_list + 3 * nl, codeB.data(), nl * 2, cudaMemcpyHostToDevice, st));
+  Blob lists;
+  lists.add(listA); lists.add(listB); lists.add(codeA); lists.add(codeB);
+  const size_t lstep = (nl * 2 + 15) / 16 * 8;   // elements from one list to the next
+  uint32_t *d_rep = (uint32_t *)sc.get(16 * (size_t)total + lists.bytes.size());
+  p->d_half = keep(8 * (size_t)total);
+  if (!d_rep || !p->d_half) { ed_free_pair(B); return ED_OK; }
+  uint32_t *d_first = d_rep + total, *d_id = d_first + total, *d_reps = d_id + total;
+  uint16_t *d_list = (uint16_t *)(d_reps + total);
+  p->ta = (uint32_t *)p->d_half;
+  p->tb = p->ta + total;
+  ED_CK(cudaMemcpyAsync(d_list, lists.bytes.data(), lists.bytes.size(), cudaMemcpyHostToDevice, st));
   const int gt = (int)std::min<uint32_t>((total + 255) / 256, (uint32_t)B->sm_count * 8);
   std::vector<uint32_t> rep(total);
   std::vector<std::vector<uint32_t>> cls(2);      // representatives of half A's (and B's) classes
   std::vector<uint32_t> bucket0[2];               // first class of each popcount
   for (int half = 0; half < 2; half++) {
     HalfParams Q{(const uint16_t *)B->d_action, B->d_dest, n, nsub, ns, hb[2 * half], hb[2 * half + 1],
-                 half && !has_swap ? hb[2] : hb[0], d_list + half * nl, (int)nl};
+                 half && !has_swap ? hb[2] : hb[0], d_list + half * lstep, (int)nl};
     half_reps<<<gt, 256, 0, st>>>(Q, total, d_rep, d_first);
     ED_CK(cudaGetLastError());
     if (half == 0 || !has_swap) {
@@ -665,7 +994,7 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
       class_ids<<<gt, 256, 0, st>>>(d_reps, nc, half ? (uint32_t)cls[0].size() : 0u, d_id);
       ED_CK(cudaGetLastError());
     }
-    half_entries<<<gt, 256, 0, st>>>(d_rep, d_first, d_id, d_list + (2 + half) * nl, total, half ? p->d_tb : p->d_ta);
+    half_entries<<<gt, 256, 0, st>>>(d_rep, d_first, d_id, d_list + (2 + half) * lstep, total, half ? p->tb : p->ta);
     ED_CK(cudaGetLastError());
   }
   const uint32_t nA = (uint32_t)cls[0].size();
@@ -700,9 +1029,9 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
   std::vector<uint8_t> tcode(ns + 1, 0);
   std::vector<int> divs;
   for (int t = 1; t <= ns; t++) if (ns % t == 0) { tcode[t] = (uint8_t)divs.size(); divs.push_back(t); }
-  p->n_w = (uint32_t)(B->denom * divs.size());
-  if (p->n_w > 65535 || divs.size() > 255) { ed_free_pair(B); return ED_OK; }
-  std::vector<double> wt(2 * (size_t)p->n_w);
+  const size_t n_w = (size_t)B->denom * divs.size();
+  if (n_w > 65535 || divs.size() > 255) { ed_free_pair(B); return ED_OK; }
+  std::vector<double> wt(2 * n_w), rwt(2 * n_w);   // and conj(chi) / sqrt(t)
   for (size_t t = 0; t < divs.size(); t++)
     for (int q = 0; q < B->denom; q++) {
       const double a = 2.0 * M_PI * (double)q / (double)B->denom, r = std::sqrt((double)divs[t]);
@@ -710,6 +1039,8 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
       if (B->is_real) { c = q ? -1.0 : 1.0; s = 0.0; }
       wt[2 * (t * B->denom + q)] = r * c;
       wt[2 * (t * B->denom + q) + 1] = r * s;
+      rwt[2 * (t * B->denom + q)] = c / r;
+      rwt[2 * (t * B->denom + q) + 1] = -s / r;
     }
   // chi of the lower half's element: [half][512] (flip bit above the element number)
   std::vector<double> chi(2 * 1024, 0.0);
@@ -732,38 +1063,43 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
       if (X == hb[0] || X == hb[1]) bond[b].x |= 1u << pos; else bond[b].y |= 1u << pos;
     }
   }
-  p->d_off = (uint32_t *)dev(4 * (size_t)nA, true);
-  p->d_mult = (uint8_t *)dev(mult.size(), true);
-  p->d_bond = (uint2 *)dev(bond.size() * 8, true);
-  p->d_chi = (double *)dev(chi.size() * 8, true);
-  p->d_w = (double *)dev(wt.size() * 8, true);
-  p->d_idx = (uint32_t *)dev((size_t)acc * 4, true);
-  p->d_meta = (uint16_t *)dev((size_t)acc * 2, true);
-  uint32_t *d_start = (uint32_t *)dev(4 * ((size_t)nA + 1), false);
-  uint32_t *d_fup = (uint32_t *)dev(4 * (size_t)nA, false);
-  uint32_t *d_up = (uint32_t *)dev(4 * up.size(), false);
-  uint32_t *d_low = (uint32_t *)dev(4 * (size_t)nA, false);
-  uint8_t *d_tcode = (uint8_t *)dev(tcode.size(), false);
-  uint32_t *d_any = (uint32_t *)dev(4, false);
-  if (oom) { ed_free_pair(B); return ED_OK; }
-  auto put = [&](void *d, const void *s, size_t bytes) { return cudaMemcpyAsync(d, s, bytes, cudaMemcpyHostToDevice, st); };
-  ED_CK(put(p->d_off, off.data(), 4 * (size_t)nA));
-  ED_CK(put(p->d_mult, mult.data(), mult.size()));
-  ED_CK(put(p->d_bond, bond.data(), bond.size() * 8));
-  ED_CK(put(p->d_chi, chi.data(), chi.size() * 8));
-  ED_CK(put(p->d_w, wt.data(), wt.size() * 8));
-  ED_CK(put(d_start, start.data(), 4 * ((size_t)nA + 1)));
-  ED_CK(put(d_fup, first_up.data(), 4 * (size_t)nA));
-  ED_CK(put(d_up, up.data(), 4 * up.size()));
-  ED_CK(put(d_low, cls[0].data(), 4 * (size_t)nA));
-  ED_CK(put(d_tcode, tcode.data(), tcode.size()));
-  ED_CK(cudaMemsetAsync(d_any, 0, 4, st));
+  // antiparallel masks by the halves' nibbles, [half][word][nibble][16] (as the nibble tables
+  // over whole states: bit k is set for every endpoint of bond k that is up)
+  const size_t n_words = bond.size() / 32;
+  p->n_hnib = (uint32_t)(m + 3) / 4;
+  std::vector<uint32_t> hnib(2 * n_words * p->n_hnib * 16, 0u);
+  for (size_t b = 0; b < bond.size(); b++)
+    for (int half = 0; half < 2; half++) {
+      const uint32_t f = half ? bond[b].y : bond[b].x;
+      for (int q = 0; q < m; q++)
+        if ((f >> q) & 1u)
+          for (int v = 0; v < 16; v++)
+            if ((v >> (q % 4)) & 1) hnib[((half * n_words + b / 32) * p->n_hnib + q / 4) * 16 + v] ^= 1u << (b % 32);
+    }
+  Blob blob;
+  const size_t o_off = blob.add(off), o_low = blob.add(cls[0]), o_mult = blob.add(mult), o_bond = blob.add(bond),
+               o_chi = blob.add(chi), o_w = blob.add(wt), o_rw = blob.add(rwt), o_hnib = blob.add(hnib), o_start = blob.add(start),
+               o_fup = blob.add(first_up), o_up = blob.add(up), o_tc = blob.add(tcode);
+  const uint32_t zero = 0;
+  const size_t o_any = blob.add(&zero, 1);
+  p->d_small = keep(blob.bytes.size());
+  p->d_slots = keep(6 * (size_t)acc);
+  if (!p->d_small || !p->d_slots) { ed_free_pair(B); return ED_OK; }
+  unsigned char *sb = (unsigned char *)p->d_small;
+  ED_CK(cudaMemcpyAsync(sb, blob.bytes.data(), blob.bytes.size(), cudaMemcpyHostToDevice, st));
+  p->off = (uint32_t *)(sb + o_off); p->low = (uint32_t *)(sb + o_low); p->mult = sb + o_mult;
+  p->bond = (uint2 *)(sb + o_bond); p->chi = (double *)(sb + o_chi); p->w = (double *)(sb + o_w); p->rw = (double *)(sb + o_rw);
+  p->half_nib = (uint32_t *)(sb + o_hnib);
+  p->idx = (uint32_t *)p->d_slots;
+  p->meta = (uint16_t *)(p->idx + acc);
+  uint32_t *d_any = (uint32_t *)(sb + o_any);
   PairSlots Q{};
-  Q.start = d_start; Q.first_up = d_fup; Q.low = d_low; Q.up = d_up; Q.n_low = nA; Q.n_slots = p->n_slots;
-  Q.K = K; Q.kel = d_list + nl; Q.tcode = d_tcode;
+  Q.start = (uint32_t *)(sb + o_start); Q.first_up = (uint32_t *)(sb + o_fup); Q.low = p->low; Q.up = (uint32_t *)(sb + o_up);
+  Q.n_low = nA; Q.n_slots = p->n_slots;
+  Q.K = K; Q.kel = d_list + lstep; Q.tcode = sb + o_tc;
   for (int q = 0; q < 4; q++) Q.hb[q] = hb[q];
   Q.up_half = has_swap ? 0 : 1;
-  Q.idx = p->d_idx; Q.meta = p->d_meta; Q.any_weight = d_any;
+  Q.idx = p->idx; Q.meta = p->meta; Q.any_weight = d_any;
   int rc = ed_launch_pair_slots(B, Q, st);
   if (rc == ED_ERR_UNSUPPORTED) { ed_free_pair(B); return ED_OK; }
   if (rc) return rc;
@@ -771,6 +1107,9 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
   ED_CK(cudaMemcpyAsync(&any, d_any, 4, cudaMemcpyDeviceToHost, st));
   ED_CK(cudaStreamSynchronize(st));
   p->weights = any != 0;
+  // the row order pays when xs outgrows the L2 and a class fills many warps
+  if (B->D >= kRowOrderMinDim && B->D / nA >= 256)
+    if ((rc = build_rows(B, p, cls[0], off, st))) return rc;
   cudaMemPoolProps props{};
   props.allocType = cudaMemAllocationTypePinned;
   props.location.type = cudaMemLocationTypeDevice;
@@ -781,8 +1120,8 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
     ed_free_pair(B);
     return ED_OK;
   }
-  uint64_t keep = ~0ull;
-  ED_CK(cudaMemPoolSetAttribute(p->pool, cudaMemPoolAttrReleaseThreshold, &keep));
+  uint64_t all = ~0ull;
+  ED_CK(cudaMemPoolSetAttribute(p->pool, cudaMemPoolAttrReleaseThreshold, &all));
   // small sectors: the pool takes its first memory here rather than in the first product,
   // where mapping it would cost several times the product itself
   const size_t first = 8 * (size_t)p->n_slots;
@@ -800,26 +1139,27 @@ namespace {
 size_t al16(size_t x) { return (x + 15) & ~(size_t)15; }
 
 template <typename V, bool kChi, bool kFlips>
-int launch_pair_t(const ed_basis *B, PairParams &P, cudaStream_t st) {
-  auto k = pair_kernel<V, kChi, kFlips>;
+int launch_pair_t(const ed_basis *B, PairParams &P, bool rows, cudaStream_t st) {
+  auto k = rows ? pair_rows_kernel<V, kChi, kFlips> : pair_kernel<V, kChi, kFlips>;
+  const int threads = rows ? kRowThreads : kThreads, per_sm = rows ? kRowBlocks : kMinBlocks;
   ED_CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, P.smem_bytes));
-  const int need = kMinBlocks * ((int)P.smem_bytes + 1536);
+  const int need = per_sm * ((int)P.smem_bytes + 1536);
   const int pct = std::min(100, (need * 100 + 228 * 1024 - 1) / (228 * 1024));
   ED_CK(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, pct));
-  const int64_t blocks = (P.r1 - P.r0 + kThreads - 1) / kThreads;
-  const int grid = (int)std::min<int64_t>(blocks, (int64_t)B->sm_count * kMinBlocks);
+  const int64_t blocks = rows ? ((int64_t)P.n_slices + threads / 32 - 1) / (threads / 32) : (P.r1 - P.r0 + threads - 1) / threads;
+  const int grid = (int)std::min<int64_t>(blocks, (int64_t)B->sm_count * per_sm);
   B->last_apply_grid = grid;
-  k<<<grid, kThreads, P.smem_bytes, st>>>(P);
+  k<<<grid, threads, P.smem_bytes, st>>>(P);
   ED_CK(cudaGetLastError());
   return ED_OK;
 }
 
 template <typename V>
-int launch_pair_v(const ed_basis *B, PairParams &P, bool chi, bool flips, cudaStream_t st) {
+int launch_pair_v(const ed_basis *B, PairParams &P, bool chi, bool flips, bool rows, cudaStream_t st) {
   if constexpr (Pv<V>::cplx) {
-    if (chi) return flips ? launch_pair_t<V, true, true>(B, P, st) : launch_pair_t<V, true, false>(B, P, st);
+    if (chi) return flips ? launch_pair_t<V, true, true>(B, P, rows, st) : launch_pair_t<V, true, false>(B, P, rows, st);
   }
-  return flips ? launch_pair_t<V, false, true>(B, P, st) : launch_pair_t<V, false, false>(B, P, st);
+  return flips ? launch_pair_t<V, false, true>(B, P, rows, st) : launch_pair_t<V, false, false>(B, P, rows, st);
 }
 
 }  // namespace
@@ -830,6 +1170,8 @@ int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, c
   const PairPlan *p = B->pair;
   if (!p) return ED_ERR_UNSUPPORTED;
   const size_t es = dtype == ED_F64 ? 8 : dtype == ED_F32 ? 4 : dtype == ED_C128 ? 16 : 8;
+  const size_t xs_bytes = al16(es * (size_t)p->n_slots);
+  const bool rows = p->n_slices && r0 == 0 && r1 == B->D && xs_bytes >= kRowOrderMinBytes;
   PairParams P{};
   P.n_classes = B->n_classes;
   int words = 0;
@@ -843,16 +1185,19 @@ int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, c
   P.n = p->n;
   P.shA0 = p->shA0; P.shA1 = p->shA1; P.shB0 = p->shB0; P.shB1 = p->shB1;
   P.bmask_hi = p->bmask_hi; P.bmask = p->bmask;
-  P.ta = p->d_ta; P.tb = p->d_tb; P.off = p->d_off;
+  P.ta = p->ta; P.tb = p->tb; P.off = p->off;
   P.n_cls = p->n_cls; P.K = p->K; P.h0 = p->h0; P.sel_off = p->sel_off;
-  P.mult = p->d_mult; P.mult_bytes = p->mult_bytes;
-  P.bond = p->d_bond;
+  P.mult = p->mult; P.mult_bytes = p->mult_bytes;
+  P.bond = p->bond;
   P.nib = B->d_nib; P.n_nib = (uint32_t)B->n_nib;
+  P.half_nib = p->half_nib; P.n_hnib = p->n_hnib;
   P.rsqrt_tab = B->d_rsqrt; P.n_sq = (uint32_t)B->nsym + 1;
   const bool cplx = dtype == ED_C128 || dtype == ED_C64;
   const bool chi = cplx && !B->is_real;
-  P.chi = p->d_chi; P.n_chi = 1024;
+  P.chi = p->chi; P.n_chi = 1024;
   P.basis = B->d_basis; P.stab = B->d_stab;
+  P.low = p->low; P.row0 = p->row0; P.slice0 = p->slice0; P.n_slices = p->n_slices;
+  P.row_b = p->row_b; P.row_i = p->row_i; P.row_m = p->row_m; P.rw = (const double2 *)p->rw;
   P.x = x; P.y = y; P.r0 = r0; P.r1 = r1; P.partial = partial;
   P.ylo = (dtype == ED_F32 || dtype == ED_C64) ? ylo : nullptr;
   size_t off = 0;
@@ -861,23 +1206,27 @@ int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, c
   put(P.off_off, 4 * (size_t)P.n_cls);
   put(P.off_mult, P.mult_bytes);
   put(P.off_bond, 8 * 32 * n_words);
-  put(P.off_nib, 4 * B->nib.size());
+  put(P.off_nib, rows ? 4 * 2 * n_words * p->n_hnib * 16 : 4 * B->nib.size());
   put(P.off_rs, 8 * (size_t)P.n_sq);
   put(P.off_chi, chi ? 16 * 1024 : 0);
-  put(P.off_mask, 4 * (size_t)words * kThreads);
+  put(P.off_mask, 4 * (size_t)words * (rows ? kRowThreads : kThreads));
+  if (rows) {
+    P.et_words = (uint32_t)(33 * n_words + 3) / 4 * 4;
+    put(P.off_et, 4 * (size_t)P.et_words * (kRowThreads / 32));
+  }
   P.smem_bytes = (uint32_t)off;
-  if (off > 110 * 1024) return ED_ERR_UNSUPPORTED;
+  if (off > (size_t)(rows ? 200 : 110) * 1024) return ED_ERR_UNSUPPORTED;
   // xs (and its remainders) for this call, from the basis's own pool in stream order, so
   // calls on several streams or threads never share it; without memory for it the search
   // kernel takes the call
   const bool lo = dtype == ED_F32 && p->weights;
-  const size_t xs_bytes = al16(es * (size_t)p->n_slots);
   char *ws = nullptr;
-  if (cudaMallocFromPoolAsync((void **)&ws, xs_bytes + (lo ? 4 * (size_t)p->n_slots : 0), p->pool, st) != cudaSuccess) {
+  if (cudaMallocFromPoolAsync((void **)&ws, 16 + xs_bytes + (lo ? 4 * (size_t)p->n_slots : 0), p->pool, st) != cudaSuccess) {
     cudaGetLastError();
     return ED_ERR_UNSUPPORTED;
   }
-  float *xslo = lo ? reinterpret_cast<float *>(ws + xs_bytes) : nullptr;
+  float *xslo = lo ? reinterpret_cast<float *>(ws + xs_bytes + 16) : nullptr;
+  P.next = reinterpret_cast<uint32_t *>(ws + xs_bytes);
   const int eg = (int)std::min<uint32_t>((p->n_slots + 255) / 256, (uint32_t)B->sm_count * 16);
   P.xs = ws;
   P.xslo = xslo;
@@ -885,8 +1234,8 @@ int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, c
   switch (dtype) {
 #define PCASE(D, V)                                                                              \
   case D:                                                                                        \
-    expand_kernel<V><<<eg, 256, 0, st>>>((const V *)x, p->d_idx, p->d_meta, (const double2 *)p->d_w, p->n_slots, (V *)ws, xslo); \
-    rc = cudaGetLastError() == cudaSuccess ? launch_pair_v<V>(B, P, chi, p->flips, st)            \
+    expand_kernel<V><<<eg, 256, 0, st>>>((const V *)x, p->idx, p->meta, (const double2 *)p->w, p->n_slots, (V *)ws, xslo, P.next); \
+    rc = cudaGetLastError() == cudaSuccess ? launch_pair_v<V>(B, P, chi, p->flips, rows, st)      \
                                            : ed_fail(ED_ERR_CUDA, "expand_kernel");              \
     break;
     PCASE(ED_F64, double)

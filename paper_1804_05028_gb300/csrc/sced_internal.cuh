@@ -403,6 +403,8 @@ struct PairSlots {
   uint16_t *meta;
   uint32_t *any_weight;
 };
+// basis.cu: out[i] = sum of in[0 .. i), *total the whole sum
+int ed_exclusive_scan(const uint32_t *in, uint64_t n, uint64_t *out, uint64_t *total, cudaStream_t st);
 int ed_launch_pair_slots(const ed_basis *B, const PairSlots &Q, cudaStream_t st);
 int ed_build_full_table(const uint8_t *d_pbit, const uint8_t *d_flip, int N, int nsym,
                         uint64_t *out, cudaStream_t st);

@@ -69,6 +69,30 @@ def test_product_of_every_type(p):
                 assert np.abs(B.apply_H_rows(x, r0, r1).cpu().numpy() - ref[r0:r1]).max() <= tol
 
 
+LARGE = [
+    T(6, momentum=(0, 0), point_irrep=1, J2=0.5, n_sublat=4, n_up=12),           # signs
+    w.chain(32, 4, k=5, n_up=11),                                                  # no involution
+    w.with_spin_flip(w.chain(32, 4, k=0, n_up=16), 1),
+    _sub(w.chain(28, 4, k=4, n_up=9), range(0, 28, 2), "chain28_even_translations"),  # no exchange
+]
+
+
+@pytest.mark.parametrize("p", LARGE, ids=lambda p: f"{p.name}_up{p.n_up}")
+def test_row_order(p):
+    """Sectors large enough for the row order by lower class (the whole product) against their
+    row ranges in basis order: the same terms summed in another order."""
+    B = _basis(p)
+    D = B.dim
+    assert D >= 1 << 18
+    for dt in ([torch.float64, torch.float32] if B.is_real else []) + [torch.complex128, torch.complex64]:
+        x = _vec(D, dt, 4)
+        y = B.apply_H(x)
+        cut = D // 3 + 1
+        ref = torch.cat([B.apply_H_rows(x, 0, cut), B.apply_H_rows(x, cut, D)])
+        tol = 2e-6 if dt in (torch.float32, torch.complex64) else 1e-12
+        assert (y - ref).abs().max() <= tol * ref.abs().max()
+
+
 def test_streams_and_capture():
     p = T(6, momentum=(0, 0), point_irrep=1, J2=0.5, n_sublat=4, n_up=6)
     B = _basis(p)
