@@ -954,6 +954,15 @@ __global__ void __launch_bounds__(256) pair_slots_kernel(const TwoParams P, cons
     }
     Q.idx[p] = idx;
     Q.meta[p] = meta;
+    if (Q.pat) {
+      uint32_t hi_v = 0, lo_v = 0;
+#pragma unroll
+      for (int X = 0; X < NSUB; X++) {
+        if (X == Q.hb[2]) hi_v = sub[X];
+        if (X == Q.hb[3]) lo_v = sub[X];
+      }
+      Q.pat[p] = u1 < 0 ? hi_v : (hi_v << n) | lo_v;
+    }
   }
 }
 

@@ -61,6 +61,7 @@ constexpr uint32_t kSpecial = 1u << 10;
 constexpr uint32_t kSignBit = 9;
 constexpr uint32_t kFlip = 1u << 8;
 constexpr uint32_t kElem = 255u;
+constexpr int kPosShift = 27;          // pair_rows_kernel's tables: a bit of B above 16 class bits
 
 struct PairParams {
   int n_classes;
@@ -86,24 +87,36 @@ struct PairParams {
   const uint64_t *basis;
   const uint16_t *stab;
   const void *x, *xs;
-  const float *xslo;             // fp32 real vectors: remainders of xs (null: all zero)
+  const float *xslo;             // fp32 real vectors: remainders of xs
+  uint32_t lo_special, lo_same;  // which slots may have one (both 0: none)
+  uint32_t n_slots;              // xs[n_slots] = 0
   void *y;
   void *ylo;
   int64_t r0, r1;
   double *partial;
   uint32_t off_off, off_mult, off_bond, off_nib, off_rs, off_chi, off_mask, smem_bytes;
-  // rows in the order of (lower class, upper pattern): pair_rows_kernel
-  const uint32_t *low;           // [n_cls] representative of the class
+  // rows in slot order: pair_rows_kernel
+  const uint32_t *low;           // [n_cls] representative of the lower class
+  const uint32_t *up;            // representatives of the upper classes, from class ubase on
+  const uint32_t *t_up;          // half table of the half the upper representatives lie on
+  uint32_t ubase;
   const uint32_t *row0;          // [n_cls + 1] first row of the class
   const uint32_t *slice0;        // [n_cls + 1] first 32-row slice of the class
+  const uint32_t *chunk_cls;     // class of every (kRowThreads / 32)th slice
   uint32_t n_slices;
-  const uint32_t *row_b;         // upper pattern
+  const uint32_t *row_b;         // pattern of the other half
   const uint32_t *row_i;         // basis index
   const uint16_t *row_m;         // weight of the row's configuration (meta of its slot)
   const double2 *rw;             // conj(chi) / sqrt(t) per weight
-  const uint32_t *half_nib;      // antiparallel masks by the halves' nibbles, [half][word][n_hnib][16]
-  uint32_t n_hnib;
-  uint32_t off_et, et_words;
+  const uint32_t *rt;            // tables of the row order, RowTables, staged as they are
+  uint32_t rt_words;
+  int kw[ED_MAXCLS][5];          // words of class c: across [0], [1); within A [1], [2); within up [3], [4)
+  uint32_t n_w, n_wa, n_hnib, m; // words, those across or within A (the first ones)
+  uint32_t n_tab, n_ucls;        // upper classes tabulated per slice, upper classes in all
+  int n_up;
+  bool no_swap, by_popcount;
+  uint32_t rt_f, rt_pos, rt_nibA, rt_nibB, rt_img, rt_left;   // offsets (words) in rt
+  uint32_t off_rt, off_et, et_words;
   uint32_t *next;                // work counter, zeroed by expand_kernel
 };
 
@@ -111,7 +124,9 @@ constexpr int kThreads = 512;
 constexpr int kMinBlocks = 2;
 constexpr int kRowThreads = 1024;      // pair_rows_kernel
 constexpr int kRowBlocks = 1;
-constexpr int kRowU = 4;
+constexpr int kRowU = 2;
+constexpr int kRowU16 = 1;
+constexpr int kRowU8 = 1;
 constexpr int64_t kRowOrderMinDim = 1 << 21;
 constexpr size_t kRowOrderMinBytes = (size_t)24 << 20;
 
@@ -143,43 +158,52 @@ __device__ __forceinline__ V ld_slot(const V *p) {
 }
 
 // one row's running sum over a coupling class: fp64, or a double-float pair for fp32
-// vectors (the fp64 pipe of this GPU issues at a small fraction of the fp32 rate)
+// vectors (the fp64 pipe of this GPU issues at a small fraction of the fp32 rate); signs come
+// in the top bit of w
+__device__ __forceinline__ float with_sign(float v, uint32_t w) {
+  return __uint_as_float(__float_as_uint(v) ^ (w & 0x80000000u));
+}
+__device__ __forceinline__ double with_sign(double v, uint32_t w) {
+  return __hiloint2double(__double2hiint(v) ^ (int)(w & 0x80000000u), __double2loint(v));
+}
 template <typename V> struct Acc;
 template <> struct Acc<double> {
-  double s = 0;
-  __device__ __forceinline__ void add(double v, uint32_t neg) { s += neg ? -v : v; }
-  __device__ __forceinline__ double re() const { return s; }
+  double s = 0, s2 = 0;   // two chains: fp64 results are slow to come back
+  __device__ __forceinline__ void add(double v, uint32_t w) {
+    const double t = s2;
+    s2 = s + with_sign(v, w);
+    s = t;
+  }
+  __device__ __forceinline__ double re() const { return s + s2; }
   __device__ __forceinline__ double im() const { return 0; }
 };
 template <> struct Acc<float> {
   float h = 0, l = 0;
-  __device__ __forceinline__ void add(float v, uint32_t neg) {
-    df_add(h, l, __uint_as_float(__float_as_uint(v) ^ (neg << 31)));
-  }
-  __device__ __forceinline__ void add_lo(float v, uint32_t neg) {
-    l = __fadd_rn(l, __uint_as_float(__float_as_uint(v) ^ (neg << 31)));
-  }
+  __device__ __forceinline__ void add(float v, uint32_t w) { df_add(h, l, with_sign(v, w)); }
+  __device__ __forceinline__ void add_lo(float v, uint32_t w) { l = __fadd_rn(l, with_sign(v, w)); }
   __device__ __forceinline__ double re() const { return df_value(h, l); }
   __device__ __forceinline__ double im() const { return 0; }
 };
 template <> struct Acc<double2> {
-  double r = 0, i = 0;
-  __device__ __forceinline__ void add(double2 v, uint32_t neg) {
-    r += neg ? -v.x : v.x;
-    i += neg ? -v.y : v.y;
+  double r = 0, i = 0, r2 = 0, i2 = 0;   // two chains
+  __device__ __forceinline__ void add(double2 v, uint32_t w) {
+    r += with_sign(v.x, w);
+    i += with_sign(v.y, w);
   }
   __device__ __forceinline__ void add(double2 v, double2 c) {
-    r = fma(c.x, v.x, fma(-c.y, v.y, r));
-    i = fma(c.x, v.y, fma(c.y, v.x, i));
+    r = fma(c.x, v.x, r);
+    r2 = fma(-c.y, v.y, r2);
+    i = fma(c.x, v.y, i);
+    i2 = fma(c.y, v.x, i2);
   }
-  __device__ __forceinline__ double re() const { return r; }
-  __device__ __forceinline__ double im() const { return i; }
+  __device__ __forceinline__ double re() const { return r + r2; }
+  __device__ __forceinline__ double im() const { return i + i2; }
 };
 template <> struct Acc<float2> {
   float rh = 0, rl = 0, ih = 0, il = 0;
-  __device__ __forceinline__ void add(float2 v, uint32_t neg) {
-    df_add(rh, rl, __uint_as_float(__float_as_uint(v.x) ^ (neg << 31)));
-    df_add(ih, il, __uint_as_float(__float_as_uint(v.y) ^ (neg << 31)));
+  __device__ __forceinline__ void add(float2 v, uint32_t w) {
+    df_add(rh, rl, with_sign(v.x, w));
+    df_add(ih, il, with_sign(v.y, w));
   }
   // chi v with chi given as (cos, remainder, sin, remainder): exact products
   __device__ __forceinline__ void add(float2 v, float4 c) {
@@ -200,44 +224,106 @@ struct PairSm {
   const uint32_t *fa, *fb;   // bits flipped in A and in B, per padded bond
 };
 
-// U terms of a row, given by the half-table entries of the exchanged configurations: the
-// first nu of them are added to acc
-template <typename V, bool kChi, bool kFlips, int U>
-__device__ __forceinline__ void pair_terms(const PairParams &P, const PairSm &S, const uint32_t (&ea)[U],
-                                           const uint32_t (&eb)[U], int nu, const V *xs,
-                                           const unsigned char *chi_sm, Acc<V> &acc) {
+// U terms in flight: the gathered values and what their sum needs (sign or chi index)
+template <typename V, int U>
+struct Terms {
   V v[U];
   float vl[U];
-  uint32_t lo[U];
+  uint32_t w[U];
+  int n;   // how many hold a term; the rest are zeros
+};
+
+// What a term gathers: its slot, what its sum needs (Terms::w), and whether the slot may hold
+// an orbit with |Stab| > 1 (fp32 real vectors then add the remainder xslo)
+struct Slot {
+  uint32_t slot, w;
+  bool lo;
+};
+
+template <bool kChi>
+__device__ __forceinline__ uint32_t lower_sign(uint32_t e, bool a_low) {
+  return kChi ? (e & (kElem | kFlip)) + (a_low ? 0u : 512u) : e << (31 - kSignBit);
+}
+
+// The slot of an exchanged configuration from its half-table entries.  |Stab| > 1 needs a
+// stabiliser on both halves, or halves that can be exchanged (one class; the difference also
+// lets a few neighbouring classes pass, whose xslo is 0).
+template <bool kChi, bool kFlips>
+__device__ __forceinline__ Slot slot_of(const PairParams &P, const PairSm &S, uint32_t ea, uint32_t eb) {
+  const uint32_t lo = min(ea, eb), hi = max(ea, eb);
+  const bool a_low = ea <= eb;
+  const uint32_t mi = (lo & kElem) * P.h0 + (hi & kElem) + (a_low ? 0u : P.sel_off);
+  Slot r;
+  r.slot = S.off[lo >> kClassShift] + P.K * (hi >> kClassShift) + S.mult[mi];
+  if (kFlips) r.slot += ((lo ^ hi) & kFlip) ? P.h0 : 0u;
+  r.w = lower_sign<kChi>(lo, a_low);
+  r.lo = (lo & hi & P.lo_special) || hi - lo < P.lo_same;
+  return r;
+}
+
+template <typename V, bool kChi, int U>
+__device__ __forceinline__ void pair_sum(const Terms<V, U> &t, const unsigned char *chi_sm, Acc<V> &acc) {
 #pragma unroll
   for (int u = 0; u < U; u++) {
-    lo[u] = min(ea[u], eb[u]);
-    const uint32_t hi = max(ea[u], eb[u]);
-    const uint32_t mi = (lo[u] & kElem) * P.h0 + (hi & kElem) + (ea[u] <= eb[u] ? 0u : P.sel_off);
-    uint32_t slot = S.off[lo[u] >> kClassShift] + P.K * (hi >> kClassShift) + S.mult[mi];
-    if (kFlips) slot += ((lo[u] ^ hi) & kFlip) ? P.h0 : 0u;
-    v[u] = ld_slot(xs + slot);
-    vl[u] = 0.f;
-    if constexpr (std::is_same<V, float>::value) {
-      // |Stab| > 1 needs a stabiliser on both halves, or halves that can be exchanged
-      if (P.xslo && ((lo[u] & hi & kSpecial) || ((lo[u] ^ hi) >> kClassShift) == 0)) vl[u] = __ldg(P.xslo + slot);
+    // adding zeros is harmless, but not free where it goes to the fp64 pipe
+    if (sizeof(typename Pv<V>::A) == 8 && u >= t.n) continue;
+    if constexpr (kChi) {
+      if constexpr (sizeof(typename Pv<V>::A) == 4)
+        acc.add(t.v[u], reinterpret_cast<const float4 *>(chi_sm)[t.w[u]]);
+      else
+        acc.add(t.v[u], reinterpret_cast<const double2 *>(chi_sm)[t.w[u]]);
+    } else {
+      acc.add(t.v[u], t.w[u]);
+      if constexpr (std::is_same<V, float>::value) acc.add_lo(t.vl[u], t.w[u]);
     }
   }
+}
+
+template <typename V>
+__device__ __forceinline__ V no_value() {
+  if constexpr (Pv<V>::cplx) { V z; z.x = 0; z.y = 0; return z; } else { return V(0); }
+}
+
+template <typename V, int U>
+__device__ __forceinline__ void no_terms(Terms<V, U> &t) {
+  t.n = 0;
 #pragma unroll
   for (int u = 0; u < U; u++) {
-    if (u < nu) {
-      if constexpr (kChi) {
-        const uint32_t ci = (lo[u] & (kElem | kFlip)) + (ea[u] <= eb[u] ? 0u : 512u);
-        if constexpr (sizeof(typename Pv<V>::A) == 4)
-          acc.add(v[u], reinterpret_cast<const float4 *>(chi_sm)[ci]);
-        else
-          acc.add(v[u], reinterpret_cast<const double2 *>(chi_sm)[ci]);
-      } else {
-        const uint32_t neg = (lo[u] >> kSignBit) & 1u;
-        acc.add(v[u], neg);
-        if constexpr (std::is_same<V, float>::value) acc.add_lo(vl[u], neg);
+    t.v[u] = no_value<V>();
+    t.vl[u] = 0.f;
+    t.w[u] = 0u;
+  }
+}
+
+// Sums n terms, U at a time; gen(slots, nu) gives the next nu.  The gathers of one round are
+// in flight while the round before is summed: two sets of registers taken in turn, as a copy
+// from one to the other would wait for the loads.  t0 holds terms still to be summed, on
+// entry and on exit, so that the gathers of one loop overlap the start of the next.
+template <typename V, bool kChi, int U, typename G>
+__device__ __forceinline__ void pair_loop(const PairParams &P, int n, G gen, const V *xs,
+                                          const unsigned char *chi_sm, Acc<V> &acc, Terms<V, U> &t0) {
+  auto step = [&](Terms<V, U> &t) {
+    Slot g[U];
+    gen(g, n);
+    t.n = n;
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      const uint32_t slot = u == 0 || u < n ? g[u].slot : P.n_slots;   // xs[n_slots] = 0
+      t.w[u] = g[u].w;
+      t.v[u] = ld_slot(xs + slot);
+      t.vl[u] = 0.f;
+      if constexpr (std::is_same<V, float>::value) {
+        if (g[u].lo) t.vl[u] = __ldg(P.xslo + slot);
       }
     }
+    n -= U;
+  };
+  while (n > 0) {
+    Terms<V, U> t1;
+    step(t1);
+    pair_sum<V, kChi, U>(t0, chi_sm, acc);
+    if (n > 0) step(t0); else no_terms(t0);
+    pair_sum<V, kChi, U>(t1, chi_sm, acc);
   }
 }
 
@@ -373,19 +459,24 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) pair_kernel(const __grid
         mask_s[(wd - w0) * kThreads] = m;
       }
       Acc<V> acc;
+      Terms<V, U> pend;
+      no_terms(pend);
       int wd = w0;
       uint32_t m = w0 < w1 ? mask_s[0] : 0u;
-      for (int left = nanti; left > 0; left -= U) {
-        uint32_t ea[U], eb[U];
+      auto gen = [&](Slot (&g)[U], int nu) {
         int kb = 0;
+        uint32_t ea[U], eb[U];
 #pragma unroll
         for (int u = 0; u < U; u++) {
-          if (u < left) kb = next_bond<kThreads>(m, wd, w0, mask_s);
+          if (u == 0 || u < nu) kb = next_bond<kThreads>(m, wd, w0, mask_s);
           ea[u] = __ldg(P.ta + (A ^ S.fa[kb]));
           eb[u] = __ldg(P.tb + (B ^ S.fb[kb]));
         }
-        pair_terms<V, kChi, kFlips, U>(P, S, ea, eb, left, xs, sm + P.off_chi, acc);
-      }
+#pragma unroll
+        for (int u = 0; u < U; u++) g[u] = slot_of<kChi, kFlips>(P, S, ea[u], eb[u]);
+      };
+      pair_loop<V, kChi, U>(P, nanti, gen, xs, sm + P.off_chi, acc, pend);
+      pair_sum<V, kChi, U>(pend, sm + P.off_chi, acc);
       row_re += P.jh[c] * acc.re();
       if constexpr (kC) row_im += P.jh[c] * acc.im();
       diag += P.jzq[c] * (double)(P.nb_cls[c] - 2 * nanti);
@@ -396,31 +487,52 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) pair_kernel(const __grid
   pair_dot<kC, kThreads>(P, dot_re, dot_im);
 }
 
-// Rows in the order of (lower class, upper pattern), for products whose xs is larger than the
-// L2 keeps.  In basis order the gathers of xs are random over the whole vector: on the 6x6
-// sector 59 bytes of DRAM traffic per gathered fp32 value and 77% of the DRAM's peak.  Rows
-// that share the lower half A reach few places: the exchanged half A' takes at most one value
-// per bond, and while class(A') stays the lower one the gather falls into that class's block
-// of slots; the whole GPU works on a few lower classes at a time, whose blocks stay in L2.
-// The half-table entries of A' are a table of the warp (one entry per bond), rows with
-// neighbouring upper patterns share the cache lines of the other half table.
+// Rows in slot order, for products whose xs is larger than the L2 keeps.  In basis order the
+// gathers of xs are random over the whole vector: on the 6x6 sector 59 bytes of DRAM traffic
+// per gathered fp32 value and 77% of the DRAM's peak (23.8 ms).  Rows that share the lower half
+// A reach few places: the exchanged half A' takes at most one value per bond, and while
+// class(A') stays the lower one the gather falls into that class's block of slots.  The GPU
+// works on one or two lower classes at a time, whose blocks (10 to 20 MB on that sector) stay
+// in L2.  That needs all SMs at the same place: blocks take slices from a counter (with a fixed
+// stride the SMs drift apart by dozens of classes, and the DRAM traffic was 120 GB instead
+// of 11).
+//
+// In slot order the rows of one upper class c lie together: b = k R(c), all k.  Terms within a
+// half keep the other class: within A the 32 rows of a warp gather from one cluster of K slots
+// (c(A'), c), and within the upper half, with the bonds taken in the frame of R(c) (the
+// bonds are invariant under the group), from one cluster (c_A, c') -- half the terms of a
+// J1-J2 row, a few cache lines instead of 32 sectors.  The half table is read at R(c) with
+// one or two bits flipped, the same few entries for all rows of the cluster:
+//     g_B b = R(c),  u' = R(c) with g_B's image of the flipped bits,  g_u u' = R(c')
+// makes g_u g_B the element that carries the exchanged half to R(c'), its number from the
+// left multiplication table of H.
 template <typename V, bool kChi, bool kFlips>
 __global__ void __launch_bounds__(kRowThreads, kRowBlocks) pair_rows_kernel(const __grid_constant__ PairParams P) {
   constexpr bool kC = Pv<V>::cplx;
-  constexpr int U = kRowU;
+  constexpr int U = sizeof(V) == 16 ? kRowU16 : sizeof(V) == 8 ? kRowU8 : kRowU;
   extern __shared__ __align__(16) unsigned char sm[];
   const PairSm S = pair_stage<V, kChi>(P, sm);
-  const int n_words = P.cls_word[P.n_classes];
-  cpy(sm, P.off_nib, P.half_nib, (uint32_t)n_words * P.n_hnib * 32);
+  cpy(sm, P.off_rt, P.rt, P.rt_words);
   __syncthreads();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const uint32_t *nibA = reinterpret_cast<const uint32_t *>(sm + P.off_nib), *nibB = nibA + n_words * P.n_hnib * 16;
+  const uint32_t *rt = reinterpret_cast<const uint32_t *>(sm + P.off_rt);
+  const uint32_t *nibA = rt + P.rt_nibA, *nibB = rt + P.rt_nibB;
+  const uint32_t *fw = rt + P.rt_f;                                        // bits of A, or of R(c)
+  const uint8_t *pos = reinterpret_cast<const uint8_t *>(rt + P.rt_pos);   // bit of B (across)
+  const uint8_t *img = reinterpret_cast<const uint8_t *>(rt + P.rt_img);   // its image under g_B
+  const uint8_t *left = reinterpret_cast<const uint8_t *>(rt + P.rt_left);
   uint32_t *mask_s = reinterpret_cast<uint32_t *>(sm + P.off_mask) + threadIdx.x;
-  uint32_t *et = reinterpret_cast<uint32_t *>(sm + P.off_et) + wid * P.et_words;   // entries of A' by bond
-  uint32_t *ma = et + n_words * 32;                                                // masks of A by word
+  // tables of the warp: per bond across the halves or within A, the entry of A' and the slot
+  // offset of its class; masks of A by word; for the slice's first upper classes c (n_tab of
+  // them), per bit of R(c) the entry with it flipped, and per bond within the upper half that
+  // with its two bits flipped
+  uint2 *et = reinterpret_cast<uint2 *>(sm + P.off_et) + wid * (P.et_words / 2);
+  uint32_t *ma = reinterpret_cast<uint32_t *>(et + P.n_wa * 32), *eup = ma + P.n_wa;
+  const uint32_t n_up2 = (P.n_w - P.n_wa) * 32, n_eup = P.m + n_up2;
   const V *xs = reinterpret_cast<const V *>(P.xs);
   double dot_re = 0.0, dot_im = 0.0;
-  uint32_t cur = 0xFFFFFFFFu;
+  uint32_t cur = 0xFFFFFFFFu, e_low = 0, off_low = 0;
+  bool st_in = false, st_across = false;
   __shared__ uint32_t chunk_s;
   for (;;) {
     __syncthreads();
@@ -429,51 +541,169 @@ __global__ void __launch_bounds__(kRowThreads, kRowBlocks) pair_rows_kernel(cons
     if (chunk_s * (kRowThreads / 32) >= P.n_slices) break;
     const uint32_t sl = chunk_s * (kRowThreads / 32) + wid;
     if (sl >= P.n_slices) continue;
-    uint32_t lo = 0, hi = P.n_cls - 1;
-    while (lo < hi) {   // the last class that starts at or before the slice
-      const uint32_t mid = (lo + hi + 1) >> 1;
-      if (__ldg(P.slice0 + mid) <= sl) lo = mid; else hi = mid - 1;
-    }
+    uint32_t lo = __ldg(P.chunk_cls + chunk_s);   // the class of the chunk's first slice
+    while (__ldg(P.slice0 + lo + 1) <= sl) lo++;
     if (lo != cur) {
       cur = lo;
       const uint32_t A = __ldg(P.low + lo);
+      e_low = __ldg(P.ta + A);
+      off_low = S.off[lo];
+      // where the lower class is known beforehand: classes are ordered by their number of up
+      // spins (the smaller of up and down spins with spin flips, where nothing is known); an
+      // exchange across the halves moves one spin.  Halves that nothing exchanges: always A.
+      const int na = __popc(A), nb = P.n_up - na;
+      st_in = P.no_swap || (P.by_popcount && na < nb);
+      st_across = P.no_swap || (P.by_popcount && na + 1 < nb - 1);
       __syncwarp();
-      for (int k = lane; k < n_words * 32; k += 32) et[k] = __ldg(P.ta + (A ^ S.fa[k]));
-      for (int wd = lane; wd < n_words; wd += 32) {
+      for (uint32_t k = lane; k < P.n_wa * 32; k += 32) {
+        const uint32_t e = __ldg(P.ta + (A ^ fw[k]));
+        et[k] = make_uint2(e | (uint32_t)pos[k] << kPosShift, S.off[e >> kClassShift]);
+      }
+      for (uint32_t wd = lane; wd < P.n_wa; wd += 32) {
         uint32_t m = 0;
         for (uint32_t q = 0; q < P.n_hnib; q++) m ^= nibA[(wd * P.n_hnib + q) * 16 + ((A >> (4 * q)) & 15u)];
         ma[wd] = m;
       }
       __syncwarp();
     }
-    const uint32_t r = __ldg(P.row0 + lo) + (sl - __ldg(P.slice0 + lo)) * 32 + lane;
-    if (r >= __ldg(P.row0 + lo + 1)) continue;
+    const uint32_t rw0 = __ldg(P.row0 + lo) + (sl - __ldg(P.slice0 + lo)) * 32;
+    const int n_row = (int)min(32u, __ldg(P.row0 + lo + 1) - rw0);
+    const uint32_t r = rw0 + min(lane, n_row - 1);   // lanes past the end repeat the last row
     const uint32_t B = __ldcs(P.row_b + r);
+    const uint32_t e_up = __ldg(P.tb + B);
+    const uint32_t c_up = (e_up >> kClassShift) - P.ubase, c0 = __shfl_sync(0xFFFFFFFFu, c_up, 0);
+    const uint32_t R = __ldg(P.up + c_up);
+    __syncwarp();
+    for (uint32_t t = 0; t < P.n_tab; t++) {
+      const uint32_t Rt = __ldg(P.up + min(c0 + t, P.n_ucls - 1));
+      uint32_t *e = eup + t * n_eup;
+      for (uint32_t q = lane; q < P.m; q += 32) e[q] = __ldg(P.t_up + (Rt ^ (1u << q)));
+      for (uint32_t k = lane; k < n_up2; k += 32) e[P.m + k] = __ldg(P.t_up + (Rt ^ fw[P.n_wa * 32 + k]));
+    }
+    __syncwarp();
+    // more classes than that occur where classes have stabilisers, and so fewer rows
+    const bool all_tab = __all_sync(0xFFFFFFFFu, c_up - c0 < P.n_tab);
+    if (lane >= n_row) continue;
+    const uint32_t *eup_r = eup + (c_up - c0) * n_eup, *eu_r = eup_r + P.m;
+    const uint32_t yB = e_up & kElem;
+    const uint8_t *img_r = img + yB * P.m, *left_y = left + yB;
+    const uint32_t slot_up = P.K * (e_up >> kClassShift);
     double diag = 0.0, row_re = 0.0, row_im = 0.0;
+    // the entry of the exchanged upper half from that of u' = R(c) with its bits flipped
+    auto carried = [&](uint32_t eu) {
+      return ((eu ^ (e_up & (kFlip | 1u << kSignBit))) & ~kElem) | left_y[(eu & kElem) * P.h0];
+    };
     for (int c = 0; c < P.n_classes; c++) {
-      const int w0 = P.cls_word[c], w1 = P.cls_word[c + 1];
       int nanti = 0;
-      for (int wd = w0; wd < w1; wd++) {
-        uint32_t m = ma[wd];
-        const uint32_t *nw = nibB + (uint32_t)wd * P.n_hnib * 16;
-        for (uint32_t q = 0; q < P.n_hnib; q++) m ^= nw[q * 16 + ((B >> (4 * q)) & 15u)];
-        nanti += __popc(m);
-        mask_s[(wd - w0) * kRowThreads] = m;
-      }
       Acc<V> acc;
-      int wd = w0;
-      uint32_t m = w0 < w1 ? mask_s[0] : 0u;
-      for (int left = nanti; left > 0; left -= U) {
-        uint32_t ea[U], eb[U];
-        int kb = 0;
-#pragma unroll
-        for (int u = 0; u < U; u++) {
-          if (u < left) kb = next_bond<kRowThreads>(m, wd, w0, mask_s);
-          ea[u] = et[kb];
-          eb[u] = __ldg(P.tb + (B ^ S.fb[kb]));
+      Terms<V, U> pend;
+      no_terms(pend);
+      {   // bonds across the halves
+        const int w0 = P.kw[c][0], w1 = P.kw[c][1];
+        int n = 0;
+        for (int wd = w0; wd < w1; wd++) {
+          uint32_t m = ma[wd];
+          const uint32_t *nw = nibB + (uint32_t)wd * P.n_hnib * 16;
+          for (uint32_t q = 0; q < P.n_hnib; q++) m ^= nw[q * 16 + ((B >> (4 * q)) & 15u)];
+          n += __popc(m);
+          mask_s[(wd - w0) * kRowThreads] = m;
         }
-        pair_terms<V, kChi, kFlips, U>(P, S, ea, eb, left, xs, sm + P.off_chi, acc);
+        nanti += n;
+        int wd = w0;
+        uint32_t m = w0 < w1 ? mask_s[0] : 0u;
+        auto across = [&](auto entry, auto is_static) {
+          auto gen = [&](Slot (&g)[U], int nu) {
+            int kb = 0;
+            uint2 e[U];
+            uint32_t eu[U];
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+              if (u == 0 || u < nu) kb = next_bond<kRowThreads>(m, wd, w0, mask_s);
+              e[u] = et[kb];
+              eu[u] = entry(img_r[e[u].x >> kPosShift]);
+            }
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+              if constexpr (decltype(is_static)::value) {   // class(A') is the lower one
+                const uint32_t k = left_y[(eu[u] & kElem) * P.h0];
+                g[u].slot = e[u].y + P.K * (eu[u] >> kClassShift) + S.mult[(e[u].x & kElem) * P.h0 + k];
+                g[u].w = lower_sign<kChi>(e[u].x, true);
+                g[u].lo = e[u].x & eu[u] & P.lo_special;
+              } else {
+                g[u] = slot_of<kChi, kFlips>(P, S, e[u].x & ((1u << kPosShift) - 1u), carried(eu[u]));
+              }
+            }
+          };
+          pair_loop<V, kChi, U>(P, n, gen, xs, sm + P.off_chi, acc, pend);
+        };
+        auto from_table = [&](uint32_t q) { return eup_r[q]; };
+        auto from_memory = [&](uint32_t q) { return __ldg(P.t_up + (R ^ (1u << q))); };
+        if (!all_tab) across(from_memory, std::false_type());
+        else if (!kFlips && st_across) across(from_table, std::true_type());
+        else across(from_table, std::false_type());
       }
+      // bonds within A
+      for (int wd = P.kw[c][1]; wd < P.kw[c][2]; wd++) {
+        uint32_t m = ma[wd];
+        const int n = __popc(m);
+        nanti += n;
+        auto within = [&](auto is_static) {
+          auto gen = [&](Slot (&g)[U], int nu) {
+            int kb = 0;
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+              if (u == 0 || u < nu) {
+                kb = wd * 32 + __ffs(m) - 1;
+                m &= m - 1;
+              }
+              const uint2 e = et[kb];
+              if constexpr (decltype(is_static)::value) {
+                g[u].slot = e.y + slot_up + S.mult[(e.x & kElem) * P.h0 + yB];
+                g[u].w = lower_sign<kChi>(e.x, true);
+                g[u].lo = e.x & e_up & P.lo_special;
+              } else {
+                g[u] = slot_of<kChi, kFlips>(P, S, e.x & ((1u << kPosShift) - 1u), e_up);
+              }
+            }
+          };
+          pair_loop<V, kChi, U>(P, n, gen, xs, sm + P.off_chi, acc, pend);
+        };
+        if (!kFlips && st_in) within(std::true_type()); else within(std::false_type());
+      }
+      // bonds within the upper half, in the frame of R(c)
+      for (int wd = P.kw[c][3]; wd < P.kw[c][4]; wd++) {
+        uint32_t m = 0;
+        const uint32_t *nw = nibB + (uint32_t)wd * P.n_hnib * 16;
+        for (uint32_t q = 0; q < P.n_hnib; q++) m ^= nw[q * 16 + ((R >> (4 * q)) & 15u)];
+        const int n = __popc(m);
+        nanti += n;
+        const uint32_t *eu_w = eu_r + (wd - (int)P.n_wa) * 32, *fw_w = fw + wd * 32;
+        auto within = [&](auto is_static) {
+          // with A unchanged and lower, k g_u^-1 for the row's own k
+          const uint8_t *mk = S.mult + P.sel_off + (uint32_t)S.mult[(e_low & kElem) * P.h0 + yB] * P.h0;
+          auto gen = [&](Slot (&g)[U], int nu) {
+            int kb = 0;
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+              if (u == 0 || u < nu) {
+                kb = __ffs(m) - 1;
+                m &= m - 1;
+              }
+              const uint32_t eu = all_tab ? eu_w[kb] : __ldg(P.t_up + (R ^ fw_w[kb]));
+              if constexpr (decltype(is_static)::value) {
+                g[u].slot = off_low + P.K * (eu >> kClassShift) + mk[eu & kElem];
+                g[u].w = lower_sign<kChi>(e_low, true);
+                g[u].lo = e_low & eu & P.lo_special;
+              } else {
+                g[u] = slot_of<kChi, kFlips>(P, S, e_low, carried(eu));
+              }
+            }
+          };
+          pair_loop<V, kChi, U>(P, n, gen, xs, sm + P.off_chi, acc, pend);
+        };
+        if (!kFlips && st_in) within(std::true_type()); else within(std::false_type());
+      }
+      pair_sum<V, kChi, U>(pend, sm + P.off_chi, acc);
       row_re += P.jh[c] * acc.re();
       if constexpr (kC) row_im += P.jh[c] * acc.im();
       diag += P.jzq[c] * (double)(P.nb_cls[c] - 2 * nanti);
@@ -498,7 +728,11 @@ template <typename V>
 __global__ void __launch_bounds__(256) expand_kernel(const V *x, const uint32_t *idx, const uint16_t *meta,
                                                      const double2 *w, uint32_t n, V *xs, float *xslo, uint32_t *next) {
   using A_ = typename Pv<V>::A;
-  if (blockIdx.x == 0 && threadIdx.x == 0) *next = 0;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    *next = 0;
+    if constexpr (Pv<V>::cplx) { xs[n].x = 0; xs[n].y = 0; } else { xs[n] = 0; }
+    if (sizeof(V) == 4 && xslo) xslo[n] = 0.f;
+  }
   for (uint32_t p = blockIdx.x * 256 + threadIdx.x; p < n; p += gridDim.x * 256) {
     const uint32_t j = __ldcs(idx + p);
     const uint32_t mt = __ldcs(meta + p);
@@ -573,17 +807,14 @@ __global__ void half_entries(const uint32_t *rep, const uint32_t *first, const u
            code[first[u] & 0x7FFFFFFFu];
 }
 
-// The rows in slot-friendly order.  Candidates are (lower class c, pattern b of the other half
-// with the right number of up spins, in increasing order), in chunks of 1024 of one class; a
-// warp owns a chunk.  A candidate stands for the basis state of its slot.  Only a class with
-// a stabiliser, or two halves of one class, give the same state several candidates: those
-// claim it with their position, the lowest wins.
+// The rows in slot order: one slot for every basis state.  A warp owns a chunk of 1024 slots
+// of one lower class.  A state has several slots when a class has a stabiliser or both halves
+// belong to one class; those slots claim it with their position, the lowest wins.
 struct RowEnum {
-  const uint32_t *ta, *tb, *low, *off, *chunk0, *list0, *list_n, *plist, *idx;
-  const uint8_t *mult;
-  uint32_t n_cls, n_chunks, K, h0;
-  uint32_t *first;       // [D] lowest claiming candidate
-  uint32_t *bits;        // [n_chunks][32] which candidates are rows
+  const uint32_t *ta, *tb, *low, *start, *chunk0, *idx, *pat;
+  uint32_t n_cls, n_chunks;
+  uint32_t *first;       // [D] lowest claiming slot
+  uint32_t *bits;        // [n_chunks][32] which slots are rows
   uint32_t *count;       // [n_chunks]
   const uint64_t *at;    // [n_chunks] first row of the chunk
   const uint16_t *meta;
@@ -603,36 +834,33 @@ __global__ void __launch_bounds__(256) enum_rows(const RowEnum Q) {
       const uint32_t mid = (lo + hi + 1) >> 1;
       if (__ldg(Q.chunk0 + mid) <= ch) lo = mid; else hi = mid - 1;
     }
-    const uint32_t ea = __ldg(Q.ta + __ldg(Q.low + lo)), off = __ldg(Q.off + lo);
-    const uint32_t j0 = (ch - __ldg(Q.chunk0 + lo)) * 1024, n = __ldg(Q.list_n + lo), l0 = __ldg(Q.list0 + lo);
+    const uint32_t ea = __ldg(Q.ta + __ldg(Q.low + lo));
+    const uint32_t p0 = __ldg(Q.start + lo) + (ch - __ldg(Q.chunk0 + lo)) * 1024, end = __ldg(Q.start + lo + 1);
     uint32_t total = 0;
     uint64_t w = kPass == kFill ? Q.at[ch] : 0;
     for (int step = 0; step < 32; step++) {
-      const uint32_t j = j0 + step * 32 + lane;
-      if (j0 + step * 32 >= n) {
-        if (kPass == kCount && lane == 0) Q.bits[ch * 32 + step] = 0;
-        continue;
-      }
+      const uint32_t p = p0 + step * 32 + lane;
       uint32_t bits = 0;
+      bool row = p < end;
       if (kPass == kFill) {
         bits = Q.bits[ch * 32 + step];
-        if (bits == 0) continue;
+        row = (bits >> lane) & 1u;
       }
-      bool row = j < n && (kPass != kFill || ((bits >> lane) & 1u));
-      uint32_t i = 0, b = 0, slot = 0;
       if (row) {
-        b = __ldg(Q.plist + l0 + j);
-        const uint32_t eb = __ldg(Q.tb + b);
-        row = (eb >> kClassShift) >= (ea >> kClassShift);
-        if (row) {
-          slot = off + Q.K * (eb >> kClassShift) + Q.mult[(ea & kElem) * Q.h0 + (eb & kElem)] +
-                                (((ea ^ eb) & kFlip) ? Q.h0 : 0u);
-          i = __ldg(Q.idx + slot);
+        const uint32_t i = __ldg(Q.idx + p);
+        if (kPass == kFill) {
+          const uint64_t at = w + __popc(bits & ((1u << lane) - 1u));
+          Q.row_b[at] = __ldg(Q.pat + p);
+          Q.row_i[at] = i;
+          Q.row_m[at] = __ldg(Q.meta + p);
+        } else {
           row = i != 0xFFFFFFFFu;
-          if (row && kPass != kFill && ((ea & kSpecial) || ((ea ^ eb) >> kClassShift) == 0)) {
-            const uint32_t e = ch * 1024 + step * 32 + lane;
-            if (kPass == kClaim) atomicMin(Q.first + i, e);
-            else row = Q.first[i] == e;
+          if (row) {
+            const uint32_t eb = __ldg(Q.tb + __ldg(Q.pat + p));
+            if (((ea | eb) & kSpecial) || ((ea ^ eb) >> kClassShift) == 0) {
+              if (kPass == kClaim) atomicMin(Q.first + i, p);
+              else row = Q.first[i] == p;
+            }
           }
         }
       }
@@ -641,17 +869,21 @@ __global__ void __launch_bounds__(256) enum_rows(const RowEnum Q) {
         if (lane == 0) Q.bits[ch * 32 + step] = m;
         total += __popc(m);
       }
-      if (kPass == kFill) {
-        if (row) {
-          const uint64_t at = w + __popc(bits & ((1u << lane) - 1u));
-          Q.row_b[at] = b;
-          Q.row_i[at] = i;
-          Q.row_m[at] = __ldg(Q.meta + slot);
-        }
-        w += __popc(bits);
-      }
+      if (kPass == kFill) w += __popc(bits);
     }
     if (kPass == kCount && lane == 0) Q.count[ch] = total;
+  }
+}
+
+__global__ void chunk_classes(const uint32_t *slice0, uint32_t n_cls, uint32_t n_chunks, uint32_t per_chunk,
+                              uint32_t *cls) {
+  for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n_chunks; k += gridDim.x * blockDim.x) {
+    uint32_t lo = 0, hi = n_cls - 1;
+    while (lo < hi) {   // the last class that starts at or before the slice
+      const uint32_t mid = (lo + hi + 1) >> 1;
+      if (__ldg(slice0 + mid) <= k * per_chunk) lo = mid; else hi = mid - 1;
+    }
+    cls[k] = lo;
   }
 }
 
@@ -668,12 +900,17 @@ struct PairPlan {
   int shA0 = 0, shA1 = 0, shB0 = 0, shB1 = 0;
   uint32_t bmask_hi = 0, bmask = 0;
   uint32_t n_cls = 0, K = 0, h0 = 0, sel_off = 0, mult_bytes = 0, n_slots = 0;
-  uint32_t n_hnib = 0, hnib_len = 0, n_slices = 0;
+  uint32_t n_slices = 0, ubase = 0, n_ucls = 0;
+  // tables of the row order (RowTables)
+  int kw[ED_MAXCLS][5] = {};
+  bool no_swap = false, any_flip = false;
+  uint32_t rt_words = 0, rt_w = 0, rt_wa = 0, n_hnib = 0, rt_f = 0, rt_pos = 0, rt_nibA = 0, rt_nibB = 0, rt_img = 0, rt_left = 0;
+  uint32_t rt_across = 0;         // most words of bonds across the halves in a class
   bool flips = false, weights = false;
   // device: the half tables, the small tables, the slots' indices and weights, the rows
   void *d_half = nullptr, *d_small = nullptr, *d_slots = nullptr, *d_rows = nullptr;
-  uint32_t *ta = nullptr, *tb = nullptr, *off = nullptr, *idx = nullptr, *low = nullptr, *half_nib = nullptr;
-  uint32_t *row0 = nullptr, *slice0 = nullptr, *row_b = nullptr, *row_i = nullptr;
+  uint32_t *ta = nullptr, *tb = nullptr, *off = nullptr, *idx = nullptr, *low = nullptr, *up = nullptr, *t_up = nullptr, *rt = nullptr;
+  uint32_t *row0 = nullptr, *slice0 = nullptr, *chunk_cls = nullptr, *row_b = nullptr, *row_i = nullptr;
   uint16_t *row_m = nullptr;
   uint8_t *mult = nullptr;
   uint2 *bond = nullptr;
@@ -722,46 +959,40 @@ struct Scratch {
 };
 
 // Row order for large sectors (see pair_rows_kernel); p->n_slices stays 0 when it is not made.
-int build_rows(ed_basis *B, PairPlan *p, const std::vector<uint32_t> &low, const std::vector<uint32_t> &off,
-               cudaStream_t st) {
-  const uint32_t nA = p->n_cls, total = 1u << p->m;
-  std::vector<uint32_t> plist(total), at(p->m + 2, 0);
-  for (uint32_t u = 0; u < total; u++) at[__builtin_popcount(u) + 1]++;
-  for (int q = 0; q <= p->m; q++) at[q + 1] += at[q];
-  std::vector<uint32_t> pos(at.begin(), at.end() - 1);
-  for (uint32_t u = 0; u < total; u++) plist[pos[__builtin_popcount(u)]++] = u;
-  std::vector<uint32_t> list0(nA), list_n(nA), chunk0(nA);
+// pat: the pattern of the other half of every slot.
+int build_rows(ed_basis *B, PairPlan *p, const std::vector<uint32_t> &start, const uint32_t *d_start,
+               const uint32_t *pat, cudaStream_t st) {
+  const uint32_t nA = p->n_cls;
+  std::vector<uint32_t> chunk0(nA);
   uint64_t chunks = 0;
   for (uint32_t c = 0; c < nA; c++) {
-    const int want = B->n_up - __builtin_popcount(low[c]);
-    list0[c] = list_n[c] = 0;
-    if (want >= 0 && want <= p->m) { list0[c] = at[want]; list_n[c] = at[want + 1] - at[want]; }
     chunk0[c] = (uint32_t)chunks;
-    chunks += (list_n[c] + 1023) / 1024;
+    chunks += ((uint64_t)start[c + 1] - start[c] + 1023) / 1024;
   }
-  if (chunks >= (1u << 22) || chunks == 0) return ED_OK;
+  if (chunks >= 0xFFFFFFFFull || chunks == 0) return ED_OK;
   Blob blob;
-  const size_t o_pl = blob.add(plist), o_l0 = blob.add(list0), o_ln = blob.add(list_n), o_c0 = blob.add(chunk0);
+  const size_t o_c0 = blob.add(chunk0);
   Scratch sc(st);
   unsigned char *d = (unsigned char *)sc.get(blob.bytes.size());
   uint32_t *d_first = (uint32_t *)sc.get(4 * (size_t)B->D), *d_bits = (uint32_t *)sc.get(128 * chunks);
   uint32_t *d_count = (uint32_t *)sc.get(4 * chunks);
   uint64_t *d_at = (uint64_t *)sc.get(8 * chunks);
   if (!d || !d_first || !d_bits || !d_count || !d_at) return ED_OK;
-  const size_t rows_bytes = 10 * (size_t)B->D + 8 * ((size_t)nA + 1);
+  const uint64_t max_chunks = (B->D / 32 + nA) / (kRowThreads / 32) + 1;
+  const size_t rows_bytes = 10 * (size_t)B->D + 8 * ((size_t)nA + 1) + 4 * max_chunks;
   if (cudaMalloc(&p->d_rows, rows_bytes) != cudaSuccess) { cudaGetLastError(); p->d_rows = nullptr; return ED_OK; }
   p->row_b = (uint32_t *)p->d_rows;
   p->row_i = p->row_b + B->D;
   p->row0 = p->row_i + B->D;
   p->slice0 = p->row0 + nA + 1;
-  p->row_m = (uint16_t *)(p->slice0 + nA + 1);
+  p->chunk_cls = p->slice0 + nA + 1;
+  p->row_m = (uint16_t *)(p->chunk_cls + max_chunks);
   ED_CK(cudaMemcpyAsync(d, blob.bytes.data(), blob.bytes.size(), cudaMemcpyHostToDevice, st));
   ED_CK(cudaMemsetAsync(d_first, 0xFF, 4 * (size_t)B->D, st));
   RowEnum Q{};
-  Q.ta = p->ta; Q.tb = p->tb; Q.low = p->low; Q.off = p->off; Q.idx = p->idx; Q.mult = p->mult;
-  Q.plist = (const uint32_t *)(d + o_pl); Q.list0 = (const uint32_t *)(d + o_l0);
-  Q.list_n = (const uint32_t *)(d + o_ln); Q.chunk0 = (const uint32_t *)(d + o_c0);
-  Q.n_cls = nA; Q.n_chunks = (uint32_t)chunks; Q.K = p->K; Q.h0 = p->h0;
+  Q.ta = p->ta; Q.tb = p->tb; Q.low = p->low; Q.idx = p->idx; Q.pat = pat; Q.start = d_start;
+  Q.chunk0 = (const uint32_t *)(d + o_c0);
+  Q.n_cls = nA; Q.n_chunks = (uint32_t)chunks;
   Q.first = d_first; Q.bits = d_bits; Q.count = d_count; Q.at = d_at; Q.meta = p->meta;
   Q.row_b = p->row_b; Q.row_i = p->row_i; Q.row_m = p->row_m;
   const int grid = (int)std::min<uint64_t>((chunks + 7) / 8, (uint64_t)B->sm_count * 8);
@@ -787,6 +1018,9 @@ int build_rows(ed_basis *B, PairPlan *p, const std::vector<uint32_t> &low, const
   }
   slice0[nA] = (uint32_t)sl;
   ED_CK(cudaMemcpyAsync(p->slice0, slice0.data(), 4 * ((size_t)nA + 1), cudaMemcpyHostToDevice, st));
+  const uint32_t n_ch = (uint32_t)((sl + kRowThreads / 32 - 1) / (kRowThreads / 32));
+  chunk_classes<<<(int)std::min<uint32_t>((n_ch + 255) / 256, 1024), 256, 0, st>>>(p->slice0, nA, n_ch, kRowThreads / 32, p->chunk_cls);
+  ED_CK(cudaGetLastError());
   ED_CK(cudaStreamSynchronize(st));
   p->n_slices = (uint32_t)sl;
   p->bytes += rows_bytes;
@@ -1063,22 +1297,88 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
       if (X == hb[0] || X == hb[1]) bond[b].x |= 1u << pos; else bond[b].y |= 1u << pos;
     }
   }
-  // antiparallel masks by the halves' nibbles, [half][word][nibble][16] (as the nibble tables
-  // over whole states: bit k is set for every endpoint of bond k that is up)
-  const size_t n_words = bond.size() / 32;
-  p->n_hnib = (uint32_t)(m + 3) / 4;
-  std::vector<uint32_t> hnib(2 * n_words * p->n_hnib * 16, 0u);
-  for (size_t b = 0; b < bond.size(); b++)
-    for (int half = 0; half < 2; half++) {
-      const uint32_t f = half ? bond[b].y : bond[b].x;
-      for (int q = 0; q < m; q++)
-        if ((f >> q) & 1u)
-          for (int v = 0; v < 16; v++)
-            if ((v >> (q % 4)) & 1) hnib[((half * n_words + b / 32) * p->n_hnib + q / 4) * 16 + v] ^= 1u << (b % 32);
+  // tables of the row order, staged in shared memory as one block of words: per bond the
+  // flipped bits (of A across the halves and within A; of the upper representative's half
+  // within that half) and the bit of B; antiparallel masks by nibbles (bit k is set for every
+  // endpoint of bond k that is up) of A and of B or the upper representative; images of B's bits
+  // under the elements of half B's list; the left multiplication table of H
+  std::vector<uint32_t> rt;
+  {
+    std::vector<uint32_t> f;
+    std::vector<uint8_t> bpos;
+    std::vector<uint32_t> mA, mB;   // bits of the bond that count in A, and in B or R(c)
+    const int iu = has_swap ? 0 : 1;   // the half of the upper representatives
+    for (int pass = 0; pass < 2; pass++) {   // bonds across and within A first
+      for (int c = 0; c < B->n_classes; c++)
+        for (int kind = pass ? 2 : 0; kind < (pass ? 3 : 2); kind++) {
+          p->kw[c][pass ? 3 : kind] = (int)f.size() / 32;
+          for (size_t b = (size_t)B->cls_word[c] * 32; b < (size_t)B->cls_word[c + 1] * 32; b++) {
+            const uint32_t fa = bond[b].x, fb = bond[b].y;
+            if (!fa && !fb) continue;   // padding
+            const uint32_t fu = iu ? fb : fa;
+            const bool across = fa && fb;
+            if (kind == 0 && across) {
+              f.push_back(fa); bpos.push_back((uint8_t)__builtin_ctz(fb)); mA.push_back(fa); mB.push_back(fb);
+            } else if (kind == 1 && !across && fa) {
+              f.push_back(fa); bpos.push_back(0); mA.push_back(fa); mB.push_back(0);
+            } else if (kind == 2 && !across && fu) {
+              f.push_back(fu); bpos.push_back(0); mA.push_back(0); mB.push_back(fu);
+            }
+          }
+          while (f.size() % 32) { f.push_back(0); bpos.push_back(0); mA.push_back(0); mB.push_back(0); }
+          p->kw[c][pass ? 4 : kind + 1] = (int)f.size() / 32;
+          if (kind == 0) p->rt_across = std::max(p->rt_across, (uint32_t)(p->kw[c][1] - p->kw[c][0]));
+        }
+      if (!pass) p->rt_wa = (uint32_t)f.size() / 32;
     }
+    p->rt_w = (uint32_t)f.size() / 32;
+    p->n_hnib = (uint32_t)(m + 3) / 4;
+    auto words = [&](const void *v, size_t bytes) -> uint32_t {
+      const uint32_t o = (uint32_t)rt.size();
+      rt.resize(rt.size() + (bytes + 3) / 4, 0u);
+      if (bytes) memcpy(rt.data() + o, v, bytes);
+      return o;
+    };
+    auto nibbles = [&](const std::vector<uint32_t> &mk) {
+      std::vector<uint32_t> t((size_t)p->rt_w * p->n_hnib * 16, 0u);
+      for (size_t b = 0; b < mk.size(); b++)
+        for (int q = 0; q < m; q++)
+          if ((mk[b] >> q) & 1u)
+            for (int v = 0; v < 16; v++)
+              if ((v >> (q % 4)) & 1) t[((b / 32) * p->n_hnib + q / 4) * 16 + v] ^= 1u << (b % 32);
+      return t;
+    };
+    const std::vector<uint32_t> tA = nibbles(mA), tB = nibbles(mB);
+    // bit q of a half pattern is a site; g carries it to a site of the half it reaches
+    auto bit_of = [&](int lab) {
+      const int X = lab / n, bit = n - 1 - lab % n;
+      return bit + ((nsub == 4 && (X == hb[0] || X == hb[2])) ? n : 0);
+    };
+    std::vector<int> label(m);
+    for (int lab = 0; lab < N; lab++) {
+      const int X = lab / n;
+      if (X == hb[2] || X == hb[3]) label[bit_of(lab)] = lab;
+    }
+    std::vector<uint8_t> im((size_t)h0 * m), lm((size_t)h0 * h0);
+    for (uint32_t y = 0; y < h0; y++)
+      for (int q = 0; q < m; q++) im[(size_t)y * m + q] = (uint8_t)bit_of(pm[(size_t)listB[y] * N + label[q]]);
+    for (uint32_t x = 0; x < h0; x++)
+      for (uint32_t y = 0; y < h0; y++) {
+        const int e = mul(H0[x], H0[y]);
+        if (e < 0 || num[e] < 0) { ed_free_pair(B); return ED_OK; }
+        lm[(size_t)x * h0 + y] = (uint8_t)num[e];
+      }
+    p->rt_f = words(f.data(), f.size() * 4);
+    p->rt_nibA = words(tA.data(), tA.size() * 4);
+    p->rt_nibB = words(tB.data(), tB.size() * 4);
+    p->rt_pos = words(bpos.data(), bpos.size());
+    p->rt_img = words(im.data(), im.size());
+    p->rt_left = words(lm.data(), lm.size());
+    p->rt_words = (uint32_t)rt.size();
+  }
   Blob blob;
   const size_t o_off = blob.add(off), o_low = blob.add(cls[0]), o_mult = blob.add(mult), o_bond = blob.add(bond),
-               o_chi = blob.add(chi), o_w = blob.add(wt), o_rw = blob.add(rwt), o_hnib = blob.add(hnib), o_start = blob.add(start),
+               o_chi = blob.add(chi), o_w = blob.add(wt), o_rw = blob.add(rwt), o_rt = blob.add(rt), o_start = blob.add(start),
                o_fup = blob.add(first_up), o_up = blob.add(up), o_tc = blob.add(tcode);
   const uint32_t zero = 0;
   const size_t o_any = blob.add(&zero, 1);
@@ -1089,7 +1389,13 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
   ED_CK(cudaMemcpyAsync(sb, blob.bytes.data(), blob.bytes.size(), cudaMemcpyHostToDevice, st));
   p->off = (uint32_t *)(sb + o_off); p->low = (uint32_t *)(sb + o_low); p->mult = sb + o_mult;
   p->bond = (uint2 *)(sb + o_bond); p->chi = (double *)(sb + o_chi); p->w = (double *)(sb + o_w); p->rw = (double *)(sb + o_rw);
-  p->half_nib = (uint32_t *)(sb + o_hnib);
+  p->rt = (uint32_t *)(sb + o_rt);
+  p->up = (uint32_t *)(sb + o_up);
+  p->t_up = has_swap ? p->ta : p->tb;
+  p->ubase = ubase;
+  p->n_ucls = (uint32_t)up.size();
+  p->no_swap = !has_swap;
+  p->any_flip = any_flip;
   p->idx = (uint32_t *)p->d_slots;
   p->meta = (uint16_t *)(p->idx + acc);
   uint32_t *d_any = (uint32_t *)(sb + o_any);
@@ -1100,6 +1406,9 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
   for (int q = 0; q < 4; q++) Q.hb[q] = hb[q];
   Q.up_half = has_swap ? 0 : 1;
   Q.idx = p->idx; Q.meta = p->meta; Q.any_weight = d_any;
+  // the row order pays when xs outgrows the L2 and a class fills many warps
+  const bool want_rows = B->D >= kRowOrderMinDim && B->D / nA >= 256 && ubase + up.size() <= 1u << (kPosShift - kClassShift);
+  if (want_rows) Q.pat = (uint32_t *)sc.get(4 * (size_t)acc);   // null without memory: no row order
   int rc = ed_launch_pair_slots(B, Q, st);
   if (rc == ED_ERR_UNSUPPORTED) { ed_free_pair(B); return ED_OK; }
   if (rc) return rc;
@@ -1107,9 +1416,8 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
   ED_CK(cudaMemcpyAsync(&any, d_any, 4, cudaMemcpyDeviceToHost, st));
   ED_CK(cudaStreamSynchronize(st));
   p->weights = any != 0;
-  // the row order pays when xs outgrows the L2 and a class fills many warps
-  if (B->D >= kRowOrderMinDim && B->D / nA >= 256)
-    if ((rc = build_rows(B, p, cls[0], off, st))) return rc;
+  if (Q.pat)
+    if ((rc = build_rows(B, p, start, Q.start, Q.pat, st))) return rc;
   cudaMemPoolProps props{};
   props.allocType = cudaMemAllocationTypePinned;
   props.location.type = cudaMemLocationTypeDevice;
@@ -1170,7 +1478,7 @@ int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, c
   const PairPlan *p = B->pair;
   if (!p) return ED_ERR_UNSUPPORTED;
   const size_t es = dtype == ED_F64 ? 8 : dtype == ED_F32 ? 4 : dtype == ED_C128 ? 16 : 8;
-  const size_t xs_bytes = al16(es * (size_t)p->n_slots);
+  const size_t xs_bytes = al16(es * ((size_t)p->n_slots + 1));
   const bool rows = p->n_slices && r0 == 0 && r1 == B->D && xs_bytes >= kRowOrderMinBytes;
   PairParams P{};
   P.n_classes = B->n_classes;
@@ -1190,13 +1498,18 @@ int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, c
   P.mult = p->mult; P.mult_bytes = p->mult_bytes;
   P.bond = p->bond;
   P.nib = B->d_nib; P.n_nib = (uint32_t)B->n_nib;
-  P.half_nib = p->half_nib; P.n_hnib = p->n_hnib;
   P.rsqrt_tab = B->d_rsqrt; P.n_sq = (uint32_t)B->nsym + 1;
   const bool cplx = dtype == ED_C128 || dtype == ED_C64;
   const bool chi = cplx && !B->is_real;
   P.chi = p->chi; P.n_chi = 1024;
   P.basis = B->d_basis; P.stab = B->d_stab;
-  P.low = p->low; P.row0 = p->row0; P.slice0 = p->slice0; P.n_slices = p->n_slices;
+  P.up = p->up; P.t_up = p->t_up; P.ubase = p->ubase; P.rt = p->rt; P.rt_words = p->rt_words;
+  memcpy(P.kw, p->kw, sizeof(P.kw));
+  P.n_w = p->rt_w; P.n_wa = p->rt_wa; P.n_up = B->n_up; P.no_swap = p->no_swap; P.by_popcount = !p->any_flip;
+  P.n_hnib = p->n_hnib; P.m = (uint32_t)p->m;
+  P.rt_f = p->rt_f; P.rt_pos = p->rt_pos; P.rt_nibA = p->rt_nibA; P.rt_nibB = p->rt_nibB; P.rt_img = p->rt_img;
+  P.rt_left = p->rt_left;
+  P.low = p->low; P.row0 = p->row0; P.slice0 = p->slice0; P.chunk_cls = p->chunk_cls; P.n_slices = p->n_slices;
   P.row_b = p->row_b; P.row_i = p->row_i; P.row_m = p->row_m; P.rw = (const double2 *)p->rw;
   P.x = x; P.y = y; P.r0 = r0; P.r1 = r1; P.partial = partial;
   P.ylo = (dtype == ED_F32 || dtype == ED_C64) ? ylo : nullptr;
@@ -1206,13 +1519,18 @@ int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, c
   put(P.off_off, 4 * (size_t)P.n_cls);
   put(P.off_mult, P.mult_bytes);
   put(P.off_bond, 8 * 32 * n_words);
-  put(P.off_nib, rows ? 4 * 2 * n_words * p->n_hnib * 16 : 4 * B->nib.size());
   put(P.off_rs, 8 * (size_t)P.n_sq);
   put(P.off_chi, chi ? 16 * 1024 : 0);
-  put(P.off_mask, 4 * (size_t)words * (rows ? kRowThreads : kThreads));
   if (rows) {
-    P.et_words = (uint32_t)(33 * n_words + 3) / 4 * 4;
+    put(P.off_rt, 4 * (size_t)P.rt_words);
+    put(P.off_mask, 4 * (size_t)p->rt_across * kRowThreads);
+    P.n_ucls = p->n_ucls;
+    P.n_tab = P.K >= 32 ? 2 : 0;   // 32 rows span two classes at most (without stabilisers)
+    P.et_words = (uint32_t)(65 * p->rt_wa + P.n_tab * (32 * (p->rt_w - p->rt_wa) + p->m) + 3) / 4 * 4;
     put(P.off_et, 4 * (size_t)P.et_words * (kRowThreads / 32));
+  } else {
+    put(P.off_nib, 4 * B->nib.size());
+    put(P.off_mask, 4 * (size_t)words * kThreads);
   }
   P.smem_bytes = (uint32_t)off;
   if (off > (size_t)(rows ? 200 : 110) * 1024) return ED_ERR_UNSUPPORTED;
@@ -1221,7 +1539,7 @@ int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, c
   // kernel takes the call
   const bool lo = dtype == ED_F32 && p->weights;
   char *ws = nullptr;
-  if (cudaMallocFromPoolAsync((void **)&ws, 16 + xs_bytes + (lo ? 4 * (size_t)p->n_slots : 0), p->pool, st) != cudaSuccess) {
+  if (cudaMallocFromPoolAsync((void **)&ws, 16 + xs_bytes + (lo ? 4 * ((size_t)p->n_slots + 1) : 0), p->pool, st) != cudaSuccess) {
     cudaGetLastError();
     return ED_ERR_UNSUPPORTED;
   }
@@ -1230,6 +1548,9 @@ int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, c
   const int eg = (int)std::min<uint32_t>((p->n_slots + 255) / 256, (uint32_t)B->sm_count * 16);
   P.xs = ws;
   P.xslo = xslo;
+  P.lo_special = lo ? kSpecial : 0u;
+  P.lo_same = lo ? 1u << kClassShift : 0u;
+  P.n_slots = p->n_slots;
   int rc = ED_OK;
   switch (dtype) {
 #define PCASE(D, V)                                                                              \

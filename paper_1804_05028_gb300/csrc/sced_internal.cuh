@@ -401,6 +401,7 @@ struct PairSlots {
   int up_half;
   uint32_t *idx;
   uint16_t *meta;
+  uint32_t *pat;         // the slot's pattern of half 1 (may be null)
   uint32_t *any_weight;
 };
 // basis.cu: out[i] = sum of in[0 .. i), *total the whole sum
