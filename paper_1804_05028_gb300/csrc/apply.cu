@@ -412,9 +412,11 @@ int ed_launch_apply(const ed_basis *B, const double *J, const double *Jz, const 
                     void *y, int dtype, int64_t r0, int64_t r1, double *partial,
                     cudaStream_t st, int mode, void *ylo) {
   if (r1 <= r0) return ED_OK;
-  if (mode == 0 && B->pair && (r1 - r0) >= B->D / 16) {
+  // The coset-arithmetic product expands the whole of x first (a pass over the slots, about
+  // 1/20 of a whole product): ranges below 1/16 of the rows go to the search kernel.
+  if (B->pair && (r1 - r0) >= B->D / 16) {
     bool done = false;
-    const int rc = ed_launch_apply_pair(B, J, Jz, x, y, dtype, r0, r1, partial, st, ylo, &done);
+    const int rc = ed_launch_apply_pair(B, J, Jz, x, y, dtype, r0, r1, partial, st, mode, ylo, &done);
     if (rc != ED_ERR_UNSUPPORTED) return rc;
   }
   {  // the specialised two-level kernels first; the generic kernel serves what they cannot

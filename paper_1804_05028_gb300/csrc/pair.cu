@@ -399,14 +399,15 @@ __device__ __forceinline__ void pair_store(const PairParams &P, const V *x, V *y
   }
 }
 
-// per-block <x, y> in a fixed order
-template <bool kC, int kT>
-__device__ __forceinline__ void pair_dot(const PairParams &P, double dot_re, double dot_im) {
+// per-block sums of n values per thread (kMode 0: <x, y>, real and imaginary part; kMode 1: the
+// classes) in a fixed order
+template <int kT>
+__device__ __forceinline__ void pair_dot(const PairParams &P, const double *v, int n) {
   if (!P.partial) return;
   __shared__ double red[kT / 32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int part = 0; part < (kC ? 2 : 1); part++) {
-    double d = part ? dot_im : dot_re;
+  for (int part = 0; part < n; part++) {
+    double d = v[part];
     for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xFFFFFFFFu, d, o);
     __syncthreads();
     if (lane == 0) red[wid] = d;
@@ -416,6 +417,21 @@ __device__ __forceinline__ void pair_dot(const PairParams &P, double dot_re, dou
       for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xFFFFFFFFu, d, o);
       if (lane == 0) P.partial[part * gridDim.x + blockIdx.x] = d;
     }
+  }
+}
+
+// Re conj(x_i) (H_c x)_i with unit exchange: the row's share of <x|H_c|x>; w is the weight
+// conj(chi) / sqrt(t) that takes the row's sum to the basis state
+template <typename V>
+__device__ __forceinline__ double class_share(const V *x, int64_t i, double diag, double jh, double2 w, double re,
+                                              double im) {
+  if constexpr (!Pv<V>::cplx) {
+    const double xi = (double)x[i];
+    return xi * (diag * xi + jh * w.x * re);
+  } else {
+    const V xv = x[i];
+    const double xr = (double)xv.x, xi = (double)xv.y;
+    return diag * (xr * xr + xi * xi) + jh * (xr * (w.x * re - w.y * im) + xi * (w.x * im + w.y * re));
   }
 }
 
@@ -429,7 +445,7 @@ __device__ __forceinline__ int next_bond(uint32_t &m, int &wd, int w0, const uin
 }
 
 // Rows in basis order: any range of rows, and sectors whose xs stays in L2.
-template <typename V, bool kChi, bool kFlips>
+template <typename V, bool kChi, bool kFlips, int kMode>
 __global__ void __launch_bounds__(kThreads, kMinBlocks) pair_kernel(const __grid_constant__ PairParams P) {
   constexpr bool kC = Pv<V>::cplx;
   constexpr int U = 2;
@@ -441,7 +457,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) pair_kernel(const __grid
   const double *rsd = reinterpret_cast<const double *>(sm + P.off_rs);
   uint32_t *mask_s = reinterpret_cast<uint32_t *>(sm + P.off_mask) + threadIdx.x;
   const V *xs = reinterpret_cast<const V *>(P.xs);
-  double dot_re = 0.0, dot_im = 0.0;
+  double dot[kMode == 1 ? ED_MAXCLS : 2] = {};
   const int64_t stride = (int64_t)gridDim.x * kThreads;
   for (int64_t i = P.r0 + (int64_t)blockIdx.x * kThreads + threadIdx.x; i < P.r1; i += stride) {
     const uint64_t s = __ldcs(reinterpret_cast<const unsigned long long *>(P.basis) + i);
@@ -477,14 +493,21 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) pair_kernel(const __grid
       };
       pair_loop<V, kChi, U>(P, nanti, gen, xs, sm + P.off_chi, acc, pend);
       pair_sum<V, kChi, U>(pend, sm + P.off_chi, acc);
-      row_re += P.jh[c] * acc.re();
-      if constexpr (kC) row_im += P.jh[c] * acc.im();
-      diag += P.jzq[c] * (double)(P.nb_cls[c] - 2 * nanti);
+      const double dg = P.jzq[c] * (double)(P.nb_cls[c] - 2 * nanti);
+      if constexpr (kMode == 1) {
+        dot[c] += class_share(reinterpret_cast<const V *>(P.x), i, dg, P.jh[c],
+                              make_double2(rsd[__ldg(P.stab + i)], 0.0), acc.re(), acc.im());
+      } else {
+        row_re += P.jh[c] * acc.re();
+        if constexpr (kC) row_im += P.jh[c] * acc.im();
+        diag += dg;
+      }
     }
-    pair_store<V>(P, reinterpret_cast<const V *>(P.x), reinterpret_cast<V *>(P.y), i, diag,
-                  rsd[__ldcs(P.stab + i)], row_re, row_im, dot_re, dot_im);
+    if constexpr (kMode == 0)
+      pair_store<V>(P, reinterpret_cast<const V *>(P.x), reinterpret_cast<V *>(P.y), i, diag,
+                    rsd[__ldcs(P.stab + i)], row_re, row_im, dot[0], dot[1]);
   }
-  pair_dot<kC, kThreads>(P, dot_re, dot_im);
+  pair_dot<kThreads>(P, dot, kMode == 1 ? P.n_classes : kC ? 2 : 1);
 }
 
 // Rows in slot order, for products whose xs is larger than the L2 keeps.  In basis order the
@@ -506,7 +529,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) pair_kernel(const __grid
 //     g_B b = R(c),  u' = R(c) with g_B's image of the flipped bits,  g_u u' = R(c')
 // makes g_u g_B the element that carries the exchanged half to R(c'), its number from the
 // left multiplication table of H.
-template <typename V, bool kChi, bool kFlips>
+template <typename V, bool kChi, bool kFlips, int kMode>
 __global__ void __launch_bounds__(kRowThreads, kRowBlocks) pair_rows_kernel(const __grid_constant__ PairParams P) {
   constexpr bool kC = Pv<V>::cplx;
   constexpr int U = sizeof(V) == 16 ? kRowU16 : sizeof(V) == 8 ? kRowU8 : kRowU;
@@ -530,7 +553,7 @@ __global__ void __launch_bounds__(kRowThreads, kRowBlocks) pair_rows_kernel(cons
   uint32_t *ma = reinterpret_cast<uint32_t *>(et + P.n_wa * 32), *eup = ma + P.n_wa;
   const uint32_t n_up2 = (P.n_w - P.n_wa) * 32, n_eup = P.m + n_up2;
   const V *xs = reinterpret_cast<const V *>(P.xs);
-  double dot_re = 0.0, dot_im = 0.0;
+  double dot[kMode == 1 ? ED_MAXCLS : 2] = {};
   uint32_t cur = 0xFFFFFFFFu, e_low = 0, off_low = 0;
   bool st_in = false, st_across = false;
   __shared__ uint32_t chunk_s;
@@ -704,10 +727,17 @@ __global__ void __launch_bounds__(kRowThreads, kRowBlocks) pair_rows_kernel(cons
         if (!kFlips && st_in) within(std::true_type()); else within(std::false_type());
       }
       pair_sum<V, kChi, U>(pend, sm + P.off_chi, acc);
-      row_re += P.jh[c] * acc.re();
-      if constexpr (kC) row_im += P.jh[c] * acc.im();
-      diag += P.jzq[c] * (double)(P.nb_cls[c] - 2 * nanti);
+      const double dg = P.jzq[c] * (double)(P.nb_cls[c] - 2 * nanti);
+      if constexpr (kMode == 1) {
+        dot[c] += class_share(reinterpret_cast<const V *>(P.x), (int64_t)__ldg(P.row_i + r), dg, P.jh[c],
+                              __ldg(P.rw + __ldg(P.row_m + r)), acc.re(), acc.im());
+      } else {
+        row_re += P.jh[c] * acc.re();
+        if constexpr (kC) row_im += P.jh[c] * acc.im();
+        diag += dg;
+      }
     }
+    if constexpr (kMode == 1) continue;
     // the sums belong to the configuration (R(lower), upper): conj(chi(h2)) takes them to the
     // representative h2 carries it to
     const double2 rw = __ldg(P.rw + __ldcs(P.row_m + r));
@@ -717,9 +747,9 @@ __global__ void __launch_bounds__(kRowThreads, kRowBlocks) pair_rows_kernel(cons
       row_re = t;
     }
     pair_store<V>(P, reinterpret_cast<const V *>(P.x), reinterpret_cast<V *>(P.y), (int64_t)__ldcs(P.row_i + r), diag,
-                  kChi ? 1.0 : rw.x, row_re, row_im, dot_re, dot_im);
+                  kChi ? 1.0 : rw.x, row_re, row_im, dot[0], dot[1]);
   }
-  pair_dot<kC, kRowThreads>(P, dot_re, dot_im);
+  pair_dot<kRowThreads>(P, dot, kMode == 1 ? P.n_classes : kC ? 2 : 1);
 }
 
 // xs[p] = w(meta[p]) x[idx[p]], w = chi sqrt(t); meta 0 is w = 1.  fp32 real vectors keep
@@ -1446,9 +1476,9 @@ namespace {
 
 size_t al16(size_t x) { return (x + 15) & ~(size_t)15; }
 
-template <typename V, bool kChi, bool kFlips>
+template <typename V, bool kChi, bool kFlips, int kMode>
 int launch_pair_t(const ed_basis *B, PairParams &P, bool rows, cudaStream_t st) {
-  auto k = rows ? pair_rows_kernel<V, kChi, kFlips> : pair_kernel<V, kChi, kFlips>;
+  auto k = rows ? pair_rows_kernel<V, kChi, kFlips, kMode> : pair_kernel<V, kChi, kFlips, kMode>;
   const int threads = rows ? kRowThreads : kThreads, per_sm = rows ? kRowBlocks : kMinBlocks;
   ED_CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, P.smem_bytes));
   const int need = per_sm * ((int)P.smem_bytes + 1536);
@@ -1462,19 +1492,25 @@ int launch_pair_t(const ed_basis *B, PairParams &P, bool rows, cudaStream_t st) 
   return ED_OK;
 }
 
-template <typename V>
-int launch_pair_v(const ed_basis *B, PairParams &P, bool chi, bool flips, bool rows, cudaStream_t st) {
+template <typename V, int kMode>
+int launch_pair_m(const ed_basis *B, PairParams &P, bool chi, bool flips, bool rows, cudaStream_t st) {
   if constexpr (Pv<V>::cplx) {
-    if (chi) return flips ? launch_pair_t<V, true, true>(B, P, rows, st) : launch_pair_t<V, true, false>(B, P, rows, st);
+    if (chi)
+      return flips ? launch_pair_t<V, true, true, kMode>(B, P, rows, st) : launch_pair_t<V, true, false, kMode>(B, P, rows, st);
   }
-  return flips ? launch_pair_t<V, false, true>(B, P, rows, st) : launch_pair_t<V, false, false>(B, P, rows, st);
+  return flips ? launch_pair_t<V, false, true, kMode>(B, P, rows, st) : launch_pair_t<V, false, false, kMode>(B, P, rows, st);
+}
+
+template <typename V>
+int launch_pair_v(const ed_basis *B, PairParams &P, bool chi, bool flips, bool rows, int mode, cudaStream_t st) {
+  return mode == 1 ? launch_pair_m<V, 1>(B, P, chi, flips, rows, st) : launch_pair_m<V, 0>(B, P, chi, flips, rows, st);
 }
 
 }  // namespace
 
 int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, const void *x, void *y,
-                         int dtype, int64_t r0, int64_t r1, double *partial, cudaStream_t st, void *ylo,
-                         bool *ylo_done) {
+                         int dtype, int64_t r0, int64_t r1, double *partial, cudaStream_t st, int mode,
+                         void *ylo, bool *ylo_done) {
   const PairPlan *p = B->pair;
   if (!p) return ED_ERR_UNSUPPORTED;
   const size_t es = dtype == ED_F64 ? 8 : dtype == ED_F32 ? 4 : dtype == ED_C128 ? 16 : 8;
@@ -1556,7 +1592,7 @@ int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, c
 #define PCASE(D, V)                                                                              \
   case D:                                                                                        \
     expand_kernel<V><<<eg, 256, 0, st>>>((const V *)x, p->idx, p->meta, (const double2 *)p->w, p->n_slots, (V *)ws, xslo, P.next); \
-    rc = cudaGetLastError() == cudaSuccess ? launch_pair_v<V>(B, P, chi, p->flips, rows, st)      \
+    rc = cudaGetLastError() == cudaSuccess ? launch_pair_v<V>(B, P, chi, p->flips, rows, mode, st)      \
                                            : ed_fail(ED_ERR_CUDA, "expand_kernel");              \
     break;
     PCASE(ED_F64, double)

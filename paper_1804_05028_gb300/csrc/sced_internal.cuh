@@ -384,8 +384,8 @@ int ed_launch_apply_fast(const ed_basis *B, const double *J, const double *Jz, c
 int ed_build_pair(ed_basis *B, cudaStream_t st);
 void ed_free_pair(ed_basis *B);
 int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, const void *x, void *y,
-                         int dtype, int64_t r0, int64_t r1, double *partial, cudaStream_t st, void *ylo,
-                         bool *ylo_done);
+                         int dtype, int64_t r0, int64_t r1, double *partial, cudaStream_t st, int mode,
+                         void *ylo, bool *ylo_done);
 // apply_fast.cu: representative, index and weight of every slot's configuration.  Slot p
 // belongs to the lower class c with start[c] <= p < start[c+1]; with r = p - start[c], the
 // upper class is first_up[c] + r / K and the element kel[r % K] carries its representative

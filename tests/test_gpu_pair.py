@@ -62,6 +62,14 @@ def test_product_of_every_type(p):
         ref = H @ xd
         tol = (2e-6 if dt in (torch.float32, torch.complex64) else 1e-12) * max(np.abs(ref).max(), 1e-30)
         assert np.abs(B.apply_H(x).cpu().numpy() - ref).max() <= tol
+        # <x|H_c|x> per class: |sum of the row shares| <= sum |x_i| |(H_c x)_i|
+        got = B.expect_classes(x, Jz=p.Jz)
+        for c in range(p.n_classes):
+            J = [0.0] * p.n_classes
+            J[c] = 1.0
+            hc = oracle.hamiltonian(p.with_couplings(J, p.Jz))[0] @ xd
+            scale = np.abs(xd) @ np.abs(hc) + np.abs(xd) @ np.abs(xd)
+            assert abs(got[c] - np.vdot(xd, hc).real) <= (2e-6 if tol > 1e-9 * np.abs(ref).max() else 1e-12) * scale
         # the rows of a range, wide enough for this product and narrower than its rule
         for r0, r1 in [(B.dim // 5, B.dim - B.dim // 7), (B.dim // 2, B.dim // 2 + max(1, B.dim // 40))]:
             r1 = min(r1, B.dim)
@@ -91,6 +99,16 @@ def test_row_order(p):
         ref = torch.cat([B.apply_H_rows(x, 0, cut), B.apply_H_rows(x, cut, D)])
         tol = 2e-6 if dt in (torch.float32, torch.complex64) else 1e-12
         assert (y - ref).abs().max() <= tol * ref.abs().max()
+        got = B.expect_classes(x)
+        xd = x.to(torch.complex128)
+        for c in range(p.n_classes):
+            J = [0.0] * p.n_classes
+            J[c] = 1.0
+            hc = B.apply_H_rows(x, 0, D - 1, J=J).to(torch.complex128)
+            ref_c = torch.vdot(xd[:-1], hc).real.item()
+            last = B.apply_H_rows(x, D - 1, D, J=J).to(torch.complex128)
+            ref_c += (xd[-1].conj() * last[0]).real.item()
+            assert abs(got[c] - ref_c) <= tol * (xd.abs()[:-1] @ hc.abs()).item()
 
 
 def test_streams_and_capture():
