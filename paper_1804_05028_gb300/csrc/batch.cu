@@ -28,6 +28,12 @@ struct BatchSector {
   void *y;
   int64_t D;
   int64_t item0;     // first work item of this sector
+  // orbit tables (kOrbit): per configuration the rank of its orbit among those of its S^z,
+  // the minimising element and whether |Stab| > 1; basis index by rank (null: the rank itself);
+  // chi per element, as signs for real sectors
+  const uint32_t *otab, *jmap;
+  const float2 *chi;
+  uint32_t sign[8];
   int cplx;
   int pad;
 };
@@ -42,6 +48,8 @@ struct ed_batch {
   uint8_t *d_bond = nullptr;
   float *d_ftab = nullptr;   // the sectors' fp32 norm and phase tables, back to back
   bool all_full = false;     // every sector has a one-sublattice (whole) table
+  bool orbit = false;        // and the orbit tables were made
+  std::vector<void *> d_orbit;   // orbit tables (per group) and index maps
   int cls_off[ED_MAXCLS + 1];
   double jh[ED_MAXCLS], jzq[ED_MAXCLS];
   const uint32_t *nib = nullptr;   // the first basis's nibble tables (shared lattice)
@@ -139,12 +147,83 @@ __device__ __forceinline__ F8 ld8(const float *p) {
 }
 static_assert(sizeof(BatchSector) % 4 == 0, "sector descriptors are copied as 32-bit words");
 
-// kFull: every sector looks its representatives up in a whole table (one sublattice), so
-// the block-wise search is not compiled in and the kernel needs far fewer registers.
+// Entry of an orbit table: rank | element << kOrbitBits | (|Stab| > 1) << 31
+constexpr int kOrbitBits = 23;
+
+// Ranks of the orbits of a whole table among those with the same number of up spins, in the
+// order of their representatives.  Blocks of 1024 configurations count their representatives
+// per popcount; the counts, scanned popcount by popcount, give each block's first rank.
+constexpr int kRankBlock = 1024;
+
+__global__ void __launch_bounds__(256) orbit_counts(const uint64_t *full, uint32_t total, uint32_t n_blocks,
+                                                    uint32_t *counts) {
+  __shared__ uint32_t h[32];
+  for (uint32_t b = blockIdx.x; b < n_blocks; b += gridDim.x) {
+    if (threadIdx.x < 32) h[threadIdx.x] = 0;
+    __syncthreads();
+    for (int q = 0; q < kRankBlock / 256; q++) {
+      const uint32_t s = b * kRankBlock + q * 256 + threadIdx.x;
+      if (s < total && (uint32_t)__ldg(full + s) == s) atomicAdd(&h[__popc(s)], 1u);
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) counts[threadIdx.x * n_blocks + b] = h[threadIdx.x];
+    __syncthreads();
+  }
+}
+
+// first[pop * n_blocks + b]: representatives before block b in the order (popcount, value)
+__global__ void __launch_bounds__(32) orbit_ranks(const uint64_t *full, uint32_t total, uint32_t n_blocks,
+                                                  const uint64_t *first, uint32_t *rank) {
+  __shared__ uint32_t next[32];
+  const int lane = threadIdx.x;
+  for (uint32_t b = blockIdx.x; b < n_blocks; b += gridDim.x) {
+    next[lane] = (uint32_t)(first[(uint64_t)lane * n_blocks + b] - first[(uint64_t)lane * n_blocks]);
+    __syncwarp();
+    for (int q = 0; q < kRankBlock / 32; q++) {
+      const uint32_t s = b * kRankBlock + q * 32 + lane;
+      const bool rep = s < total && (uint32_t)__ldg(full + s) == s;
+      const int pc = rep ? __popc(s) : 32 + lane;   // lanes without one match nobody
+      const unsigned same = __match_any_sync(0xFFFFFFFFu, pc);
+      const uint32_t before = rep ? next[pc] : 0;
+      __syncwarp();
+      if (rep) {
+        const int below = __popc(same & ((1u << lane) - 1u));
+        rank[s] = before + below;
+        if (below == 0) next[pc] = before + __popc(same);
+      }
+      __syncwarp();
+    }
+  }
+}
+
+__global__ void __launch_bounds__(256) orbit_table(const uint64_t *full, uint32_t total, const uint32_t *rank,
+                                                   uint32_t *otab) {
+  for (uint32_t s = blockIdx.x * 256 + threadIdx.x; s < total; s += gridDim.x * 256) {
+    const uint64_t e = __ldg(full + s);
+    otab[s] = __ldg(rank + (uint32_t)e) | (uint32_t)((e >> 32) & 0xFFu) << kOrbitBits |
+              ((e >> 48) > 1 ? 0x80000000u : 0u);
+  }
+}
+
+__global__ void __launch_bounds__(256) orbit_index(const uint64_t *basis, int64_t D, const uint32_t *otab,
+                                                   uint32_t *jmap) {
+  for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < D; i += (int64_t)gridDim.x * 256)
+    jmap[otab[basis[i]] & ((1u << kOrbitBits) - 1u)] = (uint32_t)i;
+}
+
+// How a sector finds a term's index.  kSearch: any split, the block-wise search and the
+// Limits lookup.  kFull: every sector has a whole table (one sublattice), so the block-wise
+// search is not compiled in.  kOrbit: whole tables small enough for orbit tables (|G| <= 256,
+// fewer than 2^23 orbits per S^z, device memory for 4 bytes per configuration and group):
+// every term's accesses run through the L1 data pipe, which bounds this kernel, so a 4-byte
+// entry with the orbit's rank replaces the 8-byte one, the prefix rank and the 16-byte record
+// of the ranked Limits; chi is one load (signs: bits of the warp's sector descriptor).
+enum Lookup { kSearch, kFull, kOrbit };
+
 // Resident blocks per SM: 6 up to k = 4; 5 for k = 8 (48 registers and a small spill),
 // which beat 4 (63 registers) by 5% and 6 (42 registers) by 3%.
-template <int K, bool kFull>
-__global__ void __launch_bounds__(kBatchThreads, kFull ? (K <= 4 ? 6 : 5) : 1)
+template <int K, Lookup kLook>
+__global__ void __launch_bounds__(kBatchThreads, kLook != kSearch ? (K <= 4 ? 6 : 5) : 1)
     batch_kernel(const BatchParams P) {
   // each warp takes its own work items and keeps its own copy of the sector descriptor,
   // so no warp waits at a block-wide barrier for another warp's rows
@@ -196,23 +275,50 @@ __global__ void __launch_bounds__(kBatchThreads, kFull ? (K <= 4 ? 6 : 5) : 1)
             am &= am - 1;
             const int pa = bond_s[2 * b], pb = bond_s[2 * b + 1];
             const uint64_t s2 = s ^ ((1ULL << pa) | (1ULL << pb));
-            RepOut R;
-            if constexpr (kFull) {
-              const uint64_t e = __ldg(S.T.full + s2);
-              R.rep = e & 0xFFFFFFFFull;
-              R.g = (int)((e >> 32) & 0xFFFF);
-              R.t = (int)(e >> 48);
+            int64_t j;
+            float w = jh, cr = 0.f, ci = 0.f;
+            bool neg = false;
+            if constexpr (kLook == kOrbit) {
+              const uint32_t e = __ldg(S.otab + s2);
+              uint32_t o = e & ((1u << kOrbitBits) - 1u);
+              if (S.jmap) {
+                o = __ldg(S.jmap + o);
+                if (o == 0xFFFFFFFFu) continue;
+              }
+              j = o;
+              if (e >> 31) w *= __ldg(S.sqrt_f + __ldg(S.I.stab + j));   // rare
+              const uint32_t g = (e >> kOrbitBits) & 0xFFu;
+              if (S.cplx) {
+                const float2 ch = __ldg(S.chi + g);
+                cr = ch.x * w;
+                ci = ch.y * w;
+              } else {
+                neg = (S.sign[g >> 5] >> (g & 31)) & 1u;
+              }
             } else {
-              R = find_rep(S.T, S.T.rep, S.T.sym_off, S.T.sym_list, S.T.dest, S.T.phase, s2);
-              if (R.mixed) continue;
+              RepOut R;
+              if constexpr (kLook == kFull) {
+                const uint64_t e = __ldg(S.T.full + s2);
+                R.rep = e & 0xFFFFFFFFull;
+                R.g = (int)((e >> 32) & 0xFFFF);
+                R.t = (int)(e >> 48);
+              } else {
+                R = find_rep(S.T, S.T.rep, S.T.sym_off, S.T.sym_list, S.T.dest, S.T.phase, s2);
+                if (R.mixed) continue;
+              }
+              j = kLook == kFull ? lookup_index32(S.I, (uint32_t)R.rep) : lookup_index(S.I, R.rep);
+              if (j < 0) continue;
+              if (R.t != 1) w *= __ldg(S.sqrt_f + R.t);   // t = |Stab| of the target, mostly 1
+              const int ph = __ldg(S.T.phase + R.g);
+              if (S.cplx) {
+                cr = __ldg(S.cs_f + 2 * ph) * w;
+                ci = __ldg(S.cs_f + 2 * ph + 1) * w;
+              } else {
+                neg = ph != 0;
+              }
             }
-            const int64_t j = kFull ? lookup_index32(S.I, (uint32_t)R.rep) : lookup_index(S.I, R.rep);
-            if (j < 0) continue;
-            float w = jh;
-            if (R.t != 1) w *= __ldg(S.sqrt_f + R.t);   // t = |Stab| of the target, mostly 1
-            const int ph = __ldg(S.T.phase + R.g);
             if (!S.cplx) {
-              const float sg = ph == 0 ? w : -w;
+              const float sg = neg ? -w : w;
               const float *xr = reinterpret_cast<const float *>(S.x) + j * K;
               if constexpr (K % 8 == 0) {
   #pragma unroll
@@ -232,7 +338,6 @@ __global__ void __launch_bounds__(kBatchThreads, kFull ? (K <= 4 ? 6 : 5) : 1)
                 for (int v = 0; v < K; v++) yr[v] += sg * xr[v];
               }
             } else {
-              const float cr = __ldg(S.cs_f + 2 * ph) * w, ci = __ldg(S.cs_f + 2 * ph + 1) * w;
               const float2 *xc = reinterpret_cast<const float2 *>(S.x) + j * K;
               if constexpr (K % 4 == 0) {   // four complex entries per 32-byte load
   #pragma unroll
@@ -332,10 +437,11 @@ int launch(ed_batch *Bt, int rows_per_item, cudaStream_t st) {
   for (int c = 0; c < Bt->n_classes; c++) { P.jh[c] = (float)Bt->jh[c]; P.jzq[c] = (float)Bt->jzq[c]; }
   ED_CK(cudaMemsetAsync(Bt->d_counter, 0, 8, st));
   const int grid = Bt->sm_count * 8;
-  switch (Bt->k * 2 + (Bt->all_full ? 1 : 0)) {
+  switch (Bt->k * 4 + (Bt->orbit ? 2 : Bt->all_full ? 1 : 0)) {
 #define BCASE(K)                                                     \
-  case 2 * K: batch_kernel<K, false><<<grid, kBatchThreads, 0, st>>>(P); break; \
-  case 2 * K + 1: batch_kernel<K, true><<<grid, kBatchThreads, 0, st>>>(P); break;
+  case 4 * K: batch_kernel<K, kSearch><<<grid, kBatchThreads, 0, st>>>(P); break; \
+  case 4 * K + 1: batch_kernel<K, kFull><<<grid, kBatchThreads, 0, st>>>(P); break; \
+  case 4 * K + 2: batch_kernel<K, kOrbit><<<grid, kBatchThreads, 0, st>>>(P); break;
     BCASE(1)
     BCASE(2)
     BCASE(4)
@@ -344,6 +450,109 @@ int launch(ed_batch *Bt, int rows_per_item, cudaStream_t st) {
     default: return ed_fail(ED_ERR_INVALID, "block width k must be 1, 2, 4 or 8");
   }
   ED_CK(cudaGetLastError());
+  return ED_OK;
+}
+
+// Orbit tables of the batch's groups and the index maps of its sectors; Bt->orbit stays false
+// (the whole-table kernel serves the batch) where they do not fit.
+int build_orbits(ed_batch *Bt) {
+  if (!Bt->all_full) return ED_OK;
+  const ed_basis *b0 = Bt->bases[0];
+  const int N = b0->N;
+  if (N < 10) return ED_OK;   // less than one block of configurations
+  const uint32_t total = 1u << N, n_blocks = total / kRankBlock;
+  struct Table { const uint64_t *full; uint32_t *otab; std::vector<uint64_t> first; };
+  std::vector<Table> tables;
+  auto drop = [&]() {
+    for (void *q : Bt->d_orbit) cudaFree(q);
+    Bt->d_orbit.clear();
+    cudaGetLastError();
+  };
+  auto get = [&](size_t bytes) -> void * {
+    void *q = nullptr;
+    if (cudaMalloc(&q, bytes) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    Bt->d_orbit.push_back(q);
+    return q;
+  };
+  for (const ed_basis *B : Bt->bases)
+    if (B->nsym > 256) return ED_OK;
+  uint32_t *d_rank = nullptr, *d_counts = nullptr;
+  uint64_t *d_first = nullptr;
+  struct Free {   // scratch, released on every path
+    uint32_t **a, **b;
+    uint64_t **c;
+    ~Free() { cudaFree(*a); cudaFree(*b); cudaFree(*c); }
+  } scratch{&d_rank, &d_counts, &d_first};
+  if (cudaMalloc(&d_rank, 4 * (size_t)total) != cudaSuccess || cudaMalloc(&d_counts, 128 * (size_t)n_blocks) != cudaSuccess ||
+      cudaMalloc(&d_first, 256 * (size_t)n_blocks) != cudaSuccess) {
+    drop();
+    return ED_OK;
+  }
+  const int grid = Bt->sm_count * 8;
+  std::vector<size_t> table_of(Bt->n);
+  for (int s = 0; s < Bt->n; s++) {
+    const ed_basis *B = Bt->bases[s];
+    size_t t = 0;
+    while (t < tables.size() && tables[t].full != B->T.full) t++;
+    table_of[s] = t;
+    if (t < tables.size()) continue;
+    Table T{B->T.full, (uint32_t *)get(4 * (size_t)total), {}};
+    if (!T.otab) { drop(); return ED_OK; }
+    orbit_counts<<<grid, 256>>>(T.full, total, n_blocks, d_counts);
+    ED_CK(cudaGetLastError());
+    uint64_t all = 0;
+    int rc = ed_exclusive_scan(d_counts, 32 * (uint64_t)n_blocks, d_first, &all, 0);
+    if (rc) return rc;
+    orbit_ranks<<<Bt->sm_count * 32, 32>>>(T.full, total, n_blocks, d_first, d_rank);
+    ED_CK(cudaGetLastError());
+    orbit_table<<<grid, 256>>>(T.full, total, d_rank, T.otab);
+    ED_CK(cudaGetLastError());
+    T.first.assign(33, all);   // orbits with fewer up spins
+    ED_CK(cudaMemcpy2D(T.first.data(), 8, d_first, 8 * (size_t)n_blocks, 8, 32, cudaMemcpyDeviceToHost));
+    for (int q = 0; q < 32; q++)
+      if (T.first[q + 1] - T.first[q] >= 1ull << kOrbitBits) { drop(); return ED_OK; }
+    tables.push_back(T);
+  }
+  size_t maps = 0;
+  std::vector<size_t> at(Bt->n, 0);
+  std::vector<float2> chi;
+  std::vector<size_t> chi_at(Bt->n, 0);
+  auto orbits = [&](int s) { const Table &T = tables[table_of[s]]; return (size_t)(T.first[Bt->bases[s]->n_up + 1] - T.first[Bt->bases[s]->n_up]); };
+  for (int s = 0; s < Bt->n; s++) {
+    const ed_basis *B = Bt->bases[s];
+    if (orbits(s) != (size_t)B->D) { at[s] = maps; maps += orbits(s); }
+    chi_at[s] = chi.size();
+    if (!B->is_real)
+      for (int g = 0; g < B->nsym; g++) {
+        const double a = 2.0 * M_PI * (double)B->phase[g] / (double)B->denom;
+        chi.push_back(make_float2((float)std::cos(a), (float)std::sin(a)));
+      }
+  }
+  uint32_t *d_maps = maps ? (uint32_t *)get(4 * maps) : nullptr;
+  float2 *d_chi = chi.empty() ? nullptr : (float2 *)get(8 * chi.size());
+  if ((maps && !d_maps) || (!chi.empty() && !d_chi)) { drop(); return ED_OK; }
+  if (maps) ED_CK(cudaMemset(d_maps, 0xFF, 4 * maps));
+  if (!chi.empty()) ED_CK(cudaMemcpy(d_chi, chi.data(), 8 * chi.size(), cudaMemcpyHostToDevice));
+  for (int s = 0; s < Bt->n; s++) {
+    const ed_basis *B = Bt->bases[s];
+    BatchSector &S = Bt->host[s];
+    S.otab = tables[table_of[s]].otab;
+    S.jmap = nullptr;
+    if (orbits(s) != (size_t)B->D) {
+      S.jmap = d_maps + at[s];
+      if (B->D > 0) {
+        orbit_index<<<(int)std::min<int64_t>((B->D + 255) / 256, grid), 256>>>(B->d_basis, B->D, S.otab, d_maps + at[s]);
+        ED_CK(cudaGetLastError());
+      }
+    }
+    S.chi = d_chi ? d_chi + chi_at[s] : nullptr;
+    for (int q = 0; q < 8; q++) S.sign[q] = 0;
+    if (B->is_real)
+      for (int g = 0; g < B->nsym; g++)
+        if (B->phase[g]) S.sign[g >> 5] |= 1u << (g & 31);
+  }
+  ED_CK(cudaDeviceSynchronize());
+  Bt->orbit = true;
   return ED_OK;
 }
 
@@ -416,6 +625,7 @@ extern "C" int ed_batch_create(ed_basis *const *bases, int32_t n, const double *
     S.rsqrt_f = S.sqrt_f + ns + 1;
     S.cs_f = S.rsqrt_f + ns + 1;
   }
+  if (const int rc = build_orbits(Bt)) { ed_batch_free(Bt); return rc; }
   *out = Bt;
   return ED_OK;
 }
@@ -519,5 +729,6 @@ extern "C" void ed_batch_free(ed_batch *Bt) {
   if (Bt->d_counter) cudaFree(Bt->d_counter);
   if (Bt->d_bond) cudaFree(Bt->d_bond);
   if (Bt->d_ftab) cudaFree(Bt->d_ftab);
+  for (void *q : Bt->d_orbit) cudaFree(q);
   delete Bt;
 }
