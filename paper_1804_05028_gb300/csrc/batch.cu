@@ -16,6 +16,7 @@
 #include <algorithm>
 #include <cmath>
 #include <chrono>
+#include <type_traits>
 #include <vector>
 
 struct BatchSector {
@@ -220,17 +221,19 @@ __global__ void __launch_bounds__(256) orbit_index(const uint64_t *basis, int64_
 // of the ranked Limits; chi is one load (signs: bits of the warp's sector descriptor).
 enum Lookup { kSearch, kFull, kOrbit };
 
-// Resident blocks per SM: 6 up to k = 4; 5 for k = 8 (48 registers and a small spill),
-// which beat 4 (63 registers) by 5% and 6 (42 registers) by 3%.
+// Resident blocks per SM: 6 up to k = 4 (40 registers); 4 for k = 8 (64 registers), which beat
+// 5 (48 registers and a small spill) by 8% with the orbit tables.
 template <int K, Lookup kLook>
-__global__ void __launch_bounds__(kBatchThreads, kLook != kSearch ? (K <= 4 ? 6 : 5) : 1)
+__global__ void __launch_bounds__(kBatchThreads, kLook != kSearch ? (K <= 4 ? 6 : 4) : 1)
     batch_kernel(const BatchParams P) {
   // each warp takes its own work items and keeps its own copy of the sector descriptor,
   // so no warp waits at a block-wide barrier for another warp's rows
   __shared__ BatchSector S_w[kBatchThreads / 32];
-  __shared__ uint8_t bond_s[2 * ED_MAXBONDS / 8];
+  using State = typename std::conditional<kLook == kSearch, uint64_t, uint32_t>::type;   // N <= 26 otherwise
+  __shared__ State bond_s[ED_MAXBONDS / 8];   // the two bits a bond's exchange flips
   const int nb = P.cls_off[P.n_classes];
-  for (int q = threadIdx.x; q < 2 * nb; q += blockDim.x) bond_s[q] = P.bond[q];
+  for (int q = threadIdx.x; q < nb; q += blockDim.x)
+    bond_s[q] = (State)1 << P.bond[2 * q] | (State)1 << P.bond[2 * q + 1];
   __syncthreads();
   const int lane = threadIdx.x & 31;
   BatchSector &S = S_w[threadIdx.x >> 5];
@@ -249,9 +252,15 @@ __global__ void __launch_bounds__(kBatchThreads, kLook != kSearch ? (K <= 4 ? 6 
       __syncwarp();
       cur = sid;
     }
+    // what every term reads of the descriptor, in registers: a shared-memory read each would
+    // take a quarter of the data pipe
+    const uint32_t *otab = S.otab, *jmap = S.jmap;
+    const float2 *chi = S.chi;
+    const void *xv = S.x;
+    const bool cplx = S.cplx != 0;
     for (int64_t i = (item - S.item0) * P.rows_per_item + lane;
          i < S.D && i < (item - S.item0 + 1) * P.rows_per_item; i += 32) {
-      const uint64_t s = __ldcs(reinterpret_cast<const unsigned long long *>(S.I.basis) + i);
+      const State s = (State)__ldcs(reinterpret_cast<const unsigned long long *>(S.I.basis) + i);
       const int ti = __ldcs(S.I.stab + i);
       float yr[K], yi[K];
 #pragma unroll
@@ -273,23 +282,22 @@ __global__ void __launch_bounds__(kBatchThreads, kLook != kSearch ? (K <= 4 ? 6 
           while (am) {
             const int b = b0 + __ffs(am) - 1;
             am &= am - 1;
-            const int pa = bond_s[2 * b], pb = bond_s[2 * b + 1];
-            const uint64_t s2 = s ^ ((1ULL << pa) | (1ULL << pb));
+            const State s2 = s ^ bond_s[b];
             int64_t j;
             float w = jh, cr = 0.f, ci = 0.f;
             bool neg = false;
             if constexpr (kLook == kOrbit) {
-              const uint32_t e = __ldg(S.otab + s2);
+              const uint32_t e = __ldg(otab + s2);
               uint32_t o = e & ((1u << kOrbitBits) - 1u);
-              if (S.jmap) {
-                o = __ldg(S.jmap + o);
+              if (jmap) {
+                o = __ldg(jmap + o);
                 if (o == 0xFFFFFFFFu) continue;
               }
               j = o;
               if (e >> 31) w *= __ldg(S.sqrt_f + __ldg(S.I.stab + j));   // rare
               const uint32_t g = (e >> kOrbitBits) & 0xFFu;
-              if (S.cplx) {
-                const float2 ch = __ldg(S.chi + g);
+              if (cplx) {
+                const float2 ch = __ldg(chi + g);
                 cr = ch.x * w;
                 ci = ch.y * w;
               } else {
@@ -310,16 +318,16 @@ __global__ void __launch_bounds__(kBatchThreads, kLook != kSearch ? (K <= 4 ? 6 
               if (j < 0) continue;
               if (R.t != 1) w *= __ldg(S.sqrt_f + R.t);   // t = |Stab| of the target, mostly 1
               const int ph = __ldg(S.T.phase + R.g);
-              if (S.cplx) {
+              if (cplx) {
                 cr = __ldg(S.cs_f + 2 * ph) * w;
                 ci = __ldg(S.cs_f + 2 * ph + 1) * w;
               } else {
                 neg = ph != 0;
               }
             }
-            if (!S.cplx) {
+            if (!cplx) {
               const float sg = neg ? -w : w;
-              const float *xr = reinterpret_cast<const float *>(S.x) + j * K;
+              const float *xr = reinterpret_cast<const float *>(xv) + j * K;
               if constexpr (K % 8 == 0) {
   #pragma unroll
                 for (int v = 0; v < K; v += 8) {
@@ -338,7 +346,7 @@ __global__ void __launch_bounds__(kBatchThreads, kLook != kSearch ? (K <= 4 ? 6 
                 for (int v = 0; v < K; v++) yr[v] += sg * xr[v];
               }
             } else {
-              const float2 *xc = reinterpret_cast<const float2 *>(S.x) + j * K;
+              const float2 *xc = reinterpret_cast<const float2 *>(xv) + j * K;
               if constexpr (K % 4 == 0) {   // four complex entries per 32-byte load
   #pragma unroll
                 for (int v = 0; v < K; v += 4) {
