@@ -270,12 +270,27 @@ __global__ void dot_kernel(const V *x, const V *y, int64_t n, double *partial) {
 // rounding remainder -- and leaves the same way, so that the update rounds nothing; the
 // norm is that of the pair.  The fp64 pipe of this GPU is too slow for a pass of fp64
 // arithmetic over the whole vector.
+// With part (may be null) a is not given but the sum of its n_part block partials of <v, w>,
+// added up by every block in the same order and stored to a_out: the host need not wait for
+// the product before it launches the update.
 template <typename V>
-__global__ void axpy_norm_kernel(V *w, const V *v, const V *vprev, double a, double b,
-                                 int64_t n, double *partial, V *wlo) {
+__global__ void __launch_bounds__(256) axpy_norm_kernel(V *w, const V *v, const V *vprev, double a, double b,
+                                                        int64_t n, double *partial, V *wlo,
+                                                        const double *part, int n_part, double *a_out) {
   using A = typename Vt<V>::A;
   constexpr bool kF = sizeof(A) == 4;
   double acc = 0;
+  if (part) {
+    __shared__ double sum_s[8];
+    double d = 0;
+    for (int k = threadIdx.x; k < n_part; k += 256) d += part[k];
+    for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xFFFFFFFFu, d, o);
+    if ((threadIdx.x & 31) == 0) sum_s[threadIdx.x >> 5] = d;
+    __syncthreads();
+    a = 0;
+    for (int k = 0; k < 8; k++) a += sum_s[k];
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a_out = a;
+  }
   float ah = 0.f, al = 0.f, bh = 0.f, bl = 0.f, nh = 0.f, nl = 0.f;
   if constexpr (kF) {
     df_split(a, ah, al);
@@ -538,10 +553,37 @@ int ed_launch_dot(const ed_basis *B, const void *x, const void *y, int dtype, do
 
 int ed_launch_axpy_norm(const ed_basis *B, void *w, const void *v, const void *vprev, double a,
                         double b, int dtype, double *partial, int nblk, cudaStream_t st,
-                        void *wlo) {
+                        void *wlo, const double *part, int n_part, double *a_out) {
   ED_DISPATCH(dtype, (axpy_norm_kernel<V><<<nblk, 256, 0, st>>>((V *)w, (const V *)v,
                                                                 (const V *)vprev, a, b, B->D,
-                                                                partial, (V *)wlo)));
+                                                                partial, (V *)wlo, part, n_part, a_out)));
+  ED_CK(cudaGetLastError());
+  return ED_OK;
+}
+
+// what the host reads of a Lanczos step, in one copy: alpha, the sweeps' corrections to it
+// (null: 0) and ||w||^2 from its block partials
+__global__ void __launch_bounds__(256) step_scalars_kernel(const double *alpha, const double *corr0, const double *corr1,
+                                                           const double *part, int n_part, double *out) {
+  __shared__ double sum_s[8];
+  double d = 0;
+  for (int k = threadIdx.x; k < n_part; k += 256) d += part[k];
+  for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xFFFFFFFFu, d, o);
+  if ((threadIdx.x & 31) == 0) sum_s[threadIdx.x >> 5] = d;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    d = 0;
+    for (int k = 0; k < 8; k++) d += sum_s[k];
+    out[0] = *alpha;
+    out[1] = corr0 ? *corr0 : 0.0;
+    out[2] = corr1 ? *corr1 : 0.0;
+    out[3] = d;
+  }
+}
+
+int ed_launch_step_scalars(const double *alpha, const double *corr0, const double *corr1, const double *part,
+                           int n_part, double *out, cudaStream_t st) {
+  step_scalars_kernel<<<1, 256, 0, st>>>(alpha, corr0, corr1, part, n_part, out);
   ED_CK(cudaGetLastError());
   return ED_OK;
 }

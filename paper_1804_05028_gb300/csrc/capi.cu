@@ -781,8 +781,11 @@ struct LanczosRun {
   int store_slots = 0;
   int reorth = ED_REORTH_LOCAL;
   double *d_ro = nullptr;  // sweep partials [m_cap * P * grid], then coefficients [m_cap * P]
-  size_t ro_coef_off = 0;
+  size_t ro_coef_off = 0, coef_len = 0;
+  double *d_scalar = nullptr;  // alpha, then the four scalars the host reads of a step
+  int nblk = 1;                // blocks of the dot products and of the three-term update
   cudaEvent_t e0, e1, r0, r1;
+  std::vector<cudaEvent_t> replay_ev;   // around every product of the replay pass
   double ms_apply = 0, ms_reorth = 0;
   void *slot(int k) const { return store + (size_t)k * elem_bytes(); }
   size_t elem_bytes() const {
@@ -792,47 +795,20 @@ struct LanczosRun {
 
 // The sweeps of step j after the three-term update of w.  Local: one sweep against v_j and
 // v_{j-1} (the second Gram-Schmidt pass of the recurrence's own projection).  Full: two
-// sweeps against every stored v_0 .. v_j (classical Gram-Schmidt, twice).  *corr gets
-// Re <v_j, w> summed over the sweeps (added to alpha_j so that the tridiagonal matrix stays
-// the projection of H), *b2 the new ||w||^2; both only when want_host (the replay pass
-// reuses the stored alpha and beta and skips the copies).
-int reorth_step(LanczosRun &L, int j, void *w, const void *v, const void *vprev, bool want_host,
-                double *corr, double *b2) {
+// sweeps against every stored v_0 .. v_j (classical Gram-Schmidt, twice).  corr[sw] points to
+// Re <v_j, w> of sweep sw (device; their sum is added to alpha_j so that the tridiagonal
+// matrix stays the projection of H); the new ||w||^2 partials are in L.d_ro.
+int reorth_step(LanczosRun &L, int j, void *w, const void *v, const void *vprev, const double *(&corr)[2]) {
   ed_basis *B = L.B;
   const int P = L.cplx ? 2 : 1;
-  const int grid = ed_reorth_grid(B);
-  double *c = L.d_ro + L.ro_coef_off;
-  ED_CK(cudaEventRecord(L.r0, L.st));
-  const int sweeps = L.reorth == ED_REORTH_FULL ? 2 : 1;
-  double cj = 0.0;
-  for (int sw = 0; sw < sweeps; sw++) {
-    int rc, jj;
-    if (L.reorth == ED_REORTH_FULL) {
-      rc = ed_launch_reorth_sweep(B, w, L.store, nullptr, nullptr, j + 1, L.dtype, L.d_ro, c, L.st, L.ylo);
-      jj = j;
-    } else {
-      rc = ed_launch_reorth_sweep(B, w, nullptr, v, vprev, j ? 2 : 1, L.dtype, L.d_ro, c, L.st, L.ylo);
-      jj = 0;
-    }
+  const bool full = L.reorth == ED_REORTH_FULL;
+  const int m = full ? j + 1 : j ? 2 : 1;
+  for (int sw = 0; sw < (full ? 2 : 1); sw++) {
+    double *c = L.d_ro + L.ro_coef_off + (size_t)sw * L.coef_len;
+    const int rc = full ? ed_launch_reorth_sweep(B, w, L.store, nullptr, nullptr, m, L.dtype, L.d_ro, c, L.st, L.ylo)
+                        : ed_launch_reorth_sweep(B, w, nullptr, v, vprev, m, L.dtype, L.d_ro, c, L.st, L.ylo);
     if (rc) return rc;
-    if (want_host) {
-      double h = 0;
-      ED_CK(cudaMemcpyAsync(&B->h_partial[0], c + (size_t)jj * P, 8, cudaMemcpyDeviceToHost, L.st));
-      ED_CK(cudaStreamSynchronize(L.st));
-      h = B->h_partial[0];
-      cj += h;
-    }
-  }
-  ED_CK(cudaEventRecord(L.r1, L.st));
-  if (want_host) {
-    double nn = 0, im = 0;
-    int rc = reduce_partials(B, L.d_ro, grid, false, L.st, &nn, &im);
-    if (rc) return rc;
-    float ms = 0;
-    ED_CK(cudaEventElapsedTime(&ms, L.r0, L.r1));
-    L.ms_reorth += ms;
-    *corr = cj;
-    *b2 = nn;
+    corr[sw] = c + (size_t)(full ? j : 0) * P;
   }
   return ED_OK;
 }
@@ -844,7 +820,7 @@ int lanczos_pass(LanczosRun &L, const ed_lanczos_opts *o, int max_steps, bool fi
                  std::vector<double> &beta, double *E0, int *steps, int *converged,
                  const std::vector<double> *coef, void *psi) {
   ed_basis *B = L.B;
-  const int nblk = B->n_partial / 2;
+  const int nblk = L.nblk;
   const bool full = L.reorth == ED_REORTH_FULL;
   void *vprev = full ? nullptr : L.v[0], *v = full ? L.slot(0) : L.v[1], *w = full ? nullptr : L.v[2];
   int rc;
@@ -868,26 +844,48 @@ int lanczos_pass(LanczosRun &L, const ed_lanczos_opts *o, int max_steps, bool fi
     if (full) { v = L.slot(j); vprev = j ? L.slot(j - 1) : nullptr; w = L.slot(j + 1); }
     if (replay) { if ((rc = ed_launch_axpy(B, psi, v, (*coef)[j], L.dtype, L.st))) return rc; }
     if (replay && j == m_total - 1) break;
-    ED_CK(cudaEventRecord(L.e0, L.st));
-    if ((rc = ed_launch_apply(B, L.J, L.Jz, v, w, L.dtype, 0, B->D, B->d_partial, L.st, 0, L.ylo))) return rc;
-    ED_CK(cudaEventRecord(L.e1, L.st));
-    double a;
-    if (replay) {
-      a = alpha_rec[j];
-    } else {
-      if ((rc = reduce_partials(B, B->d_partial, B->last_apply_grid, L.cplx, L.st, &a, nullptr))) return rc;
+    cudaEvent_t e0 = L.e0, e1 = L.e1;
+    if (replay) {   // nothing waits for a step here, so every product needs its own events
+      for (cudaEvent_t *e : {&e0, &e1}) {
+        ED_CK(cudaEventCreate(e));
+        L.replay_ev.push_back(*e);
+      }
     }
-    float ms = 0;
-    ED_CK(cudaEventSynchronize(L.e1));
-    ED_CK(cudaEventElapsedTime(&ms, L.e0, L.e1));
-    L.ms_apply += ms;
+    ED_CK(cudaEventRecord(e0, L.st));
+    if ((rc = ed_launch_apply(B, L.J, L.Jz, v, w, L.dtype, 0, B->D, B->d_partial, L.st, 0, L.ylo))) return rc;
+    ED_CK(cudaEventRecord(e1, L.st));
     const double bprev = j ? beta[j - 1] : 0.0;
-    if ((rc = ed_launch_axpy_norm(B, w, v, j ? vprev : nullptr, a, bprev, L.dtype, B->d_partial, nblk, L.st, L.ylo))) return rc;
-    double b2 = 0, corr = 0;
+    // alpha_j stays on the device until the step's scalars are read: the update sums the
+    // product's partials (its own go behind them)
+    const int n_dot = B->last_apply_grid;
+    double *part2 = B->d_partial + B->n_partial / 2;
+    if ((rc = ed_launch_axpy_norm(B, w, v, j ? vprev : nullptr, replay ? alpha_rec[j] : 0.0, bprev, L.dtype, part2, nblk,
+                                  L.st, L.ylo, replay ? nullptr : B->d_partial, n_dot, L.d_scalar))) return rc;
+    const double *corr_d[2] = {nullptr, nullptr};
+    const double *b2_part = part2;
+    int n_b2 = nblk;
     if (L.reorth != ED_REORTH_NONE) {
-      if ((rc = reorth_step(L, j, w, v, j ? vprev : nullptr, !replay, &corr, &b2))) return rc;
-    } else if (!replay) {
-      if ((rc = reduce_partials(B, B->d_partial, nblk, false, L.st, &b2, nullptr))) return rc;
+      if (!replay) ED_CK(cudaEventRecord(L.r0, L.st));
+      if ((rc = reorth_step(L, j, w, v, j ? vprev : nullptr, corr_d))) return rc;
+      if (!replay) ED_CK(cudaEventRecord(L.r1, L.st));
+      b2_part = L.d_ro;
+      n_b2 = ed_reorth_grid(B);
+    }
+    double a = 0, b2 = 0, corr = 0;
+    if (!replay) {   // the step's only wait
+      if ((rc = ed_launch_step_scalars(L.d_scalar, corr_d[0], corr_d[1], b2_part, n_b2, L.d_scalar + 1, L.st))) return rc;
+      ED_CK(cudaMemcpyAsync(B->h_partial, L.d_scalar + 1, 32, cudaMemcpyDeviceToHost, L.st));
+      ED_CK(cudaStreamSynchronize(L.st));
+      a = B->h_partial[0];
+      corr = B->h_partial[1] + B->h_partial[2];
+      b2 = B->h_partial[3];
+      float ms = 0;
+      ED_CK(cudaEventElapsedTime(&ms, L.e0, L.e1));
+      L.ms_apply += ms;
+      if (L.reorth != ED_REORTH_NONE) {
+        ED_CK(cudaEventElapsedTime(&ms, L.r0, L.r1));
+        L.ms_reorth += ms;
+      }
     }
     double b = replay ? beta[j] : std::sqrt(std::max(b2, 0.0));
     if (!replay) {
@@ -919,6 +917,14 @@ int lanczos_pass(LanczosRun &L, const ed_lanczos_opts *o, int max_steps, bool fi
     }
     if ((rc = ed_launch_scale(B, w, 1.0 / b, L.dtype, L.st, L.ylo))) return rc;
     if (!full) { void *t = vprev; vprev = v; v = w; w = t; }
+  }
+  if (!L.replay_ev.empty()) {
+    ED_CK(cudaStreamSynchronize(L.st));
+    for (size_t k = 0; k + 1 < L.replay_ev.size(); k += 2) {
+      float ms = 0;
+      ED_CK(cudaEventElapsedTime(&ms, L.replay_ev[k], L.replay_ev[k + 1]));
+      L.ms_apply += ms;
+    }
   }
   return ED_OK;
 }
@@ -985,13 +991,16 @@ extern "C" int ed_lanczos(ed_basis *B, const double *J, const double *Jz,
   const int m_cap = full ? max_steps + 1 : 2;
   const int P = L.cplx ? 2 : 1;
   L.ro_coef_off = (size_t)m_cap * P * ed_reorth_grid(B);
-  if (o.reorth != ED_REORTH_NONE &&
-      cudaMalloc(&L.d_ro, sizeof(double) * (L.ro_coef_off + (size_t)m_cap * P)) != cudaSuccess) {
+  L.coef_len = (size_t)m_cap * P;
+  // 4 rows per thread at least, as in the sweeps
+  L.nblk = (int)std::max<int64_t>(1, std::min<int64_t>(B->n_partial / 4, (B->D + 1023) / 1024));
+  if (cudaMalloc(&L.d_ro, sizeof(double) * (L.ro_coef_off + 2 * L.coef_len + 8)) != cudaSuccess) {
     cudaGetLastError();
     if (own) for (int k = 0; k < 3; k++) cudaFree(L.v[k]);
     if (L.own_ylo) cudaFree(L.ylo);
     return ed_fail(ED_ERR_OOM, "cannot allocate the reorthogonalisation scratch");
   }
+  L.d_scalar = L.d_ro + L.ro_coef_off + 2 * L.coef_len;
   if (cudaEventCreate(&L.e0) != cudaSuccess || cudaEventCreate(&L.e1) != cudaSuccess ||
       cudaEventCreate(&L.r0) != cudaSuccess || cudaEventCreate(&L.r1) != cudaSuccess) {
     cudaGetLastError();
@@ -1023,7 +1032,7 @@ extern "C" int ed_lanczos(ed_basis *B, const double *J, const double *Jz,
     if (!rc) {
       // normalise psi and take its Rayleigh quotient
       double nn, im;
-      const int nblk = B->n_partial / 2;
+      const int nblk = L.nblk;
       void *scratch = full ? L.slot(std::min(m, L.store_slots - 1)) : L.v[0];
       rc = ed_launch_dot(B, o.psi, o.psi, o.dtype, B->d_partial, nblk, L.st);
       if (!rc) rc = reduce_partials(B, B->d_partial, nblk, L.cplx, L.st, &nn, &im);
@@ -1049,6 +1058,7 @@ extern "C" int ed_lanczos(ed_basis *B, const double *J, const double *Jz,
   if (L.d_ro) cudaFree(L.d_ro);
   for (cudaEvent_t e : {L.e0, L.e1, L.r0, L.r1})
     if (e) cudaEventDestroy(e);
+  for (cudaEvent_t e : L.replay_ev) cudaEventDestroy(e);
   res->ms_total = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
   return rc;
 }

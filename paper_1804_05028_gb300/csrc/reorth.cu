@@ -21,6 +21,7 @@
 //   combine_kernel    psi = sum_k s_k u_k (the Ritz vector from a stored Krylov basis)
 #include "sced_internal.cuh"
 #include "dfloat.cuh"
+#include <algorithm>
 #include <type_traits>
 
 namespace {
@@ -88,6 +89,26 @@ __device__ __forceinline__ void md_acc(double &re, double &im, float &rh, float 
   }
 }
 
+// v[0 .. 8) summed over the warp; lane l returns the sum of v[q], q = bits 4, 3, 2 of l (most
+// significant first).  Every exchange step halves the values a lane carries: 9 fp64 additions
+// instead of 40 (the fp64 pipe takes 16 cycles for each, and small vectors spent half of
+// the multi-dot in them).
+__device__ __forceinline__ double warp_sum8(double (&v)[8], int lane) {
+#pragma unroll
+  for (int h = 4, o = 16; h >= 1; h >>= 1, o >>= 1) {
+#pragma unroll
+    for (int i = 0; i < h; i++) {
+      const bool up = lane & o;
+      const double keep = up ? v[i + h] : v[i], give = up ? v[i] : v[i + h];
+      v[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, give, o);
+    }
+  }
+  double r = v[0];
+  r += __shfl_xor_sync(0xFFFFFFFFu, r, 2);
+  r += __shfl_xor_sync(0xFFFFFFFFu, r, 1);
+  return r;
+}
+
 template <typename V>
 __device__ __forceinline__ V zero_v() {
   if constexpr (Rv<V>::cplx) { V z; z.x = 0; z.y = 0; return z; } else { return V(0); }
@@ -143,17 +164,19 @@ __global__ void __launch_bounds__(kThreads, 4) multidot_kernel(VecSet S, const V
       if (q < kn) md_acc<V>(re[q], im[q], rh[q], rl[q], ih[q], il[q], vec<V>(S, k0 + q)[i], wv, wl);
   }
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  if constexpr (kF) {
 #pragma unroll
-  for (int q = 0; q < kGroup; q++) {
-    double a0 = re[q], b0 = im[q];
-    if constexpr (kF) { a0 = df_value(rh[q], rl[q]); b0 = df_value(ih[q], il[q]); }
-    const double a = warp_sum(a0);
-    double b = 0.0;
-    if constexpr (kC) b = warp_sum(b0);
-    if (lane == 0) {
-      red[q * P][wid] = a;
-      if constexpr (kC) red[q * P + 1][wid] = b;
+    for (int q = 0; q < kGroup; q++) {
+      re[q] = df_value(rh[q], rl[q]);
+      im[q] = df_value(ih[q], il[q]);
     }
+  }
+  static_assert(kGroup == 8, "warp_sum8");
+  const double a = warp_sum8(re, lane);
+  if ((lane & 3) == 0) red[(lane >> 2) * P][wid] = a;
+  if constexpr (kC) {
+    const double c = warp_sum8(im, lane);
+    if ((lane & 3) == 0) red[(lane >> 2) * P + 1][wid] = c;
   }
   __syncthreads();
   if (threadIdx.x < kn * P) {
@@ -399,7 +422,11 @@ VecSet make_set(const void *base, int64_t stride, const void *p0, const void *p1
 
 }  // namespace
 
-int ed_reorth_grid(const ed_basis *B) { return 4 * B->sm_count; }
+// 4 blocks per SM, fewer for short vectors: a thread then still has four rows, and the block
+// sums do not outweigh them (multi-dot of 8 vectors of 1.1e5 fp64 entries: 21 us with the full grid)
+int ed_reorth_grid(const ed_basis *B) {
+  return (int)std::max<int64_t>(1, std::min<int64_t>(4 * B->sm_count, (B->D + 4 * kThreads - 1) / (4 * kThreads)));
+}
 
 // One Gram-Schmidt sweep of w against m vectors (base + k * D, or p0 and p1 when base is
 // null): coefficients c (device, m * P doubles, P = 2 for complex) and ||w||^2 block

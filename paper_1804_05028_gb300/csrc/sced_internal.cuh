@@ -366,10 +366,14 @@ int ed_launch_dot(const ed_basis *B, const void *x, const void *y, int dtype, do
                   int nblk, cudaStream_t st);
 // (w, wlo) <- (w + wlo) - a v - b vprev, ||w + wlo||^2 partials; wlo (fp32 vectors, may
 // be null) holds the low words of w: on entry those of the product (ed_launch_apply's
-// ylo), on exit those of the update
+// ylo), on exit those of the update; with part, a is the sum of its n_part partials (device),
+// also stored to a_out
 int ed_launch_axpy_norm(const ed_basis *B, void *w, const void *v, const void *vprev, double a,
                         double b, int dtype, double *partial, int nblk, cudaStream_t st,
-                        void *wlo = nullptr);
+                        void *wlo = nullptr, const double *part = nullptr, int n_part = 0,
+                        double *a_out = nullptr);
+int ed_launch_step_scalars(const double *alpha, const double *corr0, const double *corr1, const double *part,
+                           int n_part, double *out, cudaStream_t st);
 // v <- s (v + vlo), rounded once (vlo: fp32 vectors, may be null)
 int ed_launch_scale(const ed_basis *B, void *v, double s, int dtype, cudaStream_t st,
                     const void *vlo = nullptr);
