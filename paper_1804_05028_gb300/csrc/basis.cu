@@ -14,7 +14,7 @@
 //   and every lane writes its hits in order -- the output is sorted with no sort.
 // Index.  top_rank compresses the occupied values of the top r bits to a dense rank;
 // key = rank << q | next q bits; limits[key] = first position whose key is >= key
-// (lower bound in the sorted basis); the remaining low bits go to a narrow postfix
+// (marked where keys begin, then filled from the end); the remaining low bits go to a narrow postfix
 // array searched inside the bucket.  Where they fit (4x the basis's bytes, or 64 MB),
 // ranked records replace the search: one record per prefix rank and value of every bit
 // but the low 6, holding the first basis position and a 64-bit bitmap of the low-6-bit
@@ -24,6 +24,7 @@
 #include <algorithm>
 #include <chrono>
 #include <cmath>
+#include <cstring>
 #include <vector>
 
 namespace {
@@ -76,10 +77,12 @@ __device__ __forceinline__ int find_top(const EnumParams &E, uint64_t item) {
   return lo;
 }
 
+// hit_s (may be null): the count pass leaves every lane's 32-bit hit mask there, so that the
+// fill pass only has to look at the states it writes.
 template <bool kFill>
 __global__ void __launch_bounds__(256) enum_kernel(const EnumParams E, uint32_t *counts,
                                                    const uint64_t *offsets, uint64_t *basis,
-                                                   uint16_t *stab) {
+                                                   uint16_t *stab, uint32_t *hit_s) {
   const DevTables &T = E.T;
   const int lane = threadIdx.x & 31;
   const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
@@ -94,14 +97,17 @@ __global__ void __launch_bounds__(256) enum_kernel(const EnumParams E, uint32_t 
     int len = 0;
     if (r0 < total) len = (total - r0 < (uint64_t)kRun) ? (int)(total - r0) : kRun;
     uint32_t hits = 0;
-    uint64_t x = len ? unrank(E.binom, E.S, k, r0) : 0;
+    const bool known = kFill && hit_s;
+    if (known) hits = hit_s[item * 32 + lane];
+    uint64_t x = (known ? hits != 0 : len != 0) ? unrank(E.binom, E.S, k, r0) : 0;
     const uint64_t x0 = x;
-    for (int u = 0; u < len; u++) {
+    for (int u = 0; u < len && !known; u++) {
       int tt;
       if (is_kept_rep(T, T.rep, T.sym_off, T.sym_list, T.dest, T.phase, pre | x, &tt))
         hits |= 1u << u;
       x = next_comb(x);
     }
+    if (!kFill && hit_s) hit_s[item * 32 + lane] = hits;
     const int c = __popc(hits);
     if (!kFill) {
       int tot = c;
@@ -115,7 +121,7 @@ __global__ void __launch_bounds__(256) enum_kernel(const EnumParams E, uint32_t 
       }
       uint64_t w = offsets[item] + (uint64_t)(incl - c);
       x = x0;
-      for (int u = 0; u < len; u++) {
+      for (int u = 0; u < len && (hits >> u); u++) {
         if (hits & (1u << u)) {
           int tt = 0;
           is_kept_rep(T, T.rep, T.sym_off, T.sym_list, T.dest, T.phase, pre | x, &tt);
@@ -232,23 +238,73 @@ __global__ void make_rank(const uint32_t *flags, const uint64_t *scan, uint64_t 
   }
 }
 
-// limits[k] = first position whose key is >= k, by binary search for the smallest state
-// carrying key k
-__global__ void make_limits(const uint64_t *basis, int64_t D, const uint32_t *rank_top,
-                            int r_shift, int q_bits, int post_bits, uint64_t n_keys,
-                            uint32_t *limits) {
-  for (uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k <= n_keys;
-       k += (uint64_t)gridDim.x * blockDim.x) {
-    if (k == n_keys) { limits[k] = (uint32_t)D; continue; }
-    const uint64_t rk = k >> q_bits;
-    const uint64_t mid = k & ((1ULL << q_bits) - 1ULL);
-    const uint64_t thr = ((uint64_t)rank_top[rk] << r_shift) | (mid << post_bits);
-    int64_t lo = 0, hi = D;
-    while (lo < hi) {
-      const int64_t m = (lo + hi) >> 1;
-      if (basis[m] < thr) lo = m + 1; else hi = m;
+// limits[k] = first position whose key is >= k.  mark_limits notes the first position of every
+// key that occurs; fill_limits gives the others that of the next key that does: a block owns
+// 4096 keys, finds the first position beyond them by one search, and takes minima from the
+// end.  (A search per key took 43 ms on the 8.6e8-state sector.)
+__global__ void mark_limits(const uint64_t *basis, int64_t D, const uint32_t *top_rank, int r_shift,
+                            int q_bits, int post_bits, uint32_t *limits) {
+  const uint64_t qm = (1ULL << q_bits) - 1ULL;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < D;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const uint64_t s = basis[i];
+    const uint64_t k = ((uint64_t)top_rank[s >> r_shift] << q_bits) | ((s >> post_bits) & qm);
+    if (i) {
+      const uint64_t p = basis[i - 1];
+      if ((((uint64_t)top_rank[p >> r_shift] << q_bits) | ((p >> post_bits) & qm)) == k) continue;
     }
-    limits[k] = (uint32_t)lo;
+    limits[k] = (uint32_t)i;
+  }
+}
+
+constexpr int kLimitsTile = 4096;
+
+__global__ void __launch_bounds__(256) fill_limits(const uint64_t *basis, int64_t D, const uint32_t *rank_top,
+                                                   int r_shift, int q_bits, int post_bits, uint64_t n_keys,
+                                                   uint32_t *limits) {
+  constexpr int kPer = kLimitsTile / 256;
+  __shared__ uint32_t next_s[256];
+  __shared__ uint32_t beyond;
+  const uint64_t n_tiles = (n_keys + kLimitsTile) / kLimitsTile;   // keys 0 .. n_keys
+  for (uint64_t t = blockIdx.x; t < n_tiles; t += gridDim.x) {
+    const uint64_t k0 = t * kLimitsTile, end = k0 + kLimitsTile;
+    if (threadIdx.x == 0) {
+      int64_t lo = D;
+      if (end < n_keys) {   // first state whose key is >= end
+        const uint64_t thr = ((uint64_t)rank_top[end >> q_bits] << r_shift) |
+                             ((end & ((1ULL << q_bits) - 1ULL)) << post_bits);
+        int64_t hi = D;
+        lo = 0;
+        while (lo < hi) {
+          const int64_t m = (lo + hi) >> 1;
+          if (basis[m] < thr) lo = m + 1; else hi = m;
+        }
+      }
+      beyond = (uint32_t)lo;
+    }
+    // a thread owns kPer consecutive keys
+    const uint64_t mine = k0 + (uint64_t)threadIdx.x * kPer;
+    uint32_t v[kPer], first = 0xFFFFFFFFu;
+#pragma unroll
+    for (int q = kPer - 1; q >= 0; q--) {
+      v[q] = mine + q < n_keys ? limits[mine + q] : 0xFFFFFFFFu;
+      first = min(first, v[q]);
+    }
+    next_s[threadIdx.x] = first;
+    __syncthreads();
+    for (int o = 1; o < 256; o <<= 1) {   // suffix minima over the threads
+      const uint32_t u = threadIdx.x + o < 256 ? next_s[threadIdx.x + o] : 0xFFFFFFFFu;
+      __syncthreads();
+      next_s[threadIdx.x] = min(next_s[threadIdx.x], u);
+      __syncthreads();
+    }
+    uint32_t run = min(threadIdx.x < 255 ? next_s[threadIdx.x + 1] : 0xFFFFFFFFu, beyond);
+#pragma unroll
+    for (int q = kPer - 1; q >= 0; q--) {
+      run = min(run, v[q]);
+      if (mine + q <= n_keys) limits[mine + q] = run;
+    }
+    __syncthreads();
   }
 }
 
@@ -256,34 +312,24 @@ __global__ void make_limits(const uint64_t *basis, int64_t D, const uint32_t *ra
 // most 6 postfix bits a bucket is a subset of 64 values, kept as a 64-bit occupancy
 // bitmap next to the bucket's first index; the index of a state is then
 // start + popcount(bitmap below its postfix).  One 16-byte record per key:
-// {start, 0, bitmap low word, bitmap high word}.
-__global__ void ranked_starts(const uint64_t *basis, int64_t D, const uint32_t *rank_top,
-                              int r_shift, int q_bits, int post_bits, uint64_t n_keys,
-                              uint4 *rec) {
-  for (uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n_keys;
-       k += (uint64_t)gridDim.x * blockDim.x) {
-    const uint64_t rk = k >> q_bits;
-    const uint64_t mid = k & ((1ULL << q_bits) - 1ULL);
-    const uint64_t thr = ((uint64_t)rank_top[rk] << r_shift) | (mid << post_bits);
-    int64_t lo = 0, hi = D;
-    while (lo < hi) {
-      const int64_t m = (lo + hi) >> 1;
-      if (basis[m] < thr) lo = m + 1; else hi = m;
-    }
-    rec[k] = make_uint4((uint32_t)lo, 0u, 0u, 0u);
-  }
-}
-
-__global__ void ranked_bits(const uint64_t *basis, int64_t D, const uint32_t *top_rank,
-                            int r_shift, int q_bits, int post_bits, uint4 *rec) {
+// {start, 0, bitmap low word, bitmap high word}; a key that does not occur has an empty
+// bitmap, which no lookup passes, and needs no start (the records are zeroed before).  The
+// first state of a bucket writes its record.
+__global__ void ranked_records(const uint64_t *basis, int64_t D, const uint32_t *top_rank,
+                               int r_shift, int q_bits, int post_bits, uint4 *rec) {
+  const uint64_t pm = (1ULL << post_bits) - 1ULL;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < D;
        i += (int64_t)gridDim.x * blockDim.x) {
     const uint64_t s = basis[i];
-    const uint64_t rk = top_rank[s >> r_shift];
-    const uint64_t k = (rk << q_bits) | ((s >> post_bits) & ((1ULL << q_bits) - 1ULL));
-    const uint32_t pf = (uint32_t)(s & ((1ULL << post_bits) - 1ULL));
-    unsigned int *w = reinterpret_cast<unsigned int *>(rec + k) + (pf < 32 ? 2 : 3);
-    atomicOr(w, 1u << (pf & 31));
+    if (i && (basis[i - 1] >> post_bits) == (s >> post_bits)) continue;
+    uint64_t bits = 0;
+    for (int64_t j = i; j < D; j++) {
+      const uint64_t u = basis[j];
+      if ((u >> post_bits) != (s >> post_bits)) break;
+      bits |= 1ULL << (u & pm);
+    }
+    const uint64_t k = ((uint64_t)top_rank[s >> r_shift] << q_bits) | ((s >> post_bits) & ((1ULL << q_bits) - 1ULL));
+    rec[k] = make_uint4((uint32_t)i, 0u, (uint32_t)bits, (uint32_t)(bits >> 32));
   }
 }
 
@@ -306,33 +352,57 @@ __global__ void make_postfix(const uint64_t *basis, int64_t D, uint64_t mask, PT
 
 // The whole lookup table of a one-sublattice split: every configuration s < 2^N gets its
 // representative (Eq. 4, every group element applied), the first minimising element and
-// the number of minimisers.  pbit[g*N + b] is the bit that g carries bit b to.
-__global__ void full_table_kernel(const uint8_t *pbit, const uint8_t *flip, int N, int nsym,
-                                  uint64_t *out) {
-  extern __shared__ uint8_t sp[];
-  uint8_t *sf = sp + nsym * N;
-  for (int k = threadIdx.x; k < nsym * N; k += blockDim.x) sp[k] = pbit[k];
-  for (int k = threadIdx.x; k < nsym; k += blockDim.x) sf[k] = flip ? flip[k] : 0;
-  __syncthreads();
-  const uint64_t total = 1ULL << N;
-  const uint64_t all = total - 1ULL;
-  for (uint64_t s = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; s < total;
-       s += (uint64_t)gridDim.x * blockDim.x) {
-    uint64_t best = ~0ULL;
-    uint32_t gb = 0, cnt = 0;
-    for (int g = 0; g < nsym; g++) {
-      const uint8_t *pg = sp + g * N;
-      uint64_t v = 0, m = s;
-      while (m) {
-        const int b = __ffsll((long long)m) - 1;
-        m &= m - 1;
-        v |= 1ULL << pg[b];
+// the number of minimisers.  pbit[g*N + b] is the bit that g carries bit b to.  A block takes
+// kHigh x 256 configurations, a thread those with its low 8 bits: an image is the OR of the
+// image of the high bits (one per element and high part, shared memory) and that of the low
+// bits (a 256-entry table per element, read by neighbouring threads in one line), where
+// moving the spins bit by bit took 26 ms for 50 elements on 25 sites.
+__global__ void low_images(const uint8_t *pbit, int N, int nsym, uint32_t *low) {
+  const int nl = min(N, 8);
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nsym * 256; t += gridDim.x * blockDim.x) {
+    const int g = t >> 8, v = t & 255;
+    uint32_t m = 0;
+    for (int b = 0; b < nl; b++)
+      if ((v >> b) & 1) m |= 1u << pbit[g * N + b];
+    low[t] = m;
+  }
+}
+
+template <int kHigh>
+__global__ void __launch_bounds__(256) full_table_kernel(const uint8_t *pbit, const uint8_t *flip, int N, int nsym,
+                                                         const uint32_t *low, uint64_t *out) {
+  extern __shared__ uint32_t hi_s[];   // [nsym][kHigh]
+  const uint32_t total = 1u << N, all = total - 1u;   // N <= 26
+  const uint32_t n_high = N > 8 ? 1u << (N - 8) : 1u;
+  for (uint32_t h0 = blockIdx.x * kHigh; h0 < n_high; h0 += gridDim.x * kHigh) {
+    for (int t = threadIdx.x; t < nsym * kHigh; t += 256) {
+      const int g = t / kHigh;
+      uint32_t v = flip && flip[g] ? all : 0u;   // the element also reverses every spin
+      for (uint32_t m = h0 + t % kHigh; m; m &= m - 1) {
+        const int b = 8 + __ffs(m) - 1;
+        if (b < N) v ^= 1u << pbit[g * N + b];
       }
-      if (sf[g]) v ^= all;   // the element also reverses every spin
-      if (v < best) { best = v; gb = g; cnt = 1; }
-      else if (v == best) cnt++;
+      hi_s[t] = v;
     }
-    out[s] = best | ((uint64_t)gb << 32) | ((uint64_t)cnt << 48);
+    __syncthreads();
+    uint32_t best[kHigh], gb[kHigh], cnt[kHigh];
+#pragma unroll
+    for (int q = 0; q < kHigh; q++) { best[q] = 0xFFFFFFFFu; gb[q] = cnt[q] = 0; }
+    for (int g = 0; g < nsym; g++) {
+      const uint32_t lo = __ldg(low + g * 256 + threadIdx.x);
+#pragma unroll
+      for (int q = 0; q < kHigh; q++) {
+        const uint32_t v = hi_s[g * kHigh + q] ^ lo;
+        if (v < best[q]) { best[q] = v; gb[q] = g; cnt[q] = 1; }
+        else if (v == best[q]) cnt[q]++;
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < kHigh; q++) {
+      const uint64_t s = (uint64_t)(h0 + q) * 256 + threadIdx.x;
+      if (h0 + q < n_high && s < total) out[s] = best[q] | ((uint64_t)gb[q] << 32) | ((uint64_t)cnt[q] << 48);
+    }
+    __syncthreads();
   }
 }
 
@@ -351,15 +421,23 @@ int ed_exclusive_scan(const uint32_t *in, uint64_t n, uint64_t *out, uint64_t *t
 
 int ed_build_full_table(const uint8_t *d_pbit, const uint8_t *d_flip, int N, int nsym,
                         uint64_t *out, cudaStream_t st) {
-  const size_t sm = (size_t)nsym * N + nsym;
-  if (sm > 200 * 1024) return ed_fail(ED_ERR_UNSUPPORTED, "group too large for the one-block table");
+  if ((size_t)nsym * N + nsym > 200 * 1024) return ed_fail(ED_ERR_UNSUPPORTED, "group too large for the one-block table");
+  // four high parts per block, one where the group's images would not fit in shared memory
+  const bool four = sizeof(uint32_t) * 4 * (size_t)nsym <= 64 * 1024;
+  const size_t sm = sizeof(uint32_t) * (size_t)nsym * (four ? 4 : 1);
+  auto k = four ? full_table_kernel<4> : full_table_kernel<1>;
   if (sm > 48 * 1024)
-    ED_CK(cudaFuncSetAttribute(full_table_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    ED_CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   int dev = 0, nsm = 0;
   ED_CK(cudaGetDevice(&dev));
   ED_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  full_table_kernel<<<nsm * 8, 256, sm, st>>>(d_pbit, d_flip, N, nsym, out);
-  ED_CK(cudaGetLastError());
+  uint32_t *low = nullptr;
+  ED_CK(cudaMallocAsync(&low, 1024 * (size_t)nsym, st));
+  low_images<<<(nsym + 3) / 4, 256, 0, st>>>(d_pbit, N, nsym, low);
+  k<<<nsm * 8, 256, sm, st>>>(d_pbit, d_flip, N, nsym, low, out);
+  const cudaError_t e = cudaGetLastError();
+  ED_CK(cudaFreeAsync(low, st));
+  if (e != cudaSuccess) return ed_cuda_fail(e, "full_table_kernel");
   return ED_OK;
 }
 
@@ -396,39 +474,43 @@ int ed_build_device(ed_basis *B, cudaStream_t st, int bucket_target) {
   for (int a = 0; a <= 64; a++)
     for (int b = 0; b <= 64; b++) binom[a * 65 + b] = binom_host(a, b);
 
-  uint32_t *d_tv = nullptr, *d_counts = nullptr;
-  uint8_t *d_tk = nullptr;
-  uint64_t *d_ttot = nullptr, *d_titem = nullptr, *d_binom = nullptr, *d_off = nullptr;
+  // the small inputs in one upload, then the items' counts and offsets
   const size_t nt = tv.size();
-  ED_CK(cudaMallocAsync(&d_tv, nt * 4, st));
-  ED_CK(cudaMallocAsync(&d_tk, nt, st));
-  ED_CK(cudaMallocAsync(&d_ttot, nt * 8, st));
-  ED_CK(cudaMallocAsync(&d_titem, nt * 8, st));
-  ED_CK(cudaMallocAsync(&d_binom, binom.size() * 8, st));
-  ED_CK(cudaMallocAsync(&d_counts, n_items * 4, st));
-  ED_CK(cudaMallocAsync(&d_off, n_items * 8, st));
-  ED_CK(cudaMemcpyAsync(d_tv, tv.data(), nt * 4, cudaMemcpyHostToDevice, st));
-  ED_CK(cudaMemcpyAsync(d_tk, tk.data(), nt, cudaMemcpyHostToDevice, st));
-  ED_CK(cudaMemcpyAsync(d_ttot, ttot.data(), nt * 8, cudaMemcpyHostToDevice, st));
-  ED_CK(cudaMemcpyAsync(d_titem, titem.data(), nt * 8, cudaMemcpyHostToDevice, st));
-  ED_CK(cudaMemcpyAsync(d_binom, binom.data(), binom.size() * 8, cudaMemcpyHostToDevice, st));
+  std::vector<unsigned char> blob;
+  auto add = [&](const void *v, size_t bytes) {
+    const size_t o = (blob.size() + 15) / 16 * 16;
+    blob.resize(o + bytes);
+    memcpy(blob.data() + o, v, bytes);
+    return o;
+  };
+  const size_t o_tv = add(tv.data(), nt * 4), o_tk = add(tk.data(), nt), o_tt = add(ttot.data(), nt * 8),
+               o_ti = add(titem.data(), nt * 8), o_bi = add(binom.data(), binom.size() * 8);
+  const size_t o_off = (blob.size() + 15) / 16 * 16, o_cnt = o_off + n_items * 8;
+  unsigned char *d_in = nullptr;
+  ED_CK(cudaMallocAsync(&d_in, o_cnt + n_items * 4, st));
+  ED_CK(cudaMemcpyAsync(d_in, blob.data(), blob.size(), cudaMemcpyHostToDevice, st));
+  uint64_t *d_off = reinterpret_cast<uint64_t *>(d_in + o_off);
+  uint32_t *d_counts = reinterpret_cast<uint32_t *>(d_in + o_cnt);
 
   EnumParams E{};
   E.T = B->T;
   E.S = S;
   E.n_tops = (int)nt;
-  E.top_v = d_tv;
-  E.top_k = d_tk;
-  E.top_total = d_ttot;
-  E.top_item0 = d_titem;
+  E.top_v = reinterpret_cast<const uint32_t *>(d_in + o_tv);
+  E.top_k = d_in + o_tk;
+  E.top_total = reinterpret_cast<const uint64_t *>(d_in + o_tt);
+  E.top_item0 = reinterpret_cast<const uint64_t *>(d_in + o_ti);
   E.n_items = n_items;
-  E.binom = d_binom;
+  E.binom = reinterpret_cast<const uint64_t *>(d_in + o_bi);
   const uint64_t warps_needed = n_items;
   uint64_t grid64 = (warps_needed + 7) / 8;
   const uint64_t cap = (uint64_t)B->sm_count * 16;
   if (grid64 > cap) grid64 = cap;
   const unsigned grid = (unsigned)std::max<uint64_t>(grid64, 1);
-  enum_kernel<false><<<grid, 256, 0, st>>>(E, d_counts, nullptr, nullptr, nullptr);
+  // 4 bytes per 32 candidates; without memory for them the fill pass searches again
+  uint32_t *d_hits = nullptr;
+  if (cudaMallocAsync(&d_hits, n_items * 128, st) != cudaSuccess) { cudaGetLastError(); d_hits = nullptr; }
+  enum_kernel<false><<<grid, 256, 0, st>>>(E, d_counts, nullptr, nullptr, nullptr, d_hits);
   ED_CK(cudaGetLastError());
   uint64_t D = 0;
   int rc = exclusive_scan<uint32_t>(d_counts, n_items, d_off, &D, st);
@@ -441,16 +523,11 @@ int ed_build_device(ed_basis *B, cudaStream_t st, int bucket_target) {
       cudaGetLastError();
       return ed_fail(ED_ERR_OOM, "cannot allocate the basis on the device");
     }
-    enum_kernel<true><<<grid, 256, 0, st>>>(E, nullptr, d_off, B->d_basis, B->d_stab);
+    enum_kernel<true><<<grid, 256, 0, st>>>(E, nullptr, d_off, B->d_basis, B->d_stab, d_hits);
     ED_CK(cudaGetLastError());
   }
-  ED_CK(cudaFreeAsync(d_tv, st));
-  ED_CK(cudaFreeAsync(d_tk, st));
-  ED_CK(cudaFreeAsync(d_ttot, st));
-  ED_CK(cudaFreeAsync(d_titem, st));
-  ED_CK(cudaFreeAsync(d_binom, st));
-  ED_CK(cudaFreeAsync(d_counts, st));
-  ED_CK(cudaFreeAsync(d_off, st));
+  if (d_hits) ED_CK(cudaFreeAsync(d_hits, st));
+  ED_CK(cudaFreeAsync(d_in, st));
   if (D == 0) return ED_OK;
 
   // ---- prefix index ----
@@ -486,8 +563,10 @@ int ed_build_device(ed_basis *B, cudaStream_t st, int bucket_target) {
     cudaGetLastError();
     return ed_fail(ED_ERR_OOM, "cannot allocate Limits");
   }
-  make_limits<<<g1, 256, 0, st>>>(B->d_basis, B->D, d_rank_top, N - r_bits, q, post_bits,
-                                    n_keys, B->d_limits);
+  ED_CK(cudaMemsetAsync(B->d_limits, 0xFF, (n_keys + 1) * 4, st));
+  mark_limits<<<g1, 256, 0, st>>>(B->d_basis, B->D, B->d_top_rank, N - r_bits, q, post_bits, B->d_limits);
+  ED_CK(cudaGetLastError());
+  fill_limits<<<g1, 256, 0, st>>>(B->d_basis, B->D, d_rank_top, N - r_bits, q, post_bits, n_keys, B->d_limits);
   ED_CK(cudaGetLastError());
   unsigned long long *d_max = nullptr;
   ED_CK(cudaMallocAsync(&d_max, 8, st));
@@ -523,11 +602,9 @@ int ed_build_device(ed_basis *B, cudaStream_t st, int bucket_target) {
     const uint64_t rkeys = R << rq;
     if (rkeys < (1ULL << 32) && rkeys * 16 <= std::max<uint64_t>(4 * (uint64_t)D * 8, 1ULL << 26)) {
       if (cudaMalloc(&B->d_rlim, rkeys * 16) == cudaSuccess) {
-        ranked_starts<<<g1, 256, 0, st>>>(B->d_basis, B->D, d_rank_top, N - r_bits, rq, rpost, rkeys,
-                                          reinterpret_cast<uint4 *>(B->d_rlim));
-        ED_CK(cudaGetLastError());
-        ranked_bits<<<g1, 256, 0, st>>>(B->d_basis, B->D, B->d_top_rank, N - r_bits, rq, rpost,
-                                        reinterpret_cast<uint4 *>(B->d_rlim));
+        ED_CK(cudaMemsetAsync(B->d_rlim, 0, rkeys * 16, st));
+        ranked_records<<<g1, 256, 0, st>>>(B->d_basis, B->D, B->d_top_rank, N - r_bits, rq, rpost,
+                                           reinterpret_cast<uint4 *>(B->d_rlim));
         ED_CK(cudaGetLastError());
         B->rq_bits = rq;
         B->rpost_bits = rpost;

@@ -217,17 +217,38 @@ int validate(ed_basis *B, const ed_lattice *L, const ed_group *G, const ed_irrep
   return ED_OK;
 }
 
-// norm and character tables, bond positions (every split)
-int build_norm_tables(ed_basis *B, cudaStream_t st) {
-  const int ns = B->nsym;
-  auto up = [&](void **dst, const void *src, size_t bytes) -> int {
-    if (bytes == 0) { *dst = nullptr; return ED_OK; }
-    if (cudaMalloc(dst, bytes) != cudaSuccess) { cudaGetLastError(); return ed_fail(ED_ERR_OOM, "cannot allocate lookup tables"); }
-    ED_CK(cudaMemcpyAsync(*dst, src, bytes, cudaMemcpyHostToDevice, st));
-    B->table_bytes += bytes;
+// Lookup tables gathered on the host, then uploaded in one allocation and one copy (some
+// twenty of each took a good part of a small sector's build).
+struct TableSet {
+  std::vector<unsigned char> bytes;
+  std::vector<std::pair<void **, size_t>> at;
+  void add(void **dst, const void *src, size_t n) {
+    *dst = nullptr;
+    if (n == 0) return;
+    const size_t o = (bytes.size() + 255) / 256 * 256;
+    bytes.resize(o + n);
+    memcpy(bytes.data() + o, src, n);
+    at.emplace_back(dst, o);
+  }
+  int upload(ed_basis *B, cudaStream_t st) {
+    void *d = nullptr;
+    if (cudaMalloc(&d, std::max<size_t>(bytes.size(), 1)) != cudaSuccess) {
+      cudaGetLastError();
+      return ed_fail(ED_ERR_OOM, "cannot allocate lookup tables");
+    }
+    B->d_tables = d;
+    B->table_bytes += bytes.size();
+    for (auto &p : at) *p.first = (unsigned char *)d + p.second;
+    ED_CK(cudaMemcpyAsync(d, bytes.data(), bytes.size(), cudaMemcpyHostToDevice, st));
+    ED_CK(cudaStreamSynchronize(st));
     return ED_OK;
-  };
-  int rc;
+  }
+};
+
+// norm and character tables, bond positions (every split)
+void add_norm_tables(ed_basis *B, TableSet &tabs) {
+  const int ns = B->nsym;
+  auto up = [&](void **dst, const void *src, size_t n) { tabs.add(dst, src, n); };
   std::vector<double> sq(ns + 1), rs(ns + 1), cs(2 * (size_t)B->denom);
   for (int t = 0; t <= ns; t++) { sq[t] = std::sqrt((double)t); rs[t] = t ? 1.0 / std::sqrt((double)t) : 0.0; }
   for (int k = 0; k < B->denom; k++) {
@@ -235,35 +256,30 @@ int build_norm_tables(ed_basis *B, cudaStream_t st) {
     cs[2 * k] = std::cos(a);
     cs[2 * k + 1] = std::sin(a);
   }
-  if ((rc = up((void **)&B->d_sqrt, sq.data(), sq.size() * 8))) return rc;
-  if ((rc = up((void **)&B->d_rsqrt, rs.data(), rs.size() * 8))) return rc;
-  if ((rc = up((void **)&B->d_cs, cs.data(), cs.size() * 8))) return rc;
-  if ((rc = up((void **)&B->d_bond_pos, B->bond_pos.data(), B->bond_pos.size()))) return rc;
-  if ((rc = up((void **)&B->d_bond_pad, B->bond_pad.data(), B->bond_pad.size()))) return rc;
-  if ((rc = up((void **)&B->d_bond_blk, B->bond_blk.data(), B->bond_blk.size() * 4))) return rc;
-  if ((rc = up((void **)&B->d_nib, B->nib.data(), B->nib.size() * 4))) return rc;
-  ED_CK(cudaStreamSynchronize(st));
-  return ED_OK;
+  up((void **)&B->d_sqrt, sq.data(), sq.size() * 8);
+  up((void **)&B->d_rsqrt, rs.data(), rs.size() * 8);
+  up((void **)&B->d_cs, cs.data(), cs.size() * 8);
+  up((void **)&B->d_bond_pos, B->bond_pos.data(), B->bond_pos.size());
+  up((void **)&B->d_bond_pad, B->bond_pad.data(), B->bond_pad.size());
+  up((void **)&B->d_bond_blk, B->bond_blk.data(), B->bond_blk.size() * 4);
+  up((void **)&B->d_nib, B->nib.data(), B->nib.size() * 4);
 }
 
 // One sublattice: the whole table (Sec. III, "store the representative and g for every
 // state"), built on the device, or shared with another basis of the same group.
 int build_full_table(ed_basis *B, cudaStream_t st, const ed_basis *share) {
   const int N = B->N, ns = B->nsym;
-  auto up = [&](void **dst, const void *src, size_t bytes) -> int {
-    if (cudaMalloc(dst, bytes) != cudaSuccess) { cudaGetLastError(); return ed_fail(ED_ERR_OOM, "cannot allocate lookup tables"); }
-    ED_CK(cudaMemcpyAsync(*dst, src, bytes, cudaMemcpyHostToDevice, st));
-    B->table_bytes += bytes;
-    return ED_OK;
-  };
+  TableSet tabs;
   std::vector<uint8_t> pbit((size_t)ns * N);
   for (int g = 0; g < ns; g++)
     for (int b = 0; b < N; b++)   // bit b is label N-1-b; its image label perm[g][N-1-b]
       pbit[(size_t)g * N + b] = (uint8_t)(N - 1 - B->perm[(size_t)g * N + (N - 1 - b)]);
   int rc;
-  if ((rc = up((void **)&B->d_pbit, pbit.data(), pbit.size()))) return rc;
-  if ((rc = up((void **)&B->d_phase, B->phase.data(), B->phase.size() * 4))) return rc;
-  if ((rc = up((void **)&B->d_flip, B->flip.data(), B->flip.size()))) return rc;
+  tabs.add((void **)&B->d_pbit, pbit.data(), pbit.size());
+  tabs.add((void **)&B->d_phase, B->phase.data(), B->phase.size() * 4);
+  tabs.add((void **)&B->d_flip, B->flip.data(), B->flip.size());
+  add_norm_tables(B, tabs);
+  if ((rc = tabs.upload(B, st))) return rc;
   if (share && share->full_tab && share->N == N && share->nsym == ns && share->perm == B->perm &&
       share->flip == B->flip) {
     B->full_tab = share->full_tab;
@@ -286,7 +302,7 @@ int build_full_table(ed_basis *B, cudaStream_t st, const ed_basis *share) {
   T.pbit = B->d_pbit;
   T.flip = B->d_flip;
   T.phase = B->d_phase;
-  return build_norm_tables(B, st);
+  return ED_OK;
 }
 
 // Alg. 1: for every sublattice X, substate and group element, SymmetryAction_X; then
@@ -385,34 +401,30 @@ int build_tables(ed_basis *B, cudaStream_t st, const ed_basis *share) {
         }
     }
   }
-  auto up = [&](void **dst, const void *src, size_t bytes) -> int {
-    if (bytes == 0) { *dst = nullptr; return ED_OK; }
-    if (cudaMalloc(dst, bytes) != cudaSuccess) { cudaGetLastError(); return ed_fail(ED_ERR_OOM, "cannot allocate lookup tables"); }
-    ED_CK(cudaMemcpyAsync(*dst, src, bytes, cudaMemcpyHostToDevice, st));
-    B->table_bytes += bytes;
-    return ED_OK;
-  };
-  int rc;
-  if ((rc = up((void **)&B->d_rep, rep.data(), rep.size() * 4))) return rc;
-  if ((rc = up((void **)&B->d_sym_off, symoff.data(), symoff.size() * 4))) return rc;
+  TableSet tabs;
+  auto up = [&](void **dst, const void *src, size_t n) { tabs.add(dst, src, n); };
+  up((void **)&B->d_rep, rep.data(), rep.size() * 4);
+  up((void **)&B->d_sym_off, symoff.data(), symoff.size() * 4);
   if (symlist.empty()) symlist.push_back(0);
-  if ((rc = up((void **)&B->d_sym_list, symlist.data(), symlist.size() * 2))) return rc;
-  if ((rc = up((void **)&B->d_dest, dest.data(), dest.size()))) return rc;
-  if ((rc = up((void **)&B->d_phase, B->phase.data(), B->phase.size() * 4))) return rc;
-  if ((rc = up((void **)&B->d_src, src.data(), src.size()))) return rc;
+  up((void **)&B->d_sym_list, symlist.data(), symlist.size() * 2);
+  up((void **)&B->d_dest, dest.data(), dest.size());
+  up((void **)&B->d_phase, B->phase.data(), B->phase.size() * 4);
+  up((void **)&B->d_src, src.data(), src.size());
   if (two) {
     if (e2.empty()) { e2.push_back(0xFFFu); off2.push_back(0); }
     if (list2.empty()) list2.push_back(0);
-    if ((rc = up((void **)&B->d_e1, e1.data(), e1.size() * 4))) return rc;
-    if ((rc = up((void **)&B->d_rid, rid.data(), rid.size()))) return rc;
-    if ((rc = up((void **)&B->d_e2, e2.data(), e2.size() * 4))) return rc;
-    if ((rc = up((void **)&B->d_off2, off2.data(), off2.size() * 4))) return rc;
-    if ((rc = up((void **)&B->d_list2, list2.data(), list2.size() * 2))) return rc;
+    up((void **)&B->d_e1, e1.data(), e1.size() * 4);
+    up((void **)&B->d_rid, rid.data(), rid.size());
+    up((void **)&B->d_e2, e2.data(), e2.size() * 4);
+    up((void **)&B->d_off2, off2.data(), off2.size() * 4);
+    up((void **)&B->d_list2, list2.data(), list2.size() * 2);
     B->two_level = true;
     B->n_rid = nrid;
   }
-  if (u16) { if ((rc = up(&B->d_action, act16.data(), act16.size() * 2))) return rc; }
-  else { if ((rc = up(&B->d_action, act32.data(), act32.size() * 4))) return rc; }
+  if (u16) up(&B->d_action, act16.data(), act16.size() * 2);
+  else up(&B->d_action, act32.data(), act32.size() * 4);
+  add_norm_tables(B, tabs);
+  if (const int rc = tabs.upload(B, st)) return rc;
   B->sym_list_len = symlist.size();
   DevTables &T = B->T;
   T.N = N; T.nsub = nsub; T.n = n; T.nsym = ns; T.denom = B->denom;
@@ -420,17 +432,13 @@ int build_tables(ed_basis *B, cudaStream_t st, const ed_basis *share) {
   T.rep = B->d_rep; T.sym_off = B->d_sym_off; T.sym_list = B->d_sym_list;
   T.action = B->d_action; T.dest = B->d_dest; T.phase = B->d_phase;
   T.chi_trivial = 0;
-  return build_norm_tables(B, st);
+  return ED_OK;
 }
 
 void free_all(ed_basis *B) {
   ed_free_pair(B);
-  void *ptrs[] = {B->d_rep, B->d_sym_off, B->d_sym_list, B->d_action, B->d_dest, B->d_phase,
-                  B->d_src, B->d_e1, B->d_rid, B->d_e2, B->d_off2, B->d_list2, B->d_bond_pad,
-                  B->d_bond_blk, B->d_nib, B->d_pbit, B->d_flip,
-                  B->d_basis, B->d_stab, B->d_top_rank, B->d_limits, B->d_rlim,
-                  B->d_postfix == B->d_basis ? nullptr : B->d_postfix,
-                  B->d_sqrt, B->d_rsqrt, B->d_cs, B->d_bond_pos, B->d_partial,
+  void *ptrs[] = {B->d_tables, B->d_basis, B->d_stab, B->d_top_rank, B->d_limits, B->d_rlim,
+                  B->d_postfix == B->d_basis ? nullptr : B->d_postfix, B->d_partial,
                   B->d_stage_x, B->d_stage_y};
   for (void *p : ptrs) if (p) cudaFree(p);
   if (B->h_partial) cudaFreeHost(B->h_partial);

@@ -40,6 +40,8 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <map>
+#include <mutex>
 #include <new>
 #include <type_traits>
 #include <vector>
@@ -957,6 +959,7 @@ struct PairPlan {
   double *chi = nullptr, *w = nullptr, *rw = nullptr;
   uint16_t *meta = nullptr;
   cudaMemPool_t pool = nullptr;   // xs of the calls in flight, stream-ordered
+  bool own_pool = false;
   size_t bytes = 0;
 };
 
@@ -966,7 +969,7 @@ void ed_free_pair(ed_basis *B) {
   if (!p) return;
   for (void *q : {p->d_half, p->d_small, p->d_slots, p->d_rows})
     if (q) cudaFree(q);
-  if (p->pool) cudaMemPoolDestroy(p->pool);
+  if (p->pool && p->own_pool) cudaMemPoolDestroy(p->pool);
   delete p;
 }
 
@@ -997,6 +1000,33 @@ struct Scratch {
     return q;
   }
 };
+
+constexpr size_t kSharedPoolMax = (size_t)4 << 20;    // xs of fp64 vectors
+constexpr uint64_t kSharedPoolKeep = 64ull << 20;
+
+cudaMemPool_t make_pool(int device, uint64_t keep) {
+  cudaMemPoolProps props{};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = device;
+  cudaMemPool_t pool = nullptr;
+  if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+  if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+    cudaGetLastError();
+    cudaMemPoolDestroy(pool);
+    return nullptr;
+  }
+  return pool;
+}
+
+cudaMemPool_t shared_pool(int device) {
+  static std::mutex lock;
+  static std::map<int, cudaMemPool_t> pools;
+  std::lock_guard<std::mutex> hold(lock);
+  cudaMemPool_t &p = pools[device];
+  if (!p) p = make_pool(device, kSharedPoolKeep);
+  return p;
+}
 
 // Row order for large sectors (see pair_rows_kernel); p->n_slices stays 0 when it is not made.
 // pat: the pattern of the other half of every slot.
@@ -1458,21 +1488,16 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
   p->weights = any != 0;
   if (Q.pat)
     if ((rc = build_rows(B, p, start, Q.start, Q.pat, st))) return rc;
-  cudaMemPoolProps props{};
-  props.allocType = cudaMemAllocationTypePinned;
-  props.location.type = cudaMemLocationTypeDevice;
-  props.location.id = B->device;
-  if (cudaMemPoolCreate(&p->pool, &props) != cudaSuccess) {
-    cudaGetLastError();
-    p->pool = nullptr;
-    ed_free_pair(B);
-    return ED_OK;
-  }
-  uint64_t all = ~0ull;
-  ED_CK(cudaMemPoolSetAttribute(p->pool, cudaMemPoolAttrReleaseThreshold, &all));
+  // The memory of xs: large sectors keep a pool of their own, gone with the basis; small ones
+  // (a pool costs 0.2 ms, as much as the rest of their tables) share one per device, which
+  // keeps at most kSharedPoolKeep between synchronisations and gives back the rest.
+  const size_t first = 8 * ((size_t)p->n_slots + 1) + 256;
+  p->own_pool = first > kSharedPoolMax;
+  if (p->own_pool) p->pool = make_pool(B->device, ~0ull);
+  else p->pool = shared_pool(B->device);
+  if (!p->pool) { ed_free_pair(B); return ED_OK; }
   // small sectors: the pool takes its first memory here rather than in the first product,
   // where mapping it would cost several times the product itself
-  const size_t first = 8 * (size_t)p->n_slots;
   if (first <= ((size_t)64 << 20)) {
     void *q = nullptr;
     if (cudaMallocFromPoolAsync(&q, first, p->pool, st) == cudaSuccess) ED_CK(cudaFreeAsync(q, st));

@@ -288,6 +288,7 @@ struct ed_basis {
   std::vector<uint32_t> nib;           // [word][nibble][16]: antiparallel-mask contributions
   // tables
   DevTables T{};
+  void *d_tables = nullptr;            // one allocation for the lookup tables below
   uint32_t *d_rep = nullptr, *d_sym_off = nullptr;
   uint16_t *d_sym_list = nullptr;
   void *d_action = nullptr;
