@@ -138,27 +138,6 @@ __device__ __forceinline__ void cpy(unsigned char *sm, uint32_t off, const T *g,
   for (uint32_t k = threadIdx.x; k < n; k += blockDim.x) d[k] = g[k];
 }
 
-template <typename V>
-__device__ __forceinline__ V ld_slot(const V *p) {
-  if constexpr (std::is_same<V, float>::value) {
-    float f;
-    asm volatile("ld.global.nc.L1::no_allocate.f32 %0, [%1];" : "=f"(f) : "l"(p));
-    return f;
-  } else if constexpr (std::is_same<V, double>::value) {
-    double f;
-    asm volatile("ld.global.nc.L1::no_allocate.f64 %0, [%1];" : "=d"(f) : "l"(p));
-    return f;
-  } else if constexpr (std::is_same<V, float2>::value) {
-    float2 f;
-    asm volatile("ld.global.nc.L1::no_allocate.v2.f32 {%0,%1}, [%2];" : "=f"(f.x), "=f"(f.y) : "l"(p));
-    return f;
-  } else {
-    double2 f;
-    asm volatile("ld.global.nc.L1::no_allocate.v2.f64 {%0,%1}, [%2];" : "=d"(f.x), "=d"(f.y) : "l"(p));
-    return f;
-  }
-}
-
 // one row's running sum over a coupling class: fp64, or a double-float pair for fp32
 // vectors (the fp64 pipe of this GPU issues at a small fraction of the fp32 rate); signs come
 // in the top bit of w
@@ -312,7 +291,7 @@ __device__ __forceinline__ void pair_loop(const PairParams &P, int n, G gen, con
     for (int u = 0; u < U; u++) {
       const uint32_t slot = u == 0 || u < n ? g[u].slot : P.n_slots;   // xs[n_slots] = 0
       t.w[u] = g[u].w;
-      t.v[u] = ld_slot(xs + slot);
+      t.v[u] = __ldg(xs + slot);
       t.vl[u] = 0.f;
       if constexpr (std::is_same<V, float>::value) {
         if (g[u].lo) t.vl[u] = __ldg(P.xslo + slot);
@@ -381,14 +360,14 @@ __device__ __forceinline__ void pair_store(const PairParams &P, const V *x, V *y
   using A_ = typename Pv<V>::A;
   constexpr bool kF = sizeof(A_) == 4;
   if constexpr (!Pv<V>::cplx) {
-    const double xi = (double)x[i];
+    const double xi = (double)__ldcs(x + i);   // read once: keep it from pushing xs out of L2
     const double yd = diag * xi + row_re * rs;
     const A_ yi = (A_)yd;
     __stcs(y + (i - P.r0), yi);
     if (kF && P.ylo) reinterpret_cast<float *>(P.ylo)[i - P.r0] = (float)(yd - (double)yi);
     if (P.partial) dot_re += xi * (kF && P.ylo ? yd : (double)yi);
   } else {
-    const V xv = x[i];
+    const V xv = __ldcs(x + i);
     const double yr = diag * (double)xv.x + row_re * rs;
     const double yim = diag * (double)xv.y + row_im * rs;
     V yv;
@@ -561,8 +540,8 @@ __global__ void __launch_bounds__(kRowThreads, kRowBlocks) pair_rows_kernel(cons
   // offset of its class; masks of A by word; for the slice's first upper classes c (n_tab of
   // them), per bit of R(c) the entry with it flipped, and per bond within the upper half that
   // with its two bits flipped
-  uint2 *et = reinterpret_cast<uint2 *>(sm + P.off_et) + wid * (P.et_words / 2);
-  uint32_t *ma = reinterpret_cast<uint32_t *>(et + P.n_wa * 32), *eup = ma + P.n_wa;
+  uint32_t *et = reinterpret_cast<uint32_t *>(sm + P.off_et) + wid * P.et_words, *eo = et + P.n_wa * 32;
+  uint32_t *ma = eo + P.n_wa * 32, *eup = ma + P.n_wa;
   const uint32_t n_up2 = (P.n_w - P.n_wa) * 32, n_eup = P.m + n_up2;
   const V *xs = reinterpret_cast<const V *>(P.xs);
   double dot[kMode == 1 ? ED_MAXCLS : 2] = {};
@@ -570,13 +549,16 @@ __global__ void __launch_bounds__(kRowThreads, kRowBlocks) pair_rows_kernel(cons
   bool st_in = false, st_across = false;
   __shared__ uint32_t chunk_s;
   for (;;) {
+    // taken when it is worked on: a chunk taken ahead spreads the blocks over more classes
+    // (fp64 on the 6x6 sector 10.5 -> 11.0 ms)
     __syncthreads();
     if (threadIdx.x == 0) chunk_s = atomicAdd(P.next, 1u);
     __syncthreads();
-    if (chunk_s * (kRowThreads / 32) >= P.n_slices) break;
-    const uint32_t sl = chunk_s * (kRowThreads / 32) + wid;
+    const uint32_t chunk = chunk_s;
+    if (chunk * (kRowThreads / 32) >= P.n_slices) break;
+    const uint32_t sl = chunk * (kRowThreads / 32) + wid;
     if (sl >= P.n_slices) continue;
-    uint32_t lo = __ldg(P.chunk_cls + chunk_s);   // the class of the chunk's first slice
+    uint32_t lo = __ldg(P.chunk_cls + chunk);   // the class of the chunk's first slice
     while (__ldg(P.slice0 + lo + 1) <= sl) lo++;
     if (lo != cur) {
       cur = lo;
@@ -592,7 +574,8 @@ __global__ void __launch_bounds__(kRowThreads, kRowBlocks) pair_rows_kernel(cons
       __syncwarp();
       for (uint32_t k = lane; k < P.n_wa * 32; k += 32) {
         const uint32_t e = __ldg(P.ta + (A ^ fw[k]));
-        et[k] = make_uint2(e | (uint32_t)pos[k] << kPosShift, S.off[e >> kClassShift]);
+        et[k] = e | (uint32_t)pos[k] << kPosShift;
+        eo[k] = S.off[e >> kClassShift];
       }
       for (uint32_t wd = lane; wd < P.n_wa; wd += 32) {
         uint32_t m = 0;
@@ -649,23 +632,23 @@ __global__ void __launch_bounds__(kRowThreads, kRowBlocks) pair_rows_kernel(cons
         auto across = [&](auto entry, auto is_static) {
           auto gen = [&](Slot (&g)[U], int nu) {
             int kb = 0;
-            uint2 e[U];
-            uint32_t eu[U];
+            uint32_t e[U], off_a[U], eu[U];
 #pragma unroll
             for (int u = 0; u < U; u++) {
               if (u == 0 || u < nu) kb = next_bond<kRowThreads>(m, wd, w0, mask_s);
               e[u] = et[kb];
-              eu[u] = entry(img_r[e[u].x >> kPosShift]);
+              if constexpr (decltype(is_static)::value) off_a[u] = eo[kb];
+              eu[u] = entry(img_r[e[u] >> kPosShift]);
             }
 #pragma unroll
             for (int u = 0; u < U; u++) {
               if constexpr (decltype(is_static)::value) {   // class(A') is the lower one
                 const uint32_t k = left_y[(eu[u] & kElem) * P.h0];
-                g[u].slot = e[u].y + P.K * (eu[u] >> kClassShift) + S.mult[(e[u].x & kElem) * P.h0 + k];
-                g[u].w = lower_sign<kChi>(e[u].x, true);
-                g[u].lo = e[u].x & eu[u] & P.lo_special;
+                g[u].slot = off_a[u] + P.K * (eu[u] >> kClassShift) + S.mult[(e[u] & kElem) * P.h0 + k];
+                g[u].w = lower_sign<kChi>(e[u], true);
+                g[u].lo = e[u] & eu[u] & P.lo_special;
               } else {
-                g[u] = slot_of<kChi, kFlips>(P, S, e[u].x & ((1u << kPosShift) - 1u), carried(eu[u]));
+                g[u] = slot_of<kChi, kFlips>(P, S, e[u] & ((1u << kPosShift) - 1u), carried(eu[u]));
               }
             }
           };
@@ -691,13 +674,13 @@ __global__ void __launch_bounds__(kRowThreads, kRowBlocks) pair_rows_kernel(cons
                 kb = wd * 32 + __ffs(m) - 1;
                 m &= m - 1;
               }
-              const uint2 e = et[kb];
+              const uint32_t e = et[kb];
               if constexpr (decltype(is_static)::value) {
-                g[u].slot = e.y + slot_up + S.mult[(e.x & kElem) * P.h0 + yB];
-                g[u].w = lower_sign<kChi>(e.x, true);
-                g[u].lo = e.x & e_up & P.lo_special;
+                g[u].slot = eo[kb] + slot_up + S.mult[(e & kElem) * P.h0 + yB];
+                g[u].w = lower_sign<kChi>(e, true);
+                g[u].lo = e & e_up & P.lo_special;
               } else {
-                g[u] = slot_of<kChi, kFlips>(P, S, e.x & ((1u << kPosShift) - 1u), e_up);
+                g[u] = slot_of<kChi, kFlips>(P, S, e & ((1u << kPosShift) - 1u), e_up);
               }
             }
           };
@@ -764,12 +747,15 @@ __global__ void __launch_bounds__(kRowThreads, kRowBlocks) pair_rows_kernel(cons
   pair_dot<kRowThreads>(P, dot, kMode == 1 ? P.n_classes : kC ? 2 : 1);
 }
 
-// xs[p] = w(meta[p]) x[idx[p]], w = chi sqrt(t); meta 0 is w = 1.  fp32 real vectors keep
-// the rounding's remainder in xslo, so that a weight sqrt(t) costs no precision.
+// xs[p] = w(meta[p]) x[idx[p]], w = chi sqrt(t); meta 0 is w = 1.  fp32 vectors take the weights
+// as pairs of fp32 words, (re, its remainder, im, its remainder): in fp64 the products and
+// conversions kept the fp64 pipe 85% busy (0.54 ms on the 6x6 sector's 4.8e7 slots).  Real ones
+// keep the rounding's remainder in xslo, so that a weight sqrt(t) costs no precision.
 template <typename V>
 __global__ void __launch_bounds__(256) expand_kernel(const V *x, const uint32_t *idx, const uint16_t *meta,
-                                                     const double2 *w, uint32_t n, V *xs, float *xslo, uint32_t *next) {
-  using A_ = typename Pv<V>::A;
+                                                     const double2 *w, const float4 *wf, uint32_t n, V *xs,
+                                                     float *xslo, uint32_t *next) {
+  constexpr bool kF = sizeof(typename Pv<V>::A) == 4;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     *next = 0;
     if constexpr (Pv<V>::cplx) { xs[n].x = 0; xs[n].y = 0; } else { xs[n] = 0; }
@@ -784,15 +770,29 @@ __global__ void __launch_bounds__(256) expand_kernel(const V *x, const uint32_t 
     if (j != 0xFFFFFFFFu) {
       v = __ldg(x + j);
       if (mt) {
-        const double2 c = __ldg(w + mt);
-        if constexpr (Pv<V>::cplx) {
-          const double a = c.x * (double)v.x - c.y * (double)v.y, b = c.x * (double)v.y + c.y * (double)v.x;
-          v.x = (A_)a;
-          v.y = (A_)b;
+        if constexpr (kF && Pv<V>::cplx) {
+          const float4 c = __ldg(wf + mt);
+          const V u = v;
+          float h = 0.f, l = 0.f;
+          df_sub_scaled(h, l, -c.x, -c.y, u.x);
+          df_sub_scaled(h, l, c.z, c.w, u.y);
+          v.x = df_round(h, l);
+          h = l = 0.f;
+          df_sub_scaled(h, l, -c.x, -c.y, u.y);
+          df_sub_scaled(h, l, -c.z, -c.w, u.x);
+          v.y = df_round(h, l);
+        } else if constexpr (kF) {
+          const float2 c = __ldg(reinterpret_cast<const float2 *>(wf + mt));
+          const float u = v;
+          v = __fmul_rn(c.x, u);
+          lo = __fmaf_rn(c.y, u, __fmaf_rn(c.x, u, -v));
+        } else if constexpr (Pv<V>::cplx) {
+          const double2 c = __ldg(w + mt);
+          const double a = c.x * v.x - c.y * v.y, b = c.x * v.y + c.y * v.x;
+          v.x = a;
+          v.y = b;
         } else {
-          const double a = c.x * (double)v;
-          v = (A_)a;
-          lo = (float)(a - (double)v);
+          v *= __ldg(w + mt).x;
         }
       }
     }
@@ -957,6 +957,7 @@ struct PairPlan {
   uint8_t *mult = nullptr;
   uint2 *bond = nullptr;
   double *chi = nullptr, *w = nullptr, *rw = nullptr;
+  float4 *wf = nullptr;
   uint16_t *meta = nullptr;
   cudaMemPool_t pool = nullptr;   // xs of the calls in flight, stream-ordered
   bool own_pool = false;
@@ -1336,6 +1337,7 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
   const size_t n_w = (size_t)B->denom * divs.size();
   if (n_w > 65535 || divs.size() > 255) { ed_free_pair(B); return ED_OK; }
   std::vector<double> wt(2 * n_w), rwt(2 * n_w);   // and conj(chi) / sqrt(t)
+  std::vector<float4> wtf(n_w);                    // and as pairs of fp32 words
   for (size_t t = 0; t < divs.size(); t++)
     for (int q = 0; q < B->denom; q++) {
       const double a = 2.0 * M_PI * (double)q / (double)B->denom, r = std::sqrt((double)divs[t]);
@@ -1345,6 +1347,8 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
       wt[2 * (t * B->denom + q) + 1] = r * s;
       rwt[2 * (t * B->denom + q)] = c / r;
       rwt[2 * (t * B->denom + q) + 1] = -s / r;
+      const float ch = (float)(r * c), sh = (float)(r * s);
+      wtf[t * B->denom + q] = make_float4(ch, (float)(r * c - (double)ch), sh, (float)(r * s - (double)sh));
     }
   // chi of the lower half's element: [half][512] (flip bit above the element number)
   std::vector<double> chi(2 * 1024, 0.0);
@@ -1448,7 +1452,7 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
   }
   Blob blob;
   const size_t o_off = blob.add(off), o_low = blob.add(cls[0]), o_mult = blob.add(mult), o_bond = blob.add(bond),
-               o_chi = blob.add(chi), o_w = blob.add(wt), o_rw = blob.add(rwt), o_rt = blob.add(rt), o_start = blob.add(start),
+               o_chi = blob.add(chi), o_w = blob.add(wt), o_rw = blob.add(rwt), o_wf = blob.add(wtf), o_rt = blob.add(rt), o_start = blob.add(start),
                o_fup = blob.add(first_up), o_up = blob.add(up), o_tc = blob.add(tcode);
   const uint32_t zero = 0;
   const size_t o_any = blob.add(&zero, 1);
@@ -1458,7 +1462,7 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
   unsigned char *sb = (unsigned char *)p->d_small;
   ED_CK(cudaMemcpyAsync(sb, blob.bytes.data(), blob.bytes.size(), cudaMemcpyHostToDevice, st));
   p->off = (uint32_t *)(sb + o_off); p->low = (uint32_t *)(sb + o_low); p->mult = sb + o_mult;
-  p->bond = (uint2 *)(sb + o_bond); p->chi = (double *)(sb + o_chi); p->w = (double *)(sb + o_w); p->rw = (double *)(sb + o_rw);
+  p->bond = (uint2 *)(sb + o_bond); p->chi = (double *)(sb + o_chi); p->w = (double *)(sb + o_w); p->rw = (double *)(sb + o_rw); p->wf = (float4 *)(sb + o_wf);
   p->rt = (uint32_t *)(sb + o_rt);
   p->up = (uint32_t *)(sb + o_up);
   p->t_up = has_swap ? p->ta : p->tb;
@@ -1626,7 +1630,7 @@ int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, c
   switch (dtype) {
 #define PCASE(D, V)                                                                              \
   case D:                                                                                        \
-    expand_kernel<V><<<eg, 256, 0, st>>>((const V *)x, p->idx, p->meta, (const double2 *)p->w, p->n_slots, (V *)ws, xslo, P.next); \
+    expand_kernel<V><<<eg, 256, 0, st>>>((const V *)x, p->idx, p->meta, (const double2 *)p->w, p->wf, p->n_slots, (V *)ws, xslo, P.next); \
     rc = cudaGetLastError() == cudaSuccess ? launch_pair_v<V>(B, P, chi, p->flips, rows, mode, st)      \
                                            : ed_fail(ED_ERR_CUDA, "expand_kernel");              \
     break;
