@@ -33,6 +33,7 @@ struct BatchSector {
   // the minimising element and whether |Stab| > 1; basis index by rank (null: the rank itself);
   // chi per element, as signs for real sectors
   const uint32_t *otab, *jmap;
+  void *xo;          // sectors with jmap: x by orbit rank, zeros where the irrep drops the orbit
   const float2 *chi;
   uint32_t sign[8];
   int cplx;
@@ -50,7 +51,11 @@ struct ed_batch {
   float *d_ftab = nullptr;   // the sectors' fp32 norm and phase tables, back to back
   bool all_full = false;     // every sector has a one-sublattice (whole) table
   bool orbit = false;        // and the orbit tables were made
-  std::vector<void *> d_orbit;   // orbit tables (per group) and index maps
+  std::vector<void *> d_orbit;   // orbit tables (per group), index maps and xo
+  uint32_t *d_map_at = nullptr;  // sectors with an index map: its first entry, in all n_maps
+  uint32_t *d_map_sec = nullptr;
+  uint32_t n_map_sec = 0;
+  uint64_t n_maps = 0;
   int cls_off[ED_MAXCLS + 1];
   double jh[ED_MAXCLS], jzq[ED_MAXCLS];
   const uint32_t *nib = nullptr;   // the first basis's nibble tables (shared lattice)
@@ -212,13 +217,39 @@ __global__ void __launch_bounds__(256) orbit_index(const uint64_t *basis, int64_
     jmap[otab[basis[i]] & ((1u << kOrbitBits) - 1u)] = (uint32_t)i;
 }
 
+// xo of the sectors with an index map: xo[rank] = x[jmap[rank]], 0 where the orbit is dropped.
+// One streaming pass over the maps instead of a map access in every term.
+__global__ void __launch_bounds__(256) expand_orbits(const BatchSector *sec, const uint32_t *map_at, const uint32_t *map_sec,
+                                                     uint32_t n_sec, uint64_t total, int k) {
+  for (uint64_t t = (uint64_t)blockIdx.x * 256 + threadIdx.x; t < total; t += (uint64_t)gridDim.x * 256) {
+    uint32_t lo = 0, hi = n_sec - 1;
+    while (lo < hi) {
+      const uint32_t mid = (lo + hi + 1) >> 1;
+      if (__ldg(map_at + mid) <= t) lo = mid; else hi = mid - 1;
+    }
+    const BatchSector &S = sec[__ldg(map_sec + lo)];
+    const uint32_t o = (uint32_t)(t - __ldg(map_at + lo)), j = __ldg(S.jmap + o);
+    const int n = S.cplx ? 2 * k : k;   // floats of a row
+    const float *x = reinterpret_cast<const float *>(S.x) + (size_t)j * n;
+    float *xo = reinterpret_cast<float *>(S.xo) + (size_t)o * n;
+    const bool in = j != 0xFFFFFFFFu;
+    if (n % 4 == 0) {
+      for (int q = 0; q < n; q += 4)
+        *reinterpret_cast<float4 *>(xo + q) = in ? *reinterpret_cast<const float4 *>(x + q) : make_float4(0.f, 0.f, 0.f, 0.f);
+    } else {
+      for (int q = 0; q < n; q++) xo[q] = in ? x[q] : 0.f;
+    }
+  }
+}
+
 // How a sector finds a term's index.  kSearch: any split, the block-wise search and the
 // Limits lookup.  kFull: every sector has a whole table (one sublattice), so the block-wise
 // search is not compiled in.  kOrbit: whole tables small enough for orbit tables (|G| <= 256,
 // fewer than 2^23 orbits per S^z, device memory for 4 bytes per configuration and group):
 // every term's accesses run through the L1 data pipe, which bounds this kernel, so a 4-byte
 // entry with the orbit's rank replaces the 8-byte one, the prefix rank and the 16-byte record
-// of the ranked Limits; chi is one load (signs: bits of the warp's sector descriptor).
+// of the ranked Limits; chi is one load (signs: bits of the warp's sector descriptor), and where
+// an irrep drops orbits x is first spread over all ranks (expand_orbits).
 enum Lookup { kSearch, kFull, kOrbit };
 
 // Resident blocks per SM: 6 up to k = 4 (40 registers); 4 for k = 8 (64 registers), which beat
@@ -256,7 +287,8 @@ __global__ void __launch_bounds__(kBatchThreads, kLook != kSearch ? (K <= 4 ? 6 
     // take a quarter of the data pipe
     const uint32_t *otab = S.otab, *jmap = S.jmap;
     const float2 *chi = S.chi;
-    const void *xv = S.x;
+    const void *xv = kLook == kOrbit && S.xo ? S.xo : S.x;
+    if (kLook == kOrbit && S.xo) jmap = nullptr;   // the rank itself is the row of xo
     const bool cplx = S.cplx != 0;
     for (int64_t i = (item - S.item0) * P.rows_per_item + lane;
          i < S.D && i < (item - S.item0 + 1) * P.rows_per_item; i += 32) {
@@ -294,7 +326,10 @@ __global__ void __launch_bounds__(kBatchThreads, kLook != kSearch ? (K <= 4 ? 6 
                 if (o == 0xFFFFFFFFu) continue;
               }
               j = o;
-              if (e >> 31) w *= __ldg(S.sqrt_f + __ldg(S.I.stab + j));   // rare
+              if (e >> 31) {   // rare
+                const uint32_t jt = S.xo ? __ldg(S.jmap + o) : o;
+                if (jt != 0xFFFFFFFFu) w *= __ldg(S.sqrt_f + __ldg(S.I.stab + jt));
+              }
               const uint32_t g = (e >> kOrbitBits) & 0xFFu;
               if (cplx) {
                 const float2 ch = __ldg(chi + g);
@@ -445,6 +480,11 @@ int launch(ed_batch *Bt, int rows_per_item, cudaStream_t st) {
   for (int c = 0; c < Bt->n_classes; c++) { P.jh[c] = (float)Bt->jh[c]; P.jzq[c] = (float)Bt->jzq[c]; }
   ED_CK(cudaMemsetAsync(Bt->d_counter, 0, 8, st));
   const int grid = Bt->sm_count * 8;
+  if (Bt->n_map_sec) {
+    expand_orbits<<<(int)std::min<uint64_t>((Bt->n_maps + 255) / 256, grid), 256, 0, st>>>(
+        Bt->d_sec, Bt->d_map_at, Bt->d_map_sec, Bt->n_map_sec, Bt->n_maps, Bt->k);
+    ED_CK(cudaGetLastError());
+  }
   switch (Bt->k * 4 + (Bt->orbit ? 2 : Bt->all_full ? 1 : 0)) {
 #define BCASE(K)                                                     \
   case 4 * K: batch_kernel<K, kSearch><<<grid, kBatchThreads, 0, st>>>(P); break; \
@@ -541,13 +581,37 @@ int build_orbits(ed_batch *Bt) {
   if ((maps && !d_maps) || (!chi.empty() && !d_chi)) { drop(); return ED_OK; }
   if (maps) ED_CK(cudaMemset(d_maps, 0xFF, 4 * maps));
   if (!chi.empty()) ED_CK(cudaMemcpy(d_chi, chi.data(), 8 * chi.size(), cudaMemcpyHostToDevice));
+  // xo, where it fits: rows of k entries, each sector's block 32-byte aligned
+  std::vector<uint32_t> map_at, map_sec;
+  std::vector<size_t> xo_at(Bt->n, 0);
+  size_t xo_floats = 0;
+  for (int s = 0; s < Bt->n; s++)
+    if (orbits(s) != (size_t)Bt->bases[s]->D) {
+      map_at.push_back((uint32_t)at[s]);
+      map_sec.push_back((uint32_t)s);
+      xo_at[s] = xo_floats;
+      xo_floats += (orbits(s) * Bt->k * (Bt->host[s].cplx ? 2 : 1) + 7) / 8 * 8;
+    }
+  float *d_xo = nullptr;
+  if (maps && maps < (1ull << 32) && (d_xo = (float *)get(4 * xo_floats)) != nullptr &&
+      (Bt->d_map_at = (uint32_t *)get(8 * map_at.size())) != nullptr) {
+    Bt->d_map_sec = Bt->d_map_at + map_at.size();
+    ED_CK(cudaMemcpy(Bt->d_map_at, map_at.data(), 4 * map_at.size(), cudaMemcpyHostToDevice));
+    ED_CK(cudaMemcpy(Bt->d_map_sec, map_sec.data(), 4 * map_sec.size(), cudaMemcpyHostToDevice));
+    Bt->n_map_sec = (uint32_t)map_at.size();
+    Bt->n_maps = maps;
+  } else {
+    d_xo = nullptr;
+  }
   for (int s = 0; s < Bt->n; s++) {
     const ed_basis *B = Bt->bases[s];
     BatchSector &S = Bt->host[s];
     S.otab = tables[table_of[s]].otab;
     S.jmap = nullptr;
+    S.xo = nullptr;
     if (orbits(s) != (size_t)B->D) {
       S.jmap = d_maps + at[s];
+      if (d_xo) S.xo = d_xo + xo_at[s];
       if (B->D > 0) {
         orbit_index<<<(int)std::min<int64_t>((B->D + 255) / 256, grid), 256>>>(B->d_basis, B->D, S.otab, d_maps + at[s]);
         ED_CK(cudaGetLastError());
