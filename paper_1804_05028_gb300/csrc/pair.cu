@@ -73,6 +73,9 @@ struct PairParams {
   // halves of a state: (((s >> sh[0]) & bmask_hi) << n) | ((s >> sh[1]) & bmask)
   int n;
   int shA0, shA1, shB0, shB1;
+  bool blocks;                   // else by nibbles, half_x[half][n_nib][16]
+  const uint32_t *half_x;
+  uint32_t off_hx;
   uint32_t bmask_hi, bmask;
   const uint32_t *ta, *tb;       // half tables
   const uint32_t *off;           // [n_cls] slot offset of the lower class
@@ -443,7 +446,9 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) pair_kernel(const __grid
   extern __shared__ __align__(16) unsigned char sm[];
   const PairSm S = pair_stage<V, kChi>(P, sm);
   cpy(sm, P.off_nib, P.nib, (uint32_t)P.cls_word[P.n_classes] * P.n_nib * 16);
+  if (!P.blocks) cpy(sm, P.off_hx, P.half_x, P.n_nib * 32);
   __syncthreads();
+  const uint32_t *hx = reinterpret_cast<const uint32_t *>(sm + P.off_hx);
   const uint32_t *nibs = reinterpret_cast<const uint32_t *>(sm + P.off_nib);
   const double *rsd = reinterpret_cast<const double *>(sm + P.off_rs);
   uint32_t *mask_s = reinterpret_cast<uint32_t *>(sm + P.off_mask) + threadIdx.x;
@@ -452,8 +457,17 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) pair_kernel(const __grid
   const int64_t stride = (int64_t)gridDim.x * kThreads;
   for (int64_t i = P.r0 + (int64_t)blockIdx.x * kThreads + threadIdx.x; i < P.r1; i += stride) {
     const uint64_t s = __ldcs(reinterpret_cast<const unsigned long long *>(P.basis) + i);
-    const uint32_t A = (((uint32_t)(s >> P.shA0) & P.bmask_hi) << P.n) | ((uint32_t)(s >> P.shA1) & P.bmask);
-    const uint32_t B = (((uint32_t)(s >> P.shB0) & P.bmask_hi) << P.n) | ((uint32_t)(s >> P.shB1) & P.bmask);
+    uint32_t A = 0, B = 0;
+    if (P.blocks) {
+      A = (((uint32_t)(s >> P.shA0) & P.bmask_hi) << P.n) | ((uint32_t)(s >> P.shA1) & P.bmask);
+      B = (((uint32_t)(s >> P.shB0) & P.bmask_hi) << P.n) | ((uint32_t)(s >> P.shB1) & P.bmask);
+    } else {
+      for (uint32_t q = 0; q < P.n_nib; q++) {
+        const uint32_t v = (uint32_t)(s >> (4 * q)) & 15u;
+        A |= hx[q * 16 + v];
+        B |= hx[(P.n_nib + q) * 16 + v];
+      }
+    }
     double diag = 0.0, row_re = 0.0, row_im = 0.0;
     for (int c = 0; c < P.n_classes; c++) {
       const int w0 = P.cls_word[c], w1 = P.cls_word[c + 1];
@@ -802,37 +816,71 @@ __global__ void __launch_bounds__(256) expand_kernel(const V *x, const uint32_t 
 }
 
 // ------------------------------- tables (once per basis) -----------------------------
-// The half tables from the block tables: for every half pattern u the smallest image under
-// the listed elements, the number of the first of them in the list, and whether several
-// reach it.
-struct HalfParams {
-  const uint16_t *act;
-  const uint8_t *dest;
-  int n, nsub, nsym;
-  int b0, b1;          // blocks of the half (b0 most significant; b1 = -1: one block)
-  int t0;              // most significant block of the half it is carried onto
-  const uint16_t *list;
-  int n_list;
-};
-
-__device__ __forceinline__ uint32_t half_image(const HalfParams &Q, uint32_t u, int g) {
-  const uint32_t mask = (1u << Q.n) - 1u;
-  if (Q.b1 < 0) return Q.act[(((uint32_t)Q.b0 << Q.n) | u) * (uint32_t)Q.nsym + (uint32_t)g];
-  const uint32_t i0 = Q.act[(((uint32_t)Q.b0 << Q.n) | (u >> Q.n)) * (uint32_t)Q.nsym + (uint32_t)g];
-  const uint32_t i1 = Q.act[(((uint32_t)Q.b1 << Q.n) | (u & mask)) * (uint32_t)Q.nsym + (uint32_t)g];
-  return Q.dest[g * Q.nsub + Q.b0] == Q.t0 ? (i0 << Q.n) | i1 : (i1 << Q.n) | i0;
+// Images of half patterns under listed elements, eight bits at a time: img[j][chunk][value],
+// from the images of the single bits (pos[j][bit]) and, for elements that also reverse every
+// spin, the complement put into chunk 0.
+__global__ void chunk_images(const uint8_t *pos, const uint8_t *flip, int n_list, int m, uint32_t *img) {
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n_list * 768; t += gridDim.x * blockDim.x) {
+    const int j = t / 768, ch = (t / 256) % 3, v = t & 255;
+    uint32_t r = flip[j] && ch == 0 ? (1u << m) - 1u : 0u;
+    for (int b = 0; b < 8 && ch * 8 + b < m; b++)
+      if ((v >> b) & 1) r ^= 1u << pos[j * m + ch * 8 + b];
+    img[t] = r;
+  }
 }
 
-__global__ void half_reps(const HalfParams Q, uint32_t total, uint32_t *rep, uint32_t *first) {
+__device__ __forceinline__ uint32_t half_image(const uint32_t *img, uint32_t u, uint32_t j) {
+  const uint32_t *t = img + j * 768;
+  return __ldg(t + (u & 255u)) ^ __ldg(t + 256 + ((u >> 8) & 255u)) ^ __ldg(t + 512 + (u >> 16));
+}
+
+// For every half pattern u the smallest image under the listed elements, the number of the
+// first of them in the list, and whether several reach it.
+__global__ void half_reps(const uint32_t *img, uint32_t n_list, uint32_t total, uint32_t *rep, uint32_t *first) {
   for (uint32_t u = blockIdx.x * blockDim.x + threadIdx.x; u < total; u += gridDim.x * blockDim.x) {
     uint32_t best = 0xFFFFFFFFu, at = 0, cnt = 0;
-    for (int j = 0; j < Q.n_list; j++) {
-      const uint32_t v = half_image(Q, u, Q.list[j]);
-      if (v < best) { best = v; at = (uint32_t)j; cnt = 1; }
+    for (uint32_t j = 0; j < n_list; j++) {
+      const uint32_t v = half_image(img, u, j);
+      if (v < best) { best = v; at = j; cnt = 1; }
       else if (v == best) cnt++;
     }
     rep[u] = best;
     first[u] = at | (cnt > 1 ? 0x80000000u : 0u);
+  }
+}
+
+// ed_launch_pair_slots for halves that are not blocks of the split, and for splits without
+// the two-level search: Alg. 2 as printed (or the whole table of a one-sublattice split).
+// img: images of the upper representatives; spread[half][chunk][value]: a half's bits in place.
+__global__ void __launch_bounds__(256) pair_slots_any(const DevTables T, const DevIndex I, const PairSlots Q, int n_up,
+                                                      const uint32_t *img, const uint64_t *spread) {
+  for (uint64_t p = (uint64_t)blockIdx.x * 256 + threadIdx.x; p < Q.n_slots; p += (uint64_t)gridDim.x * 256) {
+    uint32_t lo = 0, hi = Q.n_low - 1;
+    while (lo < hi) {   // the last class that starts at or before p (empty ones share a start)
+      const uint32_t mid = (lo + hi + 1) >> 1;
+      if (__ldg(Q.start + mid) <= (uint32_t)p) lo = mid; else hi = mid - 1;
+    }
+    const uint32_t r = (uint32_t)p - __ldg(Q.start + lo);
+    const uint32_t a = __ldg(Q.low + lo);
+    const uint32_t b = half_image(img, __ldg(Q.up + __ldg(Q.first_up + lo) + r / Q.K), r % Q.K);
+    uint32_t idx = 0xFFFFFFFFu;
+    uint16_t meta = 0;
+    if (__popc(a) + __popc(b) == n_up) {
+      uint64_t s = 0;
+#pragma unroll
+      for (int c = 0; c < 3; c++)
+        s |= __ldg(spread + c * 256 + ((a >> (8 * c)) & 255u)) | __ldg(spread + 768 + c * 256 + ((b >> (8 * c)) & 255u));
+      const RepOut R = find_rep(T, T.rep, T.sym_off, T.sym_list, T.dest, T.phase, s);
+      const int64_t j = R.mixed ? -1 : lookup_index(I, R.rep);
+      if (j >= 0) {
+        idx = (uint32_t)j;
+        meta = (uint16_t)(T.phase[R.g] + T.denom * (int)__ldg(Q.tcode + R.t));
+        if (R.t > 1) *Q.any_weight = 1u;   // every writer stores the same value
+      }
+    }
+    Q.idx[p] = idx;
+    Q.meta[p] = meta;
+    if (Q.pat) Q.pat[p] = b;
   }
 }
 
@@ -940,6 +988,8 @@ __global__ void class_rows(const uint64_t *at, const uint32_t *chunk0, uint32_t 
 struct PairPlan {
   int n = 0, m = 0;
   int shA0 = 0, shA1 = 0, shB0 = 0, shB1 = 0;
+  bool blocks = true;
+  uint32_t *half_x = nullptr;
   uint32_t bmask_hi = 0, bmask = 0;
   uint32_t n_cls = 0, K = 0, h0 = 0, sel_off = 0, mult_bytes = 0, n_slots = 0;
   uint32_t n_slices = 0, ubase = 0, n_ucls = 0;
@@ -1105,25 +1155,59 @@ int build_rows(ed_basis *B, PairPlan *p, const std::vector<uint32_t> &start, con
 // memory is short.  Only CUDA failures other than out-of-memory are errors.
 int ed_build_pair(ed_basis *B, cudaStream_t st) {
   const int nsub = B->nsub, n = B->n, ns = B->nsym, N = B->N;
-  if (!B->two_level || (nsub != 2 && nsub != 4) || B->D == 0 || ns > 1000 || N > 44) return ED_OK;
+  if (B->D == 0 || ns > 1000 || N > 44 || N % 2) return ED_OK;
   const int m = N / 2;
-  std::vector<uint8_t> dest((size_t)ns * nsub);
-  for (int g = 0; g < ns; g++)
-    for (int X = 0; X < nsub; X++) dest[(size_t)g * nsub + X] = (uint8_t)(B->perm[(size_t)g * N + X * n] / n);
-  // halves: block sets {hb[0], hb[1]} and {hb[2], hb[3]} (one block each when nsub == 2)
+  // The half and the bit in it of every site.  First choice: blocks {hb[0], hb[1]} and
+  // {hb[2], hb[3]} of the split (one block each when it has two), whose patterns are two
+  // shifts of the state.
+  std::vector<int> half(N, -1), pos(N, 0);
   static const int kSplit[3][4] = {{0, 1, 2, 3}, {0, 2, 1, 3}, {0, 3, 1, 2}};
   int hb[4] = {0, -1, 1, -1};
   std::vector<uint8_t> swaps(ns, 0);
-  bool found = false;
-  for (int t = 0; t < (nsub == 4 ? 3 : 1) && !found; t++) {
-    if (nsub == 4) for (int q = 0; q < 4; q++) hb[q] = kSplit[t][q];
-    auto half_of = [&](int X) { return X == hb[0] || X == hb[1] ? 0 : 1; };
-    found = true;
-    for (int g = 0; g < ns && found; g++) {
-      const int to = half_of(dest[(size_t)g * nsub + hb[0]]);
-      if (nsub == 4 && half_of(dest[(size_t)g * nsub + hb[1]]) != to) found = false;
+  auto stable = [&]() {   // every element keeps the halves or exchanges them
+    int in_a = 0;
+    for (int q = 0; q < N; q++) in_a += half[q] == 0;
+    if (in_a != m) return false;
+    for (int g = 0; g < ns; g++) {
+      const int32_t *q = B->perm.data() + (size_t)g * N;
+      const int to = half[q[0]] ^ half[0];
+      for (int l = 1; l < N; l++)
+        if ((half[q[l]] ^ half[l]) != to) return false;
       swaps[g] = (uint8_t)to;
     }
+    return true;
+  };
+  bool blocks = false;
+  if (B->two_level && (nsub == 2 || nsub == 4))
+    for (int t = 0; t < (nsub == 4 ? 3 : 1) && !blocks; t++) {
+      if (nsub == 4) for (int q = 0; q < 4; q++) hb[q] = kSplit[t][q];
+      for (int l = 0; l < N; l++) {
+        const int X = l / n;
+        half[l] = X == hb[0] || X == hb[1] ? 0 : 1;
+        pos[l] = n - 1 - l % n + (nsub == 4 && (X == hb[0] || X == hb[2]) ? n : 0);
+      }
+      blocks = stable();
+    }
+  // Else the two colours of a coupling class whose bonds form a connected bipartite graph on all
+  // sites: symmetries keep the class's bonds, so they keep its colouring.
+  bool found = blocks;
+  for (int c = 0; c < B->n_classes && !found; c++) {
+    std::fill(half.begin(), half.end(), -1);
+    std::vector<int> order{0};
+    half[0] = 0;
+    bool ok = true;
+    for (size_t q = 0; q < order.size() && ok; q++)
+      for (int b = B->cls_off[c]; b < B->cls_off[c + 1] && ok; b++) {
+        const int e0 = N - 1 - B->bond_pos[2 * b], e1 = N - 1 - B->bond_pos[2 * b + 1];
+        if (e0 != order[q] && e1 != order[q]) continue;
+        const int o = e0 == order[q] ? e1 : e0;
+        if (half[o] < 0) { half[o] = 1 - half[order[q]]; order.push_back(o); }
+        else if (half[o] == half[order[q]]) ok = false;
+      }
+    if (!ok || (int)order.size() != N) continue;
+    int next[2] = {m - 1, m - 1};
+    for (int l = 0; l < N; l++) pos[l] = next[half[l]]--;
+    found = stable();
   }
   if (!found) return ED_OK;
   // the group as G0 x {1, F} when it holds the pure spin flip F (its elements then carry a
@@ -1237,8 +1321,10 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
   p->flips = pure;
   p->sel_off = n_tab == 2 ? h0 * h0 : 0u;
   p->mult_bytes = (uint32_t)mult.size();
+  p->blocks = blocks;
   const int sh = N - n;   // block X sits at bit N - (X + 1) n
-  if (nsub == 4) {
+  if (!blocks) {
+  } else if (nsub == 4) {
     p->shA0 = sh - hb[0] * n; p->shA1 = sh - hb[1] * n;
     p->shB0 = sh - hb[2] * n; p->shB1 = sh - hb[3] * n;
     p->bmask = p->bmask_hi = (1u << n) - 1u;
@@ -1257,27 +1343,47 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
   };
   const uint32_t total = 1u << m;
   const size_t nl = listA.size();
+  std::vector<int> site[2] = {std::vector<int>(m), std::vector<int>(m)};   // of a half's bits
+  for (int l = 0; l < N; l++) site[half[l]][pos[l]] = l;
+  // images of half A's bits under list A, of half B's under list B, and of the upper
+  // representatives' half under list B
+  const int up_half = has_swap ? 0 : 1;
+  auto images = [&](const std::vector<uint16_t> &list, int h) {
+    std::vector<uint8_t> v(nl * m);
+    for (size_t j = 0; j < nl; j++)
+      for (int q = 0; q < m; q++) v[j * m + q] = (uint8_t)pos[pm[(size_t)list[j] * N + site[h][q]]];
+    return v;
+  };
+  const std::vector<uint8_t> imA = images(listA, 0), imB = images(listB, 1), imK = images(listB, up_half);
+  std::vector<uint8_t> flA(nl), flB(nl);
+  for (size_t j = 0; j < nl; j++) { flA[j] = B->flip[listA[j]]; flB[j] = B->flip[listB[j]]; }
   Blob lists;
-  lists.add(listA); lists.add(listB); lists.add(codeA); lists.add(codeB);
+  lists.add(listB); lists.add(codeA); lists.add(codeB);
   const size_t lstep = (nl * 2 + 15) / 16 * 8;   // elements from one list to the next
-  uint32_t *d_rep = (uint32_t *)sc.get(16 * (size_t)total + lists.bytes.size());
+  const size_t o_im[3] = {lists.add(imA), lists.add(imB), lists.add(imK)}, o_fl[2] = {lists.add(flA), lists.add(flB)};
+  const size_t o_img = (lists.bytes.size() + 15) / 16 * 16;
+  uint32_t *d_rep = (uint32_t *)sc.get(16 * (size_t)total + o_img + 3 * 3072 * nl);
   p->d_half = keep(8 * (size_t)total);
   if (!d_rep || !p->d_half) { ed_free_pair(B); return ED_OK; }
   uint32_t *d_first = d_rep + total, *d_id = d_first + total, *d_reps = d_id + total;
-  uint16_t *d_list = (uint16_t *)(d_reps + total);
+  unsigned char *d_lists = (unsigned char *)(d_reps + total);
+  uint16_t *d_list = (uint16_t *)d_lists;
+  uint32_t *d_img = (uint32_t *)(d_lists + o_img);   // [3][nl][768]
   p->ta = (uint32_t *)p->d_half;
   p->tb = p->ta + total;
   ED_CK(cudaMemcpyAsync(d_list, lists.bytes.data(), lists.bytes.size(), cudaMemcpyHostToDevice, st));
+  for (int q = 0; q < 3; q++) {
+    chunk_images<<<(int)(3 * nl), 256, 0, st>>>(d_lists + o_im[q], d_lists + o_fl[q ? 1 : 0], (int)nl, m, d_img + q * 768 * nl);
+    ED_CK(cudaGetLastError());
+  }
   const int gt = (int)std::min<uint32_t>((total + 255) / 256, (uint32_t)B->sm_count * 8);
   std::vector<uint32_t> rep(total);
   std::vector<std::vector<uint32_t>> cls(2);      // representatives of half A's (and B's) classes
   std::vector<uint32_t> bucket0[2];               // first class of each popcount
-  for (int half = 0; half < 2; half++) {
-    HalfParams Q{(const uint16_t *)B->d_action, B->d_dest, n, nsub, ns, hb[2 * half], hb[2 * half + 1],
-                 half && !has_swap ? hb[2] : hb[0], d_list + half * lstep, (int)nl};
-    half_reps<<<gt, 256, 0, st>>>(Q, total, d_rep, d_first);
+  for (int h = 0; h < 2; h++) {
+    half_reps<<<gt, 256, 0, st>>>(d_img + h * 768 * nl, (uint32_t)nl, total, d_rep, d_first);
     ED_CK(cudaGetLastError());
-    if (half == 0 || !has_swap) {
+    if (h == 0 || !has_swap) {
       ED_CK(cudaMemcpyAsync(rep.data(), d_rep, (size_t)total * 4, cudaMemcpyDeviceToHost, st));
       ED_CK(cudaStreamSynchronize(st));
       // classes in order of (popcount of the representative, value); with spin flips the
@@ -1288,18 +1394,18 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
           const int pc = __builtin_popcount(u);
           by[any_flip ? std::min(pc, m - pc) : pc].push_back(u);
         }
-      bucket0[half].assign(m + 2, 0);
+      bucket0[h].assign(m + 2, 0);
       for (int q = 0; q <= m; q++) {
-        bucket0[half][q] = (uint32_t)cls[half].size();
-        cls[half].insert(cls[half].end(), by[q].begin(), by[q].end());
+        bucket0[h][q] = (uint32_t)cls[h].size();
+        cls[h].insert(cls[h].end(), by[q].begin(), by[q].end());
       }
-      bucket0[half][m + 1] = (uint32_t)cls[half].size();
-      const uint32_t nc = (uint32_t)cls[half].size();
-      ED_CK(cudaMemcpyAsync(d_reps, cls[half].data(), (size_t)nc * 4, cudaMemcpyHostToDevice, st));
-      class_ids<<<gt, 256, 0, st>>>(d_reps, nc, half ? (uint32_t)cls[0].size() : 0u, d_id);
+      bucket0[h][m + 1] = (uint32_t)cls[h].size();
+      const uint32_t nc = (uint32_t)cls[h].size();
+      ED_CK(cudaMemcpyAsync(d_reps, cls[h].data(), (size_t)nc * 4, cudaMemcpyHostToDevice, st));
+      class_ids<<<gt, 256, 0, st>>>(d_reps, nc, h ? (uint32_t)cls[0].size() : 0u, d_id);
       ED_CK(cudaGetLastError());
     }
-    half_entries<<<gt, 256, 0, st>>>(d_rep, d_first, d_id, d_list + (2 + half) * lstep, total, half ? p->tb : p->ta);
+    half_entries<<<gt, 256, 0, st>>>(d_rep, d_first, d_id, d_list + (1 + h) * lstep, total, h ? p->tb : p->ta);
     ED_CK(cudaGetLastError());
   }
   const uint32_t nA = (uint32_t)cls[0].size();
@@ -1366,9 +1472,8 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
     const int pe[2] = {B->bond_pad[2 * b], B->bond_pad[2 * b + 1]};
     if (pe[0] == pe[1]) continue;
     for (int q = 0; q < 2; q++) {
-      const int lab = N - 1 - pe[q], X = lab / n, bit = n - 1 - lab % n;
-      const int pos = bit + ((nsub == 4 && (X == hb[0] || X == hb[2])) ? n : 0);
-      if (X == hb[0] || X == hb[1]) bond[b].x |= 1u << pos; else bond[b].y |= 1u << pos;
+      const int l = N - 1 - pe[q];
+      (half[l] ? bond[b].y : bond[b].x) |= 1u << pos[l];
     }
   }
   // tables of the row order, staged in shared memory as one block of words: per bond the
@@ -1381,7 +1486,6 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
     std::vector<uint32_t> f;
     std::vector<uint8_t> bpos;
     std::vector<uint32_t> mA, mB;   // bits of the bond that count in A, and in B or R(c)
-    const int iu = has_swap ? 0 : 1;   // the half of the upper representatives
     for (int pass = 0; pass < 2; pass++) {   // bonds across and within A first
       for (int c = 0; c < B->n_classes; c++)
         for (int kind = pass ? 2 : 0; kind < (pass ? 3 : 2); kind++) {
@@ -1389,7 +1493,7 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
           for (size_t b = (size_t)B->cls_word[c] * 32; b < (size_t)B->cls_word[c + 1] * 32; b++) {
             const uint32_t fa = bond[b].x, fb = bond[b].y;
             if (!fa && !fb) continue;   // padding
-            const uint32_t fu = iu ? fb : fa;
+            const uint32_t fu = up_half ? fb : fa;
             const bool across = fa && fb;
             if (kind == 0 && across) {
               f.push_back(fa); bpos.push_back((uint8_t)__builtin_ctz(fb)); mA.push_back(fa); mB.push_back(fb);
@@ -1423,19 +1527,7 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
       return t;
     };
     const std::vector<uint32_t> tA = nibbles(mA), tB = nibbles(mB);
-    // bit q of a half pattern is a site; g carries it to a site of the half it reaches
-    auto bit_of = [&](int lab) {
-      const int X = lab / n, bit = n - 1 - lab % n;
-      return bit + ((nsub == 4 && (X == hb[0] || X == hb[2])) ? n : 0);
-    };
-    std::vector<int> label(m);
-    for (int lab = 0; lab < N; lab++) {
-      const int X = lab / n;
-      if (X == hb[2] || X == hb[3]) label[bit_of(lab)] = lab;
-    }
-    std::vector<uint8_t> im((size_t)h0 * m), lm((size_t)h0 * h0);
-    for (uint32_t y = 0; y < h0; y++)
-      for (int q = 0; q < m; q++) im[(size_t)y * m + q] = (uint8_t)bit_of(pm[(size_t)listB[y] * N + label[q]]);
+    std::vector<uint8_t> lm((size_t)h0 * h0);
     for (uint32_t x = 0; x < h0; x++)
       for (uint32_t y = 0; y < h0; y++) {
         const int e = mul(H0[x], H0[y]);
@@ -1446,7 +1538,7 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
     p->rt_nibA = words(tA.data(), tA.size() * 4);
     p->rt_nibB = words(tB.data(), tB.size() * 4);
     p->rt_pos = words(bpos.data(), bpos.size());
-    p->rt_img = words(im.data(), im.size());
+    p->rt_img = words(imB.data(), (size_t)h0 * m);
     p->rt_left = words(lm.data(), lm.size());
     p->rt_words = (uint32_t)rt.size();
   }
@@ -1454,6 +1546,21 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
   const size_t o_off = blob.add(off), o_low = blob.add(cls[0]), o_mult = blob.add(mult), o_bond = blob.add(bond),
                o_chi = blob.add(chi), o_w = blob.add(wt), o_rw = blob.add(rwt), o_wf = blob.add(wtf), o_rt = blob.add(rt), o_start = blob.add(start),
                o_fup = blob.add(first_up), o_up = blob.add(up), o_tc = blob.add(tcode);
+  // halves that are no blocks: their bits by the state's nibbles, and back by their bytes
+  std::vector<uint32_t> half_x;
+  std::vector<uint64_t> spread;
+  if (!blocks) {
+    half_x.assign(2 * (size_t)B->n_nib * 16, 0u);
+    spread.assign(2 * 768, 0);
+    for (int l = 0; l < N; l++) {
+      const int bit = N - 1 - l;
+      for (int v = 0; v < 16; v++)
+        if ((v >> (bit % 4)) & 1) half_x[((size_t)half[l] * B->n_nib + bit / 4) * 16 + v] |= 1u << pos[l];
+      for (int v = 0; v < 256; v++)
+        if ((v >> (pos[l] % 8)) & 1) spread[half[l] * 768 + pos[l] / 8 * 256 + v] |= 1ULL << bit;
+    }
+  }
+  const size_t o_hx = blob.add(half_x), o_sp = blob.add(spread);
   const uint32_t zero = 0;
   const size_t o_any = blob.add(&zero, 1);
   p->d_small = keep(blob.bytes.size());
@@ -1464,6 +1571,7 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
   p->off = (uint32_t *)(sb + o_off); p->low = (uint32_t *)(sb + o_low); p->mult = sb + o_mult;
   p->bond = (uint2 *)(sb + o_bond); p->chi = (double *)(sb + o_chi); p->w = (double *)(sb + o_w); p->rw = (double *)(sb + o_rw); p->wf = (float4 *)(sb + o_wf);
   p->rt = (uint32_t *)(sb + o_rt);
+  p->half_x = (uint32_t *)(sb + o_hx);
   p->up = (uint32_t *)(sb + o_up);
   p->t_up = has_swap ? p->ta : p->tb;
   p->ubase = ubase;
@@ -1476,15 +1584,21 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
   PairSlots Q{};
   Q.start = (uint32_t *)(sb + o_start); Q.first_up = (uint32_t *)(sb + o_fup); Q.low = p->low; Q.up = (uint32_t *)(sb + o_up);
   Q.n_low = nA; Q.n_slots = p->n_slots;
-  Q.K = K; Q.kel = d_list + lstep; Q.tcode = sb + o_tc;
+  Q.K = K; Q.kel = d_list; Q.tcode = sb + o_tc;
   for (int q = 0; q < 4; q++) Q.hb[q] = hb[q];
-  Q.up_half = has_swap ? 0 : 1;
+  Q.up_half = up_half;
   Q.idx = p->idx; Q.meta = p->meta; Q.any_weight = d_any;
   // the row order pays when xs outgrows the L2 and a class fills many warps
   const bool want_rows = B->D >= kRowOrderMinDim && B->D / nA >= 256 && ubase + up.size() <= 1u << (kPosShift - kClassShift);
   if (want_rows) Q.pat = (uint32_t *)sc.get(4 * (size_t)acc);   // null without memory: no row order
-  int rc = ed_launch_pair_slots(B, Q, st);
-  if (rc == ED_ERR_UNSUPPORTED) { ed_free_pair(B); return ED_OK; }
+  int rc = blocks ? ed_launch_pair_slots(B, Q, st) : ED_ERR_UNSUPPORTED;
+  if (rc == ED_ERR_UNSUPPORTED) {
+    if (blocks) { ed_free_pair(B); return ED_OK; }
+    pair_slots_any<<<(int)std::min<uint32_t>((p->n_slots + 255) / 256, (uint32_t)B->sm_count * 8), 256, 0, st>>>(
+        B->T, B->I, Q, B->n_up, d_img + 2 * 768 * nl, (const uint64_t *)(sb + o_sp));
+    ED_CK(cudaGetLastError());
+    rc = ED_OK;
+  }
   if (rc) return rc;
   uint32_t any = 0;
   ED_CK(cudaMemcpyAsync(&any, d_any, 4, cudaMemcpyDeviceToHost, st));
@@ -1568,6 +1682,7 @@ int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, c
   P.n = p->n;
   P.shA0 = p->shA0; P.shA1 = p->shA1; P.shB0 = p->shB0; P.shB1 = p->shB1;
   P.bmask_hi = p->bmask_hi; P.bmask = p->bmask;
+  P.blocks = p->blocks; P.half_x = p->half_x;
   P.ta = p->ta; P.tb = p->tb; P.off = p->off;
   P.n_cls = p->n_cls; P.K = p->K; P.h0 = p->h0; P.sel_off = p->sel_off;
   P.mult = p->mult; P.mult_bytes = p->mult_bytes;
@@ -1605,6 +1720,7 @@ int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, c
     put(P.off_et, 4 * (size_t)P.et_words * (kRowThreads / 32));
   } else {
     put(P.off_nib, 4 * B->nib.size());
+    put(P.off_hx, p->blocks ? 0 : 128 * (size_t)B->n_nib);
     put(P.off_mask, 4 * (size_t)words * kThreads);
   }
   P.smem_bytes = (uint32_t)off;

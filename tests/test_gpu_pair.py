@@ -1,5 +1,5 @@
-"""The coset-arithmetic product (csrc/pair.cu) at the edges of what it accepts: splits of two
-and four blocks, halves that are exchanged by an involution, by none, or by no element at
+"""The coset-arithmetic product (csrc/pair.cu) at the edges of what it accepts: halves made of
+the split's blocks or of a colouring of the bonds, halves that are exchanged by an involution, by none, or by no element at
 all, spin flips (as a factor of the group and tied to other elements), trivial, sign and
 complex characters, fillings whose halves hold no or all spins, every vector type, row ranges
 on both sides of the size rule, several streams at once and a captured call.  Reference: the
@@ -38,6 +38,13 @@ SECTORS = [
     T(4, momentum=(1, 2), point_irrep=0, J2=0.5, n_sublat=4, n_up=8),
     w.with_spin_flip(T(4, momentum=(2, 2), point_irrep=1, J2=0.5, n_sublat=4, n_up=8), 1),
     T(6, momentum=(0, 0), point_irrep=1, J2=0.5, n_sublat=4, n_up=4),
+    # halves that are no blocks of the split: the two colours of the nearest-neighbour bonds
+    w.chain(12, 1, k=5, n_up=6), w.chain(12, 3, k=6, n_up=5), w.chain(20, 5, k=7, n_up=9),
+    w.chain(16, 8, k=8, n_up=7), w.with_spin_flip(w.chain(12, 1, k=5, n_up=6), 1),
+    T(4, momentum=(1, 1), point_irrep=0, J2=0.5, n_sublat=1, n_up=6),
+    w.with_spin_flip(T(4, momentum=(0, 0), point_irrep=2, J2=0.5, n_sublat=1, n_up=8), 0),
+    # no such halves: the search kernels
+    w.chain(9, 3, k=2, n_up=4), T(3, momentum=(1, 2), point_irrep=0, J2=0.4, n_sublat=1, n_up=4),
 ]
 
 
@@ -82,6 +89,7 @@ LARGE = [
     w.chain(32, 4, k=5, n_up=11),                                                  # no involution
     w.with_spin_flip(w.chain(32, 4, k=0, n_up=16), 1),
     _sub(w.chain(28, 4, k=4, n_up=9), range(0, 28, 2), "chain28_even_translations"),  # no exchange
+    w.chain(30, 3, k=7, n_up=12),                                                  # halves across blocks
 ]
 
 
