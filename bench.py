@@ -47,6 +47,7 @@ WORKLOADS = {
 # the product kernels and the code that lays out the tables and the index they read
 KERNEL_SOURCES = ["paper_1804_05028_gb300/csrc/apply.cu",
                   "paper_1804_05028_gb300/csrc/apply_fast.cu",
+                  "paper_1804_05028_gb300/csrc/pair.cu",
                   "paper_1804_05028_gb300/csrc/sced_internal.cuh",
                   "paper_1804_05028_gb300/csrc/dfloat.cuh",
                   "paper_1804_05028_gb300/csrc/basis.cu",
@@ -439,9 +440,9 @@ def bench_sector(ed, torch, workload, p, steps, warmup, ctx, accuracy=True, full
                          "alg_bytes_per_launch": ab,
                          "sector_bytes_per_launch": sector_bytes(D, n_off, vb)},
             "roofline_issue": issue,
-            # per step: product, three-term update, scale, and the local sweep's
-            # multi-dot, coefficient reduction and update
-            "gpu_launches": 6 * steps + 2,
+            # per step: expansion of x and product, three-term update, scale, the local
+            # sweep's multi-dot, coefficient reduction and update, and the step's scalars
+            "gpu_launches": 8 * steps + 2,
         }
         del work
 

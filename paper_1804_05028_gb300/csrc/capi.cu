@@ -674,8 +674,10 @@ extern "C" int ed_apply_H_host(ed_basis *B, const double *J, const double *Jz, c
   // The product needs the whole of x, so the host-to-device copy comes first.  y goes
   // back in row chunks: the copy of chunk c (on a second stream) runs while chunk c+1
   // is computed, so only the last chunk's copy is exposed.
+  // A sector with the coset-arithmetic product computes y whole: every chunk would expand x
+  // again and leave the slot order (40 sites, fp32: 761 ms in 8 chunks).
   const int64_t kMinChunkRows = (int64_t)1 << 24;   // ~64 rows per thread: chunk tails stay small
-  const int n_chunks = (int)std::min<int64_t>(8, std::max<int64_t>(1, B->D / kMinChunkRows));
+  const int n_chunks = B->pair ? 1 : (int)std::min<int64_t>(8, std::max<int64_t>(1, B->D / kMinChunkRows));
   if (n_chunks > 1 && !B->copy_stream) {
     ED_CK(cudaStreamCreateWithFlags(&B->copy_stream, cudaStreamNonBlocking));
   }
@@ -802,21 +804,26 @@ struct LanczosRun {
 };
 
 // The sweeps of step j after the three-term update of w.  Local: one sweep against v_j and
-// v_{j-1} (the second Gram-Schmidt pass of the recurrence's own projection).  Full: two
-// sweeps against every stored v_0 .. v_j (classical Gram-Schmidt, twice).  corr[sw] points to
-// Re <v_j, w> of sweep sw (device; their sum is added to alpha_j so that the tridiagonal
-// matrix stays the projection of H); the new ||w||^2 partials are in L.d_ro.
-int reorth_step(LanczosRun &L, int j, void *w, const void *v, const void *vprev, const double *(&corr)[2]) {
+// v_{j-1} (the second Gram-Schmidt pass of the recurrence's own projection), whose dot
+// products the update has left in L.d_ro.  Full: two sweeps against every stored v_0 .. v_j
+// (classical Gram-Schmidt, twice).  corr[sw] points to Re <v_j, w> of sweep sw (device; their
+// sum is added to alpha_j so that the tridiagonal matrix stays the projection of H); the new
+// ||w||^2 partials, *n_b2 of them, are in L.d_ro.
+int reorth_step(LanczosRun &L, int j, void *w, const void *v, const void *vprev, const double *(&corr)[2], int *n_b2) {
   ed_basis *B = L.B;
   const int P = L.cplx ? 2 : 1;
-  const bool full = L.reorth == ED_REORTH_FULL;
-  const int m = full ? j + 1 : j ? 2 : 1;
-  for (int sw = 0; sw < (full ? 2 : 1); sw++) {
+  if (L.reorth != ED_REORTH_FULL) {
+    double *c = L.d_ro + L.ro_coef_off;
+    corr[0] = c;
+    *n_b2 = L.nblk;
+    return ed_launch_local_sweep(B, w, v, vprev, L.dtype, L.d_ro, L.nblk, c, L.st, L.ylo);
+  }
+  *n_b2 = ed_reorth_grid(B);
+  for (int sw = 0; sw < 2; sw++) {
     double *c = L.d_ro + L.ro_coef_off + (size_t)sw * L.coef_len;
-    const int rc = full ? ed_launch_reorth_sweep(B, w, L.store, nullptr, nullptr, m, L.dtype, L.d_ro, c, L.st, L.ylo)
-                        : ed_launch_reorth_sweep(B, w, nullptr, v, vprev, m, L.dtype, L.d_ro, c, L.st, L.ylo);
+    const int rc = ed_launch_reorth_sweep(B, w, L.store, nullptr, nullptr, j + 1, L.dtype, L.d_ro, c, L.st, L.ylo);
     if (rc) return rc;
-    corr[sw] = c + (size_t)(full ? j : 0) * P;
+    corr[sw] = c + (size_t)j * P;
   }
   return ED_OK;
 }
@@ -868,16 +875,16 @@ int lanczos_pass(LanczosRun &L, const ed_lanczos_opts *o, int max_steps, bool fi
     const int n_dot = B->last_apply_grid;
     double *part2 = B->d_partial + B->n_partial / 2;
     if ((rc = ed_launch_axpy_norm(B, w, v, j ? vprev : nullptr, replay ? alpha_rec[j] : 0.0, bprev, L.dtype, part2, nblk,
-                                  L.st, L.ylo, replay ? nullptr : B->d_partial, n_dot, L.d_scalar))) return rc;
+                                  L.st, L.ylo, replay ? nullptr : B->d_partial, n_dot, L.d_scalar,
+                                  L.reorth == ED_REORTH_LOCAL ? L.d_ro : nullptr))) return rc;
     const double *corr_d[2] = {nullptr, nullptr};
     const double *b2_part = part2;
     int n_b2 = nblk;
     if (L.reorth != ED_REORTH_NONE) {
       if (!replay) ED_CK(cudaEventRecord(L.r0, L.st));
-      if ((rc = reorth_step(L, j, w, v, j ? vprev : nullptr, corr_d))) return rc;
+      if ((rc = reorth_step(L, j, w, v, j ? vprev : nullptr, corr_d, &n_b2))) return rc;
       if (!replay) ED_CK(cudaEventRecord(L.r1, L.st));
       b2_part = L.d_ro;
-      n_b2 = ed_reorth_grid(B);
     }
     double a = 0, b2 = 0, corr = 0;
     if (!replay) {   // the step's only wait
@@ -998,10 +1005,10 @@ extern "C" int ed_lanczos(ed_basis *B, const double *J, const double *Jz,
   // sweep scratch: partials of up to m_cap vectors per block, then their coefficients
   const int m_cap = full ? max_steps + 1 : 2;
   const int P = L.cplx ? 2 : 1;
-  L.ro_coef_off = (size_t)m_cap * P * ed_reorth_grid(B);
-  L.coef_len = (size_t)m_cap * P;
   // 4 rows per thread at least, as in the sweeps
   L.nblk = (int)std::max<int64_t>(1, std::min<int64_t>(B->n_partial / 4, (B->D + 1023) / 1024));
+  L.ro_coef_off = std::max((size_t)m_cap * P * ed_reorth_grid(B), (size_t)2 * P * L.nblk);
+  L.coef_len = (size_t)m_cap * P;
   if (cudaMalloc(&L.d_ro, sizeof(double) * (L.ro_coef_off + 2 * L.coef_len + 8)) != cudaSuccess) {
     cudaGetLastError();
     if (own) for (int k = 0; k < 3; k++) cudaFree(L.v[k]);

@@ -132,8 +132,15 @@ constexpr int kRowBlocks = 1;
 constexpr int kRowU = 2;
 constexpr int kRowU16 = 2;
 constexpr int kRowU8 = 1;
+// and rows: below 2^21 a product is a few waves of blocks, and the row tables (10 bytes per row)
+// are not made
 constexpr int64_t kRowOrderMinDim = 1 << 21;
-constexpr size_t kRowOrderMinBytes = (size_t)24 << 20;
+// xs from which the row order pays: early where bonds within a half gather from one cluster (6x6
+// sector of 4.4e6 rows, fp32, 24 MB: 1.06 ms against 1.23 in basis order), else when xs
+// outgrows the L2 (30- and 32-site chains, 42 to 87 MB: 0.40 and 0.90 ms in basis order
+// against 0.55 and 1.16; 40-site cluster, 122 MB: 3.39 against 2.61)
+constexpr size_t kRowOrderMinBytes = (size_t)16 << 20;
+constexpr size_t kRowOrderMinBytesAcross = (size_t)96 << 20;
 
 template <typename T>
 __device__ __forceinline__ void cpy(unsigned char *sm, uint32_t off, const T *g, uint32_t n) {
@@ -1668,7 +1675,7 @@ int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, c
   if (!p) return ED_ERR_UNSUPPORTED;
   const size_t es = dtype == ED_F64 ? 8 : dtype == ED_F32 ? 4 : dtype == ED_C128 ? 16 : 8;
   const size_t xs_bytes = al16(es * ((size_t)p->n_slots + 1));
-  const bool rows = p->n_slices && r0 == 0 && r1 == B->D && xs_bytes >= kRowOrderMinBytes;
+  const bool rows = p->n_slices && r0 == 0 && r1 == B->D && xs_bytes >= (p->rt_w > p->rt_wa ? kRowOrderMinBytes : kRowOrderMinBytesAcross);
   PairParams P{};
   P.n_classes = B->n_classes;
   int words = 0;

@@ -351,6 +351,37 @@ __global__ void __launch_bounds__(kThreads, 4) update_kernel(VecSet S, const dou
   block_sum_store(nrm, partial, blockIdx.x);
 }
 
+// w <- w - c_0 u_0 - c_1 u_1 (u_1 may be null) as update_kernel does, for the local sweep: one row
+// per thread and iteration on a grid that fills the SMs' warps (0.20 ms on the 6x6 sector in
+// fp64 against 0.54 for update_kernel's four blocks of two rows per thread)
+template <typename V>
+__global__ void __launch_bounds__(kThreads) local_update_kernel(const V *u0, const V *u1, const double *c, V *w, V *wlo,
+                                                                int64_t n, double *partial) {
+  using A = typename Rv<V>::A;
+  constexpr bool kF = std::is_same<A, float>::value;
+  constexpr int P = Rv<V>::cplx ? 2 : 1;
+  double cs[2 * P];
+  float cf[4 * P];
+#pragma unroll
+  for (int t = 0; t < 2 * P; t++) {
+    cs[t] = t < P || u1 ? c[t] : 0.0;
+    if constexpr (kF) df_split(cs[t], cf[2 * t], cf[2 * t + 1]);
+  }
+  float nh = 0.f, nl = 0.f;
+  double nrm = 0.0;
+  for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kThreads) {
+    Row<V> R = row_load<V>(w, wlo, i);
+    const V a0 = u0[i];
+    V a1 = zero_v<V>();
+    if (u1) a1 = u1[i];
+    row_sub<V>(R, cs, cf, 0, a0);
+    if (u1) row_sub<V>(R, cs, cf, 1, a1);
+    row_store<V>(R, w, wlo, i, nh, nl, nrm);
+  }
+  if constexpr (kF) nrm = df_value(nh, nl);
+  block_sum_store(nrm, partial, blockIdx.x);
+}
+
 // psi = sum_k s_k u_k (real coefficients: the tridiagonal matrix is real symmetric)
 template <typename V>
 __global__ void __launch_bounds__(kThreads) combine_kernel(VecSet S, const double *s, V *psi,
@@ -448,6 +479,18 @@ int ed_launch_reorth_sweep(const ed_basis *B, void *w, const void *base, const v
     coef_kernel<<<m * P, kThreads, 0, st>>>(partial, grid, c);
     ED_CK(cudaGetLastError());
     update_kernel<V><<<grid, kThreads, smem_upd, st>>>(S, c, (V *)w, (V *)wlo, B->D, partial);
+    ED_CK(cudaGetLastError());
+  });
+  return ED_OK;
+}
+
+int ed_launch_local_sweep(const ed_basis *B, void *w, const void *v, const void *vprev, int dtype,
+                          double *partial, int nblk, double *c, cudaStream_t st, void *wlo) {
+  const int P = dtype == ED_C128 || dtype == ED_C64 ? 2 : 1;
+  coef_kernel<<<(vprev ? 2 : 1) * P, kThreads, 0, st>>>(partial, nblk, c);
+  ED_CK(cudaGetLastError());
+  RO_DISPATCH(dtype, {
+    local_update_kernel<V><<<nblk, kThreads, 0, st>>>((const V *)v, (const V *)vprev, c, (V *)w, (V *)wlo, B->D, partial);
     ED_CK(cudaGetLastError());
   });
   return ED_OK;

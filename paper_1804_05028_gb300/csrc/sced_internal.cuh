@@ -368,11 +368,17 @@ int ed_launch_dot(const ed_basis *B, const void *x, const void *y, int dtype, do
 // (w, wlo) <- (w + wlo) - a v - b vprev, ||w + wlo||^2 partials; wlo (fp32 vectors, may
 // be null) holds the low words of w: on entry those of the product (ed_launch_apply's
 // ylo), on exit those of the update; with part, a is the sum of its n_part partials (device),
-// also stored to a_out
+// also stored to a_out; with dots, the block partials of <v, w> and <vprev, w> of the updated w
+// go there, [vector][re, im][block]
 int ed_launch_axpy_norm(const ed_basis *B, void *w, const void *v, const void *vprev, double a,
                         double b, int dtype, double *partial, int nblk, cudaStream_t st,
                         void *wlo = nullptr, const double *part = nullptr, int n_part = 0,
-                        double *a_out = nullptr);
+                        double *a_out = nullptr, double *dots = nullptr);
+// one sweep of w against v and vprev (may be null) from the block partials of <v, w> and
+// <vprev, w> that ed_launch_axpy_norm left in partial (its dots); coefficients to c, ||w||^2
+// partials to partial[0, nblk)
+int ed_launch_local_sweep(const ed_basis *B, void *w, const void *v, const void *vprev, int dtype,
+                          double *partial, int nblk, double *c, cudaStream_t st, void *wlo);
 int ed_launch_step_scalars(const double *alpha, const double *corr0, const double *corr1, const double *part,
                            int n_part, double *out, cudaStream_t st);
 // v <- s (v + vlo), rounded once (vlo: fp32 vectors, may be null)
