@@ -243,7 +243,7 @@ def bench_batch(ed, torch, steps: int):
     out = {"workload": "square25 J1-J2 (J2=0.3), 572 sectors, one launch", "sectors": len(bases),
            "dim_total": int(sum(B.dim for B in bases)), "nonzeros_per_product": nnz,
            "build_s": build_s,
-           "l2": "inputs larger than L2: 6 whole-lattice tables of 268 MB each, basis %d MB"
+           "l2": "inputs larger than L2: 6 whole-lattice tables of 268 MB and 134 MB each, basis %d MB"
                  % (sum(d for d, _, _ in per) * 8 >> 20)}
     g = torch.Generator(device="cuda").manual_seed(1804)
     nz = [B for B in bases if B.dim]
@@ -440,9 +440,9 @@ def bench_sector(ed, torch, workload, p, steps, warmup, ctx, accuracy=True, full
                          "alg_bytes_per_launch": ab,
                          "sector_bytes_per_launch": sector_bytes(D, n_off, vb)},
             "roofline_issue": issue,
-            # per step: expansion of x and product, three-term update, scale, the local
-            # sweep's multi-dot, coefficient reduction and update, and the step's scalars
-            "gpu_launches": 8 * steps + 2,
+            # per step: expansion of x, product, three-term update (with the local sweep's
+            # dots), coefficient reduction, the sweep's update, the step's scalars, scale
+            "gpu_launches": 7 * steps + 2,
         }
         del work
 

@@ -7,7 +7,9 @@
 // sublattice coding (Alg. 2), s_j is located in Basis through Limits (Sec. IV), and
 // y_i += (J_c/2) chi(h) sqrt(|Stab_j|/|Stab_i|) x_j -- the conjugate-transposed form
 // of the push of Alg. 4, exact because H is Hermitian.  Each y_i is written once:
-// no atomics, no inter-block communication, fixed summation order.
+// no atomics, no inter-block communication, fixed summation order.  ed_launch_apply picks the
+// kernel: coset arithmetic (pair.cu), else the two-level search (apply_fast.cu), else the
+// search of Alg. 2 as printed (apply_h_kernel here).
 #include "sced_internal.cuh"
 #include "dfloat.cuh"
 #include <cstdlib>
@@ -490,9 +492,15 @@ int ed_launch_apply(const ed_basis *B, const double *J, const double *Jz, const 
                     void *y, int dtype, int64_t r0, int64_t r1, double *partial,
                     cudaStream_t st, int mode, void *ylo) {
   if (r1 <= r0) return ED_OK;
-  // The coset-arithmetic product expands the whole of x first (a pass over the slots, about
-  // 1/20 of a whole product): ranges below 1/16 of the rows go to the search kernel.
-  if (B->pair && (r1 - r0) >= B->D / 16) {
+  // The coset-arithmetic product expands the whole of x first, the search kernels have nothing
+  // to prepare but take longer per row.  Measured (fp32 vectors, ranges of D/17, D/128 and
+  // D/1024 rows, coset arithmetic against search): 6x6 sector, 3.2e7 states, whose xs stays
+  // mostly in L2, 0.94, 0.35, 0.28 against 3.95, 0.74, 0.40 ms; 40 sites, 8.6e8 states, 53, 23,
+  // 19 against 45, 6.2, 0.85 ms, equal near D/9; so all but the narrowest ranges up to some
+  // 3.3e7 states and ranges towards 1/8 of the rows above.  On 810 states 25 rows take 16
+  // against 20 us and 12 rows 16 against 14 us.
+  const int64_t n = r1 - r0;
+  if (B->pair && n >= 16 && n + (1 << 22) >= B->D / 8) {
     bool done = false;
     const int rc = ed_launch_apply_pair(B, J, Jz, x, y, dtype, r0, r1, partial, st, mode, ylo, &done);
     if (rc != ED_ERR_UNSUPPORTED) return rc;

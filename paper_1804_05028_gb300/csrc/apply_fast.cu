@@ -1,4 +1,7 @@
-// apply_fast.cu -- the row-pull product y = H x with a two-level representative search.
+// apply_fast.cu -- the row-pull product y = H x with a two-level representative search.  It
+// serves the sectors and calls that the coset-arithmetic product (pair.cu) does not take:
+// splits without two stable halves, tables or scratch that do not fit, and narrow ranges of
+// rows (the rule in ed_launch_apply); and it finds the representatives of that product's slots.
 //
 // Two-level search.  In Alg. 2 of arXiv:1804.05028 the candidates of a minimal block Y
 // are Sym_Y(s_Y) = K_R h: the coset of the stabiliser K_R = {k in G_0 : k R = R} of
@@ -12,7 +15,7 @@
 // character check are exact, as in the single-level search.
 //
 // Two kernels share the search:
-//   apply_tile_kernel  the product: a warp owns 32 consecutive rows and resolves their
+//   apply_tile_kernel  y = H x: a warp owns 32 consecutive rows and resolves their
 //                      exchange terms 32 at a time from term lists in shared memory (see
 //                      the comment above tile_round); the index of a representative is
 //                      one ranked Limits record (first index + popcount of a bitmap).

@@ -29,12 +29,17 @@
 // any of the equivalent choices of h gives the right term and no case is treated apart.
 // Slots whose configuration has another S^z or a vanishing projection hold 0.
 //
-// What a term costs: two half-table loads (L1/L2), one byte and one word from shared memory,
-// one gather of xs, and about 40 instructions; the two-level search it replaces executed
-// about 600 and 10 dependent loads (62.7 ms per product on the 3.2e7-state 6x6 sector, issue
-// bound).  One lane owns one row: without data-dependent searches the lanes of a warp differ
-// only in their number of antiparallel bonds.  Every y_i is written once, no atomics, fixed
-// summation order.
+// What a term costs: two half-table entries, one byte and one word from shared memory and one
+// gather of xs, 70 thread instructions in all on the 6x6 sector; the two-level search executed
+// 596 and 10 dependent loads.  One lane owns one row: without data-dependent searches the lanes
+// of a warp differ only in their number of antiparallel bonds.  Every y_i is written once, no
+// atomics, fixed summation order.
+//
+// Measured (GB300, per product, against the search kernels): 6x6 sector, 3.2e7 rows, fp32
+// 62.8 -> 8.05 ms, fp64 64.1 -> 9.6 ms; 40 sites, 8.6e8 rows, fp32 841 -> 179 ms; 2.6e6 complex
+// fp64 rows 9.8 -> 1.27 ms.  pair_rows_kernel is held by several limits at once: of their peaks
+// the L1 data pipe 60 to 70%, the requests to L2 45 to 65%, instruction issue 55% (DRAM 10%);
+// every term across the halves is one 32-byte sector from L2.
 #include "sced_internal.cuh"
 #include "dfloat.cuh"
 #include <algorithm>
@@ -113,7 +118,7 @@ struct PairParams {
   const uint32_t *row_i;         // basis index
   const uint16_t *row_m;         // weight of the row's configuration (meta of its slot)
   const double2 *rw;             // conj(chi) / sqrt(t) per weight
-  const uint32_t *rt;            // tables of the row order, RowTables, staged as they are
+  const uint32_t *rt;            // tables of the row order, staged as they are
   uint32_t rt_words;
   int kw[ED_MAXCLS][5];          // words of class c: across [0], [1); within A [1], [2); within up [3], [4)
   uint32_t n_w, n_wa, n_hnib, m; // words, those across or within A (the first ones)
@@ -125,13 +130,18 @@ struct PairParams {
   uint32_t *next;                // work counter, zeroed by expand_kernel
 };
 
-constexpr int kThreads = 512;
+constexpr int kThreads = 512;          // pair_kernel
 constexpr int kMinBlocks = 2;
-constexpr int kRowThreads = 1024;      // pair_rows_kernel
+// pair_rows_kernel: one block of 32 warps per SM, so that the shared tables are staged once and
+// all warps of the SM work on neighbouring rows (6x6 fp32 in ms, before the last steps: 9.5;
+// 2 x 512 threads 10.8, 2 x 640 10.4, 3 x 512 18.3).  Terms per round, two rounds in flight, by
+// the size of a vector entry (4 bytes: 1 / 2 / 3 / 4 terms 9.9 / 9.1 / 9.3 / 9.8 ms; 8 bytes: fp64
+// 1 / 2 terms 9.6 / 9.9 ms; 16 bytes in one round: 2 / 3 terms 40 / 43 ms on 6.4e7 rows)
+constexpr int kRowThreads = 1024;
 constexpr int kRowBlocks = 1;
 constexpr int kRowU = 2;
-constexpr int kRowU16 = 2;
 constexpr int kRowU8 = 1;
+constexpr int kRowU16 = 2;
 // and rows: below 2^21 a product is a few waves of blocks, and the row tables (10 bytes per row)
 // are not made
 constexpr int64_t kRowOrderMinDim = 1 << 21;
@@ -529,8 +539,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) pair_kernel(const __grid
 // class(A') stays the lower one the gather falls into that class's block of slots.  The GPU
 // works on one or two lower classes at a time, whose blocks (10 to 20 MB on that sector) stay
 // in L2.  That needs all SMs at the same place: blocks take slices from a counter (with a fixed
-// stride the SMs drift apart by dozens of classes, and the DRAM traffic was 120 GB instead
-// of 11).
+// stride the SMs drift apart by dozens of classes: 120 GB of DRAM reads per product, now 4).
 //
 // In slot order the rows of one upper class c lie together: b = k R(c), all k.  Terms within a
 // half keep the other class: within A the 32 rows of a warp gather from one cluster of K slots
@@ -1000,7 +1009,7 @@ struct PairPlan {
   uint32_t bmask_hi = 0, bmask = 0;
   uint32_t n_cls = 0, K = 0, h0 = 0, sel_off = 0, mult_bytes = 0, n_slots = 0;
   uint32_t n_slices = 0, ubase = 0, n_ucls = 0;
-  // tables of the row order (RowTables)
+  // tables of the row order
   int kw[ED_MAXCLS][5] = {};
   bool no_swap = false, any_flip = false;
   uint32_t rt_words = 0, rt_w = 0, rt_wa = 0, n_hnib = 0, rt_f = 0, rt_pos = 0, rt_nibA = 0, rt_nibB = 0, rt_img = 0, rt_left = 0;
