@@ -440,9 +440,9 @@ def bench_sector(ed, torch, workload, p, steps, warmup, ctx, accuracy=True, full
                          "alg_bytes_per_launch": ab,
                          "sector_bytes_per_launch": sector_bytes(D, n_off, vb)},
             "roofline_issue": issue,
-            # per step: expansion of x, product, three-term update (with the local sweep's
-            # dots), coefficient reduction, the sweep's update, the step's scalars, scale
-            "gpu_launches": 7 * steps + 2,
+            # per step: expansion of x, product, its sums by chunk, three-term update (with the
+            # local sweep's dots), coefficient reduction, the sweep's update, scalars, scale
+            "gpu_launches": 8 * steps + 2,
         }
         del work
 

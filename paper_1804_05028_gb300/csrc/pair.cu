@@ -104,6 +104,8 @@ struct PairParams {
   void *ylo;
   int64_t r0, r1;
   double *partial;
+  double *chunk_part;            // pair_rows_kernel: the sums of every chunk, [value][n_sums]
+  uint32_t n_chunks, n_sums;
   uint32_t off_off, off_mult, off_bond, off_nib, off_rs, off_chi, off_mask, smem_bytes;
   // rows in slot order: pair_rows_kernel
   const uint32_t *low;           // [n_cls] representative of the lower class
@@ -138,6 +140,7 @@ constexpr int kMinBlocks = 2;
 // the size of a vector entry (4 bytes: 1 / 2 / 3 / 4 terms 9.9 / 9.1 / 9.3 / 9.8 ms; 8 bytes: fp64
 // 1 / 2 terms 9.6 / 9.9 ms; 16 bytes in one round: 2 / 3 terms 40 / 43 ms on 6.4e7 rows)
 constexpr int kRowThreads = 1024;
+constexpr int kSumWarps = 4;           // warps that sum a chunk's <x, y>
 constexpr int kRowBlocks = 1;
 constexpr int kRowU = 2;
 constexpr int kRowU8 = 1;
@@ -410,6 +413,11 @@ __device__ __forceinline__ void pair_store(const PairParams &P, const V *x, V *y
   }
 }
 
+__device__ __forceinline__ double warp_sum(double d) {
+  for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xFFFFFFFFu, d, o);
+  return d;
+}
+
 // per-block sums of n values per thread (kMode 0: <x, y>, real and imaginary part; kMode 1: the
 // classes) in a fixed order
 template <int kT>
@@ -418,14 +426,12 @@ __device__ __forceinline__ void pair_dot(const PairParams &P, const double *v, i
   __shared__ double red[kT / 32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   for (int part = 0; part < n; part++) {
-    double d = v[part];
-    for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xFFFFFFFFu, d, o);
+    double d = warp_sum(v[part]);
     __syncthreads();
     if (lane == 0) red[wid] = d;
     __syncthreads();
     if (wid == 0) {
-      d = lane < kT / 32 ? red[lane] : 0.0;
-      for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xFFFFFFFFu, d, o);
+      d = warp_sum(lane < kT / 32 ? red[lane] : 0.0);
       if (lane == 0) P.partial[part * gridDim.x + blockIdx.x] = d;
     }
   }
@@ -578,14 +584,60 @@ __global__ void __launch_bounds__(kRowThreads, kRowBlocks) pair_rows_kernel(cons
   uint32_t cur = 0xFFFFFFFFu, e_low = 0, off_low = 0;
   bool st_in = false, st_across = false;
   __shared__ uint32_t chunk_s;
+  constexpr int kDots = kC ? 2 : 1;
+  __shared__ double red[kMode == 1 ? ED_MAXCLS : 1][kRowThreads / 32];
+  uint32_t chunk = 0xFFFFFFFFu;
   for (;;) {
+    // which block works on a chunk differs from call to call, so <x, y> is summed by chunk:
+    // the same bits every time.  The lanes' shares go through the masks' words to kSumWarps
+    // warps: fp64 additions are what this costs (6x6 sector, fp32, product with <x, y>: 8.36 ms;
+    // 8.24 with one sum per thread over whatever chunks it gets, 8.57 with every warp's 32 lanes
+    // summed by shuffles)
+    const bool sums = P.partial && chunk != 0xFFFFFFFFu;
+    if (sums) {
+      if constexpr (kMode == 1) {
+#pragma unroll
+        for (int part = 0; part < ED_MAXCLS; part++) {
+          if (part >= P.n_classes) break;
+          const double d = warp_sum(dot[part]);
+          if (lane == 0) red[part][wid] = d;
+          dot[part] = 0.0;
+        }
+      } else {
+#pragma unroll
+        for (int part = 0; part < kDots; part++) {
+          mask_s[2 * part * kRowThreads] = (uint32_t)__double2loint(dot[part]);
+          mask_s[(2 * part + 1) * kRowThreads] = (uint32_t)__double2hiint(dot[part]);
+          dot[part] = 0.0;
+        }
+      }
+    }
     // taken when it is worked on: a chunk taken ahead spreads the blocks over more classes
     // (fp64 on the 6x6 sector 10.5 -> 11.0 ms)
     __syncthreads();
     if (threadIdx.x == 0) chunk_s = atomicAdd(P.next, 1u);
+    if constexpr (kMode == 1) {
+      if (sums && wid == 1) {
+        for (int part = 0; part < P.n_classes; part++) {
+          const double d = warp_sum(red[part][lane]);
+          if (lane == 0) P.chunk_part[(size_t)part * P.n_sums + chunk] = d;
+        }
+      }
+    } else if (sums && wid >= 1 && wid <= kSumWarps) {
+      constexpr int kRows = kRowThreads / kSumWarps;
+      const uint32_t *w = reinterpret_cast<const uint32_t *>(sm + P.off_mask) + (wid - 1) * kRows + lane;
+#pragma unroll
+      for (int part = 0; part < kDots; part++, w += 2 * kRowThreads) {
+        double d = 0.0;
+#pragma unroll
+        for (int q = 0; q < kRows; q += 32) d += __hiloint2double((int)w[kRowThreads + q], (int)w[q]);
+        d = warp_sum(d);
+        if (lane == 0) P.chunk_part[(size_t)part * P.n_sums + chunk * kSumWarps + wid - 1] = d;
+      }
+    }
     __syncthreads();
-    const uint32_t chunk = chunk_s;
-    if (chunk * (kRowThreads / 32) >= P.n_slices) break;
+    chunk = chunk_s;
+    if (chunk >= P.n_chunks) break;
     const uint32_t sl = chunk * (kRowThreads / 32) + wid;
     if (sl >= P.n_slices) continue;
     uint32_t lo = __ldg(P.chunk_cls + chunk);   // the class of the chunk's first slice
@@ -774,7 +826,18 @@ __global__ void __launch_bounds__(kRowThreads, kRowBlocks) pair_rows_kernel(cons
     pair_store<V>(P, reinterpret_cast<const V *>(P.x), reinterpret_cast<V *>(P.y), (int64_t)__ldcs(P.row_i + r), diag,
                   kChi ? 1.0 : rw.x, row_re, row_im, dot[0], dot[1]);
   }
-  pair_dot<kRowThreads>(P, dot, kMode == 1 ? P.n_classes : kC ? 2 : 1);
+}
+
+// partial[value][block] from pair_rows_kernel's sums by chunk
+__global__ void __launch_bounds__(256) chunk_sum_kernel(const __grid_constant__ PairParams P, int n) {
+  double v[ED_MAXCLS] = {};
+#pragma unroll
+  for (int part = 0; part < ED_MAXCLS; part++) {
+    if (part >= n) break;
+    for (uint32_t c = blockIdx.x * 256 + threadIdx.x; c < P.n_sums; c += gridDim.x * 256)
+      v[part] += P.chunk_part[(size_t)part * P.n_sums + c];
+  }
+  pair_dot<256>(P, v, n);
 }
 
 // xs[p] = w(meta[p]) x[idx[p]], w = chi sqrt(t); meta 0 is w = 1.  fp32 vectors take the weights
@@ -1653,11 +1716,15 @@ int launch_pair_t(const ed_basis *B, PairParams &P, bool rows, cudaStream_t st) 
   const int need = per_sm * ((int)P.smem_bytes + 1536);
   const int pct = std::min(100, (need * 100 + 228 * 1024 - 1) / (228 * 1024));
   ED_CK(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, pct));
-  const int64_t blocks = rows ? ((int64_t)P.n_slices + threads / 32 - 1) / (threads / 32) : (P.r1 - P.r0 + threads - 1) / threads;
+  const int64_t blocks = rows ? (int64_t)P.n_chunks : (P.r1 - P.r0 + threads - 1) / threads;
   const int grid = (int)std::min<int64_t>(blocks, (int64_t)B->sm_count * per_sm);
   B->last_apply_grid = grid;
   k<<<grid, threads, P.smem_bytes, st>>>(P);
   ED_CK(cudaGetLastError());
+  if (rows && P.partial) {
+    chunk_sum_kernel<<<grid, 256, 0, st>>>(P, kMode == 1 ? P.n_classes : Pv<V>::cplx ? 2 : 1);
+    ED_CK(cudaGetLastError());
+  }
   return ED_OK;
 }
 
@@ -1729,7 +1796,7 @@ int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, c
   put(P.off_chi, chi ? 16 * 1024 : 0);
   if (rows) {
     put(P.off_rt, 4 * (size_t)P.rt_words);
-    put(P.off_mask, 4 * (size_t)p->rt_across * kRowThreads);
+    put(P.off_mask, 4 * std::max<size_t>(p->rt_across, cplx ? 4 : 2) * kRowThreads);   // or a row's <x, y>
     P.n_ucls = p->n_ucls;
     P.n_tab = P.K >= 32 ? 2 : 0;   // 32 rows span two classes at most (without stabilisers)
     P.et_words = (uint32_t)(65 * p->rt_wa + P.n_tab * (32 * (p->rt_w - p->rt_wa) + p->m) + 3) / 4 * 4;
@@ -1745,13 +1812,18 @@ int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, c
   // calls on several streams or threads never share it; without memory for it the search
   // kernel takes the call
   const bool lo = dtype == ED_F32 && p->weights;
+  P.n_chunks = (p->n_slices + kRowThreads / 32 - 1) / (kRowThreads / 32);
+  const size_t lo_bytes = lo ? al16(4 * ((size_t)p->n_slots + 1)) : 0;
+  P.n_sums = P.n_chunks * (mode == 1 ? 1 : kSumWarps);
+  const size_t n_sums = !rows || !partial ? 0 : (mode == 1 ? (size_t)B->n_classes : cplx ? 2 : 1) * P.n_sums;
   char *ws = nullptr;
-  if (cudaMallocFromPoolAsync((void **)&ws, 16 + xs_bytes + (lo ? 4 * ((size_t)p->n_slots + 1) : 0), p->pool, st) != cudaSuccess) {
+  if (cudaMallocFromPoolAsync((void **)&ws, 16 + xs_bytes + lo_bytes + 8 * n_sums, p->pool, st) != cudaSuccess) {
     cudaGetLastError();
     return ED_ERR_UNSUPPORTED;
   }
   float *xslo = lo ? reinterpret_cast<float *>(ws + xs_bytes + 16) : nullptr;
   P.next = reinterpret_cast<uint32_t *>(ws + xs_bytes);
+  P.chunk_part = reinterpret_cast<double *>(ws + 16 + xs_bytes + lo_bytes);
   const int eg = (int)std::min<uint32_t>((p->n_slots + 255) / 256, (uint32_t)B->sm_count * 16);
   P.xs = ws;
   P.xslo = xslo;

@@ -110,6 +110,10 @@ def test_row_order(p):
         mid = B.apply_H_rows(x, D // 2, D // 2 + 1001)      # a narrow range, x expanded whole
         assert (y[D // 2:D // 2 + 1001] - mid).abs().max() <= tol * ref.abs().max()
         got = B.expect_classes(x)
+        # blocks take the rows in any order, the sums come out the same
+        assert all(np.array_equal(got, B.expect_classes(x)) for _ in range(3))
+        runs = [B.lanczos(dtype=dt, fixed_steps=4) for _ in range(3)] if dt.is_complex != B.is_real else []
+        assert all(np.array_equal(r["alpha"], runs[0]["alpha"]) and np.array_equal(r["beta"], runs[0]["beta"]) for r in runs)
         xd = x.to(torch.complex128)
         for c in range(p.n_classes):
             J = [0.0] * p.n_classes
