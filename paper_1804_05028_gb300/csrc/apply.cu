@@ -314,10 +314,12 @@ template <> struct Dot2<float2> {
 
 // With dots (may be null) also <v, w> and <vprev, w> of the updated w: the local sweep that
 // follows would otherwise read all three vectors once more for them (a pass of 0.48 ms on the
-// 6x6 sector in fp64).  With part (may be null) a is not given but the sum of its n_part block partials of <v, w>,
-// added up by every block in the same order and stored to a_out: the host need not wait for
-// the product before it launches the update.
-template <typename V>
+// 6x6 sector in fp64); kDots tells at compile time (fp32 0.216 -> 0.188 ms, fp64 0.303 -> 0.254,
+// without dots 0.207 -> 0.151 and 0.296 -> 0.203).  With part (may be null) a is not given
+// but the sum of its n_part block partials of <v, w>, added up by every block in the same
+// order and stored to a_out: the host need not wait for the product before it launches the
+// update.
+template <typename V, bool kDots>
 __global__ void __launch_bounds__(256) axpy_norm_kernel(V *w, const V *v, const V *vprev, double a, double b,
                                                         int64_t n, double *partial, V *wlo,
                                                         const double *part, int n_part, double *a_out,
@@ -342,64 +344,76 @@ __global__ void __launch_bounds__(256) axpy_norm_kernel(V *w, const V *v, const 
     df_split(a, ah, al);
     df_split(b, bh, bl);
   }
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
+  struct Row { V w, l, v, p; };
+  auto load = [&](int64_t i) {
+    Row r = {};
+    r.w = w[i];
+    r.v = v[i];
+    if (kF && wlo) r.l = wlo[i];
+    if (vprev) r.p = vprev[i];
+    return r;
+  };
+  auto update = [&](int64_t i, const Row &in) {
     if constexpr (Vt<V>::cplx && kF) {
       // a and b are real (Hermitian tridiagonal)
-      const V w0 = w[i], v0 = v[i];
-      float rh = w0.x, rl = 0.f, ih = w0.y, il = 0.f;
-      if (wlo) { const V l0 = wlo[i]; rl = l0.x; il = l0.y; }
-      df_sub_scaled(rh, rl, ah, al, v0.x);
-      df_sub_scaled(ih, il, ah, al, v0.y);
-      V p0;
-      p0.x = p0.y = 0.f;
+      float rh = in.w.x, rl = in.l.x, ih = in.w.y, il = in.l.y;
+      df_sub_scaled(rh, rl, ah, al, in.v.x);
+      df_sub_scaled(ih, il, ah, al, in.v.y);
       if (vprev) {
-        p0 = vprev[i];
-        df_sub_scaled(rh, rl, bh, bl, p0.x);
-        df_sub_scaled(ih, il, bh, bl, p0.y);
+        df_sub_scaled(rh, rl, bh, bl, in.p.x);
+        df_sub_scaled(ih, il, bh, bl, in.p.y);
       }
       V o, r;
       df_store(rh, rl, o.x, r.x);
       df_store(ih, il, o.y, r.y);
       w[i] = o;
       if (wlo) wlo[i] = r; else { r.x = 0.f; r.y = 0.f; }
-      if (dots) { dv.add(v0, o, r); dp.add(p0, o, r); }
-      df_add_sq(nh, nl, o.x, r.x);
-      df_add_sq(nh, nl, o.y, r.y);
+      if constexpr (kDots) { dv.add(in.v, o, r); dp.add(in.p, o, r); }
+      else { df_add_sq(nh, nl, o.x, r.x); df_add_sq(nh, nl, o.y, r.y); }
     } else if constexpr (kF) {
-      float hi = w[i], lo = wlo ? wlo[i] : 0.f;
-      const float v0 = v[i], p0 = vprev ? vprev[i] : 0.f;
-      df_sub_scaled(hi, lo, ah, al, v0);
-      if (vprev) df_sub_scaled(hi, lo, bh, bl, p0);
+      float hi = in.w, lo = in.l;
+      df_sub_scaled(hi, lo, ah, al, in.v);
+      if (vprev) df_sub_scaled(hi, lo, bh, bl, in.p);
       float o, r;
       df_store(hi, lo, o, r);
       w[i] = o;
       if (wlo) wlo[i] = r; else r = 0.f;
-      if (dots) { dv.add(v0, o, r); dp.add(p0, o, r); }
-      df_add_sq(nh, nl, o, r);
+      if constexpr (kDots) { dv.add(in.v, o, r); dp.add(in.p, o, r); }
+      else df_add_sq(nh, nl, o, r);
     } else if constexpr (Vt<V>::cplx) {
-      const V w0 = w[i], v0 = v[i];
-      V p0;
-      p0.x = p0.y = 0;
-      double wr = (double)w0.x - a * (double)v0.x;
-      double wi = (double)w0.y - a * (double)v0.y;
-      if (vprev) { p0 = vprev[i]; wr -= b * (double)p0.x; wi -= b * (double)p0.y; }
+      double wr = (double)in.w.x - a * (double)in.v.x;
+      double wi = (double)in.w.y - a * (double)in.v.y;
+      if (vprev) { wr -= b * (double)in.p.x; wi -= b * (double)in.p.y; }
       V o; o.x = (A)wr; o.y = (A)wi;
       w[i] = o;
-      if (dots) { dv.add(v0, o, o); dp.add(p0, o, o); }
-      acc += (double)o.x * o.x + (double)o.y * o.y;
+      if constexpr (kDots) { dv.add(in.v, o, o); dp.add(in.p, o, o); }
+      else acc += (double)o.x * o.x + (double)o.y * o.y;
     } else {
-      const V v0 = v[i], p0 = vprev ? vprev[i] : V(0);
-      double t = (double)w[i] - a * (double)v0;
-      if (vprev) t -= b * (double)p0;
+      double t = (double)in.w - a * (double)in.v;
+      if (vprev) t -= b * (double)in.p;
       const A o = (A)t;
       w[i] = o;
-      if (dots) { dv.add(v0, o, 0); dp.add(p0, o, 0); }
-      else acc += (double)o * (double)o;   // the sweep that follows takes the norm
+      if constexpr (kDots) { dv.add(in.v, o, 0); dp.add(in.p, o, 0); }
+      else acc += (double)o * (double)o;   // with dots the sweep that follows takes the norm
+    }
+  };
+  // the loads of kU rows of a thread go out before the first row's arithmetic; the rows keep
+  // their order.  Two help fp32 with dots (6x6 sector 0.188 -> 0.164 ms), whose double-float
+  // arithmetic waits for the loads; fp64 rows, held by the fp64 pipe, lose (0.254 -> 0.347)
+  constexpr int kU = kDots && sizeof(V) == 4 ? 2 : 1;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += kU * stride) {
+    const Row r0 = load(i);
+    if (kU == 2 && i + stride < n) {
+      const Row r1 = load(i + stride);
+      update(i, r0);
+      update(i + stride, r1);
+    } else {
+      update(i, r0);
     }
   }
   if constexpr (kF) acc = df_value(nh, nl);
-  if (dots) {
+  if constexpr (kDots) {
     constexpr int P = Vt<V>::cplx ? 2 : 1;
     block_reduce_store<double>(dv.real(), dots, blockIdx.x);
     if (P == 2) block_reduce_store<double>(dv.imag(), dots, gridDim.x + blockIdx.x);
@@ -625,9 +639,8 @@ int ed_launch_dot(const ed_basis *B, const void *x, const void *y, int dtype, do
 int ed_launch_axpy_norm(const ed_basis *B, void *w, const void *v, const void *vprev, double a,
                         double b, int dtype, double *partial, int nblk, cudaStream_t st,
                         void *wlo, const double *part, int n_part, double *a_out, double *dots) {
-  ED_DISPATCH(dtype, (axpy_norm_kernel<V><<<nblk, 256, 0, st>>>((V *)w, (const V *)v,
-                                                                (const V *)vprev, a, b, B->D,
-                                                                partial, (V *)wlo, part, n_part, a_out, dots)));
+  ED_DISPATCH(dtype, ((dots ? axpy_norm_kernel<V, true> : axpy_norm_kernel<V, false>)<<<nblk, 256, 0, st>>>(
+                         (V *)w, (const V *)v, (const V *)vprev, a, b, B->D, partial, (V *)wlo, part, n_part, a_out, dots)));
   ED_CK(cudaGetLastError());
   return ED_OK;
 }
