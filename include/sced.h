@@ -164,12 +164,13 @@ int ed_find_rep(const ed_basis *basis, const uint64_t *states, int64_t n, int32_
  * ed_apply_H -- y = H x on the symmetry-adapted basis, matrix-free (Sec. IV,
  * Eqs. 12-17 restated as a row-wise pull): for each row i, its diagonal, then for
  * each antiparallel bond the exchanged configuration, its representative by sublattice
- * coding (Alg. 2), its index through Limits (the bucket's first index plus the rank of
- * the postfix in the bucket's bitmap, or a binary search in the bucket), and
- * y_i += (J/2) chi(h) sqrt(|Stab_j|/|Stab_i|) x_j.  No atomics; every y_i is written
- * once.  Deterministic: the same call gives the same bits.  The terms of 32
- * consecutive rows are summed together, so a row range that starts elsewhere
- * (ed_apply_H_rows, the chunks of ed_apply_H_host) may differ in the last bit.
+ * coding, the representative's x_j, and y_i += (J/2) chi(h) sqrt(|Stab_j|/|Stab_i|) x_j.
+ * Sectors with two stable halves name the orbit by coset arithmetic on the halves and read
+ * x from a copy in the order of those names (scratch from a stream-ordered pool of the
+ * basis, taken and given back within the call); the others search (Alg. 2) and look the
+ * index up in Limits.  Every y_i is written once.  Deterministic: the same call gives the
+ * same bits.  Whole products and row ranges (ed_apply_H_rows) may sum a row's terms in
+ * different orders and differ in the last bit.
  *   J, Jz: HOST arrays [n_classes].
  *   x, y: DEVICE arrays of dim elements of `dtype` (ED_F64 or ED_F32; the complex types
  *   for sectors with complex characters), caller-owned, must not overlap.
@@ -191,10 +192,10 @@ int ed_apply_H_rows(const ed_basis *basis, const double *J, const double *Jz, co
 
 /*
  * ed_apply_H_host -- ed_apply_H on HOST arrays x, y (dim elements of dtype): copies x
- * to device staging buffers owned by the basis, runs the product, copies y back.  Above
- * 2^25 rows the product runs in up to 8 row chunks and each chunk of y is copied back
- * (on a stream of the basis) while the next one is computed; with pinned host arrays
- * the copies then overlap the product.  Synchronous.  Not safe to call concurrently on
+ * to device staging buffers owned by the basis, runs the product, copies y back.  Sectors
+ * without coset arithmetic (see ed_apply_H) and above 2^25 rows run the product in up to 8
+ * row chunks and copy each chunk of y back (on a stream of the basis) while the next one is
+ * computed; with pinned host arrays the copies then overlap the product.  Synchronous.  Not safe to call concurrently on
  * the same basis.
  */
 int ed_apply_H_host(ed_basis *basis, const double *J, const double *Jz, const void *x_host,

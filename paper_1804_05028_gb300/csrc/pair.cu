@@ -38,7 +38,8 @@
 // Measured (GB300, per product, against the search kernels): 6x6 sector, 3.2e7 rows, fp32
 // 62.8 -> 8.05 ms, fp64 64.1 -> 9.6 ms; 40 sites, 8.6e8 rows, fp32 841 -> 179 ms; 2.6e6 complex
 // fp64 rows 9.8 -> 1.27 ms.  pair_rows_kernel is held by several limits at once: of their peaks
-// the L1 data pipe 60 to 70%, the requests to L2 45 to 65%, instruction issue 55% (DRAM 10%);
+// the L1 data pipe 65 to 70%, instruction issue 44 to 60%, the requests to L2 36% (66% where
+// every term crosses the halves), DRAM 7 to 11%;
 // every term across the halves is one 32-byte sector from L2.
 #include "sced_internal.cuh"
 #include "dfloat.cuh"

@@ -18,6 +18,8 @@
 //                     groups of 8 vectors (one group per blockIdx.y)
 //   coef_kernel       c[k] = sum over blocks of partial[k][.], one block per k
 //   update_kernel     w -= sum_k c_k u_k, partial ||w||^2 per block
+//   local_update_kernel  the same for the local sweep (m <= 2), whose dots the three-term
+//                     update takes while w passes through it
 //   combine_kernel    psi = sum_k s_k u_k (the Ritz vector from a stored Krylov basis)
 #include "sced_internal.cuh"
 #include "dfloat.cuh"
