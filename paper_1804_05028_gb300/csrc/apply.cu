@@ -200,11 +200,16 @@ __global__ void __launch_bounds__(256) apply_h_kernel(const ApplyParams P) {
   }
 }
 
+// shared memory: up to kMaxStaged with the lookup tables, else whatever the group's norm and
+// character tables take, at most what a block can have (227 KB) beside block_reduce_store's
+constexpr size_t kMaxStaged = 200 * 1024;
+constexpr size_t kMaxLaunch = 227 * 1024 - 32 * sizeof(double);
+
 template <typename V, bool kStage, int kMode = 0>
 int launch_apply_t(const ApplyParams &P, int grid, cudaStream_t st) {
   auto k = apply_h_kernel<V, kStage, kMode>;
   if (P.smem_bytes > 48 * 1024)
-    ED_CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, P.smem_bytes));
+    if (const int rc = ed_allow_smem(k, kMaxLaunch)) return rc;
   k<<<grid, 256, P.smem_bytes, st>>>(P);
   ED_CK(cudaGetLastError());
   return ED_OK;
@@ -558,10 +563,9 @@ int ed_launch_apply(const ed_basis *B, const double *J, const double *Jz, const 
                            align16((size_t)B->nsym * B->nsub);
   const size_t rest = align16((size_t)B->n_bonds * 2) + align16((size_t)(B->nsym + 1) * 2 * abytes) +
                       align16((size_t)B->denom * 2 * abytes);
-  const size_t kMaxSmem = 200 * 1024;
   // a one-sublattice split reads the whole table from global memory and has no
   // Rep/Sym/dest tables to stage
-  P.stage_tables = (!B->T.full && tab_bytes + rest <= kMaxSmem) ? 1 : 0;
+  P.stage_tables = (!B->T.full && tab_bytes + rest <= kMaxStaged) ? 1 : 0;
   P.sym_list_bytes = (uint32_t)(B->sym_list_len * 2);
   if (P.stage_tables) {
     P.off_rep = (uint32_t)off; off += align16((size_t)B->nsub * nn * 4);

@@ -971,6 +971,10 @@ __global__ void __launch_bounds__(256) pair_slots_kernel(const TwoParams P, cons
 
 size_t a16(size_t x) { return (x + 15) & ~(size_t)15; }
 
+// Most shared memory of a block: the level-2 tables staged (with or without the term lists of
+// the tile kernel), or not.
+constexpr size_t smem_most(bool e2, bool tile) { return (e2 ? (tile ? 220 : 180) : 100) * 1024; }
+
 // Parameters and shared-memory layout; e2 = stage the level-2 tables in shared memory.
 int make_params(const ed_basis *B, const double *J, const double *Jz, bool e2, TwoParams &P,
                 int tile_warps = 0) {
@@ -1036,7 +1040,7 @@ int make_params(const ed_basis *B, const double *J, const double *Jz, bool e2, T
     put(P.off_tile, (size_t)tile_warps * kTileWarpBytes);
   }
   P.smem_bytes = (uint32_t)off;
-  if (off > (e2 ? (tile_warps ? 220 : 180) : 100) * 1024) return ED_ERR_UNSUPPORTED;
+  if (off > smem_most(e2, tile_warps > 0)) return ED_ERR_UNSUPPORTED;
   return ED_OK;
 }
 
@@ -1046,11 +1050,11 @@ template <typename V, int NSUB, int kMode = 0>
 int launch_t(const TwoParams &P, bool e2, int grid, cudaStream_t st) {
   if (e2) {
     auto k = apply_two_kernel<V, NSUB, true, kMode>;
-    ED_CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, P.smem_bytes));
+    if (const int rc = ed_allow_smem(k, smem_most(true, false))) return rc;
     k<<<grid, 1024, P.smem_bytes, st>>>(P);
   } else {
     auto k = apply_two_kernel<V, NSUB, false, kMode>;
-    ED_CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, P.smem_bytes));
+    if (const int rc = ed_allow_smem(k, smem_most(false, false))) return rc;
     // ask for just the shared memory of kMinBlocks resident blocks (plus the per-block
     // reserve); the rest of the SM's 256 KB stays L1 for the SymmetryAction and level-2
     // lines (about 1% faster than the default split)
@@ -1079,11 +1083,11 @@ template <typename V, int NSUB>
 int launch_tile_t(const TwoParams &P, bool e2, int grid, cudaStream_t st) {
   if (e2) {
     auto k = apply_tile_kernel<V, NSUB, true>;
-    ED_CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, P.smem_bytes));
+    if (const int rc = ed_allow_smem(k, smem_most(true, true))) return rc;
     k<<<grid, kTileThreadsE2, P.smem_bytes, st>>>(P);
   } else {
     auto k = apply_tile_kernel<V, NSUB, false>;
-    ED_CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, P.smem_bytes));
+    if (const int rc = ed_allow_smem(k, smem_most(false, true))) return rc;
     const int need = kTileMinBlocks * ((int)P.smem_bytes + 1536);
     const int pct = std::min(100, (need * 100 + 228 * 1024 - 1) / (228 * 1024));
     ED_CK(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, pct));
@@ -1184,7 +1188,7 @@ int ed_launch_find_rep_two(const ed_basis *B, const uint64_t *states, int64_t n,
 #define L2CASE(K, C)                                                                           \
   case K * 2 + C: {                                                                            \
     auto k = find_rep_two_kernel<K, C>;                                                        \
-    ED_CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, P.smem_bytes)); \
+    if (const int rc = ed_allow_smem(k, smem_most(C, false))) return rc; \
     k<<<grid, 256, P.smem_bytes, st>>>(P, B->I, states, n, rep, phase, stab, index);           \
     break;                                                                                     \
   }
@@ -1211,7 +1215,7 @@ int ed_launch_pair_slots(const ed_basis *B, const PairSlots &Q, cudaStream_t st)
 #define PSCASE(K, C)                                                                           \
   case K * 2 + C: {                                                                            \
     auto k = pair_slots_kernel<K, C>;                                                          \
-    ED_CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, P.smem_bytes)); \
+    if (const int rc = ed_allow_smem(k, smem_most(C, false))) return rc; \
     k<<<grid, 256, P.smem_bytes, st>>>(P, B->I, Q, B->n_up);                                   \
     break;                                                                                     \
   }

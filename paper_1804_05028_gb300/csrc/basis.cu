@@ -421,13 +421,14 @@ int ed_exclusive_scan(const uint32_t *in, uint64_t n, uint64_t *out, uint64_t *t
 
 int ed_build_full_table(const uint8_t *d_pbit, const uint8_t *d_flip, int N, int nsym,
                         uint64_t *out, cudaStream_t st) {
-  if ((size_t)nsym * N + nsym > 200 * 1024) return ed_fail(ED_ERR_UNSUPPORTED, "group too large for the one-block table");
+  constexpr size_t kMaxImages = 200 * 1024;
+  if ((size_t)nsym * N + nsym > kMaxImages) return ed_fail(ED_ERR_UNSUPPORTED, "group too large for the one-block table");
   // four high parts per block, one where the group's images would not fit in shared memory
   const bool four = sizeof(uint32_t) * 4 * (size_t)nsym <= 64 * 1024;
   const size_t sm = sizeof(uint32_t) * (size_t)nsym * (four ? 4 : 1);
   auto k = four ? full_table_kernel<4> : full_table_kernel<1>;
   if (sm > 48 * 1024)
-    ED_CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    if (const int rc = ed_allow_smem(k, kMaxImages)) return rc;
   int dev = 0, nsm = 0;
   ED_CK(cudaGetDevice(&dev));
   ED_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));

@@ -135,6 +135,8 @@ struct PairParams {
 
 constexpr int kThreads = 512;          // pair_kernel
 constexpr int kMinBlocks = 2;
+constexpr size_t kPairMaxSmem = 110 * 1024;   // a block's tables, two blocks per SM
+constexpr size_t kRowsMaxSmem = 200 * 1024;   // pair_rows_kernel, one block per SM
 // pair_rows_kernel: one block of 32 warps per SM, so that the shared tables are staged once and
 // all warps of the SM work on neighbouring rows (6x6 fp32 in ms, before the last steps: 9.5;
 // 2 x 512 threads 10.8, 2 x 640 10.4, 3 x 512 18.3).  Terms per round, two rounds in flight, by
@@ -1713,7 +1715,7 @@ template <typename V, bool kChi, bool kFlips, int kMode>
 int launch_pair_t(const ed_basis *B, PairParams &P, bool rows, cudaStream_t st) {
   auto k = rows ? pair_rows_kernel<V, kChi, kFlips, kMode> : pair_kernel<V, kChi, kFlips, kMode>;
   const int threads = rows ? kRowThreads : kThreads, per_sm = rows ? kRowBlocks : kMinBlocks;
-  ED_CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, P.smem_bytes));
+  if (const int rc = ed_allow_smem(k, rows ? kRowsMaxSmem : kPairMaxSmem)) return rc;
   const int need = per_sm * ((int)P.smem_bytes + 1536);
   const int pct = std::min(100, (need * 100 + 228 * 1024 - 1) / (228 * 1024));
   ED_CK(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, pct));
@@ -1808,7 +1810,7 @@ int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, c
     put(P.off_mask, 4 * (size_t)words * kThreads);
   }
   P.smem_bytes = (uint32_t)off;
-  if (off > (size_t)(rows ? 200 : 110) * 1024) return ED_ERR_UNSUPPORTED;
+  if (off > (rows ? kRowsMaxSmem : kPairMaxSmem)) return ED_ERR_UNSUPPORTED;
   // xs (and its remainders) for this call, from the basis's own pool in stream order, so
   // calls on several streams or threads never share it; without memory for it the search
   // kernel takes the call

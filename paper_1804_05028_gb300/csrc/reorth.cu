@@ -503,11 +503,12 @@ int ed_launch_combine(const ed_basis *B, void *psi, const void *base, int m, con
                       int dtype, cudaStream_t st) {
   const VecSet S = make_set(base, B->D, nullptr, nullptr, m);
   const size_t smem = 2 * sizeof(double) * (size_t)m;
-  if (smem > 200 * 1024) return ed_fail(ED_ERR_UNSUPPORTED, "too many vectors to combine");
+  constexpr size_t kMaxCombine = 200 * 1024;
+  if (smem > kMaxCombine) return ed_fail(ED_ERR_UNSUPPORTED, "too many vectors to combine");
   RO_DISPATCH(dtype, {
     auto k = combine_kernel<V>;
     if (smem > 48 * 1024)
-      ED_CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+      if (const int rc = ed_allow_smem(k, kMaxCombine)) return rc;
     k<<<ed_reorth_grid(B), kThreads, smem, st>>>(S, s, (V *)psi, B->D);
     ED_CK(cudaGetLastError());
   });

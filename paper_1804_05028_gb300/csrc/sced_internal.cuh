@@ -348,6 +348,16 @@ int ed_cuda_fail(cudaError_t e, const char *what);
     if (_e != cudaSuccess) return ed_cuda_fail(_e, #call);            \
   } while (0)
 
+// Lets kernel k take up to `most` bytes of dynamic shared memory, the largest that any of its
+// launches asks for.  The limit belongs to the kernel on the device, not to the launch that
+// follows: with the bytes of the call at hand a thread could lower it between another thread's
+// call here and its launch, which then fails.
+template <typename K>
+inline int ed_allow_smem(K k, size_t most) {
+  ED_CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
+  return ED_OK;
+}
+
 // kernels.cu / basis.cu entry points used by capi.cu
 int ed_build_device(ed_basis *B, cudaStream_t st, int bucket_target);
 // mode 0: y = H x (partial: optional <x, y> block partials); mode 1: per-class block partials

@@ -153,3 +153,34 @@ def test_streams_and_capture():
         torch.cuda.synchronize()
         assert torch.equal(y, r)
     del g
+
+
+def test_threads_with_other_table_sizes():
+    """Two host threads whose sectors take different amounts of shared memory in one kernel: what
+    one thread sets for its launch leaves the other's as it was."""
+    import threading
+    ps = [w.chain(8, 2, k=0, n_up=4), T(6, momentum=(0, 0), point_irrep=0, J2=0.5, n_sublat=4, n_up=4),   # coset arithmetic
+          w.chain(9, 3, k=0, n_up=4), w.chain(33, 3, k=0, n_up=3)]                                        # search
+    errors = []
+
+    def work(p):
+        try:
+            B = _basis(p)
+            x = _vec(B.dim, torch.float64, 5)
+            s = torch.cuda.Stream()
+            s.wait_stream(torch.cuda.default_stream())
+            y, ref = torch.empty_like(x), B.apply_H(x, stream=s)
+            for _ in range(3000):
+                B.apply_H(x, y, stream=s)
+            s.synchronize()
+            assert torch.equal(y, ref)
+        except Exception as e:   # noqa: BLE001 -- reported by the main thread
+            errors.append(e)
+
+    for pair in (ps[:2], ps[2:]):
+        threads = [threading.Thread(target=work, args=(p,)) for p in pair]
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join()
+    assert not errors, errors
