@@ -43,6 +43,7 @@
 // every term across the halves is one 32-byte sector from L2.
 #include "sced_internal.cuh"
 #include "dfloat.cuh"
+#include "pair_rules.h"
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -848,7 +849,7 @@ __global__ void __launch_bounds__(256) chunk_sum_kernel(const __grid_constant__ 
 // conversions kept the fp64 pipe 85% busy (0.54 ms on the 6x6 sector's 4.8e7 slots).  Real ones
 // keep the rounding's remainder in xslo, so that a weight sqrt(t) costs no precision.
 template <typename V>
-__global__ void __launch_bounds__(256) expand_kernel(const V *x, const uint32_t *idx, const uint16_t *meta,
+__global__ void __launch_bounds__(pair_rules::kExpandThreads) expand_kernel(const V *x, const uint32_t *idx, const uint16_t *meta,
                                                      const double2 *w, const float4 *wf, uint32_t n, V *xs,
                                                      float *xslo, uint32_t *next) {
   constexpr bool kF = sizeof(typename Pv<V>::A) == 4;
@@ -857,7 +858,8 @@ __global__ void __launch_bounds__(256) expand_kernel(const V *x, const uint32_t 
     if constexpr (Pv<V>::cplx) { xs[n].x = 0; xs[n].y = 0; } else { xs[n] = 0; }
     if (sizeof(V) == 4 && xslo) xslo[n] = 0.f;
   }
-  for (uint32_t p = blockIdx.x * 256 + threadIdx.x; p < n; p += gridDim.x * 256) {
+  constexpr uint32_t kT = pair_rules::kExpandThreads;
+  for (uint32_t p = blockIdx.x * kT + threadIdx.x; p < n; p += gridDim.x * kT) {
     const uint32_t j = __ldcs(idx + p);
     const uint32_t mt = __ldcs(meta + p);
     V v;
@@ -1512,7 +1514,7 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
     first_up[c] = lo;
     off[c] = (uint32_t)acc - K * (ubase + lo);    // modulo 2^32: slot = off + K upper + k
     acc += (uint64_t)K * (hi - lo);
-    if (acc >= 0xFFFFFF00ull) { ed_free_pair(B); return ED_OK; }
+    if (acc > pair_rules::kMaxSlots) { ed_free_pair(B); return ED_OK; }
   }
   start[nA] = (uint32_t)acc;
   const uint64_t cap = std::max<uint64_t>(4 * (uint64_t)B->D, 1u << 22);
@@ -1827,7 +1829,7 @@ int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, c
   float *xslo = lo ? reinterpret_cast<float *>(ws + xs_bytes + 16) : nullptr;
   P.next = reinterpret_cast<uint32_t *>(ws + xs_bytes);
   P.chunk_part = reinterpret_cast<double *>(ws + 16 + xs_bytes + lo_bytes);
-  const int eg = (int)std::min<uint32_t>((p->n_slots + 255) / 256, (uint32_t)B->sm_count * 16);
+  const int eg = (int)pair_rules::expand_blocks(p->n_slots, (uint32_t)B->sm_count);
   P.xs = ws;
   P.xslo = xslo;
   P.lo_special = lo ? kSpecial : 0u;
@@ -1837,7 +1839,7 @@ int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, c
   switch (dtype) {
 #define PCASE(D, V)                                                                              \
   case D:                                                                                        \
-    expand_kernel<V><<<eg, 256, 0, st>>>((const V *)x, p->idx, p->meta, (const double2 *)p->w, p->wf, p->n_slots, (V *)ws, xslo, P.next); \
+    expand_kernel<V><<<eg, pair_rules::kExpandThreads, 0, st>>>((const V *)x, p->idx, p->meta, (const double2 *)p->w, p->wf, p->n_slots, (V *)ws, xslo, P.next); \
     rc = cudaGetLastError() == cudaSuccess ? launch_pair_v<V>(B, P, chi, p->flips, rows, mode, st)      \
                                            : ed_fail(ED_ERR_CUDA, "expand_kernel");              \
     break;

@@ -1,0 +1,60 @@
+"""The size rules of the coset-arithmetic product (csrc/pair_rules.h), compiled for the host."""
+import os
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1804_05028_gb300", "csrc")
+
+
+def run(tmp_path, body):
+    """What a program made of the rules and `body` prints."""
+    src, exe = tmp_path / "t.cpp", tmp_path / "t"
+    src.write_text('#include "pair_rules.h"\n#include <cstdio>\nusing namespace pair_rules;\n' + body)
+    subprocess.run(["g++", "-std=c++17", "-O1", "-Wall", "-Werror", "-I", CSRC, str(src), "-o", str(exe)], check=True)
+    return subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout
+
+
+# the last step of expand_kernel's loop: every thread's first position at or past the end, in the
+# 32 bits the kernel counts in
+LAST_STEP = """
+static bool ends(uint64_t slots, uint32_t sms) {
+  const uint32_t n = (uint32_t)slots, stride = expand_blocks(slots, sms) * kExpandThreads;
+  for (uint32_t t = 0; t < stride && t < n; t++) {
+    const uint32_t last = t + (n - 1 - t) / stride * stride;
+    if ((uint32_t)(last + stride) < n) return false;   // wrapped to the front
+  }
+  return true;
+}
+"""
+
+
+@pytest.mark.parametrize("sms", [1, 132, 152, 4096, 100000])
+def test_expansion_ends(tmp_path, sms):
+    out = run(tmp_path, LAST_STEP + """
+int main() {
+  const uint64_t n[] = {1, 255, 256, 257, 1u << 22, kMaxSlots - 1, kMaxSlots};
+  for (uint64_t v : n) printf("%%d", ends(v, %d));
+}
+""" % sms)
+    assert out == "1111111"
+
+
+def test_row_enumeration_ends(tmp_path):
+    """enum_rows' warps look at 1024 slots from any start inside a class."""
+    out = run(tmp_path, """
+int main() {
+  const uint32_t end = (uint32_t)kMaxSlots;
+  for (uint32_t p0 = end - 1024; p0 < end; p0++)
+    for (uint32_t q = 0; q < 1024; q++)
+      if ((uint32_t)(p0 + q) < p0) { printf("wraps"); return 0; }
+  printf("ends");
+}
+""")
+    assert out == "ends"
+
+
+def test_emulation_sees_the_wrap(tmp_path):
+    """Slots within one stride of 2^32 are what the bound keeps out."""
+    out = run(tmp_path, LAST_STEP + 'int main() { printf("%d", ends(0xFFFFFF00ull, 152)); }')
+    assert out == "0"
