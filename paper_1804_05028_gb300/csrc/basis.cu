@@ -199,9 +199,9 @@ int exclusive_scan(const TI *in, uint64_t n, uint64_t *out, uint64_t *total, cud
     scan_block_apply<TI><<<1, 256, 0, st>>>(in, n, nullptr, out);
     ED_CK(cudaGetLastError());
   } else {
-    uint64_t *sums = nullptr, *offs = nullptr;
-    ED_CK(cudaMallocAsync(&sums, nb * 8, st));
-    ED_CK(cudaMallocAsync(&offs, nb * 8, st));
+    Scratch sc(st);
+    uint64_t *sums = (uint64_t *)sc.get(nb * 8), *offs = (uint64_t *)sc.get(nb * 8);
+    if (!sums || !offs) return ed_fail(ED_ERR_OOM, "cannot allocate the scan's block sums");
     scan_block_sums<TI><<<(unsigned)nb, 256, 0, st>>>(in, n, sums);
     ED_CK(cudaGetLastError());
     uint64_t sub_total = 0;
@@ -209,8 +209,6 @@ int exclusive_scan(const TI *in, uint64_t n, uint64_t *out, uint64_t *total, cud
     if (rc) return rc;
     scan_block_apply<TI><<<(unsigned)nb, 256, 0, st>>>(in, n, offs, out);
     ED_CK(cudaGetLastError());
-    ED_CK(cudaFreeAsync(sums, st));
-    ED_CK(cudaFreeAsync(offs, st));
   }
   // total = out[n-1] + in[n-1]
   uint64_t last_out = 0;
@@ -487,8 +485,9 @@ int ed_build_device(ed_basis *B, cudaStream_t st, int bucket_target) {
   const size_t o_tv = add(tv.data(), nt * 4), o_tk = add(tk.data(), nt), o_tt = add(ttot.data(), nt * 8),
                o_ti = add(titem.data(), nt * 8), o_bi = add(binom.data(), binom.size() * 8);
   const size_t o_off = (blob.size() + 15) / 16 * 16, o_cnt = o_off + n_items * 8;
-  unsigned char *d_in = nullptr;
-  ED_CK(cudaMallocAsync(&d_in, o_cnt + n_items * 4, st));
+  Scratch sc(st);
+  unsigned char *d_in = (unsigned char *)sc.get(o_cnt + n_items * 4);
+  if (!d_in) return ed_fail(ED_ERR_OOM, "cannot allocate the enumeration's scratch");
   ED_CK(cudaMemcpyAsync(d_in, blob.data(), blob.size(), cudaMemcpyHostToDevice, st));
   uint64_t *d_off = reinterpret_cast<uint64_t *>(d_in + o_off);
   uint32_t *d_counts = reinterpret_cast<uint32_t *>(d_in + o_cnt);
@@ -508,9 +507,9 @@ int ed_build_device(ed_basis *B, cudaStream_t st, int bucket_target) {
   const uint64_t cap = (uint64_t)B->sm_count * 16;
   if (grid64 > cap) grid64 = cap;
   const unsigned grid = (unsigned)std::max<uint64_t>(grid64, 1);
-  // 4 bytes per 32 candidates; without memory for them the fill pass searches again
-  uint32_t *d_hits = nullptr;
-  if (cudaMallocAsync(&d_hits, n_items * 128, st) != cudaSuccess) { cudaGetLastError(); d_hits = nullptr; }
+  // 4 bytes per 32 candidates (3 bytes per state at most, less than the index takes later);
+  // without memory for them the fill pass searches again
+  uint32_t *d_hits = (uint32_t *)sc.get(n_items * 128);
   enum_kernel<false><<<grid, 256, 0, st>>>(E, d_counts, nullptr, nullptr, nullptr, d_hits);
   ED_CK(cudaGetLastError());
   uint64_t D = 0;
@@ -527,17 +526,17 @@ int ed_build_device(ed_basis *B, cudaStream_t st, int bucket_target) {
     enum_kernel<true><<<grid, 256, 0, st>>>(E, nullptr, d_off, B->d_basis, B->d_stab, d_hits);
     ED_CK(cudaGetLastError());
   }
-  if (d_hits) ED_CK(cudaFreeAsync(d_hits, st));
-  ED_CK(cudaFreeAsync(d_in, st));
+  sc.release(d_hits);
+  sc.release(d_in);
   if (D == 0) return ED_OK;
 
   // ---- prefix index ----
   const int r_bits = std::min(N, 12);
   const uint64_t ntop = 1ULL << r_bits;
-  uint32_t *d_flags = nullptr, *d_rank_top = nullptr;
-  uint64_t *d_scan = nullptr;
-  ED_CK(cudaMallocAsync(&d_flags, ntop * 4, st));
-  ED_CK(cudaMallocAsync(&d_scan, ntop * 8, st));
+  const auto no_scratch = [] { return ed_fail(ED_ERR_OOM, "cannot allocate the index's scratch"); };
+  uint32_t *d_flags = (uint32_t *)sc.get(ntop * 4);
+  uint64_t *d_scan = (uint64_t *)sc.get(ntop * 8);
+  if (!d_flags || !d_scan) return no_scratch();
   ED_CK(cudaMemsetAsync(d_flags, 0, ntop * 4, st));
   const int g1 = B->sm_count * 8;
   mark_tops<<<g1, 256, 0, st>>>(B->d_basis, B->D, N - r_bits, d_flags);
@@ -549,7 +548,8 @@ int ed_build_device(ed_basis *B, cudaStream_t st, int bucket_target) {
     cudaGetLastError();
     return ed_fail(ED_ERR_OOM, "cannot allocate the prefix rank table");
   }
-  ED_CK(cudaMallocAsync(&d_rank_top, R * 4, st));
+  uint32_t *d_rank_top = (uint32_t *)sc.get(R * 4);
+  if (!d_rank_top) return no_scratch();
   make_rank<<<g1, 256, 0, st>>>(d_flags, d_scan, ntop, B->d_top_rank, d_rank_top);
   ED_CK(cudaGetLastError());
   // q: about bucket_target states per key, limited by the bits left
@@ -569,8 +569,8 @@ int ed_build_device(ed_basis *B, cudaStream_t st, int bucket_target) {
   ED_CK(cudaGetLastError());
   fill_limits<<<g1, 256, 0, st>>>(B->d_basis, B->D, d_rank_top, N - r_bits, q, post_bits, n_keys, B->d_limits);
   ED_CK(cudaGetLastError());
-  unsigned long long *d_max = nullptr;
-  ED_CK(cudaMallocAsync(&d_max, 8, st));
+  unsigned long long *d_max = (unsigned long long *)sc.get(8);
+  if (!d_max) return no_scratch();
   ED_CK(cudaMemsetAsync(d_max, 0, 8, st));
   max_bucket_kernel<<<g1, 256, 0, st>>>(B->d_limits, n_keys, d_max);
   ED_CK(cudaGetLastError());
@@ -616,10 +616,7 @@ int ed_build_device(ed_basis *B, cudaStream_t st, int bucket_target) {
       }
     }
   }
-  ED_CK(cudaFreeAsync(d_flags, st));
-  ED_CK(cudaFreeAsync(d_scan, st));
-  ED_CK(cudaFreeAsync(d_rank_top, st));
-  ED_CK(cudaFreeAsync(d_max, st));
+  for (void *q : {(void *)d_flags, (void *)d_scan, (void *)d_rank_top, (void *)d_max}) sc.release(q);
   ED_CK(cudaStreamSynchronize(st));
   B->n_keys = (int64_t)n_keys;
   B->max_bucket = (int64_t)mb;

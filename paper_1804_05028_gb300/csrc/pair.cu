@@ -1122,20 +1122,6 @@ struct Blob {
   template <typename T> size_t add(const std::vector<T> &v) { return add(v.data(), v.size()); }
 };
 
-// stream-ordered scratch of the build, returned on every path
-struct Scratch {
-  cudaStream_t st;
-  std::vector<void *> v;
-  explicit Scratch(cudaStream_t s) : st(s) {}
-  ~Scratch() { for (void *q : v) cudaFreeAsync(q, st); }
-  void *get(size_t bytes) {
-    void *q = nullptr;
-    if (cudaMallocAsync(&q, std::max<size_t>(bytes, 16), st) != cudaSuccess) { cudaGetLastError(); return nullptr; }
-    v.push_back(q);
-    return q;
-  }
-};
-
 constexpr size_t kSharedPoolMax = (size_t)4 << 20;    // xs of fp64 vectors
 constexpr uint64_t kSharedPoolKeep = 64ull << 20;
 

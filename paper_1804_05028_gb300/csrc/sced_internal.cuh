@@ -358,6 +358,26 @@ inline int ed_allow_smem(K k, size_t most) {
   return ED_OK;
 }
 
+// Stream-ordered scratch, given back in stream order when it goes out of scope (on errors too).
+struct Scratch {
+  cudaStream_t st;
+  std::vector<void *> v;
+  explicit Scratch(cudaStream_t s) : st(s) {}
+  Scratch(const Scratch &) = delete;
+  ~Scratch() { for (void *q : v) cudaFreeAsync(q, st); }
+  // null when there is no memory
+  void *get(size_t bytes) {
+    void *q = nullptr;
+    if (cudaMallocAsync(&q, bytes < 16 ? 16 : bytes, st) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    v.push_back(q);
+    return q;
+  }
+  void release(void *q) {
+    for (size_t k = 0; q && k < v.size(); k++)
+      if (v[k] == q) { cudaFreeAsync(q, st); v.erase(v.begin() + k); return; }
+  }
+};
+
 // kernels.cu / basis.cu entry points used by capi.cu
 int ed_build_device(ed_basis *B, cudaStream_t st, int bucket_target);
 // mode 0: y = H x (partial: optional <x, y> block partials); mode 1: per-class block partials
