@@ -430,13 +430,12 @@ int ed_build_full_table(const uint8_t *d_pbit, const uint8_t *d_flip, int N, int
   int dev = 0, nsm = 0;
   ED_CK(cudaGetDevice(&dev));
   ED_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  uint32_t *low = nullptr;
-  ED_CK(cudaMallocAsync(&low, 1024 * (size_t)nsym, st));
+  Scratch sc(st);
+  uint32_t *low = (uint32_t *)sc.get(1024 * (size_t)nsym);
+  if (!low) return ed_fail(ED_ERR_OOM, "cannot allocate the images of the one-block table");
   low_images<<<(nsym + 3) / 4, 256, 0, st>>>(d_pbit, N, nsym, low);
   k<<<nsm * 8, 256, sm, st>>>(d_pbit, d_flip, N, nsym, low, out);
-  const cudaError_t e = cudaGetLastError();
-  ED_CK(cudaFreeAsync(low, st));
-  if (e != cudaSuccess) return ed_cuda_fail(e, "full_table_kernel");
+  ED_CK(cudaGetLastError());
   return ED_OK;
 }
 
@@ -519,7 +518,7 @@ int ed_build_device(ed_basis *B, cudaStream_t st, int bucket_target) {
     return ed_fail(ED_ERR_UNSUPPORTED, "sector dimension must be below 2^32");
   B->D = (int64_t)D;
   if (D > 0) {
-    if (cudaMalloc(&B->d_basis, D * 8) != cudaSuccess || cudaMalloc(&B->d_stab, D * 2) != cudaSuccess) {
+    if (ed_malloc(&B->d_basis, D * 8) != cudaSuccess || ed_malloc(&B->d_stab, D * 2) != cudaSuccess) {
       cudaGetLastError();
       return ed_fail(ED_ERR_OOM, "cannot allocate the basis on the device");
     }
@@ -544,7 +543,7 @@ int ed_build_device(ed_basis *B, cudaStream_t st, int bucket_target) {
   uint64_t R = 0;
   rc = exclusive_scan<uint32_t>(d_flags, ntop, d_scan, &R, st);
   if (rc) return rc;
-  if (cudaMalloc(&B->d_top_rank, ntop * 4) != cudaSuccess) {
+  if (ed_malloc(&B->d_top_rank, ntop * 4) != cudaSuccess) {
     cudaGetLastError();
     return ed_fail(ED_ERR_OOM, "cannot allocate the prefix rank table");
   }
@@ -560,7 +559,7 @@ int ed_build_device(ed_basis *B, cudaStream_t st, int bucket_target) {
   while ((double)R * std::ldexp(1.0, q) > 4.0e9) q--;   // keys must fit in uint32
   const int post_bits = N - r_bits - q;
   const uint64_t n_keys = R << q;
-  if (cudaMalloc(&B->d_limits, (n_keys + 1) * 4) != cudaSuccess) {
+  if (ed_malloc(&B->d_limits, (n_keys + 1) * 4) != cudaSuccess) {
     cudaGetLastError();
     return ed_fail(ED_ERR_OOM, "cannot allocate Limits");
   }
@@ -582,7 +581,7 @@ int ed_build_device(ed_basis *B, cudaStream_t st, int bucket_target) {
     B->d_postfix = B->d_basis;   // full states are the postfixes
   } else {
     // 32 bytes of zero padding: the bucket reader loads whole 16-byte chunks
-    if (cudaMalloc(&B->d_postfix, (size_t)D * post_bytes + 32) != cudaSuccess) {
+    if (ed_malloc(&B->d_postfix, (size_t)D * post_bytes + 32) != cudaSuccess) {
       cudaGetLastError();
       return ed_fail(ED_ERR_OOM, "cannot allocate postfixes");
     }
@@ -602,7 +601,7 @@ int ed_build_device(ed_basis *B, cudaStream_t st, int bucket_target) {
     const int rpost = N - r_bits - rq;
     const uint64_t rkeys = R << rq;
     if (rkeys < (1ULL << 32) && rkeys * 16 <= std::max<uint64_t>(4 * (uint64_t)D * 8, 1ULL << 26)) {
-      if (cudaMalloc(&B->d_rlim, rkeys * 16) == cudaSuccess) {
+      if (ed_malloc(&B->d_rlim, rkeys * 16) == cudaSuccess) {
         ED_CK(cudaMemsetAsync(B->d_rlim, 0, rkeys * 16, st));
         ranked_records<<<g1, 256, 0, st>>>(B->d_basis, B->D, B->d_top_rank, N - r_bits, rq, rpost,
                                            reinterpret_cast<uint4 *>(B->d_rlim));

@@ -518,7 +518,7 @@ int build_orbits(ed_batch *Bt) {
   };
   auto get = [&](size_t bytes) -> void * {
     void *q = nullptr;
-    if (cudaMalloc(&q, bytes) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    if (ed_malloc(&q, bytes) != cudaSuccess) { cudaGetLastError(); return nullptr; }
     Bt->d_orbit.push_back(q);
     return q;
   };
@@ -531,8 +531,8 @@ int build_orbits(ed_batch *Bt) {
     uint64_t **c;
     ~Free() { cudaFree(*a); cudaFree(*b); cudaFree(*c); }
   } scratch{&d_rank, &d_counts, &d_first};
-  if (cudaMalloc(&d_rank, 4 * (size_t)total) != cudaSuccess || cudaMalloc(&d_counts, 128 * (size_t)n_blocks) != cudaSuccess ||
-      cudaMalloc(&d_first, 256 * (size_t)n_blocks) != cudaSuccess) {
+  if (ed_malloc(&d_rank, 4 * (size_t)total) != cudaSuccess || ed_malloc(&d_counts, 128 * (size_t)n_blocks) != cudaSuccess ||
+      ed_malloc(&d_first, 256 * (size_t)n_blocks) != cudaSuccess) {
     drop();
     return ED_OK;
   }
@@ -677,10 +677,10 @@ extern "C" int ed_batch_create(ed_basis *const *bases, int32_t n, const double *
       ftab.push_back((float)std::sin(a));
     }
   }
-  if (cudaMalloc(&Bt->d_sec, sizeof(BatchSector) * n) != cudaSuccess ||
-      cudaMalloc(&Bt->d_item0, 8 * (size_t)n) != cudaSuccess || cudaMalloc(&Bt->d_counter, 8) != cudaSuccess ||
-      cudaMalloc(&Bt->d_bond, std::max<size_t>(b0->bond_pos.size(), 1)) != cudaSuccess ||
-      cudaMalloc(&Bt->d_ftab, ftab.size() * 4) != cudaSuccess) {
+  if (ed_malloc(&Bt->d_sec, sizeof(BatchSector) * n) != cudaSuccess ||
+      ed_malloc(&Bt->d_item0, 8 * (size_t)n) != cudaSuccess || ed_malloc(&Bt->d_counter, 8) != cudaSuccess ||
+      ed_malloc(&Bt->d_bond, std::max<size_t>(b0->bond_pos.size(), 1)) != cudaSuccess ||
+      ed_malloc(&Bt->d_ftab, ftab.size() * 4) != cudaSuccess) {
     cudaGetLastError();
     ed_batch_free(Bt);
     return ed_fail(ED_ERR_OOM, "cannot allocate the batch");

@@ -8,6 +8,8 @@
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
+#include <map>
+#include <mutex>
 #include <string>
 #include <unordered_map>
 #include <vector>
@@ -22,6 +24,42 @@ int ed_fail(int code, const std::string &msg) {
 int ed_cuda_fail(cudaError_t e, const char *what) {
   g_err = std::string("CUDA error in ") + what + ": " + cudaGetErrorString(e);
   return ED_ERR_CUDA;
+}
+
+cudaMemPool_t ed_make_pool(int device, uint64_t keep) {
+  cudaMemPoolProps props{};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = device;
+  cudaMemPool_t pool = nullptr;
+  if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+  if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+    cudaGetLastError();
+    cudaMemPoolDestroy(pool);
+    return nullptr;
+  }
+  return pool;
+}
+
+cudaMemPool_t ed_shared_pool(int device) {
+  static std::mutex lock;
+  static std::map<int, cudaMemPool_t> pools;
+  std::lock_guard<std::mutex> hold(lock);
+  cudaMemPool_t &p = pools[device];
+  if (!p) p = ed_make_pool(device, 64ull << 20);
+  return p;
+}
+
+cudaError_t ed_malloc(void **p, size_t bytes) {
+  const cudaError_t e = cudaMalloc(p, bytes);
+  if (e != cudaErrorMemoryAllocation) return e;
+  cudaGetLastError();
+  int dev = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceSynchronize() == cudaSuccess) {
+    cudaMemPool_t pool = ed_shared_pool(dev);
+    if (pool) cudaMemPoolTrimTo(pool, 0);
+  }
+  return cudaMalloc(p, bytes);
 }
 
 
@@ -232,7 +270,7 @@ struct TableSet {
   }
   int upload(ed_basis *B, cudaStream_t st) {
     void *d = nullptr;
-    if (cudaMalloc(&d, std::max<size_t>(bytes.size(), 1)) != cudaSuccess) {
+    if (ed_malloc(&d, std::max<size_t>(bytes.size(), 1)) != cudaSuccess) {
       cudaGetLastError();
       return ed_fail(ED_ERR_OOM, "cannot allocate lookup tables");
     }
@@ -285,7 +323,7 @@ int build_full_table(ed_basis *B, cudaStream_t st, const ed_basis *share) {
     B->full_tab = share->full_tab;
   } else {
     uint64_t *t = nullptr;
-    if (cudaMalloc(&t, ((size_t)1 << N) * 8) != cudaSuccess) {
+    if (ed_malloc(&t, ((size_t)1 << N) * 8) != cudaSuccess) {
       cudaGetLastError();
       return ed_fail(ED_ERR_OOM, "cannot allocate the one-sublattice table");
     }
@@ -572,7 +610,7 @@ extern "C" int ed_build_basis(const ed_lattice *L, const ed_group *G, const ed_i
   if ((rc = ed_build_device(B, st, bucket))) { free_all(B); delete B; return rc; }
   if ((rc = ed_build_pair(B, st))) { free_all(B); delete B; return rc; }
   B->n_partial = ED_MAXCLS * B->sm_count * 8;   // per-class partials of the widest grid
-  if (cudaMalloc(&B->d_partial, (size_t)B->n_partial * 8) != cudaSuccess ||
+  if (ed_malloc(&B->d_partial, (size_t)B->n_partial * 8) != cudaSuccess ||
       cudaMallocHost(&B->h_partial, (size_t)B->n_partial * 8) != cudaSuccess) {
     cudaGetLastError();
     free_all(B);
@@ -665,7 +703,7 @@ extern "C" int ed_apply_H_host(ed_basis *B, const double *J, const double *Jz, c
     if (B->d_stage_y) cudaFree(B->d_stage_y);
     B->d_stage_x = B->d_stage_y = nullptr;
     B->stage_bytes = 0;
-    if (cudaMalloc(&B->d_stage_x, bytes) != cudaSuccess || cudaMalloc(&B->d_stage_y, bytes) != cudaSuccess) {
+    if (ed_malloc(&B->d_stage_x, bytes) != cudaSuccess || ed_malloc(&B->d_stage_y, bytes) != cudaSuccess) {
       cudaGetLastError();
       return ed_fail(ED_ERR_OOM, "cannot allocate staging vectors");
     }
@@ -737,13 +775,14 @@ extern "C" int ed_count_terms(const ed_basis *B, int64_t *n_flip, int64_t *n_off
   *n_flip = *n_offdiag = 0;
   if (B->D == 0) return ED_OK;
   cudaStream_t st = (cudaStream_t)stream;
-  unsigned long long *d = nullptr, h[2] = {0, 0};
-  ED_CK(cudaMallocAsync(&d, 16, st));
+  unsigned long long h[2] = {0, 0};
+  Scratch sc(st);
+  unsigned long long *d = (unsigned long long *)sc.get(16);
+  if (!d) return ed_fail(ED_ERR_OOM, "cannot allocate the counters");
   ED_CK(cudaMemsetAsync(d, 0, 16, st));
   int rc = ed_launch_count(B, d, st);
   if (rc) return rc;
   ED_CK(cudaMemcpyAsync(h, d, 16, cudaMemcpyDeviceToHost, st));
-  ED_CK(cudaFreeAsync(d, st));
   ED_CK(cudaStreamSynchronize(st));
   *n_flip = (int64_t)h[0];
   *n_offdiag = (int64_t)h[1];
@@ -983,7 +1022,7 @@ extern "C" int ed_lanczos(ed_basis *B, const double *J, const double *Jz,
   }
   for (int k = 0; k < 3 && !full; k++) {
     if (!own) { L.v[k] = (char *)o.work + k * bytes; continue; }
-    if (cudaMalloc(&L.v[k], bytes) != cudaSuccess) {
+    if (ed_malloc(&L.v[k], bytes) != cudaSuccess) {
       cudaGetLastError();
       for (int q = 0; q < k; q++) cudaFree(L.v[q]);
       return ed_fail(ED_ERR_OOM, "cannot allocate Lanczos vectors");
@@ -994,7 +1033,7 @@ extern "C" int ed_lanczos(ed_basis *B, const double *J, const double *Jz,
   if (o.dtype == ED_F32 || o.dtype == ED_C64) {
     if (!full && !own && o.work_bytes >= (int64_t)(4 * bytes)) {
       L.ylo = (char *)o.work + 3 * bytes;
-    } else if (cudaMalloc(&L.ylo, bytes) == cudaSuccess) {
+    } else if (ed_malloc(&L.ylo, bytes) == cudaSuccess) {
       L.own_ylo = true;
     } else {
       cudaGetLastError();
@@ -1009,7 +1048,7 @@ extern "C" int ed_lanczos(ed_basis *B, const double *J, const double *Jz,
   L.nblk = (int)std::max<int64_t>(1, std::min<int64_t>(B->n_partial / 4, (B->D + 1023) / 1024));
   L.ro_coef_off = std::max((size_t)m_cap * P * ed_reorth_grid(B), (size_t)2 * P * L.nblk);
   L.coef_len = (size_t)m_cap * P;
-  if (cudaMalloc(&L.d_ro, sizeof(double) * (L.ro_coef_off + 2 * L.coef_len + 8)) != cudaSuccess) {
+  if (ed_malloc(&L.d_ro, sizeof(double) * (L.ro_coef_off + 2 * L.coef_len + 8)) != cudaSuccess) {
     cudaGetLastError();
     if (own) for (int k = 0; k < 3; k++) cudaFree(L.v[k]);
     if (L.own_ylo) cudaFree(L.ylo);

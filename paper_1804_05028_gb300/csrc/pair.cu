@@ -47,8 +47,6 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
-#include <map>
-#include <mutex>
 #include <new>
 #include <type_traits>
 #include <vector>
@@ -1123,31 +1121,6 @@ struct Blob {
 };
 
 constexpr size_t kSharedPoolMax = (size_t)4 << 20;    // xs of fp64 vectors
-constexpr uint64_t kSharedPoolKeep = 64ull << 20;
-
-cudaMemPool_t make_pool(int device, uint64_t keep) {
-  cudaMemPoolProps props{};
-  props.allocType = cudaMemAllocationTypePinned;
-  props.location.type = cudaMemLocationTypeDevice;
-  props.location.id = device;
-  cudaMemPool_t pool = nullptr;
-  if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) { cudaGetLastError(); return nullptr; }
-  if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
-    cudaGetLastError();
-    cudaMemPoolDestroy(pool);
-    return nullptr;
-  }
-  return pool;
-}
-
-cudaMemPool_t shared_pool(int device) {
-  static std::mutex lock;
-  static std::map<int, cudaMemPool_t> pools;
-  std::lock_guard<std::mutex> hold(lock);
-  cudaMemPool_t &p = pools[device];
-  if (!p) p = make_pool(device, kSharedPoolKeep);
-  return p;
-}
 
 // Row order for large sectors (see pair_rows_kernel); p->n_slices stays 0 when it is not made.
 // pat: the pattern of the other half of every slot.
@@ -1171,7 +1144,7 @@ int build_rows(ed_basis *B, PairPlan *p, const std::vector<uint32_t> &start, con
   if (!d || !d_first || !d_bits || !d_count || !d_at) return ED_OK;
   const uint64_t max_chunks = (B->D / 32 + nA) / (kRowThreads / 32) + 1;
   const size_t rows_bytes = 10 * (size_t)B->D + 8 * ((size_t)nA + 1) + 4 * max_chunks;
-  if (cudaMalloc(&p->d_rows, rows_bytes) != cudaSuccess) { cudaGetLastError(); p->d_rows = nullptr; return ED_OK; }
+  if (ed_malloc(&p->d_rows, rows_bytes) != cudaSuccess) { cudaGetLastError(); p->d_rows = nullptr; return ED_OK; }
   p->row_b = (uint32_t *)p->d_rows;
   p->row_i = p->row_b + B->D;
   p->row0 = p->row_i + B->D;
@@ -1407,7 +1380,7 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
   Scratch sc(st);
   auto keep = [&](size_t bytes) -> void * {
     void *q = nullptr;
-    if (cudaMalloc(&q, bytes) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    if (ed_malloc(&q, bytes) != cudaSuccess) { cudaGetLastError(); return nullptr; }
     p->bytes += bytes;
     return q;
   };
@@ -1677,12 +1650,11 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
   if (Q.pat)
     if ((rc = build_rows(B, p, start, Q.start, Q.pat, st))) return rc;
   // The memory of xs: large sectors keep a pool of their own, gone with the basis; small ones
-  // (a pool costs 0.2 ms, as much as the rest of their tables) share one per device, which
-  // keeps at most kSharedPoolKeep between synchronisations and gives back the rest.
+  // (a pool costs 0.2 ms, as much as the rest of their tables) take it from the device's shared one.
   const size_t first = 8 * ((size_t)p->n_slots + 1) + 256;
   p->own_pool = first > kSharedPoolMax;
-  if (p->own_pool) p->pool = make_pool(B->device, ~0ull);
-  else p->pool = shared_pool(B->device);
+  if (p->own_pool) p->pool = ed_make_pool(B->device, ~0ull);
+  else p->pool = ed_shared_pool(B->device);
   if (!p->pool) { ed_free_pair(B); return ED_OK; }
   // small sectors: the pool takes its first memory here rather than in the first product,
   // where mapping it would cost several times the product itself

@@ -358,17 +358,37 @@ inline int ed_allow_smem(K k, size_t most) {
   return ED_OK;
 }
 
-// Stream-ordered scratch, given back in stream order when it goes out of scope (on errors too).
+// A memory pool of the device that keeps up to `keep` bytes over synchronisations (null on
+// failure), and the pool that all builds and the products of small sectors share: it keeps at
+// most 64 MB and gives the rest back.
+cudaMemPool_t ed_make_pool(int device, uint64_t keep);
+cudaMemPool_t ed_shared_pool(int device);
+// cudaMalloc; where that fails, once more after the shared pool has given back what it keeps
+cudaError_t ed_malloc(void **p, size_t bytes);
+template <typename T>
+inline cudaError_t ed_malloc(T **p, size_t bytes) { return ed_malloc(reinterpret_cast<void **>(p), bytes); }
+
+// Stream-ordered scratch of the current device, given back in stream order when it goes out of
+// scope (on errors too).  From the shared pool: the device's default pool unmaps its memory at
+// every synchronisation, and mapping it again took 75 us each of the three to five times that a
+// build comes back for more.
 struct Scratch {
   cudaStream_t st;
+  cudaMemPool_t pool;
   std::vector<void *> v;
-  explicit Scratch(cudaStream_t s) : st(s) {}
+  explicit Scratch(cudaStream_t s) : st(s), pool(nullptr) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess) pool = ed_shared_pool(dev);
+  }
   Scratch(const Scratch &) = delete;
   ~Scratch() { for (void *q : v) cudaFreeAsync(q, st); }
   // null when there is no memory
   void *get(size_t bytes) {
     void *q = nullptr;
-    if (cudaMallocAsync(&q, bytes < 16 ? 16 : bytes, st) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    if (!pool || cudaMallocFromPoolAsync(&q, bytes < 16 ? 16 : bytes, pool, st) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
     v.push_back(q);
     return q;
   }
