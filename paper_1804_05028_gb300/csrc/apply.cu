@@ -511,15 +511,7 @@ int ed_launch_apply(const ed_basis *B, const double *J, const double *Jz, const 
                     void *y, int dtype, int64_t r0, int64_t r1, double *partial,
                     cudaStream_t st, int mode, void *ylo) {
   if (r1 <= r0) return ED_OK;
-  // The coset-arithmetic product expands the whole of x first, the search kernels have nothing
-  // to prepare but take longer per row.  Measured (fp32 vectors, ranges of D/17, D/128 and
-  // D/1024 rows, coset arithmetic against search): 6x6 sector, 3.2e7 states, whose xs stays
-  // mostly in L2, 0.94, 0.35, 0.28 against 3.95, 0.74, 0.40 ms; 40 sites, 8.6e8 states, 53, 23,
-  // 19 against 45, 6.2, 0.85 ms, equal near D/9; so all but the narrowest ranges up to some
-  // 3.3e7 states and ranges towards 1/8 of the rows above.  On 810 states 25 rows take 16
-  // against 20 us and 12 rows 16 against 14 us.
-  const int64_t n = r1 - r0;
-  if (B->pair && n >= 16 && n + (1 << 22) >= B->D / 8) {
+  {  // coset arithmetic where the sector has a plan and the call is large enough for it
     bool done = false;
     const int rc = ed_launch_apply_pair(B, J, Jz, x, y, dtype, r0, r1, partial, st, mode, ylo, &done);
     if (rc != ED_ERR_UNSUPPORTED) return rc;

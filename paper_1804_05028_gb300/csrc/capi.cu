@@ -609,6 +609,8 @@ extern "C" int ed_build_basis(const ed_lattice *L, const ed_group *G, const ed_i
   const int bucket = (opts && opts->bucket_target > 0) ? opts->bucket_target : 1;
   if ((rc = ed_build_device(B, st, bucket))) { free_all(B); delete B; return rc; }
   if ((rc = ed_build_pair(B, st))) { free_all(B); delete B; return rc; }
+  if (B->N > 1)
+    B->terms_per_row = 2.0 * B->n_bonds * B->n_up * (B->N - B->n_up) / ((double)B->N * (B->N - 1));
   B->n_partial = ED_MAXCLS * B->sm_count * 8;   // per-class partials of the widest grid
   if (ed_malloc(&B->d_partial, (size_t)B->n_partial * 8) != cudaSuccess ||
       cudaMallocHost(&B->h_partial, (size_t)B->n_partial * 8) != cudaSuccess) {

@@ -93,11 +93,14 @@ struct PairParams {
   const double *rsqrt_tab;
   uint32_t n_sq;
   const double *chi;             // complex sectors: (cos, sin) of chi per half and element
-  uint32_t n_chi;
   const uint64_t *basis;
   const uint16_t *stab;
   const void *x, *xs;
   const float *xslo;             // fp32 real vectors: remainders of xs
+  const uint32_t *slot_idx;      // what xs is made of: basis index and weight number of a slot,
+  const uint16_t *slot_meta;     // and the weights chi sqrt(t) (fp32 vectors: pairs of words)
+  const double2 *w;
+  const float4 *wf;
   uint32_t lo_special, lo_same;  // which slots may have one (both 0: none)
   uint32_t n_slots;              // xs[n_slots] = 0
   void *y;
@@ -301,32 +304,87 @@ __device__ __forceinline__ void no_terms(Terms<V, U> &t) {
   }
 }
 
+// What xs holds of v = x_j: w(mt) v with w = chi sqrt(t), mt 0 being w = 1.  fp32 vectors take the
+// weights as pairs of fp32 words, (re, its remainder, im, its remainder): in fp64 the products
+// and conversions kept the fp64 pipe 85% busy (expansion of the 6x6 sector's 4.8e7 slots: 0.54
+// ms).  Real ones give the rounding's remainder in lo, so that a weight sqrt(t) costs no precision.
+template <typename V>
+__device__ __forceinline__ V weighted(V v, uint32_t mt, const double2 *w, const float4 *wf, float &lo) {
+  constexpr bool kF = sizeof(typename Pv<V>::A) == 4;
+  lo = 0.f;
+  if (!mt) return v;
+  if constexpr (kF && Pv<V>::cplx) {
+    const float4 c = __ldg(wf + mt);
+    const V u = v;
+    float h = 0.f, l = 0.f;
+    df_sub_scaled(h, l, -c.x, -c.y, u.x);
+    df_sub_scaled(h, l, c.z, c.w, u.y);
+    v.x = df_round(h, l);
+    h = l = 0.f;
+    df_sub_scaled(h, l, -c.x, -c.y, u.y);
+    df_sub_scaled(h, l, -c.z, -c.w, u.x);
+    v.y = df_round(h, l);
+  } else if constexpr (kF) {
+    const float2 c = __ldg(reinterpret_cast<const float2 *>(wf + mt));
+    const float u = v;
+    v = __fmul_rn(c.x, u);
+    lo = __fmaf_rn(c.y, u, __fmaf_rn(c.x, u, -v));
+  } else if constexpr (Pv<V>::cplx) {
+    const double2 c = __ldg(w + mt);
+    const double a = c.x * v.x - c.y * v.y, b = c.x * v.y + c.y * v.x;
+    v.x = a;
+    v.y = b;
+  } else {
+    v *= __ldg(w + mt).x;
+  }
+  return v;
+}
+
 // Sums n terms, U at a time; gen(slots, nu) gives the next nu.  The gathers of one round are
 // in flight while the round before is summed: two sets of registers taken in turn, as a copy
 // from one to the other would wait for the loads.  t0 holds terms still to be summed, on
 // entry and on exit, so that the gathers of one loop overlap the start of the next.
-template <typename V, bool kChi, int U, typename G>
+template <typename V, bool kChi, int U, bool kDirect, typename G>
 __device__ __forceinline__ void pair_loop(const PairParams &P, int n, G gen, const V *xs,
                                           const unsigned char *chi_sm, Acc<V> &acc, Terms<V, U> &t0) {
   auto step = [&](Terms<V, U> &t) {
     Slot g[U];
     gen(g, n);
     t.n = n;
+    if constexpr (kDirect) {
+      uint32_t j[U], mt[U];
 #pragma unroll
-    for (int u = 0; u < U; u++) {
-      const uint32_t slot = u == 0 || u < n ? g[u].slot : P.n_slots;   // xs[n_slots] = 0
-      t.w[u] = g[u].w;
-      t.v[u] = __ldg(xs + slot);
-      t.vl[u] = 0.f;
-      if constexpr (std::is_same<V, float>::value) {
-        if (g[u].lo) t.vl[u] = __ldg(P.xslo + slot);
+      for (int u = 0; u < U; u++) {
+        const bool in = u == 0 || u < n;
+        j[u] = in ? __ldg(P.slot_idx + g[u].slot) : 0xFFFFFFFFu;
+        mt[u] = in ? __ldg(P.slot_meta + g[u].slot) : 0u;
+        t.w[u] = g[u].w;
+      }
+#pragma unroll
+      for (int u = 0; u < U; u++) {
+        t.v[u] = no_value<V>();
+        float lo = 0.f;
+        if (j[u] != 0xFFFFFFFFu) t.v[u] = weighted<V>(__ldg(xs + j[u]), mt[u], P.w, P.wf, lo);
+        t.vl[u] = g[u].lo ? lo : 0.f;
+      }
+    } else {
+#pragma unroll
+      for (int u = 0; u < U; u++) {
+        const uint32_t slot = u == 0 || u < n ? g[u].slot : P.n_slots;   // xs[n_slots] = 0
+        t.w[u] = g[u].w;
+        t.v[u] = __ldg(xs + slot);
+        t.vl[u] = 0.f;
+        if constexpr (std::is_same<V, float>::value) {
+          if (g[u].lo) t.vl[u] = __ldg(P.xslo + slot);
+        }
       }
     }
     n -= U;
   };
-  if constexpr (sizeof(V) == 16) {
+  if constexpr (sizeof(V) == 16 || kDirect) {
     // 16-byte values leave no registers for a second set, and the fp64 pipe is the bound
-    // (pair_kernel on 2.6e6 complex rows: 1.32 ms, with two sets 1.41)
+    // (pair_kernel on 2.6e6 complex rows: 1.32 ms, with two sets 1.41); direct terms need
+    // their index and weight in registers and wait for them in any case
     while (n > 0) {
       Terms<V, U> t1;
       step(t1);
@@ -358,7 +416,9 @@ __device__ __forceinline__ PairSm pair_stage(const PairParams &P, unsigned char 
   }
   cpy(sm, P.off_rs, P.rsqrt_tab, P.n_sq);
   if constexpr (kChi) {
-    for (uint32_t k = threadIdx.x; k < P.n_chi; k += blockDim.x) {
+    // the elements there are: h0 numbers, with and without the flip bit, for either half
+    for (uint32_t q = threadIdx.x; q < 4 * P.h0; q += blockDim.x) {
+      const uint32_t k = q / P.h0 * 256 + q % P.h0;
       const double c = P.chi[2 * k], s = P.chi[2 * k + 1];
       if constexpr (sizeof(typename Pv<V>::A) == 4) {
         const float ch = (float)c, sh = (float)s;
@@ -463,11 +523,12 @@ __device__ __forceinline__ int next_bond(uint32_t &m, int &wd, int w0, const uin
   return k;
 }
 
-// Rows in basis order: any range of rows, and sectors whose xs stays in L2.
-template <typename V, bool kChi, bool kFlips, int kMode>
+// Rows in basis order: any range of rows, and sectors whose xs stays in L2.  kDirect: no xs; a term
+// reads its slot's index, its weight and x one after the other (see pair_rules.h for when).
+template <typename V, bool kChi, bool kFlips, int kMode, bool kDirect>
 __global__ void __launch_bounds__(kThreads, kMinBlocks) pair_kernel(const __grid_constant__ PairParams P) {
   constexpr bool kC = Pv<V>::cplx;
-  constexpr int U = 2;
+  constexpr int U = kDirect ? 4 : 2;
   extern __shared__ __align__(16) unsigned char sm[];
   const PairSm S = pair_stage<V, kChi>(P, sm);
   cpy(sm, P.off_nib, P.nib, (uint32_t)P.cls_word[P.n_classes] * P.n_nib * 16);
@@ -477,7 +538,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) pair_kernel(const __grid
   const uint32_t *nibs = reinterpret_cast<const uint32_t *>(sm + P.off_nib);
   const double *rsd = reinterpret_cast<const double *>(sm + P.off_rs);
   uint32_t *mask_s = reinterpret_cast<uint32_t *>(sm + P.off_mask) + threadIdx.x;
-  const V *xs = reinterpret_cast<const V *>(P.xs);
+  const V *xs = reinterpret_cast<const V *>(kDirect ? P.x : P.xs);
   double dot[kMode == 1 ? ED_MAXCLS : 2] = {};
   const int64_t stride = (int64_t)gridDim.x * kThreads;
   for (int64_t i = P.r0 + (int64_t)blockIdx.x * kThreads + threadIdx.x; i < P.r1; i += stride) {
@@ -521,7 +582,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) pair_kernel(const __grid
 #pragma unroll
         for (int u = 0; u < U; u++) g[u] = slot_of<kChi, kFlips>(P, S, ea[u], eb[u]);
       };
-      pair_loop<V, kChi, U>(P, nanti, gen, xs, sm + P.off_chi, acc, pend);
+      pair_loop<V, kChi, U, kDirect>(P, nanti, gen, xs, sm + P.off_chi, acc, pend);
       pair_sum<V, kChi, U>(pend, sm + P.off_chi, acc);
       const double dg = P.jzq[c] * (double)(P.nb_cls[c] - 2 * nanti);
       if constexpr (kMode == 1) {
@@ -736,7 +797,7 @@ __global__ void __launch_bounds__(kRowThreads, kRowBlocks) pair_rows_kernel(cons
               }
             }
           };
-          pair_loop<V, kChi, U>(P, n, gen, xs, sm + P.off_chi, acc, pend);
+          pair_loop<V, kChi, U, false>(P, n, gen, xs, sm + P.off_chi, acc, pend);
         };
         auto from_table = [&](uint32_t q) { return eup_r[q]; };
         auto from_memory = [&](uint32_t q) { return __ldg(P.t_up + (R ^ (1u << q))); };
@@ -768,7 +829,7 @@ __global__ void __launch_bounds__(kRowThreads, kRowBlocks) pair_rows_kernel(cons
               }
             }
           };
-          pair_loop<V, kChi, U>(P, n, gen, xs, sm + P.off_chi, acc, pend);
+          pair_loop<V, kChi, U, false>(P, n, gen, xs, sm + P.off_chi, acc, pend);
         };
         if (!kFlips && st_in) within(std::true_type()); else within(std::false_type());
       }
@@ -801,7 +862,7 @@ __global__ void __launch_bounds__(kRowThreads, kRowBlocks) pair_rows_kernel(cons
               }
             }
           };
-          pair_loop<V, kChi, U>(P, n, gen, xs, sm + P.off_chi, acc, pend);
+          pair_loop<V, kChi, U, false>(P, n, gen, xs, sm + P.off_chi, acc, pend);
         };
         if (!kFlips && st_in) within(std::true_type()); else within(std::false_type());
       }
@@ -842,56 +903,23 @@ __global__ void __launch_bounds__(256) chunk_sum_kernel(const __grid_constant__ 
   pair_dot<256>(P, v, n);
 }
 
-// xs[p] = w(meta[p]) x[idx[p]], w = chi sqrt(t); meta 0 is w = 1.  fp32 vectors take the weights
-// as pairs of fp32 words, (re, its remainder, im, its remainder): in fp64 the products and
-// conversions kept the fp64 pipe 85% busy (0.54 ms on the 6x6 sector's 4.8e7 slots).  Real ones
-// keep the rounding's remainder in xslo, so that a weight sqrt(t) costs no precision.
+// xs[p] = w(meta[p]) x[idx[p]]
 template <typename V>
 __global__ void __launch_bounds__(pair_rules::kExpandThreads) expand_kernel(const V *x, const uint32_t *idx, const uint16_t *meta,
                                                      const double2 *w, const float4 *wf, uint32_t n, V *xs,
                                                      float *xslo, uint32_t *next) {
-  constexpr bool kF = sizeof(typename Pv<V>::A) == 4;
+  constexpr uint32_t kT = pair_rules::kExpandThreads;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     *next = 0;
-    if constexpr (Pv<V>::cplx) { xs[n].x = 0; xs[n].y = 0; } else { xs[n] = 0; }
+    xs[n] = no_value<V>();
     if (sizeof(V) == 4 && xslo) xslo[n] = 0.f;
   }
-  constexpr uint32_t kT = pair_rules::kExpandThreads;
   for (uint32_t p = blockIdx.x * kT + threadIdx.x; p < n; p += gridDim.x * kT) {
     const uint32_t j = __ldcs(idx + p);
     const uint32_t mt = __ldcs(meta + p);
-    V v;
-    if constexpr (Pv<V>::cplx) { v.x = 0; v.y = 0; } else { v = 0; }
+    V v = no_value<V>();
     float lo = 0.f;
-    if (j != 0xFFFFFFFFu) {
-      v = __ldg(x + j);
-      if (mt) {
-        if constexpr (kF && Pv<V>::cplx) {
-          const float4 c = __ldg(wf + mt);
-          const V u = v;
-          float h = 0.f, l = 0.f;
-          df_sub_scaled(h, l, -c.x, -c.y, u.x);
-          df_sub_scaled(h, l, c.z, c.w, u.y);
-          v.x = df_round(h, l);
-          h = l = 0.f;
-          df_sub_scaled(h, l, -c.x, -c.y, u.y);
-          df_sub_scaled(h, l, -c.z, -c.w, u.x);
-          v.y = df_round(h, l);
-        } else if constexpr (kF) {
-          const float2 c = __ldg(reinterpret_cast<const float2 *>(wf + mt));
-          const float u = v;
-          v = __fmul_rn(c.x, u);
-          lo = __fmaf_rn(c.y, u, __fmaf_rn(c.x, u, -v));
-        } else if constexpr (Pv<V>::cplx) {
-          const double2 c = __ldg(w + mt);
-          const double a = c.x * v.x - c.y * v.y, b = c.x * v.y + c.y * v.x;
-          v.x = a;
-          v.y = b;
-        } else {
-          v *= __ldg(w + mt).x;
-        }
-      }
-    }
+    if (j != 0xFFFFFFFFu) v = weighted<V>(__ldg(x + j), mt, w, wf, lo);
     xs[p] = v;
     if (sizeof(V) == 4 && xslo) xslo[p] = lo;
   }
@@ -1671,16 +1699,31 @@ namespace {
 
 size_t al16(size_t x) { return (x + 15) & ~(size_t)15; }
 
+template <typename V>
+int launch_expand(const ed_basis *B, const PairParams &P, cudaStream_t st) {
+  const uint32_t blocks = pair_rules::expand_blocks(P.n_slots, (uint32_t)B->sm_count);
+  expand_kernel<V><<<blocks, pair_rules::kExpandThreads, 0, st>>>(
+      (const V *)P.x, P.slot_idx, P.slot_meta, P.w, P.wf, P.n_slots, (V *)const_cast<void *>(P.xs),
+      const_cast<float *>(P.xslo), P.next);
+  ED_CK(cudaGetLastError());
+  return ED_OK;
+}
+
 template <typename V, bool kChi, bool kFlips, int kMode>
 int launch_pair_t(const ed_basis *B, PairParams &P, bool rows, cudaStream_t st) {
-  auto k = rows ? pair_rows_kernel<V, kChi, kFlips, kMode> : pair_kernel<V, kChi, kFlips, kMode>;
+  auto k = rows ? pair_rows_kernel<V, kChi, kFlips, kMode>
+                : P.xs ? pair_kernel<V, kChi, kFlips, kMode, false> : pair_kernel<V, kChi, kFlips, kMode, true>;
   const int threads = rows ? kRowThreads : kThreads, per_sm = rows ? kRowBlocks : kMinBlocks;
-  if (const int rc = ed_allow_smem(k, rows ? kRowsMaxSmem : kPairMaxSmem)) return rc;
-  const int need = per_sm * ((int)P.smem_bytes + 1536);
-  const int pct = std::min(100, (need * 100 + 228 * 1024 - 1) / (228 * 1024));
-  ED_CK(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, pct));
   const int64_t blocks = rows ? (int64_t)P.n_chunks : (P.r1 - P.r0 + threads - 1) / threads;
   const int grid = (int)std::min<int64_t>(blocks, (int64_t)B->sm_count * per_sm);
+  // small calls are held by the host: 48 KB need no permission, and a block per SM no split
+  if (P.smem_bytes > 48 * 1024)
+    if (const int rc = ed_allow_smem(k, rows ? kRowsMaxSmem : kPairMaxSmem)) return rc;
+  if (grid > B->sm_count || rows) {
+    const int need = per_sm * ((int)P.smem_bytes + 1536);
+    const int pct = std::min(100, (need * 100 + 228 * 1024 - 1) / (228 * 1024));
+    ED_CK(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, pct));
+  }
   B->last_apply_grid = grid;
   k<<<grid, threads, P.smem_bytes, st>>>(P);
   ED_CK(cudaGetLastError());
@@ -1712,9 +1755,12 @@ int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, c
                          void *ylo, bool *ylo_done) {
   const PairPlan *p = B->pair;
   if (!p) return ED_ERR_UNSUPPORTED;
+  const pair_rules::Route route = pair_rules::route(r1 - r0, B->D, B->terms_per_row, p->n_slots, dtype == ED_C128,
+                                                    B->T.full && mode == 0 && !B->is_real && dtype == ED_C64);
+  if (route == pair_rules::kSearch) return ED_ERR_UNSUPPORTED;
   const size_t es = dtype == ED_F64 ? 8 : dtype == ED_F32 ? 4 : dtype == ED_C128 ? 16 : 8;
   const size_t xs_bytes = al16(es * ((size_t)p->n_slots + 1));
-  const bool rows = p->n_slices && r0 == 0 && r1 == B->D && xs_bytes >= (p->rt_w > p->rt_wa ? kRowOrderMinBytes : kRowOrderMinBytesAcross);
+  const bool rows = route == pair_rules::kExpanded && p->n_slices && r0 == 0 && r1 == B->D && xs_bytes >= (p->rt_w > p->rt_wa ? kRowOrderMinBytes : kRowOrderMinBytesAcross);
   PairParams P{};
   P.n_classes = B->n_classes;
   int words = 0;
@@ -1737,7 +1783,7 @@ int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, c
   P.rsqrt_tab = B->d_rsqrt; P.n_sq = (uint32_t)B->nsym + 1;
   const bool cplx = dtype == ED_C128 || dtype == ED_C64;
   const bool chi = cplx && !B->is_real;
-  P.chi = p->chi; P.n_chi = 1024;
+  P.chi = p->chi;
   P.basis = B->d_basis; P.stab = B->d_stab;
   P.up = p->up; P.t_up = p->t_up; P.ubase = p->ubase; P.rt = p->rt; P.rt_words = p->rt_words;
   memcpy(P.kw, p->kw, sizeof(P.kw));
@@ -1771,35 +1817,35 @@ int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, c
   }
   P.smem_bytes = (uint32_t)off;
   if (off > (rows ? kRowsMaxSmem : kPairMaxSmem)) return ED_ERR_UNSUPPORTED;
-  // xs (and its remainders) for this call, from the basis's own pool in stream order, so
-  // calls on several streams or threads never share it; without memory for it the search
-  // kernel takes the call
   const bool lo = dtype == ED_F32 && p->weights;
-  P.n_chunks = (p->n_slices + kRowThreads / 32 - 1) / (kRowThreads / 32);
-  const size_t lo_bytes = lo ? al16(4 * ((size_t)p->n_slots + 1)) : 0;
-  P.n_sums = P.n_chunks * (mode == 1 ? 1 : kSumWarps);
-  const size_t n_sums = !rows || !partial ? 0 : (mode == 1 ? (size_t)B->n_classes : cplx ? 2 : 1) * P.n_sums;
-  char *ws = nullptr;
-  if (cudaMallocFromPoolAsync((void **)&ws, 16 + xs_bytes + lo_bytes + 8 * n_sums, p->pool, st) != cudaSuccess) {
-    cudaGetLastError();
-    return ED_ERR_UNSUPPORTED;
-  }
-  float *xslo = lo ? reinterpret_cast<float *>(ws + xs_bytes + 16) : nullptr;
-  P.next = reinterpret_cast<uint32_t *>(ws + xs_bytes);
-  P.chunk_part = reinterpret_cast<double *>(ws + 16 + xs_bytes + lo_bytes);
-  const int eg = (int)pair_rules::expand_blocks(p->n_slots, (uint32_t)B->sm_count);
-  P.xs = ws;
-  P.xslo = xslo;
   P.lo_special = lo ? kSpecial : 0u;
   P.lo_same = lo ? 1u << kClassShift : 0u;
   P.n_slots = p->n_slots;
+  P.slot_idx = p->idx; P.slot_meta = p->meta; P.w = (const double2 *)p->w; P.wf = p->wf;
+  P.n_chunks = (p->n_slices + kRowThreads / 32 - 1) / (kRowThreads / 32);
+  P.n_sums = P.n_chunks * (mode == 1 ? 1 : kSumWarps);
+  // xs (and its remainders) for this call, from the basis's own pool in stream order, so
+  // calls on several streams or threads never share it; without memory for it the search
+  // kernel takes the call
+  char *ws = nullptr;
+  if (route == pair_rules::kExpanded) {
+    const size_t lo_bytes = lo ? al16(4 * ((size_t)p->n_slots + 1)) : 0;
+    const size_t n_sums = !rows || !partial ? 0 : (mode == 1 ? (size_t)B->n_classes : cplx ? 2 : 1) * P.n_sums;
+    if (cudaMallocFromPoolAsync((void **)&ws, 16 + xs_bytes + lo_bytes + 8 * n_sums, p->pool, st) != cudaSuccess) {
+      cudaGetLastError();
+      return ED_ERR_UNSUPPORTED;
+    }
+    P.xs = ws;
+    P.next = reinterpret_cast<uint32_t *>(ws + xs_bytes);
+    if (lo) P.xslo = reinterpret_cast<float *>(ws + 16 + xs_bytes);
+    P.chunk_part = reinterpret_cast<double *>(ws + 16 + xs_bytes + lo_bytes);
+  }
   int rc = ED_OK;
   switch (dtype) {
-#define PCASE(D, V)                                                                              \
-  case D:                                                                                        \
-    expand_kernel<V><<<eg, pair_rules::kExpandThreads, 0, st>>>((const V *)x, p->idx, p->meta, (const double2 *)p->w, p->wf, p->n_slots, (V *)ws, xslo, P.next); \
-    rc = cudaGetLastError() == cudaSuccess ? launch_pair_v<V>(B, P, chi, p->flips, rows, mode, st)      \
-                                           : ed_fail(ED_ERR_CUDA, "expand_kernel");              \
+#define PCASE(D, V)                                                     \
+  case D:                                                               \
+    rc = ws ? launch_expand<V>(B, P, st) : ED_OK;                       \
+    if (!rc) rc = launch_pair_v<V>(B, P, chi, p->flips, rows, mode, st); \
     break;
     PCASE(ED_F64, double)
     PCASE(ED_F32, float)
@@ -1808,8 +1854,10 @@ int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, c
 #undef PCASE
     default: rc = ed_fail(ED_ERR_INVALID, "unknown dtype");
   }
-  const cudaError_t fe = cudaFreeAsync(ws, st);
-  if (!rc && fe != cudaSuccess) rc = ed_cuda_fail(fe, "cudaFreeAsync");
+  if (ws) {
+    const cudaError_t fe = cudaFreeAsync(ws, st);
+    if (!rc && fe != cudaSuccess) rc = ed_cuda_fail(fe, "cudaFreeAsync");
+  }
   if (!rc && ylo_done) *ylo_done = P.ylo != nullptr;
   return rc;
 }

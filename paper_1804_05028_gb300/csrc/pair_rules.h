@@ -18,4 +18,36 @@ inline uint32_t expand_blocks(uint64_t n_slots, uint32_t sm_count) {
   return (uint32_t)(b < kExpandMaxBlocks ? b : kExpandMaxBlocks);
 }
 
+// How a product over `rows` rows (or the class expectations, over all of them) finds its terms.
+enum Route {
+  kSearch,     // the representative of every term by search: nothing to prepare
+  kDirect,     // coset arithmetic; a term reads its slot's index, its weight and x
+  kExpanded,   // coset arithmetic; x is first spread over all slots, then a term is one read
+};
+
+// Expanding costs a pass over the slots and a call to the memory pool, reading directly two more
+// accesses per term.  Measured (us, search / direct / expanded; GB300):
+//   3.2e7 states fp32, 16 rows 136 / 41 / 278, 2.6e5 rows 847 / 320 / 354, 1e6 2486 / 1272 / 655
+//   7.1e6 states c64 (chain), 16 rows 23 / 16 / 62, 2.6e5 rows 117 / 63 / 83, 1e6 334 / 180 / 151
+//   6.4e7 states c64, D/1024 rows 253 / 90 / 399, D/128 856 / 522 / 563, D/9 9712 / 11004 / 4084
+//   810 states fp64, all rows 31 / 12 / 15; 9252 states 45 / 14 / 15
+// so directly up to one term per four slots, and on sectors so small that the second launch
+// outweighs the reads: up to 2^14 slots and some fifteen terms per row (497 states c64 45 / 14 / 16),
+// but not in complex fp64 (497 states 58 / 21 / 17), whose products wait for the weights.
+// One-block splits read a term's representative from a whole table, and in complex fp32, where
+// coset arithmetic multiplies twice by a character, small sectors of few terms are done sooner
+// so: 9225 states 16.5 / 18 / 19 (fp32 17 / 12 / 15), class expectations 43 / 42.5 / 43.5.
+// At 8.6e8 states every read is a DRAM sector and the search is as fast for narrow ranges
+// (us, D/4096 rows 238 / 298 / 17384, D/9 82 / 145 / 77 ms).  Fewer rows than half a warp leave
+// both kernels waiting for one memory access after the other (775 states c64, 8 rows 12 / 12 / 15).
+inline Route route(int64_t rows, int64_t dim, double terms_per_row, uint64_t n_slots, bool complex_fp64,
+                   bool table_complex_fp32 = false) {
+  if (rows < 16) return kSearch;
+  if (table_complex_fp32 && n_slots <= 1u << 14 && terms_per_row <= 11.0) return kSearch;
+  if (dim > (int64_t)1 << 27) return rows >= dim / 8 ? kExpanded : kSearch;
+  if ((double)rows * terms_per_row <= 0.25 * (double)n_slots) return kDirect;
+  if (n_slots <= 1u << 14 && terms_per_row <= 15.0 && !complex_fp64) return kDirect;
+  return kExpanded;
+}
+
 }  // namespace pair_rules

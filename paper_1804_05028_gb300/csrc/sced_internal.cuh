@@ -337,6 +337,7 @@ struct ed_basis {
   std::vector<cudaEvent_t> chunk_done;  // one per row chunk of ed_apply_H_host
   double build_ms = 0;
   PairPlan *pair = nullptr;            // null: the split has no two stable halves
+  double terms_per_row = 0;            // exchange terms of a row: antiparallel bonds, on average
 };
 
 // error reporting (capi.cu)

@@ -125,6 +125,26 @@ def test_row_order(p):
             assert abs(got[c] - ref_c) <= tol * (xd.abs()[:-1] @ hc.abs()).item()
 
 
+DIRECT = [
+    T(6, momentum=(0, 0), point_irrep=1, J2=0.5, n_sublat=4, n_up=6), T(6, momentum=(1, 2), point_irrep=0, J2=0.5, n_sublat=4, n_up=6),
+    w.chain(28, 4, k=5, n_up=7), w.chain(30, 3, k=15, n_up=7), w.with_spin_flip(w.chain(24, 4, k=0, n_up=12), 1),
+    _sub(w.chain(28, 4, k=4, n_up=7), range(0, 28, 2), "chain28_even_translations"),
+]
+
+
+@pytest.mark.parametrize("p", DIRECT, ids=lambda p: f"{p.name}_up{p.n_up}")
+def test_direct_rows(p):
+    """Narrow ranges read x through the slots, the whole product expands it first: the same values
+    summed in the same order, so the same bits (16 rows: the fewest; 17 and 33: a ragged warp)."""
+    B = _basis(p)
+    D = B.dim
+    for dt in ([torch.float64, torch.float32] if B.is_real else []) + [torch.complex128, torch.complex64]:
+        x = _vec(D, dt, 6)
+        y = B.apply_H(x)
+        for r0, n in [(0, 16), (D // 3, 17), (D - 33, 33), (D // 2, 66)]:
+            assert torch.equal(B.apply_H_rows(x, r0, r0 + n), y[r0:r0 + n])
+
+
 def test_streams_and_capture():
     p = T(6, momentum=(0, 0), point_irrep=1, J2=0.5, n_sublat=4, n_up=6)
     B = _basis(p)

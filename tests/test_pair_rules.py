@@ -58,3 +58,22 @@ def test_emulation_sees_the_wrap(tmp_path):
     """Slots within one stride of 2^32 are what the bound keeps out."""
     out = run(tmp_path, LAST_STEP + 'int main() { printf("%d", ends(0xFFFFFF00ull, 152)); }')
     assert out == "0"
+
+
+def test_routes(tmp_path):
+    """Which way a product goes: s(earch), d(irect) or e(xpanded)."""
+    out = run(tmp_path, """
+static void q(int64_t rows, int64_t dim, double terms, uint64_t slots, bool c128 = false, bool tab = false) {
+  putchar("sde"[route(rows, dim, terms, slots, c128, tab)]);
+}
+int main() {
+  q(15, 15, 5, 20); q(15, 1 << 20, 10, 1 << 20);                         // less than half a warp
+  q(16, 16, 5, 20); q(810, 810, 8.5, 1100); q(810, 810, 8.5, 1100, true);   // small sectors
+  q(810, 810, 8.5, 1100, false, true); q(153, 153, 17, 300, false, true);   // one block, complex fp32
+  q(153, 153, 17, 300); q(16384, 16384, 10, 16385);
+  q(250000, 10000000, 10, 10000000); q(250001, 10000000, 10, 10000000);      // a term per four slots
+  const int64_t big = 1ll << 27;
+  q(16, big, 40, big); q(16, big + 8, 40, big); q(big / 8, big + 8, 40, big); q(big / 8 + 1, big + 8, 40, big);
+}
+""")
+    assert out == "ss" + "dde" + "se" + "ee" + "de" + "dsse"
