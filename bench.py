@@ -49,6 +49,7 @@ KERNEL_SOURCES = ["paper_1804_05028_gb300/csrc/apply.cu",
                   "paper_1804_05028_gb300/csrc/apply_fast.cu",
                   "paper_1804_05028_gb300/csrc/pair.cu",
                   "paper_1804_05028_gb300/csrc/pair_rules.h",
+                  "paper_1804_05028_gb300/csrc/character.h",
                   "paper_1804_05028_gb300/csrc/sced_internal.cuh",
                   "paper_1804_05028_gb300/csrc/dfloat.cuh",
                   "paper_1804_05028_gb300/csrc/basis.cu",

@@ -12,6 +12,7 @@
 // the counter reset and the launch are replayed from a captured CUDA graph.  The number
 // of rows per work item is picked by timing a few candidates on the first call.
 #include "sced_internal.cuh"
+#include "character.h"
 
 #include <algorithm>
 #include <cmath>
@@ -572,8 +573,9 @@ int build_orbits(ed_batch *Bt) {
     chi_at[s] = chi.size();
     if (!B->is_real)
       for (int g = 0; g < B->nsym; g++) {
-        const double a = 2.0 * M_PI * (double)B->phase[g] / (double)B->denom;
-        chi.push_back(make_float2((float)std::cos(a), (float)std::sin(a)));
+        double c, s1;
+        ed_character(B->phase[g], B->denom, &c, &s1);
+        chi.push_back(make_float2((float)c, (float)s1));
       }
   }
   uint32_t *d_maps = maps ? (uint32_t *)get(4 * maps) : nullptr;
@@ -672,9 +674,10 @@ extern "C" int ed_batch_create(ed_basis *const *bases, int32_t n, const double *
     for (int t = 0; t <= B->nsym; t++) ftab.push_back((float)std::sqrt((double)t));
     for (int t = 0; t <= B->nsym; t++) ftab.push_back(t ? (float)(1.0 / std::sqrt((double)t)) : 0.f);
     for (int q = 0; q < B->denom; q++) {
-      const double a = 2.0 * M_PI * (double)q / (double)B->denom;
-      ftab.push_back((float)std::cos(a));
-      ftab.push_back((float)std::sin(a));
+      double c, s1;
+      ed_character(q, B->denom, &c, &s1);
+      ftab.push_back((float)c);
+      ftab.push_back((float)s1);
     }
   }
   if (ed_malloc(&Bt->d_sec, sizeof(BatchSector) * n) != cudaSuccess ||

@@ -3,6 +3,7 @@
 // H x entry points and the Lanczos driver (Sec. IV: the product dominates; dots,
 // scalings and the tridiagonal eigenproblem are cheap and stay simple).
 #include "sced_internal.cuh"
+#include "character.h"
 #include <algorithm>
 #include <chrono>
 #include <cmath>
@@ -289,11 +290,7 @@ void add_norm_tables(ed_basis *B, TableSet &tabs) {
   auto up = [&](void **dst, const void *src, size_t n) { tabs.add(dst, src, n); };
   std::vector<double> sq(ns + 1), rs(ns + 1), cs(2 * (size_t)B->denom);
   for (int t = 0; t <= ns; t++) { sq[t] = std::sqrt((double)t); rs[t] = t ? 1.0 / std::sqrt((double)t) : 0.0; }
-  for (int k = 0; k < B->denom; k++) {
-    const double a = 2.0 * M_PI * (double)k / (double)B->denom;
-    cs[2 * k] = std::cos(a);
-    cs[2 * k + 1] = std::sin(a);
-  }
+  for (int k = 0; k < B->denom; k++) ed_character(k, B->denom, &cs[2 * k], &cs[2 * k + 1]);
   up((void **)&B->d_sqrt, sq.data(), sq.size() * 8);
   up((void **)&B->d_rsqrt, rs.data(), rs.size() * 8);
   up((void **)&B->d_cs, cs.data(), cs.size() * 8);

@@ -43,6 +43,7 @@
 // every term across the halves is one 32-byte sector from L2.
 #include "sced_internal.cuh"
 #include "dfloat.cuh"
+#include "character.h"
 #include "pair_rules.h"
 #include <algorithm>
 #include <cmath>
@@ -1517,8 +1518,9 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
   std::vector<float4> wtf(n_w);                    // and as pairs of fp32 words
   for (size_t t = 0; t < divs.size(); t++)
     for (int q = 0; q < B->denom; q++) {
-      const double a = 2.0 * M_PI * (double)q / (double)B->denom, r = std::sqrt((double)divs[t]);
-      double c = std::cos(a), s = std::sin(a);
+      const double r = std::sqrt((double)divs[t]);
+      double c, s;
+      ed_character(q, B->denom, &c, &s);
       if (B->is_real) { c = q ? -1.0 : 1.0; s = 0.0; }
       wt[2 * (t * B->denom + q)] = r * c;
       wt[2 * (t * B->denom + q) + 1] = r * s;
@@ -1533,9 +1535,7 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
     for (size_t j = 0; j < nl; j++) {
       const int g = half ? listB[j] : listA[j];
       const uint32_t e = (half ? codeB[j] : codeA[j]) & (kElem | kFlip);
-      const double a = 2.0 * M_PI * (double)B->phase[g] / (double)B->denom;
-      chi[2 * (512 * half + e)] = std::cos(a);
-      chi[2 * (512 * half + e) + 1] = std::sin(a);
+      ed_character(B->phase[g], B->denom, &chi[2 * (512 * half + e)], &chi[2 * (512 * half + e) + 1]);
     }
   // bonds as flipped bits of the two halves
   std::vector<uint2> bond(B->bond_pad.size() / 2, make_uint2(0, 0));
