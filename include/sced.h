@@ -190,6 +190,20 @@ int ed_apply_H(const ed_basis *basis, const double *J, const double *Jz, const v
 int ed_apply_H_rows(const ed_basis *basis, const double *J, const double *Jz, const void *x,
                     void *y, int32_t dtype, int64_t row_begin, int64_t row_end, void *stream);
 
+/* Which kernel a product takes (ed_apply_route). */
+#define ED_ROUTE_SEARCH 0      /* the representative of every term by search */
+#define ED_ROUTE_DIRECT 1      /* coset arithmetic; terms read x through the slots' indices */
+#define ED_ROUTE_EXPANDED 2    /* coset arithmetic on x spread over the slots, rows in basis order */
+#define ED_ROUTE_SLOT_ORDER 3  /* the same, rows in slot order */
+
+/*
+ * ed_apply_route -- which of them a product over rows [row_begin, row_end) takes (classes != 0:
+ * ed_expect_classes, over all rows) while device memory for its scratch is there; a test hook,
+ * computed on the host.  *route: one of ED_ROUTE_*.  Errors: ED_ERR_INVALID (as ed_apply_H_rows).
+ */
+int ed_apply_route(const ed_basis *basis, int32_t dtype, int64_t row_begin, int64_t row_end,
+                   int32_t classes, int32_t *route);
+
 /*
  * ed_apply_H_host -- ed_apply_H on HOST arrays x, y (dim elements of dtype): copies x
  * to device staging buffers owned by the basis, runs the product, copies y back.  Sectors

@@ -27,7 +27,7 @@ REORTH = {"local": 0, "none": 1, "full": 2}
 LIB_PATH = _build.LIB
 # every function declared in include/sced.h
 SYMBOLS = ["ed_build_basis", "ed_free_basis", "ed_basis_info", "ed_basis_export",
-           "ed_find_rep", "ed_apply_H", "ed_apply_H_rows", "ed_apply_H_host", "ed_lanczos",
+           "ed_find_rep", "ed_apply_H", "ed_apply_H_rows", "ed_apply_route", "ed_apply_H_host", "ed_lanczos",
            "ed_dot", "ed_count_terms", "ed_expect_classes", "ed_dot_noalloc", "ed_batch_create",
            "ed_batch_set_vectors", "ed_batch_apply", "ed_batch_info", "ed_batch_free",
            "ed_axpy_norm", "ed_scale", "ed_last_error", "ed_version"]
@@ -119,6 +119,7 @@ def lib():
             L.ed_find_rep.argtypes = [vp, vp, i64, i32, vp, vp, vp, vp, vp, vp]
             L.ed_apply_H.argtypes = [vp, vp, vp, vp, vp, i32, vp]
             L.ed_apply_H_rows.argtypes = [vp, vp, vp, vp, vp, i32, i64, i64, vp]
+            L.ed_apply_route.argtypes = [vp, i32, i64, i64, i32, ctypes.POINTER(i32)]
             L.ed_apply_H_host.argtypes = [vp, vp, vp, vp, vp, i32, vp]
             L.ed_lanczos.argtypes = [vp, vp, vp, vp, vp]
             L.ed_dot.argtypes = [vp, vp, vp, i32, vp, vp]
@@ -300,6 +301,16 @@ class Basis:
         _check(lib().ed_apply_H_rows(self._h, cJ, cJz, px, py, _dtype_code(x),
                                      int(row_begin), int(row_end), _stream(stream)))
         return y
+
+    def apply_route(self, dtype, row_begin=0, row_end=None, classes=False) -> str:
+        """Which kernel a product of this torch dtype over these rows takes ("search",
+        "direct", "expanded" or "slot order"); a test hook."""
+        import torch
+        route = ctypes.c_int32()
+        end = self.dim if row_end is None else row_end
+        _check(lib().ed_apply_route(self._h, _dtype_code(torch.empty(0, dtype=dtype)), int(row_begin), int(end),
+                                    int(classes), ctypes.byref(route)))
+        return ("search", "direct", "expanded", "slot order")[route.value]
 
     def apply_H_host(self, x, y=None, J=None, Jz=None, stream=None):
         """y = H x for HOST numpy arrays (or pinned CPU tensors); copies inside the call."""

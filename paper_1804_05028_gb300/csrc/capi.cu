@@ -688,6 +688,16 @@ extern "C" int ed_apply_H(const ed_basis *B, const double *J, const double *Jz, 
   return ed_apply_H_rows(B, J, Jz, x, y, dtype, 0, B->D, stream);
 }
 
+extern "C" int ed_apply_route(const ed_basis *B, int32_t dtype, int64_t r0, int64_t r1, int32_t classes,
+                              int32_t *route) {
+  if (!B || !route) return ed_fail(ED_ERR_INVALID, "null argument");
+  const int rc = check_dtype(B, dtype);
+  if (rc) return rc;
+  if (r0 < 0 || r1 > B->D || r0 > r1) return ed_fail(ED_ERR_INVALID, "row range outside the basis");
+  *route = ed_pair_route(B, dtype, r0, r1, classes ? 1 : 0);
+  return ED_OK;
+}
+
 extern "C" int ed_apply_H_host(ed_basis *B, const double *J, const double *Jz, const void *xh,
                                void *yh, int32_t dtype, void *stream) {
   if (!B || !J || !Jz) return ed_fail(ED_ERR_INVALID, "null argument");

@@ -1748,25 +1748,65 @@ int launch_pair_v(const ed_basis *B, PairParams &P, bool chi, bool flips, bool r
   return mode == 1 ? launch_pair_m<V, 1>(B, P, chi, flips, rows, st) : launch_pair_m<V, 0>(B, P, chi, flips, rows, st);
 }
 
+// Shared memory of a block, as offsets in P and in bytes.
+size_t pair_layout(const ed_basis *B, bool cplx, bool chi, bool rows, PairParams &P) {
+  const PairPlan *p = B->pair;
+  size_t off = 0;
+  auto put = [&](uint32_t &o, size_t bytes) { o = (uint32_t)off; off += al16(bytes); };
+  int words = 0;
+  for (int c = 0; c < B->n_classes; c++) words = std::max(words, B->cls_word[c + 1] - B->cls_word[c]);
+  put(P.off_off, 4 * (size_t)p->n_cls);
+  put(P.off_mult, p->mult_bytes);
+  put(P.off_bond, 8 * 32 * (size_t)B->cls_word[B->n_classes]);
+  put(P.off_rs, 8 * ((size_t)B->nsym + 1));
+  put(P.off_chi, chi ? 16 * 1024 : 0);
+  if (rows) {
+    put(P.off_rt, 4 * (size_t)p->rt_words);
+    put(P.off_mask, 4 * std::max<size_t>(p->rt_across, cplx ? 4 : 2) * kRowThreads);   // or a row's <x, y>
+    P.n_tab = p->K >= 32 ? 2 : 0;   // 32 rows span two classes at most (without stabilisers)
+    P.et_words = (uint32_t)(65 * p->rt_wa + P.n_tab * (32 * (p->rt_w - p->rt_wa) + p->m) + 3) / 4 * 4;
+    put(P.off_et, 4 * (size_t)P.et_words * (kRowThreads / 32));
+  } else {
+    put(P.off_nib, 4 * B->nib.size());
+    put(P.off_hx, p->blocks ? 0 : 128 * (size_t)B->n_nib);
+    put(P.off_mask, 4 * (size_t)words * kThreads);
+  }
+  P.smem_bytes = (uint32_t)off;
+  return off;
+}
+
+size_t elem_bytes(int dtype) { return dtype == ED_F32 ? 4 : dtype == ED_C128 ? 16 : 8; }
+
 }  // namespace
+
+int ed_pair_route(const ed_basis *B, int dtype, int64_t r0, int64_t r1, int mode) {
+  const PairPlan *p = B->pair;
+  if (!p || r1 <= r0) return ED_ROUTE_SEARCH;
+  const bool cplx = dtype == ED_C128 || dtype == ED_C64, chi = cplx && !B->is_real;
+  const pair_rules::Route way = pair_rules::route(r1 - r0, B->D, B->terms_per_row, p->n_slots, dtype == ED_C128,
+                                                  B->T.full && mode == 0 && !B->is_real && dtype == ED_C64);
+  PairParams P{};
+  if (way == pair_rules::kSearch || pair_layout(B, cplx, chi, false, P) > kPairMaxSmem) return ED_ROUTE_SEARCH;
+  if (way == pair_rules::kDirect) return ED_ROUTE_DIRECT;
+  const size_t least = p->rt_w > p->rt_wa ? kRowOrderMinBytes : kRowOrderMinBytesAcross;
+  if (p->n_slices && r0 == 0 && r1 == B->D && al16(elem_bytes(dtype) * ((size_t)p->n_slots + 1)) >= least &&
+      pair_layout(B, cplx, chi, true, P) <= kRowsMaxSmem)
+    return ED_ROUTE_SLOT_ORDER;
+  return ED_ROUTE_EXPANDED;
+}
 
 int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, const void *x, void *y,
                          int dtype, int64_t r0, int64_t r1, double *partial, cudaStream_t st, int mode,
                          void *ylo, bool *ylo_done) {
   const PairPlan *p = B->pair;
-  if (!p) return ED_ERR_UNSUPPORTED;
-  const pair_rules::Route route = pair_rules::route(r1 - r0, B->D, B->terms_per_row, p->n_slots, dtype == ED_C128,
-                                                    B->T.full && mode == 0 && !B->is_real && dtype == ED_C64);
-  if (route == pair_rules::kSearch) return ED_ERR_UNSUPPORTED;
-  const size_t es = dtype == ED_F64 ? 8 : dtype == ED_F32 ? 4 : dtype == ED_C128 ? 16 : 8;
-  const size_t xs_bytes = al16(es * ((size_t)p->n_slots + 1));
-  const bool rows = route == pair_rules::kExpanded && p->n_slices && r0 == 0 && r1 == B->D && xs_bytes >= (p->rt_w > p->rt_wa ? kRowOrderMinBytes : kRowOrderMinBytesAcross);
+  int route = ed_pair_route(B, dtype, r0, r1, mode);
+  if (route == ED_ROUTE_SEARCH) return ED_ERR_UNSUPPORTED;
+  bool rows = route == ED_ROUTE_SLOT_ORDER;
+  const size_t xs_bytes = al16(elem_bytes(dtype) * ((size_t)p->n_slots + 1));
   PairParams P{};
   P.n_classes = B->n_classes;
-  int words = 0;
   for (int c = 0; c <= B->n_classes; c++) P.cls_word[c] = B->cls_word[c];
   for (int c = 0; c < B->n_classes; c++) {
-    words = std::max(words, B->cls_word[c + 1] - B->cls_word[c]);
     P.nb_cls[c] = B->cls_off[c + 1] - B->cls_off[c];
     P.jh[c] = 0.5 * J[c];
     P.jzq[c] = 0.25 * J[c] * Jz[c];
@@ -1785,7 +1825,7 @@ int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, c
   const bool chi = cplx && !B->is_real;
   P.chi = p->chi;
   P.basis = B->d_basis; P.stab = B->d_stab;
-  P.up = p->up; P.t_up = p->t_up; P.ubase = p->ubase; P.rt = p->rt; P.rt_words = p->rt_words;
+  P.up = p->up; P.t_up = p->t_up; P.ubase = p->ubase; P.n_ucls = p->n_ucls; P.rt = p->rt; P.rt_words = p->rt_words;
   memcpy(P.kw, p->kw, sizeof(P.kw));
   P.n_w = p->rt_w; P.n_wa = p->rt_wa; P.n_up = B->n_up; P.no_swap = p->no_swap; P.by_popcount = !p->any_flip;
   P.n_hnib = p->n_hnib; P.m = (uint32_t)p->m;
@@ -1795,28 +1835,7 @@ int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, c
   P.row_b = p->row_b; P.row_i = p->row_i; P.row_m = p->row_m; P.rw = (const double2 *)p->rw;
   P.x = x; P.y = y; P.r0 = r0; P.r1 = r1; P.partial = partial;
   P.ylo = (dtype == ED_F32 || dtype == ED_C64) ? ylo : nullptr;
-  size_t off = 0;
-  auto put = [&](uint32_t &o, size_t bytes) { o = (uint32_t)off; off += al16(bytes); };
-  const size_t n_words = (size_t)B->cls_word[B->n_classes];
-  put(P.off_off, 4 * (size_t)P.n_cls);
-  put(P.off_mult, P.mult_bytes);
-  put(P.off_bond, 8 * 32 * n_words);
-  put(P.off_rs, 8 * (size_t)P.n_sq);
-  put(P.off_chi, chi ? 16 * 1024 : 0);
-  if (rows) {
-    put(P.off_rt, 4 * (size_t)P.rt_words);
-    put(P.off_mask, 4 * std::max<size_t>(p->rt_across, cplx ? 4 : 2) * kRowThreads);   // or a row's <x, y>
-    P.n_ucls = p->n_ucls;
-    P.n_tab = P.K >= 32 ? 2 : 0;   // 32 rows span two classes at most (without stabilisers)
-    P.et_words = (uint32_t)(65 * p->rt_wa + P.n_tab * (32 * (p->rt_w - p->rt_wa) + p->m) + 3) / 4 * 4;
-    put(P.off_et, 4 * (size_t)P.et_words * (kRowThreads / 32));
-  } else {
-    put(P.off_nib, 4 * B->nib.size());
-    put(P.off_hx, p->blocks ? 0 : 128 * (size_t)B->n_nib);
-    put(P.off_mask, 4 * (size_t)words * kThreads);
-  }
-  P.smem_bytes = (uint32_t)off;
-  if (off > (rows ? kRowsMaxSmem : kPairMaxSmem)) return ED_ERR_UNSUPPORTED;
+  pair_layout(B, cplx, chi, rows, P);
   const bool lo = dtype == ED_F32 && p->weights;
   P.lo_special = lo ? kSpecial : 0u;
   P.lo_same = lo ? 1u << kClassShift : 0u;
@@ -1825,20 +1844,24 @@ int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, c
   P.n_chunks = (p->n_slices + kRowThreads / 32 - 1) / (kRowThreads / 32);
   P.n_sums = P.n_chunks * (mode == 1 ? 1 : kSumWarps);
   // xs (and its remainders) for this call, from the basis's own pool in stream order, so
-  // calls on several streams or threads never share it; without memory for it the search
-  // kernel takes the call
+  // calls on several streams or threads never share it.  Without memory for it terms read x
+  // through the slots; the largest sectors are searched sooner than that (pair_rules.h).
   char *ws = nullptr;
-  if (route == pair_rules::kExpanded) {
+  if (route != ED_ROUTE_DIRECT) {
     const size_t lo_bytes = lo ? al16(4 * ((size_t)p->n_slots + 1)) : 0;
     const size_t n_sums = !rows || !partial ? 0 : (mode == 1 ? (size_t)B->n_classes : cplx ? 2 : 1) * P.n_sums;
     if (cudaMallocFromPoolAsync((void **)&ws, 16 + xs_bytes + lo_bytes + 8 * n_sums, p->pool, st) != cudaSuccess) {
       cudaGetLastError();
-      return ED_ERR_UNSUPPORTED;
+      ws = nullptr;
+      if (B->D > pair_rules::kMaxDirectDim) return ED_ERR_UNSUPPORTED;
+      rows = false;
+      pair_layout(B, cplx, chi, false, P);
+    } else {
+      P.xs = ws;
+      P.next = reinterpret_cast<uint32_t *>(ws + xs_bytes);
+      if (lo) P.xslo = reinterpret_cast<float *>(ws + 16 + xs_bytes);
+      P.chunk_part = reinterpret_cast<double *>(ws + 16 + xs_bytes + lo_bytes);
     }
-    P.xs = ws;
-    P.next = reinterpret_cast<uint32_t *>(ws + xs_bytes);
-    if (lo) P.xslo = reinterpret_cast<float *>(ws + 16 + xs_bytes);
-    P.chunk_part = reinterpret_cast<double *>(ws + 16 + xs_bytes + lo_bytes);
   }
   int rc = ED_OK;
   switch (dtype) {

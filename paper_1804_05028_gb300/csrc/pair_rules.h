@@ -40,11 +40,13 @@ enum Route {
 // At 8.6e8 states every read is a DRAM sector and the search is as fast for narrow ranges
 // (us, D/4096 rows 238 / 298 / 17384, D/9 82 / 145 / 77 ms).  Fewer rows than half a warp leave
 // both kernels waiting for one memory access after the other (775 states c64, 8 rows 12 / 12 / 15).
+constexpr int64_t kMaxDirectDim = (int64_t)1 << 27;
+
 inline Route route(int64_t rows, int64_t dim, double terms_per_row, uint64_t n_slots, bool complex_fp64,
                    bool table_complex_fp32 = false) {
   if (rows < 16) return kSearch;
   if (table_complex_fp32 && n_slots <= 1u << 14 && terms_per_row <= 11.0) return kSearch;
-  if (dim > (int64_t)1 << 27) return rows >= dim / 8 ? kExpanded : kSearch;
+  if (dim > kMaxDirectDim) return rows >= dim / 8 ? kExpanded : kSearch;
   if ((double)rows * terms_per_row <= 0.25 * (double)n_slots) return kDirect;
   if (n_slots <= 1u << 14 && terms_per_row <= 15.0 && !complex_fp64) return kDirect;
   return kExpanded;

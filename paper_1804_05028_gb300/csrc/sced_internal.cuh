@@ -442,9 +442,11 @@ int ed_launch_apply_fast(const ed_basis *B, const double *J, const double *Jz, c
                          void *y, int dtype, int64_t r0, int64_t r1, double *partial,
                          cudaStream_t st, int mode, void *ylo = nullptr, bool *ylo_done = nullptr);
 // pair.cu: the coset-arithmetic product, its tables (built once per basis) and their release;
-// ed_launch_apply_pair returns ED_ERR_UNSUPPORTED when the sector has no plan
+// ed_launch_apply_pair returns ED_ERR_UNSUPPORTED when the search kernels take the call
 int ed_build_pair(ed_basis *B, cudaStream_t st);
 void ed_free_pair(ed_basis *B);
+// the ED_ROUTE_* of a product (mode 0) or of the class expectations (mode 1)
+int ed_pair_route(const ed_basis *B, int dtype, int64_t r0, int64_t r1, int mode);
 int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, const void *x, void *y,
                          int dtype, int64_t r0, int64_t r1, double *partial, cudaStream_t st, int mode,
                          void *ylo, bool *ylo_done);

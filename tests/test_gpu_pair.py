@@ -204,3 +204,48 @@ def test_threads_with_other_table_sizes():
         for t in threads:
             t.join()
     assert not errors, errors
+
+
+def _searched(B, x, y, tol, n=48):
+    """Rows of y against the search kernels, which take ranges of fewer than 16 rows and share no
+    table with the coset arithmetic but the basis."""
+    D, scale = B.dim, y.abs().max()
+    assert B.apply_route(x.dtype, 0, 15) == "search"
+    for r0 in np.linspace(0, D - 15, n).astype(np.int64).tolist():
+        assert (B.apply_H_rows(x, r0, r0 + 15) - y[r0:r0 + 15]).abs().max() <= tol * scale
+
+
+def test_tables_too_wide_for_the_slot_order():
+    """Third-neighbour bonds and complex characters on the 40-site cluster: the slot order would
+    need 209 KB of shared memory, the rows in basis order 93; with two couplings it fits."""
+    two = w.tilted_square_40(momentum=(0, 0), point_irrep=1, n_sublat=4, J2=0.5, n_up=10)
+    cl = w._Cluster((6, 2), (-2, 6))
+    at = {cl.key(int(x), int(y)): lab for lab, (x, y) in enumerate(two.coords)}
+    third = [(lab, at[cl.key(int(x) + dx, int(y) + dy)]) for lab, (x, y) in enumerate(two.coords) for dx, dy in ((2, 0), (0, 2))]
+    three = dataclasses.replace(two, bonds=np.concatenate([two.bonds, np.array(third, np.int32)]),
+                                bond_class=np.concatenate([two.bond_class, np.full(len(third), 2, np.int32)]),
+                                n_classes=3, J=(1.0, 0.5, 0.3), Jz=(1.0, 0.8, 0.6))
+    for p, route in ((two, "slot order"), (three, "expanded")):
+        B = _basis(p)
+        for dt, tol in ((torch.complex64, 2e-6), (torch.complex128, 1e-12)):
+            assert B.apply_route(dt) == route and B.apply_route(dt, classes=True) == route
+            x = _vec(B.dim, dt, 7)
+            _searched(B, x, B.apply_H(x), tol)
+        B.close()
+
+
+def test_product_without_scratch():
+    """Where the pool has no room for x over the slots, terms read it through their indices: the
+    same bits as in basis order."""
+    B = _basis(w.chain(32, 4, k=0, n_up=14))          # 59 MB; builds leave up to 64 MB for the widest type in the pool
+    x = _vec(B.dim, torch.float32, 8)
+    y, z = torch.empty_like(x), torch.empty_like(x)
+    assert B.apply_route(torch.float32) == "expanded"
+    torch.cuda.synchronize()
+    hold = torch.empty(torch.cuda.mem_get_info()[0] - (8 << 20), dtype=torch.uint8, device="cuda")
+    B.apply_H(x, y)
+    torch.cuda.synchronize()
+    left = torch.cuda.mem_get_info()[0]
+    del hold
+    torch.cuda.empty_cache()
+    assert torch.equal(B.apply_H(x, z), y) and left <= 16 << 20
