@@ -1,11 +1,13 @@
 """The coset-arithmetic product (csrc/pair.cu) at the edges of what it accepts: halves made of
-the split's blocks or of a colouring of the bonds, halves that are exchanged by an involution, by none, or by no element at
-all, spin flips (as a factor of the group and tied to other elements), trivial, sign and
-complex characters, fillings whose halves hold no or all spins, every vector type, row ranges
-on both sides of the size rule, several streams at once and a captured call.  Reference: the
-oracle's explicit matrix.  Bounds: as in test_gpu_parity, a row sums at most a few hundred
-terms of size max|J| |x|, so fp64 stays near 1e-15 relative (1e-12 asked) and fp32 within a
-few roundings (2e-6 asked)."""
+the split's blocks or of a colouring of the bonds, halves that are exchanged by an involution,
+by other elements only or by none, spin flips (as a factor of the group and tied to other
+elements), trivial, sign and complex characters, fillings whose halves hold no or all spins,
+every vector type, row ranges on both sides of the size rules, each of the ways a product is
+taken (asked for, so that a rule that moves does not empty a test), several streams and host
+threads at once and a captured call.  Reference: the oracle's explicit matrix on small sectors,
+on large ones the search kernels.  Bounds: as in test_gpu_parity, a row sums at most a few
+hundred terms of size max|J| |x|, so fp64 stays near 1e-15 relative (1e-12 asked) and fp32
+within a few roundings (2e-6 asked)."""
 import dataclasses
 
 import numpy as np
@@ -77,37 +79,86 @@ def test_product_of_every_type(p):
             hc = oracle.hamiltonian(p.with_couplings(J, p.Jz))[0] @ xd
             scale = np.abs(xd) @ np.abs(hc) + np.abs(xd) @ np.abs(xd)
             assert abs(got[c] - np.vdot(xd, hc).real) <= (2e-6 if tol > 1e-9 * np.abs(ref).max() else 1e-12) * scale
-        # the rows of a range: most of them, the fewest that this product takes, one less
+        # the rows of a range: most of them, the fewest that coset arithmetic takes, one less
         for r0, r1 in [(B.dim // 5, B.dim - B.dim // 7), (B.dim // 2, B.dim // 2 + 16), (B.dim // 2, B.dim // 2 + 15)]:
             r1 = min(r1, B.dim)
             if r0 < r1:
                 assert np.abs(B.apply_H_rows(x, r0, r1).cpu().numpy() - ref[r0:r1]).max() <= tol
 
 
+def _searched(B, x, y, tol, n=48):
+    """Rows of y against the search kernels, which take ranges of fewer than 16 rows and share no
+    table with the coset arithmetic but the basis."""
+    D, scale = B.dim, y.abs().max()
+    assert B.apply_route(x.dtype, 0, 15) == "search"
+    for r0 in np.linspace(0, D - 15, n).astype(np.int64).tolist():
+        assert (B.apply_H_rows(x, r0, r0 + 15) - y[r0:r0 + 15]).abs().max() <= tol * scale
+
+
+def _ops(p, even, odd):
+    """The elements of a 6x6 group whose translation keeps the checkerboard and whose point
+    operation is in `even`, or exchanges it and is in `odd`; operation of each."""
+    sel, ops = [], []
+    for g, name in enumerate(p.sym_names):
+        op, t = name.split("+t")
+        if op in (odd if sum(eval(t)) % 2 else even):
+            sel.append(g)
+            ops.append(op)
+    return sel, ops
+
+
+def _no_involution(n_up):
+    """Quarter turns about plaquettes, which exchange the checkerboard halves and square to half
+    turns, half turns and translations inside the halves; characters i^(quarter turns)."""
+    p = T(6, momentum=(0, 0), point_irrep=0, J2=0.5, n_sublat=4, n_up=n_up)
+    sel, ops = _ops(p, ("E", "C2"), ("C4", "C4^3"))
+    q = _sub(p, sel, "square36_quarter_turns")
+    turns = {"E": 0, "C4": 1, "C2": 2, "C4^3": 3}
+    return dataclasses.replace(q, phase_denom=4, phase_num=np.array([turns[o] for o in ops], np.int32))
+
+
+def _halves_kept(momentum, n_up):
+    p = T(6, momentum=momentum, point_irrep=1, J2=0.5, n_sublat=4, n_up=n_up)
+    return _sub(p, _ops(p, w.C4V_NAMES, ())[0], f"square36_k{momentum}_halves_kept")
+
+
+# what the slot order distinguishes: characters (signs or complex), tables for two upper classes
+# per slice (32 or more elements between the halves) or none, an involution that exchanges the
+# halves, another exchange (a second multiplication table) or none, spin flips as a factor of the
+# group or tied to its elements, halves of blocks or of colours; and the types that reach it
+ALL = [torch.float64, torch.float32, torch.complex128, torch.complex64]
 LARGE = [
-    T(6, momentum=(0, 0), point_irrep=1, J2=0.5, n_sublat=4, n_up=12),           # signs
-    w.chain(32, 4, k=5, n_up=11),                                                  # no involution
-    w.with_spin_flip(w.chain(32, 4, k=0, n_up=16), 1),
-    _sub(w.chain(28, 4, k=4, n_up=9), range(0, 28, 2), "chain28_even_translations"),  # no exchange
-    w.chain(30, 3, k=7, n_up=12),                                                  # halves across blocks
+    (T(6, momentum=(0, 0), point_irrep=1, J2=0.5, n_sublat=4, n_up=12), ALL),
+    (T(6, momentum=(1, 1), point_irrep=1, J2=0.5, n_sublat=4, n_up=11), ALL[2:]),
+    (T(6, momentum=(1, 2), point_irrep=0, J2=0.5, n_sublat=4, n_up=10), ALL[2:]),
+    (_no_involution(11), ALL[2:]),
+    (w.chain(32, 4, k=5, n_up=12), ALL[2:3]),
+    (_halves_kept((0, 0), 12), ALL),
+    (_halves_kept((1, 1), 10), ALL[2:]),
+    (w.with_spin_flip(w.chain(32, 4, k=0, n_up=16), 1), [torch.float64, torch.complex64]),
+    (w.with_spin_flip(w.chain(32, 4, k=5, n_up=16), 0), ALL[2:]),
+    (dataclasses.replace(w.chain(32, 4, k=3, n_up=16), flip=(np.arange(32) % 2).astype(np.uint8), name="chain32_flip_tied"), ALL[2:]),
+    (w.chain(36, 3, k=7, n_up=11), ALL[2:]),
 ]
 
 
-@pytest.mark.parametrize("p", LARGE, ids=lambda p: f"{p.name}_up{p.n_up}")
-def test_row_order(p):
-    """Sectors large enough for the row order by lower class (the whole product) against their
-    row ranges in basis order: the same terms summed in another order."""
+@pytest.mark.parametrize("p,types", LARGE, ids=lambda v: f"{v.name}_up{v.n_up}" if hasattr(v, "n_up") else "")
+def test_row_order(p, types):
+    """Whole products in slot order against the search kernels on sampled rows, and against row
+    ranges in basis order everywhere: the same terms summed in another order."""
     B = _basis(p)
     D = B.dim
-    assert D >= 1 << 18
-    for dt in ([torch.float64, torch.float32] if B.is_real else []) + [torch.complex128, torch.complex64]:
+    for dt in types:
+        assert B.apply_route(dt) == "slot order" and B.apply_route(dt, classes=True) == "slot order"
         x = _vec(D, dt, 4)
         y = B.apply_H(x)
-        cut = D // 3 + 1
-        ref = torch.cat([B.apply_H_rows(x, 0, cut), B.apply_H_rows(x, cut, D)])
         tol = 2e-6 if dt in (torch.float32, torch.complex64) else 1e-12
+        _searched(B, x, y, tol)
+        cut = D // 3 + 1
+        assert B.apply_route(dt, 0, cut) == "expanded"
+        ref = torch.cat([B.apply_H_rows(x, 0, cut), B.apply_H_rows(x, cut, D)])
         assert (y - ref).abs().max() <= tol * ref.abs().max()
-        mid = B.apply_H_rows(x, D // 2, D // 2 + 1001)      # a narrow range, x expanded whole
+        mid = B.apply_H_rows(x, D // 2, D // 2 + 1001)      # a narrow range
         assert (y[D // 2:D // 2 + 1001] - mid).abs().max() <= tol * ref.abs().max()
         got = B.expect_classes(x)
         # blocks take the rows in any order, the sums come out the same
@@ -123,6 +174,7 @@ def test_row_order(p):
             last = B.apply_H_rows(x, D - 1, D, J=J).to(torch.complex128)
             ref_c += (xd[-1].conj() * last[0]).real.item()
             assert abs(got[c] - ref_c) <= tol * (xd.abs()[:-1] @ hc.abs()).item()
+    B.close()
 
 
 DIRECT = [
@@ -204,15 +256,6 @@ def test_threads_with_other_table_sizes():
         for t in threads:
             t.join()
     assert not errors, errors
-
-
-def _searched(B, x, y, tol, n=48):
-    """Rows of y against the search kernels, which take ranges of fewer than 16 rows and share no
-    table with the coset arithmetic but the basis."""
-    D, scale = B.dim, y.abs().max()
-    assert B.apply_route(x.dtype, 0, 15) == "search"
-    for r0 in np.linspace(0, D - 15, n).astype(np.int64).tolist():
-        assert (B.apply_H_rows(x, r0, r0 + 15) - y[r0:r0 + 15]).abs().max() <= tol * scale
 
 
 def test_tables_too_wide_for_the_slot_order():
