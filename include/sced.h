@@ -104,7 +104,9 @@ typedef struct {
   int32_t postfix_bits;       /* bits compared by the in-bucket binary search */
   int64_t n_keys;             /* Limits buckets */
   int64_t max_bucket;         /* largest bucket */
-  int64_t table_bytes;        /* device bytes of Rep/Sym/SymmetryAction tables */
+  int64_t table_bytes;        /* device bytes of Rep/Sym/SymmetryAction tables and, for coset
+                                 arithmetic, of its tables and one call's scratch (the pool of a
+                                 large basis keeps up to twice that scratch) */
   int64_t index_bytes;        /* device bytes of the prefix rank table, Limits and postfixes */
   int64_t basis_bytes;        /* device bytes of Basis and |Stab| */
   int64_t sym_list_len;       /* total entries of the Sym_X lists */
@@ -167,9 +169,11 @@ int ed_find_rep(const ed_basis *basis, const uint64_t *states, int64_t n, int32_
  * coding, the representative's x_j, and y_i += (J/2) chi(h) sqrt(|Stab_j|/|Stab_i|) x_j.
  * Sectors with two stable halves name the orbit by coset arithmetic on the halves and read
  * x from a copy in the order of those names (scratch from a stream-ordered pool of the
- * basis, taken and given back within the call); the others search (Alg. 2) and look the
- * index up in Limits.  Every y_i is written once.  Deterministic: the same call gives the
- * same bits.  Whole products and row ranges (ed_apply_H_rows) may sum a row's terms in
+ * basis, taken and given back within the call; narrow ranges and small sectors read x through
+ * the names' indices instead); the others search (Alg. 2) and look the index up in Limits.
+ * Every y_i is written once.  Deterministic: the same call gives the same bits, as long as
+ * device memory for the scratch is there (without it another kernel takes the call and may sum
+ * a row's terms in another order).  Whole products and row ranges (ed_apply_H_rows) may sum a row's terms in
  * different orders and differ in the last bit.
  *   J, Jz: HOST arrays [n_classes].
  *   x, y: DEVICE arrays of dim elements of `dtype` (ED_F64 or ED_F32; the complex types

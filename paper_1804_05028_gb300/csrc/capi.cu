@@ -51,7 +51,7 @@ cudaMemPool_t ed_shared_pool(int device) {
   return p;
 }
 
-cudaError_t ed_malloc(void **p, size_t bytes) {
+cudaError_t ed_malloc(void **p, size_t bytes, const ed_basis *B) {
   const cudaError_t e = cudaMalloc(p, bytes);
   if (e != cudaErrorMemoryAllocation) return e;
   cudaGetLastError();
@@ -59,6 +59,7 @@ cudaError_t ed_malloc(void **p, size_t bytes) {
   if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceSynchronize() == cudaSuccess) {
     cudaMemPool_t pool = ed_shared_pool(dev);
     if (pool) cudaMemPoolTrimTo(pool, 0);
+    if (B) ed_trim_pair(B);
   }
   return cudaMalloc(p, bytes);
 }
@@ -712,7 +713,7 @@ extern "C" int ed_apply_H_host(ed_basis *B, const double *J, const double *Jz, c
     if (B->d_stage_y) cudaFree(B->d_stage_y);
     B->d_stage_x = B->d_stage_y = nullptr;
     B->stage_bytes = 0;
-    if (ed_malloc(&B->d_stage_x, bytes) != cudaSuccess || ed_malloc(&B->d_stage_y, bytes) != cudaSuccess) {
+    if (ed_malloc(&B->d_stage_x, bytes, B) != cudaSuccess || ed_malloc(&B->d_stage_y, bytes, B) != cudaSuccess) {
       cudaGetLastError();
       return ed_fail(ED_ERR_OOM, "cannot allocate staging vectors");
     }
@@ -1031,7 +1032,7 @@ extern "C" int ed_lanczos(ed_basis *B, const double *J, const double *Jz,
   }
   for (int k = 0; k < 3 && !full; k++) {
     if (!own) { L.v[k] = (char *)o.work + k * bytes; continue; }
-    if (ed_malloc(&L.v[k], bytes) != cudaSuccess) {
+    if (ed_malloc(&L.v[k], bytes, B) != cudaSuccess) {
       cudaGetLastError();
       for (int q = 0; q < k; q++) cudaFree(L.v[q]);
       return ed_fail(ED_ERR_OOM, "cannot allocate Lanczos vectors");
@@ -1042,7 +1043,7 @@ extern "C" int ed_lanczos(ed_basis *B, const double *J, const double *Jz,
   if (o.dtype == ED_F32 || o.dtype == ED_C64) {
     if (!full && !own && o.work_bytes >= (int64_t)(4 * bytes)) {
       L.ylo = (char *)o.work + 3 * bytes;
-    } else if (ed_malloc(&L.ylo, bytes) == cudaSuccess) {
+    } else if (ed_malloc(&L.ylo, bytes, B) == cudaSuccess) {
       L.own_ylo = true;
     } else {
       cudaGetLastError();
@@ -1057,7 +1058,7 @@ extern "C" int ed_lanczos(ed_basis *B, const double *J, const double *Jz,
   L.nblk = (int)std::max<int64_t>(1, std::min<int64_t>(B->n_partial / 4, (B->D + 1023) / 1024));
   L.ro_coef_off = std::max((size_t)m_cap * P * ed_reorth_grid(B), (size_t)2 * P * L.nblk);
   L.coef_len = (size_t)m_cap * P;
-  if (ed_malloc(&L.d_ro, sizeof(double) * (L.ro_coef_off + 2 * L.coef_len + 8)) != cudaSuccess) {
+  if (ed_malloc(&L.d_ro, sizeof(double) * (L.ro_coef_off + 2 * L.coef_len + 8), B) != cudaSuccess) {
     cudaGetLastError();
     if (own) for (int k = 0; k < 3; k++) cudaFree(L.v[k]);
     if (L.own_ylo) cudaFree(L.ylo);

@@ -1135,6 +1135,10 @@ void ed_free_pair(ed_basis *B) {
   delete p;
 }
 
+void ed_trim_pair(const ed_basis *B) {
+  if (B->pair && B->pair->pool && B->pair->own_pool) cudaMemPoolTrimTo(B->pair->pool, 0);
+}
+
 namespace {
 
 // host tables gathered into one upload; at(k) is table k's place in it
@@ -1508,6 +1512,13 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
   const uint64_t cap = std::max<uint64_t>(4 * (uint64_t)B->D, 1u << 22);
   if (acc == 0 || acc > cap) { ed_free_pair(B); return ED_OK; }
   p->n_slots = (uint32_t)acc;
+  pair_rules::Plan room{true, true};
+  if (!pair_rules::always_fits((uint64_t)B->D, acc)) {
+    size_t free_bytes = 0, all = 0;
+    ED_CK(cudaMemGetInfo(&free_bytes, &all));
+    room = pair_rules::fits(free_bytes, (uint64_t)B->D, acc, B->is_real);
+    if (!room.pair) { ed_free_pair(B); return ED_OK; }
+  }
   // weights chi sqrt(t): index phase + denom * (number of t among the divisors of |G|)
   std::vector<uint8_t> tcode(ns + 1, 0);
   std::vector<int> divs;
@@ -1660,7 +1671,7 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
   Q.up_half = up_half;
   Q.idx = p->idx; Q.meta = p->meta; Q.any_weight = d_any;
   // the row order pays when xs outgrows the L2 and a class fills many warps
-  const bool want_rows = B->D >= kRowOrderMinDim && B->D / nA >= 256 && ubase + up.size() <= 1u << (kPosShift - kClassShift);
+  const bool want_rows = room.rows && B->D >= kRowOrderMinDim && B->D / nA >= 256 && ubase + up.size() <= 1u << (kPosShift - kClassShift);
   if (want_rows) Q.pat = (uint32_t *)sc.get(4 * (size_t)acc);   // null without memory: no row order
   int rc = blocks ? ed_launch_pair_slots(B, Q, st) : ED_ERR_UNSUPPORTED;
   if (rc == ED_ERR_UNSUPPORTED) {
@@ -1681,7 +1692,7 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
   // (a pool costs 0.2 ms, as much as the rest of their tables) take it from the device's shared one.
   const size_t first = 8 * ((size_t)p->n_slots + 1) + 256;
   p->own_pool = first > kSharedPoolMax;
-  if (p->own_pool) p->pool = ed_make_pool(B->device, ~0ull);
+  if (p->own_pool) p->pool = ed_make_pool(B->device, pair_rules::pool_keep(p->n_slots, B->is_real));
   else p->pool = ed_shared_pool(B->device);
   if (!p->pool) { ed_free_pair(B); return ED_OK; }
   // small sectors: the pool takes its first memory here rather than in the first product,
@@ -1691,7 +1702,7 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
     if (cudaMallocFromPoolAsync(&q, first, p->pool, st) == cudaSuccess) ED_CK(cudaFreeAsync(q, st));
     else cudaGetLastError();
   }
-  B->table_bytes += p->bytes;
+  B->table_bytes += p->bytes + (p->own_pool ? pair_rules::xs_most(p->n_slots, B->is_real) : 0);
   return ED_OK;
 }
 

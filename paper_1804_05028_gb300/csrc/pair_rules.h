@@ -52,4 +52,16 @@ inline Route route(int64_t rows, int64_t dim, double terms_per_row, uint64_t n_s
   return kExpanded;
 }
 
+// Device memory.  A plan is made where, beside it, there is still room for the vectors of a
+// Lanczos run and its ground state: the tables (6 bytes per slot) and one call's xs, then the row
+// order (10 bytes per state).  The pool of a basis keeps the xs of two calls in its widest type.
+struct Plan { bool pair, rows; };
+inline uint64_t xs_most(uint64_t n_slots, bool is_real) { return (is_real ? 8 : 16) * (n_slots + 1); }
+inline uint64_t pool_keep(uint64_t n_slots, bool is_real) { return 2 * xs_most(n_slots, is_real) + (16ull << 20); }
+inline Plan fits(uint64_t free_bytes, uint64_t dim, uint64_t n_slots, bool is_real) {
+  const uint64_t vectors = 4 * (is_real ? 8 : 16) * dim, pair = 6 * n_slots + xs_most(n_slots, is_real);
+  return {pair + vectors <= free_bytes, pair + 10 * dim + vectors <= free_bytes};
+}
+inline bool always_fits(uint64_t dim, uint64_t n_slots) { return 22 * n_slots + 10 * dim < (64ull << 20); }
+
 }  // namespace pair_rules

@@ -364,10 +364,13 @@ inline int ed_allow_smem(K k, size_t most) {
 // most 64 MB and gives the rest back.
 cudaMemPool_t ed_make_pool(int device, uint64_t keep);
 cudaMemPool_t ed_shared_pool(int device);
-// cudaMalloc; where that fails, once more after the shared pool has given back what it keeps
-cudaError_t ed_malloc(void **p, size_t bytes);
+// cudaMalloc; where that fails, once more after the shared pool and that of basis B (may be null)
+// have given back what they keep
+cudaError_t ed_malloc(void **p, size_t bytes, const ed_basis *B = nullptr);
 template <typename T>
-inline cudaError_t ed_malloc(T **p, size_t bytes) { return ed_malloc(reinterpret_cast<void **>(p), bytes); }
+inline cudaError_t ed_malloc(T **p, size_t bytes, const ed_basis *B = nullptr) {
+  return ed_malloc(reinterpret_cast<void **>(p), bytes, B);
+}
 
 // Stream-ordered scratch of the current device, given back in stream order when it goes out of
 // scope (on errors too).  From the shared pool: the device's default pool unmaps its memory at
@@ -445,6 +448,7 @@ int ed_launch_apply_fast(const ed_basis *B, const double *J, const double *Jz, c
 // ed_launch_apply_pair returns ED_ERR_UNSUPPORTED when the search kernels take the call
 int ed_build_pair(ed_basis *B, cudaStream_t st);
 void ed_free_pair(ed_basis *B);
+void ed_trim_pair(const ed_basis *B);   // its pool gives back what no call in flight holds
 // the ED_ROUTE_* of a product (mode 0) or of the class expectations (mode 1)
 int ed_pair_route(const ed_basis *B, int dtype, int64_t r0, int64_t r1, int mode);
 int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, const void *x, void *y,

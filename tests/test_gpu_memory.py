@@ -64,3 +64,37 @@ def test_pool_gives_way_to_a_build():
         B.apply_H(x, y)
         B.close()
     assert (y - ref).abs().max() <= 2e-6 * ref.abs().max()
+
+
+def test_plan_leaves_room_for_a_lanczos_run():
+    """The tables of coset arithmetic (140 MB here) are not made where the run's vectors would
+    then find no room: the sector is searched, as without them."""
+    p = w.square_torus(6, momentum=(0, 0), point_irrep=0, J2=0.5, n_sublat=4, n_up=12)
+    B = build(p)
+    i = B.info()
+    ref = B.lanczos(fixed_steps=3, seed=3)["E0"]
+    assert B.apply_route(torch.float64) == "slot order"
+    B.close()
+    with memory_left(i["basis_bytes"] + i["index_bytes"] + 190 * MB):
+        B = build(p)
+        route = B.apply_route(torch.float64)
+        e = B.lanczos(fixed_steps=3, seed=3)["E0"]
+        B.close()
+    assert route == "search" and abs(e - ref) <= 1e-12 * abs(ref)
+
+
+def test_pool_of_a_basis_is_bounded():
+    """Sixteen products in flight take sixteen times the scratch, of which two times stay."""
+    p = w.square_torus(6, momentum=(0, 0), point_irrep=0, J2=0.5, n_sublat=4, n_up=12)
+    B = build(p)
+    x = torch.rand(B.dim, dtype=torch.float64, device="cuda")
+    ys = [torch.empty_like(x) for _ in range(16)]
+    streams = [torch.cuda.Stream() for _ in ys]
+    B.apply_H(x, ys[0])
+    before = free_bytes()
+    for y, s in zip(ys, streams):
+        B.apply_H(x, y, stream=s)
+    held = before - free_bytes()
+    assert all(torch.equal(y, ys[0]) for y in ys)
+    assert held <= 2 * 8 * 2 * B.dim + 40 * MB      # slots: less than twice the states
+    B.close()

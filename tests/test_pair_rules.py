@@ -10,7 +10,7 @@ CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
 def run(tmp_path, body):
     """What a program made of the rules and `body` prints."""
     src, exe = tmp_path / "t.cpp", tmp_path / "t"
-    src.write_text('#include "pair_rules.h"\n#include <cstdio>\nusing namespace pair_rules;\n' + body)
+    src.write_text('#include "pair_rules.h"\n#include <cstdio>\n#include <initializer_list>\nusing namespace pair_rules;\n' + body)
     subprocess.run(["g++", "-std=c++17", "-O1", "-Wall", "-Werror", "-I", CSRC, str(src), "-o", str(exe)], check=True)
     return subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout
 
@@ -77,3 +77,17 @@ int main() {
 }
 """)
     assert out == "ss" + "dde" + "se" + "ee" + "de" + "dsse"
+
+
+def test_memory(tmp_path):
+    """A plan only beside the vectors of a Lanczos run; the pool's bound."""
+    out = run(tmp_path, """
+int main() {
+  const uint64_t D = 861602748, n = 920000000, GB = 1000000000;
+  for (uint64_t f : {264 * GB, 48 * GB, 41 * GB, 38 * GB}) printf("%d%d ", fits(f, D, n, true).pair, fits(f, D, n, true).rows);
+  const uint64_t E = 4200000000ull;      // 284 GB less 95 GB of basis and index
+  printf("%d %d%d ", fits(189 * GB, E, E, true).pair, always_fits(1000, 2000), always_fits(D, n));
+  printf("%d", pool_keep(n, true) <= 16 * n + (17u << 20) && pool_keep(n, false) <= 32 * n + (17u << 20));
+}
+""")
+    assert out == "11 10 10 00 0 10 1"
