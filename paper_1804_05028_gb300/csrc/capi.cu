@@ -870,7 +870,7 @@ int reorth_step(LanczosRun &L, int j, void *w, const void *v, const void *vprev,
   *n_b2 = ed_reorth_grid(B);
   for (int sw = 0; sw < 2; sw++) {
     double *c = L.d_ro + L.ro_coef_off + (size_t)sw * L.coef_len;
-    const int rc = ed_launch_reorth_sweep(B, w, L.store, nullptr, nullptr, j + 1, L.dtype, L.d_ro, c, L.st, L.ylo);
+    const int rc = ed_launch_reorth_sweep(B, w, L.store, j + 1, L.dtype, L.d_ro, c, L.st, L.ylo);
     if (rc) return rc;
     corr[sw] = c + (size_t)j * P;
   }

@@ -38,18 +38,16 @@ constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr int kGroup = 8;     // vectors per block of the multi-dot (blockIdx.y)
 
-// the m vectors: base + k * stride (a Krylov store), or the two explicit pointers p0, p1
+// the m vectors of a Krylov store: base + k * stride
 struct VecSet {
   const void *base;
   int64_t stride;
-  const void *p0, *p1;
   int m;
 };
 
 template <typename V>
 __device__ __forceinline__ const V *vec(const VecSet &S, int k) {
-  if (S.base) return reinterpret_cast<const V *>(S.base) + (size_t)k * (size_t)S.stride;
-  return reinterpret_cast<const V *>(k ? S.p1 : S.p0);
+  return reinterpret_cast<const V *>(S.base) + (size_t)k * (size_t)S.stride;
 }
 
 __device__ __forceinline__ double warp_sum(double d) {
@@ -443,16 +441,6 @@ __global__ void __launch_bounds__(kThreads) combine_kernel(VecSet S, const doubl
     default: return ed_fail(ED_ERR_INVALID, "unknown dtype");     \
   }
 
-VecSet make_set(const void *base, int64_t stride, const void *p0, const void *p1, int m) {
-  VecSet S;
-  S.base = base;
-  S.stride = stride;
-  S.p0 = p0;
-  S.p1 = p1;
-  S.m = m;
-  return S;
-}
-
 }  // namespace
 
 // 4 blocks per SM, fewer for short vectors: a thread then still has four rows, and the block
@@ -461,17 +449,15 @@ int ed_reorth_grid(const ed_basis *B) {
   return (int)std::max<int64_t>(1, std::min<int64_t>(4 * B->sm_count, (B->D + 4 * kThreads - 1) / (4 * kThreads)));
 }
 
-// One Gram-Schmidt sweep of w against m vectors (base + k * D, or p0 and p1 when base is
-// null): coefficients c (device, m * P doubles, P = 2 for complex) and ||w||^2 block
+// One Gram-Schmidt sweep of w against m vectors (base + k * D): coefficients c (device, m * P doubles, P = 2 for complex) and ||w||^2 block
 // partials in partial[0 .. grid).  partial must hold m * P * grid doubles.
-int ed_launch_reorth_sweep(const ed_basis *B, void *w, const void *base, const void *p0,
-                           const void *p1, int m, int dtype, double *partial, double *c,
-                           cudaStream_t st, void *wlo) {
+int ed_launch_reorth_sweep(const ed_basis *B, void *w, const void *base, int m, int dtype,
+                           double *partial, double *c, cudaStream_t st, void *wlo) {
   if (m <= 0) return ED_OK;
   const bool cplx = dtype == ED_C128 || dtype == ED_C64;
   const int P = cplx ? 2 : 1;
   const int grid = ed_reorth_grid(B);
-  const VecSet S = make_set(base, B->D, p0, p1, m);
+  const VecSet S{base, B->D, m};
   const size_t smem_upd = 2 * sizeof(double) * (size_t)m * P;   // fp64 + two fp32 words
   if (smem_upd > 48 * 1024) return ed_fail(ED_ERR_UNSUPPORTED, "too many vectors in one sweep");
   const dim3 dgrid(grid, (m + kGroup - 1) / kGroup);
@@ -501,7 +487,7 @@ int ed_launch_local_sweep(const ed_basis *B, void *w, const void *v, const void 
 // psi = sum_k s[k] (base + k * D), s a DEVICE array of m doubles.
 int ed_launch_combine(const ed_basis *B, void *psi, const void *base, int m, const double *s,
                       int dtype, cudaStream_t st) {
-  const VecSet S = make_set(base, B->D, nullptr, nullptr, m);
+  const VecSet S{base, B->D, m};
   const size_t smem = 2 * sizeof(double) * (size_t)m;
   constexpr size_t kMaxCombine = 200 * 1024;
   if (smem > kMaxCombine) return ed_fail(ED_ERR_UNSUPPORTED, "too many vectors to combine");
