@@ -31,7 +31,8 @@ struct BatchSector {
   int64_t D;
   int64_t item0;     // first work item of this sector
   // orbit tables (kOrbit): per configuration the rank of its orbit among those of its S^z,
-  // the minimising element and whether |Stab| > 1; basis index by rank (null: the rank itself);
+  // the minimising element and whether |Stab| > 1; basis index by rank where the irrep drops
+  // orbits (null: the rank itself);
   // chi per element, as signs for real sectors
   const uint32_t *otab, *jmap;
   void *xo;          // sectors with jmap: x by orbit rank, zeros where the irrep drops the orbit
@@ -246,7 +247,8 @@ __global__ void __launch_bounds__(256) expand_orbits(const BatchSector *sec, con
 // How a sector finds a term's index.  kSearch: any split, the block-wise search and the
 // Limits lookup.  kFull: every sector has a whole table (one sublattice), so the block-wise
 // search is not compiled in.  kOrbit: whole tables small enough for orbit tables (|G| <= 256,
-// fewer than 2^23 orbits per S^z, device memory for 4 bytes per configuration and group):
+// fewer than 2^23 orbits per S^z, device memory for 4 bytes per configuration and group and a
+// copy of x):
 // every term's accesses run through the L1 data pipe, which bounds this kernel, so a 4-byte
 // entry with the orbit's rank replaces the 8-byte one, the prefix rank and the 16-byte record
 // of the ranked Limits; chi is one load (signs: bits of the warp's sector descriptor), and where
@@ -286,10 +288,9 @@ __global__ void __launch_bounds__(kBatchThreads, kLook != kSearch ? (K <= 4 ? 6 
     }
     // what every term reads of the descriptor, in registers: a shared-memory read each would
     // take a quarter of the data pipe
-    const uint32_t *otab = S.otab, *jmap = S.jmap;
+    const uint32_t *otab = S.otab;
     const float2 *chi = S.chi;
-    const void *xv = kLook == kOrbit && S.xo ? S.xo : S.x;
-    if (kLook == kOrbit && S.xo) jmap = nullptr;   // the rank itself is the row of xo
+    const void *xv = kLook == kOrbit && S.xo ? S.xo : S.x;   // either way the rank is the row
     const bool cplx = S.cplx != 0;
     for (int64_t i = (item - S.item0) * P.rows_per_item + lane;
          i < S.D && i < (item - S.item0 + 1) * P.rows_per_item; i += 32) {
@@ -321,14 +322,10 @@ __global__ void __launch_bounds__(kBatchThreads, kLook != kSearch ? (K <= 4 ? 6 
             bool neg = false;
             if constexpr (kLook == kOrbit) {
               const uint32_t e = __ldg(otab + s2);
-              uint32_t o = e & ((1u << kOrbitBits) - 1u);
-              if (jmap) {
-                o = __ldg(jmap + o);
-                if (o == 0xFFFFFFFFu) continue;
-              }
+              const uint32_t o = e & ((1u << kOrbitBits) - 1u);
               j = o;
               if (e >> 31) {   // rare
-                const uint32_t jt = S.xo ? __ldg(S.jmap + o) : o;
+                const uint32_t jt = S.jmap ? __ldg(S.jmap + o) : o;
                 if (jt != 0xFFFFFFFFu) w *= __ldg(S.sqrt_f + __ldg(S.I.stab + jt));
               }
               const uint32_t g = (e >> kOrbitBits) & 0xFFu;
@@ -583,7 +580,7 @@ int build_orbits(ed_batch *Bt) {
   if ((maps && !d_maps) || (!chi.empty() && !d_chi)) { drop(); return ED_OK; }
   if (maps) ED_CK(cudaMemset(d_maps, 0xFF, 4 * maps));
   if (!chi.empty()) ED_CK(cudaMemcpy(d_chi, chi.data(), 8 * chi.size(), cudaMemcpyHostToDevice));
-  // xo, where it fits: rows of k entries, each sector's block 32-byte aligned
+  // xo: rows of k entries, each sector's block 32-byte aligned
   std::vector<uint32_t> map_at, map_sec;
   std::vector<size_t> xo_at(Bt->n, 0);
   size_t xo_floats = 0;
@@ -595,15 +592,16 @@ int build_orbits(ed_batch *Bt) {
       xo_floats += (orbits(s) * Bt->k * (Bt->host[s].cplx ? 2 : 1) + 7) / 8 * 8;
     }
   float *d_xo = nullptr;
-  if (maps && maps < (1ull << 32) && (d_xo = (float *)get(4 * xo_floats)) != nullptr &&
-      (Bt->d_map_at = (uint32_t *)get(8 * map_at.size())) != nullptr) {
-    Bt->d_map_sec = Bt->d_map_at + map_at.size();
+  if (maps) {
+    d_xo = (float *)get(4 * xo_floats);
+    uint32_t *d_at = (uint32_t *)get(8 * map_at.size());
+    if (!d_xo || !d_at || maps >= 1ull << 32) { drop(); return ED_OK; }
+    Bt->d_map_at = d_at;
+    Bt->d_map_sec = d_at + map_at.size();
     ED_CK(cudaMemcpy(Bt->d_map_at, map_at.data(), 4 * map_at.size(), cudaMemcpyHostToDevice));
     ED_CK(cudaMemcpy(Bt->d_map_sec, map_sec.data(), 4 * map_sec.size(), cudaMemcpyHostToDevice));
     Bt->n_map_sec = (uint32_t)map_at.size();
     Bt->n_maps = maps;
-  } else {
-    d_xo = nullptr;
   }
   for (int s = 0; s < Bt->n; s++) {
     const ed_basis *B = Bt->bases[s];
@@ -613,7 +611,7 @@ int build_orbits(ed_batch *Bt) {
     S.xo = nullptr;
     if (orbits(s) != (size_t)B->D) {
       S.jmap = d_maps + at[s];
-      if (d_xo) S.xo = d_xo + xo_at[s];
+      S.xo = d_xo + xo_at[s];
       if (B->D > 0) {
         orbit_index<<<(int)std::min<int64_t>((B->D + 255) / 256, grid), 256>>>(B->d_basis, B->D, S.otab, d_maps + at[s]);
         ED_CK(cudaGetLastError());

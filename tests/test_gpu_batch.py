@@ -150,6 +150,32 @@ def test_batched_sublattice_sectors(k):
     bt.close()
 
 
+@pytest.mark.parametrize("k", [1, 2, 4, 8])
+def test_whole_tables_without_orbit_tables(k):
+    """Nine sites in one block: whole tables too small for orbit tables (fewer than 1024
+    configurations), looked up through the ranked Limits; every S^z and momentum of the 3x3
+    torus against the oracle's explicit matrix."""
+    import paper_1804_05028_gb300 as ed
+    T = w.square_torus
+    probs = [T(3, momentum=m, point_irrep=i, J2=0.4, n_sublat=1, n_up=u) for u in (1, 4, 5, 7)
+             for m in ((0, 0), (1, 0), (1, 2)) for i in range(w.n_point_irreps((3, 0), (0, 3), m))]
+    bases = ed.build_sectors(probs)
+    g = torch.Generator(device="cuda").manual_seed(11)
+    xs = [torch.randn(B.dim * k, dtype=torch.float32 if B.is_real else torch.complex64, device="cuda", generator=g) for B in bases]
+    ys = [torch.full_like(x, float("nan")) for x in xs]
+    bt = ed.Batch(bases, k=k)
+    bt.set_vectors(xs, ys)
+    bt.apply()
+    torch.cuda.synchronize()
+    for p, B, x, y in zip(probs, bases, xs, ys):
+        if B.dim == 0:
+            continue
+        H, _, _ = oracle.hamiltonian(p)
+        ref = H @ x.view(B.dim, k).cpu().numpy().astype(np.complex128)
+        assert np.abs(y.view(B.dim, k).cpu().numpy() - ref).max() <= 2e-6 * max(np.abs(ref).max(), 1.0)
+    bt.close()
+
+
 def test_whole_table_batch_against_oracle(sectors):
     """The whole-table batched kernel (the variant the 572-sector launch runs) against the
     oracle's stored matrix directly, every column of every block width, on four sectors:
