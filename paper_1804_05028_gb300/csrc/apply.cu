@@ -509,16 +509,16 @@ static size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
 
 int ed_launch_apply(const ed_basis *B, const double *J, const double *Jz, const void *x,
                     void *y, int dtype, int64_t r0, int64_t r1, double *partial,
-                    cudaStream_t st, int mode, void *ylo) {
+                    cudaStream_t st, int mode, void *ylo, int *n_blocks) {
   if (r1 <= r0) return ED_OK;
   {  // coset arithmetic where the sector has a plan and the call is large enough for it
     bool done = false;
-    const int rc = ed_launch_apply_pair(B, J, Jz, x, y, dtype, r0, r1, partial, st, mode, ylo, &done);
+    const int rc = ed_launch_apply_pair(B, J, Jz, x, y, dtype, r0, r1, partial, st, mode, ylo, &done, n_blocks);
     if (rc != ED_ERR_UNSUPPORTED) return rc;
   }
   {  // the specialised two-level kernels first; the generic kernel serves what they cannot
     bool done = false;
-    const int rc = ed_launch_apply_fast(B, J, Jz, x, y, dtype, r0, r1, partial, st, mode, ylo, &done);
+    const int rc = ed_launch_apply_fast(B, J, Jz, x, y, dtype, r0, r1, partial, st, mode, ylo, &done, n_blocks);
     if (rc != ED_ERR_UNSUPPORTED) {
       if (!rc && ylo && !done)
         ED_CK(cudaMemsetAsync(ylo, 0, (size_t)(r1 - r0) * (dtype == ED_C64 ? 8 : 4), st));
@@ -575,7 +575,7 @@ int ed_launch_apply(const ed_basis *B, const double *J, const double *Jz, const 
   // fixed grid: a whole number of CTAs per SM, grid-stride over rows
   const int grid = grid_for(B, r1 - r0, 8);
   if (partial && grid > B->n_partial / 2) return ed_fail(ED_ERR_INVALID, "partial buffer too small");
-  B->last_apply_grid = grid;
+  if (n_blocks) *n_blocks = grid;
   const bool sg = P.stage_tables != 0;
   if (mode == 1) {
     if (!partial || B->n_classes * grid > B->n_partial) return ed_fail(ED_ERR_INVALID, "partial buffer too small");

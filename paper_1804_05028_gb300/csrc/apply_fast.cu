@@ -1111,7 +1111,7 @@ int launch_tile_v(const TwoParams &P, bool e2, int nsub, int grid, cudaStream_t 
 // |G| <= 4096); returns ED_ERR_UNSUPPORTED otherwise (the caller uses the generic kernel).
 int ed_launch_apply_fast(const ed_basis *B, const double *J, const double *Jz, const void *x,
                          void *y, int dtype, int64_t r0, int64_t r1, double *partial,
-                         cudaStream_t st, int mode, void *ylo, bool *ylo_done) {
+                         cudaStream_t st, int mode, void *ylo, bool *ylo_done, int *n_blocks) {
   TwoParams P;
   bool e2 = true;
   int rc = make_params(B, J, Jz, e2, P);
@@ -1137,7 +1137,7 @@ int ed_launch_apply_fast(const ed_basis *B, const double *J, const double *Jz, c
       if (need < grid) grid = (int)need;
       if (grid < 1) grid = 1;
       if (partial && grid > B->n_partial / 2) return ed_fail(ED_ERR_INVALID, "partial buffer too small");
-      B->last_apply_grid = grid;
+      if (n_blocks) *n_blocks = grid;
       switch (dtype) {
         case ED_F32: return launch_tile_v<float>(Q, qe2, B->nsub, grid, st);
         case ED_C64: return launch_tile_v<float2>(Q, qe2, B->nsub, grid, st);
@@ -1154,7 +1154,7 @@ int ed_launch_apply_fast(const ed_basis *B, const double *J, const double *Jz, c
   if (need < grid) grid = (int)need;
   if (grid < 1) grid = 1;
   if (partial && grid > B->n_partial / 2) return ed_fail(ED_ERR_INVALID, "partial buffer too small");
-  B->last_apply_grid = grid;
+  if (n_blocks) *n_blocks = grid;
   if (mode == 1) {
     if (!partial || B->n_classes * grid > B->n_partial) return ed_fail(ED_ERR_INVALID, "partial buffer too small");
     switch (dtype) {

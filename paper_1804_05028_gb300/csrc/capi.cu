@@ -809,8 +809,8 @@ extern "C" int ed_expect_classes(ed_basis *B, const double *Jz, const void *x, i
   if (!x) return ed_fail(ED_ERR_INVALID, "null vector");
   cudaStream_t st = (cudaStream_t)stream;
   std::vector<double> unit(B->n_classes, 1.0);
-  if ((rc = ed_launch_apply(B, unit.data(), Jz, x, nullptr, dtype, 0, B->D, B->d_partial, st, 1))) return rc;
-  const int g = B->last_apply_grid;
+  int g = 0;
+  if ((rc = ed_launch_apply(B, unit.data(), Jz, x, nullptr, dtype, 0, B->D, B->d_partial, st, 1, nullptr, &g))) return rc;
   ED_CK(cudaMemcpyAsync(B->h_partial, B->d_partial, (size_t)B->n_classes * g * 8,
                         cudaMemcpyDeviceToHost, st));
   ED_CK(cudaStreamSynchronize(st));
@@ -916,12 +916,12 @@ int lanczos_pass(LanczosRun &L, const ed_lanczos_opts *o, int max_steps, bool fi
       }
     }
     ED_CK(cudaEventRecord(e0, L.st));
-    if ((rc = ed_launch_apply(B, L.J, L.Jz, v, w, L.dtype, 0, B->D, B->d_partial, L.st, 0, L.ylo))) return rc;
+    int n_dot = 0;
+    if ((rc = ed_launch_apply(B, L.J, L.Jz, v, w, L.dtype, 0, B->D, B->d_partial, L.st, 0, L.ylo, &n_dot))) return rc;
     ED_CK(cudaEventRecord(e1, L.st));
     const double bprev = j ? beta[j - 1] : 0.0;
     // alpha_j stays on the device until the step's scalars are read: the update sums the
     // product's partials (its own go behind them)
-    const int n_dot = B->last_apply_grid;
     double *part2 = B->d_partial + B->n_partial / 2;
     if ((rc = ed_launch_axpy_norm(B, w, v, j ? vprev : nullptr, replay ? alpha_rec[j] : 0.0, bprev, L.dtype, part2, nblk,
                                   L.st, L.ylo, replay ? nullptr : B->d_partial, n_dot, L.d_scalar,
@@ -1101,9 +1101,10 @@ extern "C" int ed_lanczos(ed_basis *B, const double *J, const double *Jz,
       rc = ed_launch_dot(B, o.psi, o.psi, o.dtype, B->d_partial, nblk, L.st);
       if (!rc) rc = reduce_partials(B, B->d_partial, nblk, L.cplx, L.st, &nn, &im);
       if (!rc) rc = ed_launch_scale(B, o.psi, 1.0 / std::sqrt(nn), o.dtype, L.st);
-      if (!rc) rc = ed_launch_apply(B, J, Jz, o.psi, scratch, o.dtype, 0, B->D, B->d_partial, L.st);
+      int n_dot = 0;
+      if (!rc) rc = ed_launch_apply(B, J, Jz, o.psi, scratch, o.dtype, 0, B->D, B->d_partial, L.st, 0, nullptr, &n_dot);
       double rq = 0;
-      if (!rc) rc = reduce_partials(B, B->d_partial, B->last_apply_grid, L.cplx, L.st, &rq, nullptr);
+      if (!rc) rc = reduce_partials(B, B->d_partial, n_dot, L.cplx, L.st, &rq, nullptr);
       res->rq = rq;
     }
   }

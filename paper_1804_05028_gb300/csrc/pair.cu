@@ -1721,7 +1721,7 @@ int launch_expand(const ed_basis *B, const PairParams &P, cudaStream_t st) {
 }
 
 template <typename V, bool kChi, bool kFlips, int kMode>
-int launch_pair_t(const ed_basis *B, PairParams &P, bool rows, cudaStream_t st) {
+int launch_pair_t(const ed_basis *B, PairParams &P, bool rows, cudaStream_t st, int *n_blocks) {
   auto k = rows ? pair_rows_kernel<V, kChi, kFlips, kMode>
                 : P.xs ? pair_kernel<V, kChi, kFlips, kMode, false> : pair_kernel<V, kChi, kFlips, kMode, true>;
   const int threads = rows ? kRowThreads : kThreads, per_sm = rows ? kRowBlocks : kMinBlocks;
@@ -1735,7 +1735,7 @@ int launch_pair_t(const ed_basis *B, PairParams &P, bool rows, cudaStream_t st) 
     const int pct = std::min(100, (need * 100 + 228 * 1024 - 1) / (228 * 1024));
     ED_CK(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, pct));
   }
-  B->last_apply_grid = grid;
+  if (n_blocks) *n_blocks = grid;
   k<<<grid, threads, P.smem_bytes, st>>>(P);
   ED_CK(cudaGetLastError());
   if (rows && P.partial) {
@@ -1746,17 +1746,18 @@ int launch_pair_t(const ed_basis *B, PairParams &P, bool rows, cudaStream_t st) 
 }
 
 template <typename V, int kMode>
-int launch_pair_m(const ed_basis *B, PairParams &P, bool chi, bool flips, bool rows, cudaStream_t st) {
+int launch_pair_m(const ed_basis *B, PairParams &P, bool chi, bool flips, bool rows, cudaStream_t st, int *n_blocks) {
   if constexpr (Pv<V>::cplx) {
     if (chi)
-      return flips ? launch_pair_t<V, true, true, kMode>(B, P, rows, st) : launch_pair_t<V, true, false, kMode>(B, P, rows, st);
+      return flips ? launch_pair_t<V, true, true, kMode>(B, P, rows, st, n_blocks) : launch_pair_t<V, true, false, kMode>(B, P, rows, st, n_blocks);
   }
-  return flips ? launch_pair_t<V, false, true, kMode>(B, P, rows, st) : launch_pair_t<V, false, false, kMode>(B, P, rows, st);
+  return flips ? launch_pair_t<V, false, true, kMode>(B, P, rows, st, n_blocks) : launch_pair_t<V, false, false, kMode>(B, P, rows, st, n_blocks);
 }
 
 template <typename V>
-int launch_pair_v(const ed_basis *B, PairParams &P, bool chi, bool flips, bool rows, int mode, cudaStream_t st) {
-  return mode == 1 ? launch_pair_m<V, 1>(B, P, chi, flips, rows, st) : launch_pair_m<V, 0>(B, P, chi, flips, rows, st);
+int launch_pair_v(const ed_basis *B, PairParams &P, bool chi, bool flips, bool rows, int mode, cudaStream_t st,
+                  int *n_blocks) {
+  return mode == 1 ? launch_pair_m<V, 1>(B, P, chi, flips, rows, st, n_blocks) : launch_pair_m<V, 0>(B, P, chi, flips, rows, st, n_blocks);
 }
 
 // Shared memory of a block, as offsets in P and in bytes.
@@ -1808,7 +1809,7 @@ int ed_pair_route(const ed_basis *B, int dtype, int64_t r0, int64_t r1, int mode
 
 int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, const void *x, void *y,
                          int dtype, int64_t r0, int64_t r1, double *partial, cudaStream_t st, int mode,
-                         void *ylo, bool *ylo_done) {
+                         void *ylo, bool *ylo_done, int *n_blocks) {
   const PairPlan *p = B->pair;
   int route = ed_pair_route(B, dtype, r0, r1, mode);
   if (route == ED_ROUTE_SEARCH) return ED_ERR_UNSUPPORTED;
@@ -1879,7 +1880,7 @@ int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, c
 #define PCASE(D, V)                                                     \
   case D:                                                               \
     rc = ws ? launch_expand<V>(B, P, st) : ED_OK;                       \
-    if (!rc) rc = launch_pair_v<V>(B, P, chi, p->flips, rows, mode, st); \
+    if (!rc) rc = launch_pair_v<V>(B, P, chi, p->flips, rows, mode, st, n_blocks); \
     break;
     PCASE(ED_F64, double)
     PCASE(ED_F32, float)

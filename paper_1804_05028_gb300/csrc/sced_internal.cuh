@@ -329,7 +329,6 @@ struct ed_basis {
   // scratch
   double *d_partial = nullptr;
   int n_partial = 0;
-  mutable int last_apply_grid = 0;     // grid of the last product (number of dot partials)
   double *h_partial = nullptr;   // pinned
   void *d_stage_x = nullptr, *d_stage_y = nullptr;
   size_t stage_bytes = 0;
@@ -409,9 +408,11 @@ int ed_build_device(ed_basis *B, cudaStream_t st, int bucket_target);
 // ylo (fp32 / complex fp32 vectors only, may be null): receives the remainder of rounding
 // each y_i to fp32, so that y + ylo holds the product to about 48 bits; zeroed when the
 // kernel that runs cannot produce it
+// n_blocks (may be null): the number of blocks, that is of partials per sum; not kept in the basis,
+// where another thread's product could change it
 int ed_launch_apply(const ed_basis *B, const double *J, const double *Jz, const void *x, void *y,
                     int dtype, int64_t r0, int64_t r1, double *partial, cudaStream_t st,
-                    int mode = 0, void *ylo = nullptr);
+                    int mode = 0, void *ylo = nullptr, int *n_blocks = nullptr);
 int ed_launch_find_rep(const ed_basis *B, const uint64_t *states, int64_t n, uint64_t *rep,
                        int32_t *sym, int32_t *phase, int32_t *stab, int64_t *index,
                        cudaStream_t st);
@@ -443,7 +444,7 @@ int ed_launch_axpy(const ed_basis *B, void *y, const void *x, double a, int dtyp
 int ed_launch_start(const ed_basis *B, void *v, uint64_t seed, int dtype, cudaStream_t st);
 int ed_launch_apply_fast(const ed_basis *B, const double *J, const double *Jz, const void *x,
                          void *y, int dtype, int64_t r0, int64_t r1, double *partial,
-                         cudaStream_t st, int mode, void *ylo = nullptr, bool *ylo_done = nullptr);
+                         cudaStream_t st, int mode, void *ylo, bool *ylo_done, int *n_blocks);
 // pair.cu: the coset-arithmetic product, its tables (built once per basis) and their release;
 // ed_launch_apply_pair returns ED_ERR_UNSUPPORTED when the search kernels take the call
 int ed_build_pair(ed_basis *B, cudaStream_t st);
@@ -453,7 +454,7 @@ void ed_trim_pair(const ed_basis *B);   // its pool gives back what no call in f
 int ed_pair_route(const ed_basis *B, int dtype, int64_t r0, int64_t r1, int mode);
 int ed_launch_apply_pair(const ed_basis *B, const double *J, const double *Jz, const void *x, void *y,
                          int dtype, int64_t r0, int64_t r1, double *partial, cudaStream_t st, int mode,
-                         void *ylo, bool *ylo_done);
+                         void *ylo, bool *ylo_done, int *n_blocks);
 // apply_fast.cu: representative, index and weight of every slot's configuration.  Slot p
 // belongs to the lower class c with start[c] <= p < start[c+1]; with r = p - start[c], the
 // upper class is first_up[c] + r / K and the element kel[r % K] carries its representative

@@ -292,3 +292,29 @@ def test_product_without_scratch():
     del hold
     torch.cuda.empty_cache()
     assert torch.equal(B.apply_H(x, z), y) and left <= 16 << 20
+
+
+def test_lanczos_beside_products_of_another_thread():
+    """A product on the same basis from another thread, over another number of blocks, does not
+    change how many block sums a Lanczos step adds up."""
+    import threading
+    B = _basis(w.chain(20, 2, k=0, n_up=10))
+    x = _vec(B.dim, torch.float64, 10)
+    ref = B.lanczos(fixed_steps=8, seed=2)
+    stop = threading.Event()
+
+    def narrow():
+        s = torch.cuda.Stream()
+        y = torch.empty(64, dtype=x.dtype, device="cuda")
+        while not stop.is_set():
+            B.apply_H_rows(x, 100, 164, y=y, stream=s)
+        s.synchronize()
+
+    t = threading.Thread(target=narrow)
+    t.start()
+    try:
+        runs = [B.lanczos(fixed_steps=8, seed=2) for _ in range(400)]
+    finally:
+        stop.set()
+        t.join()
+    assert all(np.array_equal(r["alpha"], ref["alpha"]) and np.array_equal(r["beta"], ref["beta"]) for r in runs)
