@@ -1153,7 +1153,9 @@ struct Blob {
   template <typename T> size_t add(const std::vector<T> &v) { return add(v.data(), v.size()); }
 };
 
-constexpr size_t kSharedPoolMax = (size_t)4 << 20;    // xs of fp64 vectors
+// xs of fp64 vectors that a pool shared with other bases serves: one of its own costs a build 0.1
+// ms, 5% of that of the 28-site chain (1.4e6 states, 11 MB)
+constexpr size_t kSharedPoolMax = (size_t)16 << 20;
 
 // Row order for large sectors (see pair_rows_kernel); p->n_slices stays 0 when it is not made.
 // pat: the pattern of the other half of every slot.
@@ -1689,7 +1691,7 @@ int ed_build_pair(ed_basis *B, cudaStream_t st) {
   if (Q.pat)
     if ((rc = build_rows(B, p, start, Q.start, Q.pat, st))) return rc;
   // The memory of xs: large sectors keep a pool of their own, gone with the basis; small ones
-  // (a pool costs 0.2 ms, as much as the rest of their tables) take it from the device's shared one.
+  // take it from the device's shared one.
   const size_t first = 8 * ((size_t)p->n_slots + 1) + 256;
   p->own_pool = first > kSharedPoolMax;
   if (p->own_pool) p->pool = ed_make_pool(B->device, pair_rules::pool_keep(p->n_slots, B->is_real));
@@ -1796,7 +1798,7 @@ int ed_pair_route(const ed_basis *B, int dtype, int64_t r0, int64_t r1, int mode
   if (!p || r1 <= r0) return ED_ROUTE_SEARCH;
   const bool cplx = dtype == ED_C128 || dtype == ED_C64, chi = cplx && !B->is_real;
   const pair_rules::Route way = pair_rules::route(r1 - r0, B->D, B->terms_per_row, p->n_slots, dtype == ED_C128,
-                                                  B->T.full && mode == 0 && !B->is_real && dtype == ED_C64);
+                                                  B->T.full && B->N <= 22 && mode == 0 && !B->is_real && dtype == ED_C64);
   PairParams P{};
   if (way == pair_rules::kSearch || pair_layout(B, cplx, chi, false, P) > kPairMaxSmem) return ED_ROUTE_SEARCH;
   if (way == pair_rules::kDirect) return ED_ROUTE_DIRECT;

@@ -32,11 +32,13 @@ enum Route {
 //   6.4e7 states c64, D/1024 rows 253 / 90 / 399, D/128 856 / 522 / 563, D/9 9712 / 11004 / 4084
 //   810 states fp64, all rows 31 / 12 / 15; 9252 states 45 / 14 / 15
 // so directly up to one term per four slots, and on sectors so small that the second launch
-// outweighs the reads: up to 2^14 slots and some fifteen terms per row (497 states c64 45 / 14 / 16),
-// but not in complex fp64 (497 states 58 / 21 / 17), whose products wait for the weights.
-// One-block splits read a term's representative from a whole table, and in complex fp32, where
-// coset arithmetic multiplies twice by a character, small sectors of few terms are done sooner
-// so: 9225 states 16.5 / 18 / 19 (fp32 17 / 12 / 15), class expectations 43 / 42.5 / 43.5.
+// outweighs the reads: up to 2^14 slots and some fifteen terms per row (497 states c64 45 / 14 / 16).
+// Complex fp64 multiplies each by its weight in the fp64 pipe and gains on the smallest only (168
+// states 25 / 12 / 14, 497 states 58 / 21 / 17; 66 states of 13 terms 195 / 21 / 21).
+// One-block splits read a term's representative from a whole table.  Where that stays in L2 (up to
+// 22 sites), small sectors of few terms are done sooner so in complex fp32, where coset arithmetic
+// multiplies twice by a character: 20 sites, 9225 states 16.5 / 18 / 19 (fp32 17 / 12 / 15); 26
+// sites, 8844 states 20 / 16 / 17.
 // At 8.6e8 states every read is a DRAM sector and the search is as fast for narrow ranges
 // (us, D/4096 rows 238 / 298 / 17384, D/9 82 / 145 / 77 ms).  Fewer rows than half a warp leave
 // both kernels waiting for one memory access after the other (775 states c64, 8 rows 12 / 12 / 15).
@@ -48,7 +50,8 @@ inline Route route(int64_t rows, int64_t dim, double terms_per_row, uint64_t n_s
   if (table_complex_fp32 && n_slots <= 1u << 14 && terms_per_row <= 11.0) return kSearch;
   if (dim > kMaxDirectDim) return rows >= dim / 8 ? kExpanded : kSearch;
   if ((double)rows * terms_per_row <= 0.25 * (double)n_slots) return kDirect;
-  if (n_slots <= 1u << 14 && terms_per_row <= 15.0 && !complex_fp64) return kDirect;
+  if (n_slots > 1u << 14) return kExpanded;
+  if (complex_fp64 ? terms_per_row <= 11.0 && (double)rows * terms_per_row <= 1500.0 : terms_per_row <= 15.0) return kDirect;
   return kExpanded;
 }
 

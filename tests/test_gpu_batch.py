@@ -152,8 +152,8 @@ def test_batched_sublattice_sectors(k):
 
 @pytest.mark.parametrize("k", [1, 2, 4, 8])
 def test_whole_tables_without_orbit_tables(k):
-    """Nine sites in one block: whole tables too small for orbit tables (fewer than 1024
-    configurations), looked up through the ranked Limits; every S^z and momentum of the 3x3
+    """Nine sites in one block: whole tables without orbit tables (fewer than 1024 configurations
+    and, in all, states), looked up through the ranked Limits; every S^z and momentum of the 3x3
     torus against the oracle's explicit matrix."""
     import paper_1804_05028_gb300 as ed
     T = w.square_torus

@@ -70,13 +70,14 @@ int main() {
   q(15, 15, 5, 20); q(15, 1 << 20, 10, 1 << 20);                         // less than half a warp
   q(16, 16, 5, 20); q(810, 810, 8.5, 1100); q(810, 810, 8.5, 1100, true);   // small sectors
   q(810, 810, 8.5, 1100, false, true); q(153, 153, 17, 300, false, true);   // one block, complex fp32
+  q(168, 168, 6.6, 300, true); q(66, 66, 13, 130, true); q(300, 300, 6, 600, true);   // complex fp64
   q(153, 153, 17, 300); q(16384, 16384, 10, 16385);
   q(250000, 10000000, 10, 10000000); q(250001, 10000000, 10, 10000000);      // a term per four slots
   const int64_t big = 1ll << 27;
   q(16, big, 40, big); q(16, big + 8, 40, big); q(big / 8, big + 8, 40, big); q(big / 8 + 1, big + 8, 40, big);
 }
 """)
-    assert out == "ss" + "dde" + "se" + "ee" + "de" + "dsse"
+    assert out == "ss" + "dde" + "se" + "dee" + "ee" + "de" + "dsse"
 
 
 def test_memory(tmp_path):
