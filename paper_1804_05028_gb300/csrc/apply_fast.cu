@@ -1,7 +1,8 @@
 // apply_fast.cu -- the row-pull product y = H x with a two-level representative search.  It
 // serves the sectors and calls that the coset-arithmetic product (pair.cu) does not take:
-// splits without two stable halves, tables or scratch that do not fit, and narrow ranges of
-// rows (the rule in ed_launch_apply); and it finds the representatives of that product's slots.
+// splits without two stable halves, tables or memory that do not fit, fewer than 16 rows, and
+// narrow ranges of the largest sectors (pair_rules.h); and it finds the representatives of that
+// product's slots.
 //
 // Two-level search.  In Alg. 2 of arXiv:1804.05028 the candidates of a minimal block Y
 // are Sym_Y(s_Y) = K_R h: the coset of the stabiliser K_R = {k in G_0 : k R = R} of

@@ -21,7 +21,8 @@
 // The product first expands x into xs (one streaming pass over the slots: xs = chi(h2)
 // sqrt(|Stab_j|) x_j, j the basis index and h2 the element that carry the slot's
 // configuration to its representative, tabulated once per basis), then every row sums
-// chi(h) xs[slot] over its antiparallel bonds.
+// chi(h) xs[slot] over its antiparallel bonds.  Where that pass would outweigh the rows
+// (pair_rules.h), a term reads the slot's index, its weight and x instead.
 //
 // Several slots may hold the same orbit: a lower class with a nontrivial stabiliser lists
 // every image of the upper pattern, an upper class with one lists the same pattern under
