@@ -264,6 +264,7 @@ __global__ void __launch_bounds__(kBatchThreads, kLook != kSearch ? (K <= 4 ? 6 
   // so no warp waits at a block-wide barrier for another warp's rows
   __shared__ BatchSector S_w[kBatchThreads / 32];
   using State = typename std::conditional<kLook == kSearch, uint64_t, uint32_t>::type;   // N <= 26 otherwise
+  using Row = typename std::conditional<kLook == kOrbit, uint32_t, int64_t>::type;   // a rank has 23 bits
   __shared__ State bond_s[ED_MAXBONDS / 8];   // the two bits a bond's exchange flips
   const int nb = P.cls_off[P.n_classes];
   for (int q = threadIdx.x; q < nb; q += blockDim.x)
@@ -292,8 +293,8 @@ __global__ void __launch_bounds__(kBatchThreads, kLook != kSearch ? (K <= 4 ? 6 
     const float2 *chi = S.chi;
     const void *xv = kLook == kOrbit && S.xo ? S.xo : S.x;   // either way the rank is the row
     const bool cplx = S.cplx != 0;
-    for (int64_t i = (item - S.item0) * P.rows_per_item + lane;
-         i < S.D && i < (item - S.item0 + 1) * P.rows_per_item; i += 32) {
+    const Row r0 = (Row)((item - S.item0) * P.rows_per_item), r1 = min((Row)S.D, (Row)(r0 + P.rows_per_item));
+    for (Row i = r0 + lane; i < r1; i += 32) {
       const State s = (State)__ldcs(reinterpret_cast<const unsigned long long *>(S.I.basis) + i);
       const int ti = __ldcs(S.I.stab + i);
       float yr[K], yi[K];
@@ -317,7 +318,7 @@ __global__ void __launch_bounds__(kBatchThreads, kLook != kSearch ? (K <= 4 ? 6 
             const int b = b0 + __ffs(am) - 1;
             am &= am - 1;
             const State s2 = s ^ bond_s[b];
-            int64_t j;
+            Row j;
             float w = jh, cr = 0.f, ci = 0.f;
             bool neg = false;
             if constexpr (kLook == kOrbit) {
